@@ -72,10 +72,6 @@ struct hann_ctx {
     // plaintexts encoded and transformed per launch group: small enough that the group's intermediates stay in L2
     int encode_group = 1 << 20;
     int host_limbs = 0;  // limbs of every score polynomial that hann_score_level_host downloads (L: all)
-    // key-switch lift launches of at most this many CTAs (after the split) are cut along their targets: 160 keeps it to the
-    // ModDown lifts of a single item; hann_rotate_sum raises it to 320 for levels of one or two blocks, whose launches
-    // otherwise leave most of the machine idle
-    int lift_split_ctas = 160;
     // debugging aid: guards behind every workspace sub-buffer (see Arena in api.cu), filled when carved, checked on request
     int canaries = 0;
     std::vector<u64*> guards;

@@ -573,7 +573,15 @@ __global__ void __launch_bounds__(kThreads, AR::kMinBlocks) k_ntt_inv_a(NttArgs 
 // Both the digit decomposition (ModUp) and ModDown take a polynomial back to coefficients, lift every coefficient to a
 // centred integer and re-reduce it into other moduli, whose forward transforms follow.  The last inverse round leaves a
 // thread with rows g + G1*e of its column -- exactly the words the first forward round needs -- so the lift and pass A of
-// all target transforms run from registers; the coefficient-domain polynomials never travel to memory.
+// all target transforms run from there; the coefficient-domain polynomials never travel to memory.
+//
+// A CTA is 128 threads on C = 128 >> R2 adjacent columns.  The sixteen centred coefficients of a thread wait in shared
+// memory between the targets (every thread reads back only what it wrote), which leaves 96 registers per thread and five
+// independent CTAs per SM (six spill and lose 2 %): the kernel is a chain of short rounds with a CTA-wide exchange between
+// them, and its bound is the latency of that chain unless enough of them run side by side.  A binary64 coefficient enters a
+// binary64 target as it is; only the 60-bit special prime costs integer work, and its rounds are rolled (fwd_round4_smem).
+// Sum of the launches of a pass, against CTAs of 256 threads with the coefficients in registers and a Barrett reduction per
+// target: 493 -> 382 us (seven blocks, N = 2^16, L = 4), 5.18 -> 2.89 ms (membership circuit, N = 2^15, L = 12).
 
 struct LiftArgs {
     u64* src;             // source polynomials after inverse pass B' (private format of their modulus)
@@ -587,71 +595,141 @@ struct LiftArgs {
     const LimbConst* lt;
 };
 
+constexpr int kLiftThreads = 128;
+#ifndef HANN_LIFT_MINBLOCKS
+#define HANN_LIFT_MINBLOCKS 5
+#endif
+
+// word of (row, column) in the exchange tile: with eight columns the rows of two groups would meet in the same banks
+template <int R2>
+__device__ __forceinline__ int lift_word(int row, int c) {
+    constexpr int logC = 7 - R2;
+    return (row << logC) + c + (R2 == 4 ? (row >> 4) << 3 : 0);
+}
+
+// the centred coefficients of a source polynomial: balanced binary64 integers (class 0) or signed integers (class 2)
+__device__ __forceinline__ u64 lift_centred(const ArithF64& ar, double x, const LimbConst*) {
+    return (u64)__double_as_longlong(ar.reduce(ar.mulmod(ar.reduce(x), ar.ninv)));
+}
+__device__ __forceinline__ u64 lift_centred(const ArithInt<false>& ar, u64 x, const LimbConst* lc) {
+    const u64 v = ar.scaled_output(x, ar.ninv);
+    return v > lc->half ? v - ar.q : v;
+}
+
 template <int R1, int R2, class AR>
-__device__ __forceinline__ void lift_inverse(const LiftArgs& A, const AR ar, const typename AR::TW* __restrict__ tw, const u64* __restrict__ base,
-                                             u64* __restrict__ sm, int g, int c, bool active, u64 (&v)[1 << R1]) {
-    constexpr int G1 = 1 << R2, G2 = 1 << R1;
+__device__ __forceinline__ void lift_inverse(const AR ar, const LimbConst* lc, const typename AR::TW* __restrict__ tw,
+                                             const u64* __restrict__ base, u64* __restrict__ sm, u64* __restrict__ vs, int g, int c) {
+    constexpr int G1 = 1 << R2, G2 = 1 << R1, logC = 7 - R2, C = 1 << logC;
     constexpr int RR2 = R2 == 0 ? 1 : R2;
-    const typename AR::TW ninv = ar.ninv;
     if (R2 != 0) {
-        for (int w = threadIdx.x; w < (G2 << 4); w += blockDim.x) {
-            const int cc = w & 15, gg = w >> 4;
+#pragma unroll
+        for (int w = threadIdx.x; w < (G2 << logC); w += kLiftThreads) {
+            const int cc = w & (C - 1), gg = w >> logC;
             typename AR::T x[1 << RR2];
 #pragma unroll
             for (int e = 0; e < (1 << RR2); e++) x[e] = ar.from_mid(base[(size_t)((gg << RR2) + e) * 256 + cc]);
             inv_round<RR2>(ar, x, tw, (unsigned)(G2 + gg));
 #pragma unroll
-            for (int e = 0; e < (1 << RR2); e++) sm[(((gg << RR2) + e) << 4) + cc] = ar.to_mid(x[e]);
+            for (int e = 0; e < (1 << RR2); e++) sm[lift_word<R2>((gg << RR2) + e, cc)] = ar.to_mid(x[e]);
         }
         __syncthreads();
     }
-    if (active) {
-        typename AR::T x[1 << R1];
+    typename AR::T x[1 << R1];
 #pragma unroll
-        for (int e = 0; e < (1 << R1); e++) x[e] = ar.from_mid(R2 == 0 ? base[(size_t)(g + G1 * e) * 256 + c] : sm[((g + G1 * e) << 4) + c]);
-        inv_round<R1>(ar, x, tw, 1u);
+    for (int e = 0; e < (1 << R1); e++) x[e] = ar.from_mid(R2 == 0 ? base[(size_t)(g + G1 * e) * 256 + c] : sm[lift_word<R2>(g + G1 * e, c)]);
+    inv_round<R1>(ar, x, tw, 1u);
 #pragma unroll
-        for (int e = 0; e < (1 << R1); e++) v[e] = ar.scaled_output(x[e], ninv);
+    for (int e = 0; e < (1 << R1); e++) vs[e * kLiftThreads] = lift_centred(ar, x[e], lc);
+}
+
+// the same for the integer class, its rounds of four stages in place in the exchange tile (see fwd_round4_smem)
+template <int R1, int R2>
+__device__ __forceinline__ void lift_inverse_int(const ArithInt<false> ar, const LimbConst* lc, const ulonglong2* __restrict__ tw,
+                                                 const u64* __restrict__ base, u64* __restrict__ sm, u64* __restrict__ vs, int g, int c) {
+    if constexpr (R1 == 4) {
+        constexpr int G1 = 1 << R2, logC = 7 - R2, C = 1 << logC;
+        if constexpr (R2 == 4) {
+            const auto word = [=](int e) { return sm + lift_word<R2>((g << 4) + e, c); };
+#pragma unroll 4
+            for (int e = 0; e < 16; e++) *word(e) = base[(size_t)((g << 4) + e) * 256 + c];
+            inv_round4_smem(ar, word, tw, (unsigned)(16 + g));
+        } else if constexpr (R2 > 0) {
+#pragma unroll 1
+            for (int w = threadIdx.x; w < (16 << logC); w += kLiftThreads) {
+                const int cc = w & (C - 1), gg = w >> logC;
+                u64 x[1 << R2];
+#pragma unroll
+                for (int e = 0; e < (1 << R2); e++) x[e] = base[(size_t)((gg << R2) + e) * 256 + cc];
+                inv_round<R2>(ar, x, tw, (unsigned)(16 + gg));
+#pragma unroll
+                for (int e = 0; e < (1 << R2); e++) sm[lift_word<R2>((gg << R2) + e, cc)] = x[e];
+            }
+        } else {
+#pragma unroll 4
+            for (int e = 0; e < 16; e++) sm[lift_word<R2>(e, c)] = base[(size_t)e * 256 + c];
+        }
+        if (R2 != 0) __syncthreads();
+        const auto word = [=](int e) { return sm + lift_word<R2>(g + G1 * e, c); };
+        inv_round4_smem(ar, word, tw, 1u);
+#pragma unroll 2
+        for (int e = 0; e < 16; e++) vs[e * kLiftThreads] = lift_centred(ar, *word(e), lc);
+    } else {
+        lift_inverse<R1, R2>(ar, lc, tw, base, sm, vs, g, c);
     }
 }
 
-__device__ __forceinline__ double lifted_value(const ArithF64& ar, u64 r, bool neg, u64 q) {
-    const double d = ar.from_canonical(r);
-    return neg ? -d : d;
-}
-template <bool S>
-__device__ __forceinline__ u64 lifted_value(const ArithInt<S>&, u64 r, bool neg, u64 q) { return (neg && r) ? q - r : r; }
+// a centred coefficient as input of a target's forward rounds.  SRC: arithmetic class of the source (0: a balanced binary64
+// integer, else a signed 64-bit integer).
+template <int SRC>
+struct Lifted {
+    bool same, fold;
+    // binary64 targets take values up to 0.53 q as they are (the bounds of ntt.cu then reach 7.62 q after eight stages);
+    // `fold`: the source modulus is too large for that against this target's
+    __device__ __forceinline__ double operator()(const ArithF64& ar, u64 v, const LimbConst*) const {
+        if (SRC == 0) {
+            const double x = __longlong_as_double((long long)v);
+            return fold ? ar.reduce(x) : x;
+        }
+        // quotient below 2^51 rounded on the FP64 pipe, remainder exact modulo 2^64
+        const long long s = (long long)v;
+        const long long k = __double_as_longlong(__fma_rn((double)s, ar.qinv, ArithF64::kRound)) - 0x4338000000000000LL;
+        const long long r = s - k * ar.qi;
+        return __dsub_rn(__longlong_as_double(r + 0x4338000000000000LL), ArithF64::kRound);
+    }
+    template <bool S>
+    __device__ __forceinline__ u64 operator()(const ArithInt<S>& ar, u64 v, const LimbConst* lc) const {
+        long long s = (long long)v;
+        if (SRC == 0) s = __double_as_longlong(__dadd_rn(__longlong_as_double((long long)v), ArithF64::kRound)) - 0x4338000000000000LL;
+        if (SRC == 0 || same) return (u64)(s + ((s >> 63) & (long long)ar.q));  // |s| < 2^49 < q, or already centred modulo q
+        return reduce_signed(s, *lc);
+    }
+};
 
-template <int R1, int R2, class AR>
-__device__ __forceinline__ void lift_forward(const AR ar, const LimbConst* lc, bool same_modulus, const typename AR::TW* __restrict__ tw,
-                                             u64* __restrict__ base, u64* __restrict__ sm, int g, int c, bool active,
-                                             const u64 (&v)[1 << R1], u64 src_q, u64 src_half) {
-    constexpr int G1 = 1 << R2, G2 = 1 << R1;
+template <int R1, int R2, class AR, class LIFT>
+__device__ __forceinline__ void lift_forward(const AR ar, const LimbConst* lc, const LIFT lift, const typename AR::TW* __restrict__ tw,
+                                             u64* __restrict__ base, u64* __restrict__ sm, const u64* __restrict__ vs, int g, int c) {
+    constexpr int G1 = 1 << R2, G2 = 1 << R1, logC = 7 - R2, C = 1 << logC;
     constexpr int RR2 = R2 == 0 ? 1 : R2;
-    if (active) {
+    {
         typename AR::T x[1 << R1];
 #pragma unroll
-        for (int e = 0; e < (1 << R1); e++) {
-            // centred lift of the coefficient (sign and magnitude), reduced into this modulus
-            const bool neg = v[e] > src_half;
-            const u64 mag = neg ? src_q - v[e] : v[e];
-            x[e] = same_modulus ? ar.from_canonical(v[e]) : lifted_value(ar, barrett64(mag, *lc), neg, lc->q);
-        }
+        for (int e = 0; e < (1 << R1); e++) x[e] = lift(ar, vs[e * kLiftThreads], lc);
         fwd_round<R1, AR, R1>(ar, x, tw, 1u);
 #pragma unroll
         for (int e = 0; e < (1 << R1); e++) {
             if (R2 == 0) base[(size_t)(g + G1 * e) * 256 + c] = ar.to_mid(x[e]);
-            else sm[((g + G1 * e) << 4) + c] = ar.to_mid(x[e]);
+            else sm[lift_word<R2>(g + G1 * e, c)] = ar.to_exch(x[e]);
         }
     }
     if (R2 != 0) {
         __syncthreads();
-        for (int w = threadIdx.x; w < (G2 << 4); w += blockDim.x) {
-            const int cc = w & 15, gg = w >> 4;
+#pragma unroll
+        for (int w = threadIdx.x; w < (G2 << logC); w += kLiftThreads) {
+            const int cc = w & (C - 1), gg = w >> logC;
             typename AR::T x[1 << RR2];
 #pragma unroll
-            for (int e = 0; e < (1 << RR2); e++) x[e] = ar.from_mid(sm[(((gg << RR2) + e) << 4) + cc]);
-            fwd_round<RR2, AR, RR2>(ar, x, tw, (unsigned)(G2 + gg));
+            for (int e = 0; e < (1 << RR2); e++) x[e] = ar.from_mid(sm[lift_word<R2>((gg << RR2) + e, cc)]);
+            fwd_round<RR2, AR, 5 - R1>(ar, x, tw, (unsigned)(G2 + gg));
 #pragma unroll
             for (int e = 0; e < (1 << RR2); e++) base[(size_t)((gg << RR2) + e) * 256 + cc] = ar.to_mid(x[e]);
         }
@@ -659,43 +737,92 @@ __device__ __forceinline__ void lift_forward(const AR ar, const LimbConst* lc, b
     }
 }
 
-template <int R1, int R2>
-__global__ void __launch_bounds__(256, 2) k_ks_lift(LiftArgs A) {
-    extern __shared__ u64 sm[];
-    constexpr int G1 = 1 << R2;
-    const int N = 1 << A.logN;
-    const long long sp = blockIdx.y;
-    const int c0 = blockIdx.x << 4;
-    const int c = threadIdx.x & 15, g = threadIdx.x >> 4;
-    const bool active = g < G1;
-    const int sl = (int)((A.src_limb4 >> (4 * (sp % A.src_period))) & 15);
-    const LimbConst* slc = A.lt + sl;
-    const u64* sbase = A.src + sp * A.src_stride + c0;
-    u64 v[1 << R1];
-    if (slc->q < (1ULL << 50)) {
-        const ArithF64 ar(slc);
-        lift_inverse<R1, R2>(A, ar, (const double2*)A.tw_inv_f64 + ((size_t)sl << A.logN), sbase, sm, g, c, active, v);
+// integer targets, their rounds of four stages in place in the exchange tile
+template <int R1, int R2, class AR, class LIFT>
+__device__ __forceinline__ void lift_forward_int(const AR ar, const LimbConst* lc, const LIFT lift, const ulonglong2* __restrict__ tw,
+                                                 u64* __restrict__ base, u64* __restrict__ sm, const u64* __restrict__ vs, int g, int c) {
+    if constexpr (R1 == 4) {
+        constexpr int G1 = 1 << R2, logC = 7 - R2, C = 1 << logC;
+        const auto first = [=](int e) { return sm + lift_word<R2>(g + G1 * e, c); };
+#pragma unroll 2
+        for (int e = 0; e < 16; e++) *first(e) = lift(ar, vs[e * kLiftThreads], lc);
+        fwd_round4_smem(ar, first, tw, 1u);
+        if (R2 != 0) __syncthreads();
+        if constexpr (R2 == 4) {
+            const auto second = [=](int e) { return sm + lift_word<R2>((g << 4) + e, c); };
+            fwd_round4_smem(ar, second, tw, (unsigned)(16 + g));
+#pragma unroll 4
+            for (int e = 0; e < 16; e++) base[(size_t)((g << 4) + e) * 256 + c] = *second(e);
+        } else if constexpr (R2 > 0) {
+#pragma unroll 1
+            for (int w = threadIdx.x; w < (16 << logC); w += kLiftThreads) {
+                const int cc = w & (C - 1), gg = w >> logC;
+                u64 x[1 << R2];
+#pragma unroll
+                for (int e = 0; e < (1 << R2); e++) x[e] = sm[lift_word<R2>((gg << R2) + e, cc)];
+                fwd_round<R2>(ar, x, tw, (unsigned)(16 + gg));
+#pragma unroll
+                for (int e = 0; e < (1 << R2); e++) base[(size_t)((gg << R2) + e) * 256 + cc] = x[e];
+            }
+        } else {
+#pragma unroll 4
+            for (int e = 0; e < 16; e++) base[(size_t)e * 256 + c] = *first(e);
+        }
+        if (R2 != 0) __syncthreads();  // the exchange tile is free for the next target
     } else {
-        const ArithInt<false> ar(slc);
-        lift_inverse<R1, R2>(A, ar, (const ulonglong2*)A.tw_inv_int + ((size_t)sl << A.logN), sbase, sm, g, c, active, v);
+        lift_forward<R1, R2>(ar, lc, lift, tw, base, sm, vs, g, c);
     }
-    if (R2 != 0) __syncthreads();  // every thread is done with the exchange tile of the inverse rounds
+}
+
+template <int R1, int R2, int SRC>
+__device__ __forceinline__ void lift_targets(const LiftArgs& A, int sl, long long sp, int c0, u64* sm, const u64* vs, int g, int c) {
+    const int N = 1 << A.logN;
+    const u64 src_q = A.lt[sl].q;
     // a launch too small to fill the machine is cut along the targets as well: gridDim.z CTAs repeat the inverse rounds and
     // share out the targets, which shortens the chain one CTA runs
     for (int ti = blockIdx.z; ti < A.n_tgt; ti += gridDim.z) {
         const int tl = A.tgt_limb0 + ti;
         const LimbConst* tlc = A.lt + tl;
+        const u64 q = tlc->q;
         u64* dbase = A.dst + (sp * A.n_tgt + ti) * (long long)N + c0;
-        if (tlc->q < (1ULL << 50)) {
+        Lifted<SRC> lift;
+        lift.same = tl == sl;
+        lift.fold = src_q > q + (q >> 5);
+        if (q < (1ULL << 50)) {
             const ArithF64 ar(tlc);
-            lift_forward<R1, R2>(ar, tlc, tl == sl, (const double2*)A.tw_fwd_f64 + ((size_t)tl << A.logN), dbase, sm, g, c, active, v, slc->q, slc->half);
-        } else if (tlc->q < (1ULL << 57)) {
+            lift_forward<R1, R2>(ar, tlc, lift, (const double2*)A.tw_fwd_f64 + ((size_t)tl << A.logN), dbase, sm, vs, g, c);
+        } else if (q < (1ULL << 57)) {
             const ArithInt<true> ar(tlc);
-            lift_forward<R1, R2>(ar, tlc, tl == sl, (const ulonglong2*)A.tw_fwd_int + ((size_t)tl << A.logN), dbase, sm, g, c, active, v, slc->q, slc->half);
+            lift_forward_int<R1, R2>(ar, tlc, lift, (const ulonglong2*)A.tw_fwd_int + ((size_t)tl << A.logN), dbase, sm, vs, g, c);
         } else {
             const ArithInt<false> ar(tlc);
-            lift_forward<R1, R2>(ar, tlc, tl == sl, (const ulonglong2*)A.tw_fwd_int + ((size_t)tl << A.logN), dbase, sm, g, c, active, v, slc->q, slc->half);
+            lift_forward_int<R1, R2>(ar, tlc, lift, (const ulonglong2*)A.tw_fwd_int + ((size_t)tl << A.logN), dbase, sm, vs, g, c);
         }
+    }
+}
+
+template <int R1, int R2>
+__global__ void __launch_bounds__(kLiftThreads, HANN_LIFT_MINBLOCKS) k_ks_lift(LiftArgs A) {
+    extern __shared__ u64 sm[];
+    constexpr int logC = 7 - R2, C = 1 << logC;
+    const long long sp = blockIdx.y;
+    const int c0 = blockIdx.x << logC;
+    const int c = threadIdx.x & (C - 1), g = threadIdx.x >> logC;
+    const int sl = (int)((A.src_limb4 >> (4 * (sp % A.src_period))) & 15);
+    const LimbConst* slc = A.lt + sl;
+    const u64* sbase = A.src + sp * A.src_stride + c0;
+    u64* vs = sm + threadIdx.x;                        // [2^R1][128]: the thread's centred coefficients
+    u64* tile = sm + (kLiftThreads << R1);             // exchange tile
+    if (slc->q < (1ULL << 50)) {
+        const ArithF64 ar(slc);
+        lift_inverse<R1, R2>(ar, slc, (const double2*)A.tw_inv_f64 + ((size_t)sl << A.logN), sbase, tile, vs, g, c);
+        if (R2 != 0) __syncthreads();  // every thread is done with the exchange tile of the inverse rounds
+        lift_targets<R1, R2, 0>(A, sl, sp, c0, tile, vs, g, c);
+    } else {
+        const ArithInt<false> ar(slc);
+        lift_inverse_int<R1, R2>(ar, slc, (const ulonglong2*)A.tw_inv_int + ((size_t)sl << A.logN), sbase, tile, vs, g, c);
+        if (R2 != 0) __syncthreads();
+        lift_targets<R1, R2, 2>(A, sl, sp, c0, tile, vs, g, c);
     }
 }
 
@@ -1010,6 +1137,22 @@ int launch_ntt_inv(hann_ctx* c, u64* data, int64_t npoly, int64_t stride, const 
 
 bool ks_lift_available(const hann_ctx* c) { return c->logN >= 9; }
 
+// CTAs that share out the targets of a tile: smallest (waves x rounds of a CTA, the inverse rounds counting as one target),
+// ties to fewer CTAs
+static int lift_zsplit(long ctas, int n_tgt) {
+    const long slots = 148 * HANN_LIFT_MINBLOCKS;
+    int zs = 1;
+    long best = -1;
+    for (int z = 1; z <= n_tgt; z++) {
+        const long cost = ((ctas * z + slots - 1) / slots) * (1 + (n_tgt + z - 1) / z);
+        if (best < 0 || cost < best) {
+            best = cost;
+            zs = z;
+        }
+    }
+    return zs;
+}
+
 // After inverse pass B' of the nsrc source polynomials (launch_ntt_inv_pass_b): finish their inverse transforms, lift the
 // coefficients (centred) into the n_tgt moduli tgt_limb0 .. and run pass A of the target transforms.  The caller finishes
 // with launch_ntt_fwd_pass_b over the targets.
@@ -1030,9 +1173,8 @@ int launch_ks_lift(hann_ctx* c, u64* src, int64_t src_stride, int64_t nsrc, cons
     A.tw_fwd_int = c->tw_fwd;
     A.tw_fwd_f64 = c->tw_fwd_f64;
     A.lt = c->lt_dev;
-    const int a = c->logN - 8;
-    const size_t smem = a > 4 ? (size_t)(1 << a) * 16 * 8 : 0;
-    const int threads = a >= 8 ? 256 : (a == 7 ? 128 : 64);
+    const int a = c->logN - 8, R1 = a < 4 ? a : 4, R2 = a - R1, tiles = 256 >> (7 - R2);
+    const size_t smem = (size_t)8 * (2 * (kLiftThreads << R1) + (R2 == 4 ? 128 : 0));
     for (int64_t s0 = 0; s0 < nsrc; s0 += 65535) {
         const int ns = (int)std::min<int64_t>(65535, nsrc - s0);
         // the source limb of polynomial s0 + y is nibble (s0 + y) % period: 65535 is not a multiple of every period, so shift
@@ -1042,8 +1184,7 @@ int launch_ks_lift(hann_ctx* c, u64* src, int64_t src_stride, int64_t nsrc, cons
         Ap.src_limb4 = 0;
         for (int i = 0; i < src_lm.period && i < 16; i++) Ap.src_limb4 |= (u64)src_lm.limb[(s0 + i) % src_lm.period] << (4 * i);
         KProf kp(c, KC_LIFT_DIGITS);
-        const int zsplit = (16L * ns * n_tgt <= c->lift_split_ctas) ? n_tgt : 1;  // see hann_ctx::lift_split_ctas
-        pick_lift(a)<<<dim3(16, ns, zsplit), threads, smem, c->stream>>>(Ap);
+        pick_lift(a)<<<dim3(tiles, ns, lift_zsplit((long)tiles * ns, n_tgt)), kLiftThreads, smem, c->stream>>>(Ap);
     }
     return check_launch(c, "ks_lift");
 }

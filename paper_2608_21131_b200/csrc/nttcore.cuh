@@ -192,6 +192,48 @@ __device__ __forceinline__ void inv_round_f(const AR& ar, typename AR::T (&x)[1 
     }
 }
 
+// A round of FOUR stages of the integer classes on sixteen words that stay in shared memory, four at a time: two stages per
+// quad, eight quads in a rolled loop.  Unrolled like the binary64 rounds, an integer round is about a thousand instructions that
+// a warp runs through once, and a launch of few CTAs then spends most of its time fetching them (ncu: "no instruction" was ten
+// of thirteen stall cycles of a two-polynomial ModDown lift).  word(e): address of word e; tw: the table entries of the round,
+// base as in fwd_round / inv_round.
+template <class AR, class WORD>
+__device__ __forceinline__ void fwd_round4_smem(const AR& ar, const WORD& word, const typename AR::TW* __restrict__ tw, unsigned base) {
+#pragma unroll 1
+    for (int it = 0; it < 8; it++) {
+        const int k = it & 3, e0 = it < 4 ? k : 4 * k, st = it < 4 ? 4 : 1;
+        const unsigned b = it < 4 ? base : 4 * base + k;
+        u64 x0 = *word(e0), x1 = *word(e0 + st), x2 = *word(e0 + 2 * st), x3 = *word(e0 + 3 * st);
+        const typename AR::TW w = tw[b], wa = tw[2 * b], wb = tw[2 * b + 1];
+        ar.fwd(x0, x2, w);
+        ar.fwd(x1, x3, w);
+        ar.fwd(x0, x1, wa);
+        ar.fwd(x2, x3, wb);
+        *word(e0) = x0;
+        *word(e0 + st) = x1;
+        *word(e0 + 2 * st) = x2;
+        *word(e0 + 3 * st) = x3;
+    }
+}
+template <class AR, class WORD>
+__device__ __forceinline__ void inv_round4_smem(const AR& ar, const WORD& word, const typename AR::TW* __restrict__ tw, unsigned base) {
+#pragma unroll 1
+    for (int it = 0; it < 8; it++) {
+        const int k = it & 3, e0 = it < 4 ? 4 * k : k, st = it < 4 ? 1 : 4;
+        const unsigned b = it < 4 ? 4 * base + k : base;
+        u64 x0 = *word(e0), x1 = *word(e0 + st), x2 = *word(e0 + 2 * st), x3 = *word(e0 + 3 * st);
+        const typename AR::TW w = tw[b], wa = tw[2 * b], wb = tw[2 * b + 1];
+        ar.inv(x0, x1, wa);
+        ar.inv(x2, x3, wb);
+        ar.inv(x0, x2, w);
+        ar.inv(x1, x3, w);
+        *word(e0) = x0;
+        *word(e0 + st) = x1;
+        *word(e0 + 2 * st) = x2;
+        *word(e0 + 3 * st) = x3;
+    }
+}
+
 template <int R2>
 __device__ __forceinline__ int pad(int pos) { return R2 == 0 ? pos : pos + (pos >> R2); }
 
