@@ -192,8 +192,10 @@ int upload_secret(hann_ctx* c, const int8_t* s_host, int nlimbs, int8_t* s8, u64
 // left to the caller because its sources and targets differ between the callers.
 // gather_src (optional): the polynomials to switch still lie at gather_src + item * gather_stride (L limbs each); they are
 // brought into c1c on the way (by the inverse pass itself where its bulk-copy kernel applies, by a strided copy otherwise).
+// leave_pass_b (rings of 2^10 points and more): pass B of the lifted polynomials is left to launch_ks_finish.
 int ks_digits_to_lifted(hann_ctx* c, u64* c1c, int64_t items, u64* digits, int64_t digit_stride, int rot0, int rot_inc,
-                        int64_t u_items, u64* u, u64* lifted, const u64* gather_src = nullptr, int64_t gather_stride = 0) {
+                        int64_t u_items, u64* u, u64* lifted, const u64* gather_src = nullptr, int64_t gather_stride = 0,
+                        bool leave_pass_b = false) {
     const int L = c->L, N = c->N;
     const int64_t LN = (int64_t)L * N;
     const bool fused_gather = gather_src && ks_lift_available(c) && ntt_inv_pass_b_gathers(c, gather_src, c1c) && (gather_stride & 1) == 0;
@@ -209,7 +211,7 @@ int ks_digits_to_lifted(hann_ctx* c, u64* c1c, int64_t items, u64* digits, int64
         RET(launch_ks_inner(c, digits, digit_stride, rot0, rot_inc, u_items, u));
         RET(launch_ntt_inv_pass_b(c, u + (int64_t)L * N, u_items * 2, (int64_t)(L + 1) * N, limbmap_single(L)));
         RET(launch_ks_lift(c, u + (int64_t)L * N, (int64_t)(L + 1) * N, u_items * 2, limbmap_single(L), lifted, L, 0));
-        RET(launch_ntt_fwd_pass_b(c, lifted, u_items * 2 * L, N, limbmap_q(c)));
+        if (!leave_pass_b) RET(launch_ntt_fwd_pass_b(c, lifted, u_items * 2 * L, N, limbmap_q(c)));
         return HANN_OK;
     }
     RET(launch_ntt_inv(c, c1c, items * L, N, limbmap_q(c)));
@@ -220,6 +222,31 @@ int ks_digits_to_lifted(hann_ctx* c, u64* c1c, int64_t items, u64* digits, int64
     RET(launch_ntt_inv(c, u + (int64_t)L * N, u_items * 2, (int64_t)(L + 1) * N, limbmap_single(L)));
     RET(launch_moddown_lift(c, u, u_items * 2, lifted));
     RET(launch_ntt_fwd(c, lifted, u_items * 2 * L, N, limbmap_q(c)));
+    return HANN_OK;
+}
+
+// The same round on rings of 2^10 points and more (ksfused.cu), with the sum over nz rotations taken before the ModDown: polynomial
+// (z, item) to switch lies at src + item * src_it + z * src_z (transform domain, L limbs; left as it is unless it is c1c itself, which
+// the inverse pass overwrites: then nz = 1) and goes under the key of rotation rot0 + z * rot_zinc.  The automorphism is applied to
+// the sums, so what is left to the caller is launch_ks_finish.  Buffers, in words: c1c nz * items * LN, digits nz * items * L * L1N,
+// u items * 2 L1N, lifted items * 2 LN.
+int ks_round_fused(hann_ctx* c, const u64* src, int64_t src_it, int64_t src_z, int64_t items, int nz, int rot0, int rot_zinc, u64* c1c, u64* digits,
+                   u64* u, u64* lifted) {
+    const int L = c->L, N = c->N;
+    const int64_t LN = (int64_t)L * N, L1N = (int64_t)(L + 1) * N;
+    const bool in_place = src == c1c;
+    if (in_place) {
+        RET(launch_ntt_inv_pass_b(c, c1c, items * L, N, limbmap_q(c)));
+    } else if (ntt_inv_pass_b_gathers(c, src, c1c) && ((src_it | src_z) & 1) == 0) {
+        RET(launch_ntt_inv_pass_b_from(c, src, src_it, c1c, nz * items * L, N, limbmap_q(c), items, src_z));
+    } else {
+        for (int z = 0; z < nz; z++) RET(launch_copy2d(c, c1c + z * items * LN, LN, src + z * src_z, src_it, LN, items));
+        RET(launch_ntt_inv_pass_b(c, c1c, nz * items * L, N, limbmap_q(c)));
+    }
+    // a digit's transform modulo its own prime is the polynomial that came in, where that still exists
+    RET(launch_ks_lift(c, c1c, N, nz * items * L, limbmap_q(c), digits, in_place ? L + 1 : L, 0, !in_place));
+    RET(launch_ks_apply(c, digits, in_place ? nullptr : src, src_it, src_z, items, nz, rot0, rot_zinc, u));
+    RET(launch_ks_lift(c, u + LN, L1N, items * 2, limbmap_single(L), lifted, L, 0));
     return HANN_OK;
 }
 
@@ -285,6 +312,14 @@ extern "C" int hann_ctx_create(const hann_params* prm, hann_ctx** out) {
         lc.ninv = hm::invmod((u64)N % q, q);
         lc.ninv_s = hm::shoup(lc.ninv, q);
         lc.half = q / 2;
+        lc.qd = (double)q;
+        lc.halfd = (double)lc.half;
+        lc.qinv = 1.0 / lc.qd;
+        {
+            const u64 c51 = (1ULL << 51) % q;
+            lc.c51_bal = c51 > lc.half ? -(double)(q - c51) : (double)c51;
+            lc.c51_q = lc.c51_bal / lc.qd;
+        }
         {
             const double nb = lc.ninv > q / 2 ? -(double)(q - lc.ninv) : (double)lc.ninv;
             lc.ninv_bal = nb;
@@ -294,8 +329,11 @@ extern "C" int hann_ctx_create(const hann_params* prm, hann_ctx** out) {
             lc.pmod = prm->p % q;
             lc.pinv = hm::invmod(lc.pmod, q);
             lc.pinv_s = hm::shoup(lc.pinv, q);
+            lc.pinv_bal = lc.pinv > q / 2 ? -(double)(q - lc.pinv) : (double)lc.pinv;
+            lc.pinv_q = lc.pinv_bal / (double)q;
         } else {
             lc.pmod = 0; lc.pinv = 0; lc.pinv_s = 0;
+            lc.pinv_bal = lc.pinv_q = 0;
         }
         const u64 psi = hm::find_psi(q, N), ipsi = hm::invmod(psi, q);
         pw[0] = ipw[0] = 1;
@@ -382,7 +420,7 @@ extern "C" int hann_ctx_create(const hann_params* prm, hann_ctx** out) {
     if (ok) ok = cudaEventCreateWithFlags(&c->prep_done, cudaEventDisableTiming) == cudaSuccess;
     if (ok) ok = ntt_configure(c) == HANN_OK;
     // a -DHANN_DEBUG build: the range checks of the kernels report through this context's error word
-    if (ok) ok = debug_bind_keyswitch(c->kflag) == 0 && debug_bind_project(c->kflag) == 0 && debug_bind_encode(c->kflag) == 0;
+    if (ok) ok = debug_bind_keyswitch(c->kflag) == 0 && debug_bind_project(c->kflag) == 0 && debug_bind_encode(c->kflag) == 0 && debug_bind_ksfused(c->kflag) == 0;
     if (ok) {
         // look up the built-in scratch of hann_keyswitch_static now, while this device is current, so that the request-time
         // call only reads a cached address (a failure here is reported by that call, not by context creation)
@@ -1079,8 +1117,10 @@ static int rotate_hoisted(hann_ctx* c, const char* who, const u64* ct, int rot0,
     u64* lifted = ar.take<u64>((int64_t)count * 2 * LN);
     if (!c1c || !digits || !u || !lifted) return fail(c, HANN_EWORKSPACE, (std::string(who) + ": workspace too small").c_str());
     // one digit set, count keys: item i uses rotation rot0 + i
-    RET(ks_digits_to_lifted(c, c1c, 1, digits, 0, rot0, 1, count, u, lifted, ct + LN, 2 * LN));
-    RET(launch_moddown_combine(c, u, lifted, count, rot0, 1, ct, 0, nullptr, 0, out, out + LN, ctw));
+    const bool fin = ks_fused_available(c);
+    RET(ks_digits_to_lifted(c, c1c, 1, digits, 0, rot0, 1, count, u, lifted, ct + LN, 2 * LN, fin));
+    if (fin) RET(launch_ks_finish(c, u, lifted, count, true, rot0, 1, 1, ct, 0, 0, nullptr, 0, out, out + LN, ctw));
+    else RET(launch_moddown_combine(c, u, lifted, count, rot0, 1, ct, 0, nullptr, 0, out, out + LN, ctw));
     return HANN_OK;
 }
 
@@ -1206,6 +1246,11 @@ extern "C" int hann_score_level_ctdb(hann_ctx* c, const void* baby_dev, const vo
         RET(launch_mac_ct(c, (const u64*)baby_dev, ctdb + i0 * c->B * ctw, ni, d));
         // relinearise: (d0 + ks0, d1 + ks1) with (ks0, ks1) the key switch of d2 under the key of s^2 ("rotation 0": no
         // automorphism)
+        if (ks_fused_available(c)) {
+            RET(ks_round_fused(c, d + 2 * LN, 3 * LN, 0, ni, 1, 0, 0, c1c, digits, u, lifted));
+            RET(launch_ks_finish(c, u, lifted, ni, false, 0, 0, 1, nullptr, 0, 0, d, 3 * LN, inner + i0 * ctw, inner + i0 * ctw + LN, ctw));
+            continue;
+        }
         RET(launch_copy2d(c, c1c, LN, d + 2 * LN, 3 * LN, LN, ni));
         RET(ks_digits_to_lifted(c, c1c, ni, digits, (int64_t)L * L1N, 0, 0, ni, u, lifted));
         RET(launch_moddown_combine(c, u, lifted, ni, 0, 0, nullptr, 0, d, 3 * LN, inner + i0 * ctw, inner + i0 * ctw + LN, ctw));
@@ -1243,6 +1288,11 @@ extern "C" int hann_multiply(hann_ctx* c, const void* a_dev, const void* b_dev, 
         const int64_t ni = std::min(ch, count - i0);
         RET(launch_mul_ct(c, a + i0 * ctw, b + i0 * ctw, ni, d));
         // relinearise: (d0 + ks0, d1 + ks1), (ks0, ks1) the key switch of d2 under the key of s^2 ("rotation 0")
+        if (ks_fused_available(c)) {
+            RET(ks_round_fused(c, d + 2 * LN, 3 * LN, 0, ni, 1, 0, 0, c1c, digits, u, lifted));
+            RET(launch_ks_finish(c, u, lifted, ni, false, 0, 0, 1, nullptr, 0, 0, d, 3 * LN, out + i0 * ctw, out + i0 * ctw + LN, ctw));
+            continue;
+        }
         RET(launch_copy2d(c, c1c, LN, d + 2 * LN, 3 * LN, LN, ni));
         RET(ks_digits_to_lifted(c, c1c, ni, digits, (int64_t)L * L1N, 0, 0, ni, u, lifted));
         RET(launch_moddown_combine(c, u, lifted, ni, 0, 0, nullptr, 0, d, 3 * LN, out + i0 * ctw, out + i0 * ctw + LN, ctw));
@@ -1267,6 +1317,7 @@ extern "C" int hann_rotate_sum(hann_ctx* c, const void* inner_dev, int64_t n_blo
     }
     if (!c->keytab_host[B]) return fail(c, HANN_ENOKEY, "hann_rotate_sum: the key of rotation B is not loaded");
     if (!ws || ((uintptr_t)ws & 255)) return fail(c, HANN_EWORKSPACE, "hann_rotate_sum: workspace missing or not 256-byte aligned");
+    const bool fused = ks_fused_available(c);
     // Horner over the giant steps for blocks [b_lo, b_hi), as many blocks per round as the given part of the workspace
     // holds, on the context's current stream
     auto run_range = [&](int64_t b_lo, int64_t b_hi, char* wsp, int64_t wsp_bytes) -> int {
@@ -1287,6 +1338,14 @@ extern "C" int hann_rotate_sum(hann_ctx* c, const void* inner_dev, int64_t n_blo
             for (int g = G - 2; g >= 0; g--) {
                 u64* out = (g % 2 == 0) ? score + b0 * ctw : tmp;
                 // c1 of every accumulator, still in the transform domain; the key-switch round takes it from there
+                if (fused) {
+                    RET(ks_round_fused(c, old + LN, old_stride, 0, nb, 1, B, 0, c1c, digits, u, lifted));
+                    RET(launch_ks_finish(c, u, lifted, nb, false, B, 0, 1, old, old_stride, 0, inner + (b0 * G + g) * ctw, (int64_t)G * ctw, out,
+                                         out + LN, ctw));
+                    old = out;
+                    old_stride = ctw;
+                    continue;
+                }
                 RET(ks_digits_to_lifted(c, c1c, nb, digits, (int64_t)L * L1N, B, 0, nb, u, lifted, old + LN, old_stride));
                 RET(launch_moddown_combine(c, u, lifted, nb, B, 0, old, old_stride, inner + (b0 * G + g) * ctw, (int64_t)G * ctw, out,
                                            out + LN, ctw));
@@ -1346,7 +1405,7 @@ extern "C" int hann_rotate_sum_lazy(hann_ctx* c, const void* inner_dev, int64_t 
     for (int g = 1; g < G; g++)
         if (!c->keytab_host[g * B]) return fail(c, HANN_ENOKEY, "hann_rotate_sum_lazy: the keys of rotations B, 2B, .., (G-1)B must be loaded");
     if (!ws || ((uintptr_t)ws & 255)) return fail(c, HANN_EWORKSPACE, "hann_rotate_sum_lazy: workspace missing or not 256-byte aligned");
-    const bool lift = ks_lift_available(c);
+    const bool lift = ks_lift_available(c), fused = ks_fused_available(c);
     // blocks [b_lo, b_hi), as many per round as the given part of the workspace holds, on the context's current stream
     auto run_range = [&](int64_t b_lo, int64_t b_hi, char* wsp, int64_t wsp_bytes) -> int {
         int64_t ch = (wsp_bytes - kSlack) / (lazy_block_words(c) * 8);
@@ -1362,14 +1421,22 @@ extern "C" int hann_rotate_sum_lazy(hann_ctx* c, const void* inner_dev, int64_t 
         if (!c1c || !digits || !u || !up || !lifted) return fail(c, HANN_EWORKSPACE, "hann_rotate_sum_lazy: workspace too small");
         for (int64_t b0 = b_lo; b0 < b_hi; b0 += ch) {
             const int64_t nb = std::min(ch, b_hi - b0), items = nb * (G - 1);
+            const u64* in0 = inner + b0 * G * ctw;
+            if (fused) {
+                // all giant steps summed under their own keys and automorphisms before one ModDown per block
+                RET(ks_round_fused(c, in0 + ctw + LN, (int64_t)G * ctw, ctw, nb, G - 1, B, B, c1c, digits, u, lifted));
+                RET(launch_ks_finish(c, u, lifted, nb, false, B, B, G - 1, in0 + ctw, (int64_t)G * ctw, ctw, in0, (int64_t)G * ctw, score + b0 * ctw,
+                                     score + b0 * ctw + LN, ctw));
+                continue;
+            }
             // c1 of term (g, blk), still in the transform domain, into c1c[(g - 1) * nb + blk]
             bool all_fused = lift;
             for (int g = 1; g < G; g++) {
                 const u64* src = inner + (b0 * G + g) * ctw + LN;
                 u64* dst = c1c + (int64_t)(g - 1) * nb * LN;
-                const bool fused = lift && ntt_inv_pass_b_gathers(c, src, dst);
-                all_fused = all_fused && fused;
-                if (fused) RET(launch_ntt_inv_pass_b_from(c, src, (int64_t)G * ctw, dst, nb * L, N, limbmap_q(c)));
+                const bool gathers = lift && ntt_inv_pass_b_gathers(c, src, dst);
+                all_fused = all_fused && gathers;
+                if (gathers) RET(launch_ntt_inv_pass_b_from(c, src, (int64_t)G * ctw, dst, nb * L, N, limbmap_q(c)));
                 else RET(launch_copy2d(c, dst, LN, src, (int64_t)G * ctw, LN, nb));
             }
             if (lift) {
@@ -1558,8 +1625,13 @@ extern "C" int hann_fold(hann_ctx* c, void* ct_dev, int stride, int steps, void*
     for (int t = 0; t < steps; t++) {
         const int r = stride << t;
         // nxt = cur + rot_r(cur): the Horner step of the rotate-and-sum with the ciphertext itself as the addend
-        RET(ks_digits_to_lifted(c, kb.c1c, 1, kb.digits, (int64_t)L * L1N, r, 0, 1, kb.u, kb.lifted, cur + LN, ctw));
-        RET(launch_moddown_combine(c, kb.u, kb.lifted, 1, r, 0, cur, ctw, cur, ctw, nxt, nxt + LN, ctw));
+        if (ks_fused_available(c)) {
+            RET(ks_round_fused(c, cur + LN, ctw, 0, 1, 1, r, 0, kb.c1c, kb.digits, kb.u, kb.lifted));
+            RET(launch_ks_finish(c, kb.u, kb.lifted, 1, false, r, 0, 1, cur, ctw, 0, cur, ctw, nxt, nxt + LN, ctw));
+        } else {
+            RET(ks_digits_to_lifted(c, kb.c1c, 1, kb.digits, (int64_t)L * L1N, r, 0, 1, kb.u, kb.lifted, cur + LN, ctw));
+            RET(launch_moddown_combine(c, kb.u, kb.lifted, 1, r, 0, cur, ctw, cur, ctw, nxt, nxt + LN, ctw));
+        }
         std::swap(cur, nxt);
     }
     if (cur != (u64*)ct_dev) RET(launch_copy2d(c, (u64*)ct_dev, ctw, cur, ctw, ctw, 1));
@@ -1634,6 +1706,10 @@ extern "C" int hann_keyswitch(hann_ctx* c, int rot, const void* poly_dev, void* 
     // the stored key is phi_k^{-1}(evk): switch phi_k^{-1}(d) and apply phi_k to the result
     const unsigned kinv = c->h_galois[(c->n - rot) % c->n];
     RET(launch_permute(c, (const u64*)poly_dev, c1c, L, kinv));
+    if (ks_fused_available(c)) {
+        RET(ks_round_fused(c, c1c, (int64_t)L * c->N, 0, 1, 1, rot, 0, c1c, digits, u, lifted));
+        return launch_ks_finish(c, u, lifted, 1, false, 0, 0, 1, nullptr, 0, 0, nullptr, 0, (u64*)ks0_dev, (u64*)ks1_dev, 0);
+    }
     RET(ks_digits_to_lifted(c, c1c, 1, digits, 0, rot, 0, 1, u, lifted));
     RET(launch_moddown_combine(c, u, lifted, 1, rot, 0, nullptr, 0, nullptr, 0, (u64*)ks0_dev, (u64*)ks1_dev, 0));
     return HANN_OK;

@@ -148,6 +148,7 @@ int launch_guard_verify(hann_ctx* c, u64* const* guards, int64_t count, unsigned
 int debug_bind_keyswitch(int* word);
 int debug_bind_project(int* word);
 int debug_bind_encode(int* word);
+int debug_bind_ksfused(int* word);
 
 // ---- launchers: each enqueues on ctx->stream, counts its launches and returns HANN_OK or HANN_ECUDA
 int check_launch(hann_ctx* c, const char* what);
@@ -162,10 +163,11 @@ int launch_copy2d(hann_ctx* c, u64* dst, int64_t dst_pitch, const u64* src, int6
 int launch_unpack_half(hann_ctx* c, const u64* half, int64_t npoly, u64* full);
 int launch_ntt_inv_pass_b(hann_ctx* c, u64* data, int64_t npoly, int64_t stride, const LimbMap& lm);
 bool ntt_inv_pass_b_gathers(const hann_ctx* c, const void* src, const void* dst);
-int launch_ntt_inv_pass_b_from(hann_ctx* c, const u64* src, int64_t src_gstride, u64* data, int64_t npoly, int64_t stride, const LimbMap& lm);
+int launch_ntt_inv_pass_b_from(hann_ctx* c, const u64* src, int64_t src_gstride, u64* data, int64_t npoly, int64_t stride, const LimbMap& lm,
+                               int64_t src_per = 0, int64_t src_zstride = 0);
 bool ks_lift_available(const hann_ctx* c);
 int launch_wait_selftest(hann_ctx* c, unsigned long long limit_ns, unsigned long long* waited_ns_dev);
-int launch_ks_lift(hann_ctx* c, u64* src, int64_t src_stride, int64_t nsrc, const LimbMap& src_lm, u64* dst, int n_tgt, int tgt_limb0);
+int launch_ks_lift(hann_ctx* c, u64* src, int64_t src_stride, int64_t nsrc, const LimbMap& src_lm, u64* dst, int n_tgt, int tgt_limb0, bool skip_own = false);
 // encode a block and run pass A of the transforms in one kernel when the parameters allow it (returns false if not)
 bool encode_fused_available(const hann_ctx* c);
 int launch_encode_rows_fused(hann_ctx* c, const float* rows, int64_t rows_in_block, int dim, int p_first, int count, u64* out,
@@ -195,6 +197,11 @@ int launch_mac_batch(hann_ctx* c, const u64* baby, int n_queries, const u64* pt,
 int launch_lift_digits(hann_ctx* c, const u64* src, int64_t src_stride, int64_t nitems, u64* digits);
 int launch_ks_inner(hann_ctx* c, const u64* digits, int64_t digit_stride, int rot0, int rot_inc, int64_t nitems, u64* u);
 int launch_moddown_lift(hann_ctx* c, const u64* u, int64_t npoly, u64* lifted);
+// fused key switch of rings of 2^10 points and more (ksfused.cu)
+bool ks_fused_available(const hann_ctx* c);
+int launch_ks_apply(hann_ctx* c, const u64* digits, const u64* own, int64_t own_it, int64_t own_z, int64_t items, int nz, int rot0, int rot_zinc, u64* u);
+int launch_ks_finish(hann_ctx* c, const u64* u, const u64* lifted, int64_t items, bool perm_items, int rot0, int rot_inc, int nz, const u64* c0,
+                     int64_t c0_it, int64_t c0_z, const u64* add, int64_t add_it, u64* out0, u64* out1, int64_t out_it);
 // lazy giant steps (items laid out giant step after giant step, see keyswitch.cu)
 int launch_ks_inner_batches(hann_ctx* c, const u64* digits, int64_t digit_stride, int rot0, int rot_zinc, int nz, int64_t per_z, u64* u);
 int launch_giant_sum_p(hann_ctx* c, const u64* u, int64_t nblk, u64* up);

@@ -1,0 +1,498 @@
+// Hybrid key switching on rings of 2^10 points and more, after the lift (ntt.cu): the second half of every digit's forward
+// transform, the product with the key and the sum over rotations in one kernel; the second half of the ModDown transforms and
+// the final combination in another.  Neither the transformed digits nor the transformed ModDown polynomials travel to memory.
+//
+// Positions.  A polynomial is stored in chunks of 256 words with their low nibbles swapped (see galois_src): word m = 16 b + a of
+// a chunk holds logical position 16 a + b.  Sixteen lanes (a half-warp) transform one chunk of one polynomial in two register
+// rounds; lane j holds logical positions j + 16 e in the first forward round and 16 j + e in the second.  In shared memory logical
+// position 16 a + b is kept at word 16 a + (b ^ a), which both rounds and the word-by-word passes reach without bank conflicts
+// (swz).  An automorphism maps every chunk of 256 positions onto one chunk, so a CTA that owns a chunk of the result reads
+// one chunk of every source and permutes inside it.
+#include "internal.h"
+#include "debugcheck.cuh"
+#include "nttcore.cuh"
+
+namespace {
+
+__device__ __forceinline__ int swz(int m) { return ((m & 15) << 4) | ((m >> 4) ^ (m & 15)); }
+
+// The words 16 e + j of a chunk (logical positions 16 j + e) under an automorphism: their sources share the chunk and the low nibble
+// of the word; the high nibble, bit-reversed, advances by k times the bit-reversed e.
+struct LaneSource {
+    int base;  // first word of the source chunk + the low nibble
+    unsigned t0, k;
+    __device__ __forceinline__ static int brev4(unsigned v) { return (int)((0xF7B3D591E6A2C480ULL >> (4 * v)) & 15); }
+    __device__ __forceinline__ LaneSource(int first, unsigned k_, int logN) : k(k_) {
+        const int s = galois_src(first, k_, logN, 1);
+        base = s & ~0xF0;
+        t0 = brev4((s >> 4) & 15);
+    }
+    __device__ __forceinline__ int high(int e) const { return brev4((t0 + brev4(e) * k) & 15); }
+    __device__ __forceinline__ int word(int e) const { return base + 16 * high(e); }
+};
+
+// table entries of a chunk's second pass (cbase = 2^a + chunk number) in the order of the two rounds: entries 0..14 for the first
+// round (broadcast to the lanes of a chunk), entry 16 (r + 1) + j, r = 2^u - 1 + il, for stage u of the second
+template <class TW>
+__device__ __forceinline__ void stage_twiddles(TW* __restrict__ tc, const TW* __restrict__ tw, unsigned cbase) {
+#pragma unroll 4
+    for (int e = threadIdx.x; e < 256; e += blockDim.x) {
+        const int r = e < 16 ? e : (e >> 4) - 1, u = 31 - __clz(r + 1), il = r + 1 - (1 << u);
+        const unsigned idx = e < 16 ? (cbase << u) + il : (cbase << (4 + u)) + ((e & 15) << u) + il;
+        if (r < 15) tc[e] = tw[idx];
+    }
+}
+
+// 16-byte asynchronous copies of the 2 L key chunks (256 words each, L1N words apart) of a modulus into shared memory
+__device__ __forceinline__ void stage_keys(u64* __restrict__ ks, const u64* __restrict__ key, long long L1N, int L) {
+    const unsigned dst = (unsigned)__cvta_generic_to_shared(ks);
+    for (int v = threadIdx.x; v < 2 * L * 128; v += blockDim.x) {
+        const u64* src = key + (long long)(v >> 7) * L1N + (v & 127) * 2;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + v * 16), "l"(src) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// the eight stages of a chunk: x[e] enters as word j + 16 e (pass-A format) and leaves as logical position 16 j + e, unreduced
+// (below 8q)
+__device__ __forceinline__ void chunk_forward(const ArithF64& ar, double (&x)[16], const double2* tc, u64* sb, int j, unsigned hmask) {
+    fwd_round_f<4, ArithF64, 4>(ar, x, [=](int st, int il) { return tc[(1 << st) - 1 + il]; });
+#pragma unroll
+    for (int e = 0; e < 16; e++) sb[16 * e + (j ^ e)] = ar.to_exch(x[e]);
+    __syncwarp(hmask);
+#pragma unroll
+    for (int e = 0; e < 16; e++) x[e] = ar.from_mid(sb[16 * j + (e ^ j)]);
+    fwd_round_f<4, ArithF64, 1>(ar, x, [=](int u, int il) { return tc[(((1 << u) + il) << 4) + j]; });
+}
+// the same in place for the integer classes, rolled (see fwd_round4_smem): x[e] enters at the word of position j + 16 e; canonical
+// residues at the words of the swizzled layout
+template <class AR>
+__device__ __forceinline__ void chunk_forward_int(const AR& ar, const ulonglong2* tc, u64* sb, int j, unsigned hmask) {
+    fwd_round4_staged(ar, [=](int e) { return sb + 16 * e + (j ^ e); }, tc, 1, 0);
+    __syncwarp(hmask);
+    const auto second = [=](int e) { return sb + 16 * j + (e ^ j); };
+    fwd_round4_staged(ar, second, tc + 16, 16, j);
+#pragma unroll 2
+    for (int e = 0; e < 16; e++) *second(e) = ar.to_canonical(*second(e));
+}
+
+struct ApplyArgs {
+    const u64* digits;  // pass-A output of digit (z, item, j) for modulus i: ((z * items + item) * L + j) * n_tgt + target of i
+    int n_tgt;          // L + 1 targets per digit, or L: a digit's own modulus is left out and read from `own`
+    const u64* own;     // the polynomials being switched, transform domain: own + item * own_it + z * own_z + j * N (or null)
+    long long own_it, own_z;
+    const u64* const* keytab;
+    const unsigned* galois;
+    int rot0, rot_zinc, nz;  // rotation of z
+    long long items;
+    u64* u;  // [item][2][L+1][N]: limbs below L canonical (below 2^50: balanced binary64 integers), the special prime's after its
+             // inverse pass B' (private format)
+    int N, logN, L;
+    const void *tw_fwd_f64, *tw_fwd_int, *tw_inv_f64, *tw_inv_int;
+    const LimbConst* lt;
+};
+
+// u[item][c][i] = sum over z of phi_z( sum_j digit(z, item, j) * key_z[j][c] )  modulo i, for chunk blockIdx.x of the result, modulus
+// i = L - blockIdx.y (the special prime, which has the longest chain, first) and IB items.  A half-warp transforms one digit's
+// chunk; then every thread multiplies positions of all items with key words it loads once.
+//
+// Bound: issue slots and FP64 pipe together (ncu, two items x three z at N = 2^16, L = 4: FP64 27 %, issue 51 %, 96 registers and 20
+// warps per SM; 80 registers and 24 warps were 2 to 3 % slower).  The table entries and key words of a chunk are staged in shared
+// memory (the keys asynchronously, under the transform), which took the single-item launch from 91 to 51 us: read from global
+// memory they sat in the chain.  The sums are reduced on the FP64 pipe: the 128-bit integer reduction was as long as the products.
+// Against pass B, key product and permuted sum as kernels of their own (seven blocks, three giant steps, N = 2^16, L = 4):
+// 513 -> 390 us with the finish kernel below, and four of twenty digit transforms less in the lift.
+template <int IB, int T>
+__global__ void __launch_bounds__(T, 640 / T) k_ks_apply(ApplyArgs A) {
+    extern __shared__ __align__(16) u64 sm[];
+    const int L = A.L, N = A.N, t = blockIdx.x, i = L - (int)blockIdx.y;
+    const long long L1N = (long long)(L + 1) * N;
+    double2* tc = (double2*)sm;                  // [256]
+    u64* ks = sm + 512;                          // [L][2][256] key words
+    u64* buf = ks + (size_t)L * 512;             // [IB * L][256] digits
+    u64* acc = buf + (size_t)IB * L * 256;       // [IB][2][256] sums
+    const long long it0 = (long long)blockIdx.z * IB;
+    const int nit = A.items - it0 < IB ? (int)(A.items - it0) : IB;
+    const int hw = threadIdx.x >> 4, j = threadIdx.x & 15;
+    const unsigned hmask = 0xFFFFu << (threadIdx.x & 16);
+    const LimbConst* lc = A.lt + i;
+    const u64 q = lc->q;
+    const bool f64 = q < (1ULL << 50);
+    const unsigned m0 = (unsigned)(N >> 8);
+    const int it = hw / L, dj = hw - it * L;
+    const bool valid = it < nit, own = A.own && dj == i;
+    u64* sb = buf + hw * 256;
+    const ArithF64 ar(lc);
+    const double2 c51 = make_double2(lc->c51_bal, lc->c51_q);
+    int staged = -1;
+    for (int z = 0; z < A.nz; z++) {
+        const unsigned k = A.galois[A.rot0 + z * A.rot_zinc];
+        const int sc = k == 1u ? t : galois_src(t << 8, k, A.logN, 1) >> 8;
+        const u64* p = own ? A.own + (it0 + it) * A.own_it + z * A.own_z + (long long)i * N
+                           : A.digits + (((z * A.items + it0 + it) * L + dj) * A.n_tgt + (A.n_tgt > L || i < dj ? i : i - 1)) * N;
+        p += (sc << 8);
+        if (z) __syncthreads();  // the products of the previous rotation have been taken
+        double x[16];  // binary64 or integer words alike
+        if (valid) {
+#pragma unroll
+            for (int e = 0; e < 16; e++) x[e] = __longlong_as_double((long long)p[j + 16 * e]);
+        }
+        stage_keys(ks, A.keytab[A.rot0 + z * A.rot_zinc] + (long long)i * N + (sc << 8), L1N, L);
+        if (staged != sc) {
+            if (f64) stage_twiddles(tc, (const double2*)A.tw_fwd_f64 + ((size_t)i << A.logN), m0 + sc);
+            else stage_twiddles((ulonglong2*)tc, (const ulonglong2*)A.tw_fwd_int + ((size_t)i << A.logN), m0 + sc);
+        }
+        staged = sc;
+        __syncthreads();
+        if (valid && own) {  // canonical words of the transform itself
+#pragma unroll
+            for (int e = 0; e < 16; e++) {
+                const u64 v = (u64)__double_as_longlong(x[e]);
+                sb[16 * j + (e ^ j)] = f64 ? (u64)__double_as_longlong(ar.inv_input(v)) : v;
+            }
+        } else if (valid && f64) {
+            chunk_forward(ar, x, tc, sb, j, hmask);
+#pragma unroll
+            for (int e = 0; e < 16; e++) sb[16 * j + (e ^ j)] = (u64)__double_as_longlong(ar.reduce(x[e]));
+        } else if (valid) {
+#pragma unroll
+            for (int e = 0; e < 16; e++) sb[16 * e + (j ^ e)] = (u64)__double_as_longlong(x[e]);
+            if (q < (1ULL << 57)) chunk_forward_int(ArithInt<true>(lc), (const ulonglong2*)tc, sb, j, hmask);
+            else chunk_forward_int(ArithInt<false>(lc), (const ulonglong2*)tc, sb, j, hmask);
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+        for (int m = threadIdx.x; m < 256; m += blockDim.x) {
+            int s = m;
+            if (k != 1u) {
+                const int src = galois_src((t << 8) + m, k, A.logN, 1);
+                if (!HANN_CHECK_INDEX((src >> 8) - sc, 1)) continue;
+                s = src & 255;
+            }
+            const u64* kp = ks + s;
+            const u64* xp = buf + swz(s);
+            u64* ac = acc + swz(m);
+            if (f64) {
+                // exact sums of at most eight products in two binary64 words (acc2_fma), reduced on the FP64 pipe; chains of more
+                // than eight primes run one item per CTA and add up several such sums
+                double r[IB][2];
+#pragma unroll
+                for (int b = 0; b < IB; b++) {
+                    r[b][0] = z ? __longlong_as_double((long long)ac[b * 512]) : 0.0;
+                    r[b][1] = z ? __longlong_as_double((long long)ac[b * 512 + 256]) : 0.0;
+                }
+                for (int d0 = 0; d0 < L; d0 += 8) {
+                    double ah[IB][2], al[IB][2];
+#pragma unroll
+                    for (int b = 0; b < IB; b++) ah[b][0] = ah[b][1] = kAcc2Start, al[b][0] = al[b][1] = 0;
+                    const int d1 = d0 + 8 < L ? d0 + 8 : L;
+#pragma unroll 4
+                    for (int d = d0; d < d1; d++) {
+                        const double k0 = residue_to_f64(kp[d << 9]), k1 = residue_to_f64(kp[(d << 9) + 256]);
+#pragma unroll
+                        for (int b = 0; b < IB; b++) {
+                            const double xv = __longlong_as_double((long long)xp[(b * L + d) << 8]);
+                            acc2_fma(ah[b][0], al[b][0], k0, xv);
+                            acc2_fma(ah[b][1], al[b][1], k1, xv);
+                        }
+                    }
+#pragma unroll
+                    for (int b = 0; b < IB; b++)
+#pragma unroll
+                        for (int c = 0; c < 2; c++) r[b][c] = ar.reduce(__dadd_rn(r[b][c], ar.acc2_value(ah[b][c], al[b][c], c51)));
+                    if (IB > 1) break;
+                }
+#pragma unroll
+                for (int b = 0; b < IB; b++) {
+                    ac[b * 512] = (u64)__double_as_longlong(r[b][0]);
+                    ac[b * 512 + 256] = (u64)__double_as_longlong(r[b][1]);
+                }
+            } else {
+                u64 hi[IB][2], lo[IB][2];
+#pragma unroll
+                for (int b = 0; b < IB; b++) hi[b][0] = hi[b][1] = lo[b][0] = lo[b][1] = 0;
+#pragma unroll 1
+                for (int d = 0; d < L; d++) {
+                    const u64 k0 = kp[d << 9], k1 = kp[(d << 9) + 256];
+#pragma unroll
+                    for (int b = 0; b < IB; b++) {
+                        const u64 xv = xp[(b * L + d) << 8];
+                        mac128(hi[b][0], lo[b][0], xv, k0);
+                        mac128(hi[b][1], lo[b][1], xv, k1);
+                    }
+                }
+#pragma unroll
+                for (int b = 0; b < IB; b++)
+#pragma unroll
+                    for (int c = 0; c < 2; c++) {
+                        const u64 r = reduce128(hi[b][c], lo[b][c], *lc);
+                        u64* a = ac + (b * 2 + c) * 256;
+                        *a = z ? addmod(*a, r, q) : r;
+                    }
+            }
+        }
+    }
+    u64* out = A.u + it0 * 2 * L1N + (long long)i * N + (t << 8);
+    if (i < L) {  // every thread stores the sums it made
+        for (int m = threadIdx.x; m < 256; m += blockDim.x)
+            for (int v = 0; v < 2 * nit; v++) out[v * L1N + m] = acc[v * 256 + swz(m)];
+        return;
+    }
+    // the special prime's sums go straight into the inverse pass B' of their chunk
+    __syncthreads();
+    for (int v = hw; v < 2 * nit; v += blockDim.x >> 4) {
+        u64* sv = acc + v * 256;
+        u64* o = out + v * L1N;
+        if (f64) {
+            const double2* tw = (const double2*)A.tw_inv_f64 + ((size_t)i << A.logN);
+            double x[16];
+#pragma unroll
+            for (int e = 0; e < 16; e++) x[e] = ar.from_mid(sv[16 * j + (e ^ j)]);
+            inv_round<4>(ar, x, tw, ((m0 + t) << 4) + j);
+#pragma unroll
+            for (int e = 0; e < 16; e++) sv[16 * j + (e ^ j)] = ar.to_mid(x[e]);
+            __syncwarp(hmask);
+#pragma unroll
+            for (int e = 0; e < 16; e++) x[e] = ar.from_mid(sv[16 * e + (j ^ e)]);
+            inv_round<4>(ar, x, tw, m0 + t);
+#pragma unroll
+            for (int e = 0; e < 16; e++) o[j + 16 * e] = ar.to_mid(x[e]);
+        } else {
+            const ArithInt<false> ar(lc);
+            const ulonglong2* tw = (const ulonglong2*)A.tw_inv_int + ((size_t)i << A.logN);
+            inv_round4_smem(ar, [=](int e) { return sv + 16 * j + (e ^ j); }, tw, ((m0 + t) << 4) + j);
+            __syncwarp(hmask);
+            const auto second = [=](int e) { return sv + 16 * e + (j ^ e); };
+            inv_round4_smem(ar, second, tw, m0 + t);
+#pragma unroll 8
+            for (int e = 0; e < 16; e++) o[j + 16 * e] = *second(e);
+        }
+    }
+}
+
+struct FinishArgs {
+    const u64* lifted;  // [item][2][L][N], pass-A format
+    const u64* u;       // [item][2][L+1][N]
+    const u64* add;     // optional: add + item * add_it + component * L N, in the order of the result
+    long long add_it;
+    const u64* c0;      // optional, first component only: the sum over z of phi_z(c0 + item * c0_it + z * c0_z)
+    long long c0_it, c0_z;
+    int rot0, rot_inc, nz;  // rotation of z; with PERM, of the item
+    u64 *out0, *out1;
+    long long out_it;
+    const unsigned* galois;
+    long long items;
+    int N, logN, L, n;
+    const void *tw_fwd_f64, *tw_fwd_int;
+    const LimbConst* lt;
+};
+
+// out[item][c][i] = (u - lifted) p^{-1} + add + phi(c0), modulus i = blockIdx.y, chunk blockIdx.x, a half-warp per (item, component):
+// pass B of the lifted ModDown polynomials with the combination behind its last round.
+// PERM: u, lifted and c0 are still in the order before the automorphism, which differs from item to item (hoisted rotations); the
+// finished words are permuted in shared memory and stored to the item's own chunk of the result.
+//
+// 31 rotations at N = 2^16, L = 4: 170 us (pass B and the combination as two kernels) -> 103 us; the integer reductions of the
+// combination and a 16-fold unrolled tail (instruction fetch) cost most of that on the way.
+template <bool PERM>
+__global__ void __launch_bounds__(256, 3) k_ks_finish(FinishArgs A) {
+    extern __shared__ __align__(16) u64 sm[];
+    const int L = A.L, N = A.N, t = blockIdx.x, i = blockIdx.y;
+    const long long LN = (long long)L * N, L1N = LN + N;
+    double2* tc = (double2*)sm;
+    const int hw = threadIdx.x >> 4, j = threadIdx.x & 15;
+    const unsigned hmask = 0xFFFFu << (threadIdx.x & 16);
+    u64* sb = sm + 512 + hw * 256;
+    const LimbConst* lc = A.lt + i;
+    const u64 q = lc->q;
+    const unsigned m0 = (unsigned)(N >> 8);
+    const bool f64 = q < (1ULL << 50);
+    const ArithF64 ar(lc);
+    const double2 pinv = make_double2(lc->pinv_bal, lc->pinv_q);
+    const u64 pinv_i = lc->pinv, pinv_s = lc->pinv_s;
+    if (f64) stage_twiddles(tc, (const double2*)A.tw_fwd_f64 + ((size_t)i << A.logN), m0 + t);
+    else stage_twiddles((ulonglong2*)tc, (const ulonglong2*)A.tw_fwd_int + ((size_t)i << A.logN), m0 + t);
+    __syncthreads();
+    const long long units = 2 * A.items, ustep = (long long)gridDim.z * (blockDim.x >> 4);
+    for (long long v = (long long)blockIdx.z * (blockDim.x >> 4) + hw; v < units; v += ustep) {
+        const long long item = v >> 1;
+        const int c = (int)(v & 1);
+        const u64* p = A.lifted + (v * L + i) * N + (t << 8);
+        const u64* up = A.u + v * L1N + (long long)i * N + (t << 8) + j;
+        const u64* ap = A.add ? A.add + item * A.add_it + c * LN + (long long)i * N + (t << 8) + j : nullptr;
+        const u64* cp = A.c0 && c == 0 ? A.c0 + item * A.c0_it + (long long)i * N : nullptr;
+        u64* o = (c == 0 ? A.out0 : A.out1) + item * A.out_it + (long long)i * N;
+        double x[16];
+#pragma unroll
+        for (int e = 0; e < 16; e++) x[e] = __longlong_as_double((long long)p[j + 16 * e]);
+        __syncwarp(hmask);  // the words of the half-warp's previous polynomial have been taken
+        // then words 16 e + j, eight at a time: the combination is long and a rolled loop keeps its instructions few
+        if (f64) {
+            chunk_forward(ar, x, tc, sb, j, hmask);
+#pragma unroll
+            for (int e = 0; e < 16; e++) sb[16 * j + (e ^ j)] = (u64)__double_as_longlong(ar.reduce(x[e]));
+#pragma unroll 1
+            for (int e0 = 0; e0 < 16; e0 += 8) {
+                double uw[8], a[8];
+#pragma unroll
+                for (int e = 0; e < 8; e++) {
+                    const u64 v = up[16 * (e0 + e)];
+                    uw[e] = PERM ? ar.from_canonical(v) : ar.from_mid(v);
+                }
+#pragma unroll
+                for (int e = 0; e < 8; e++) a[e] = ap ? ar.from_canonical(ap[16 * (e0 + e)]) : 0.0;
+                if (PERM && cp) {
+#pragma unroll
+                    for (int e = 0; e < 8; e++) a[e] = ar.from_canonical(cp[(t << 8) + 16 * (e0 + e) + j]);
+                } else if (cp) {
+                    for (int z = 0; z < A.nz; z++) {
+                        const LaneSource ls((t << 8) + j, A.galois[A.rot0 + z * A.rot_inc], A.logN);
+#pragma unroll
+                        for (int e = 0; e < 8; e++) {
+                            const int w = ls.word(e0 + e);
+                            if (!HANN_CHECK_INDEX(w, N)) continue;
+                            a[e] = __dadd_rn(a[e], ar.from_canonical(cp[z * A.c0_z + w]));
+                            if ((z & 3) == 3) a[e] = ar.reduce(a[e]);
+                        }
+                    }
+                }
+#pragma unroll
+                for (int e = 0; e < 8; e++) {
+                    // |u - reduce(x)| <= 1.5 q, the product lies below 0.7 q, the added words below 5 q
+                    u64* w = sb + 16 * j + ((e0 + e) ^ j);
+                    const double y = ar.mulmod_small(__dsub_rn(uw[e], __longlong_as_double((long long)*w)), pinv);
+                    const u64 r = ar.to_canonical(__dadd_rn(y, a[e]));
+                    if (PERM) *w = r;
+                    else o[(t << 8) + 16 * (e0 + e) + j] = r;
+                }
+            }
+        } else {
+#pragma unroll
+            for (int e = 0; e < 16; e++) sb[16 * e + (j ^ e)] = (u64)__double_as_longlong(x[e]);
+            if (q < (1ULL << 57)) chunk_forward_int(ArithInt<true>(lc), (const ulonglong2*)tc, sb, j, hmask);
+            else chunk_forward_int(ArithInt<false>(lc), (const ulonglong2*)tc, sb, j, hmask);
+#pragma unroll 2
+            for (int e = 0; e < 16; e++) {
+                u64* w = sb + 16 * j + (e ^ j);
+                u64 r = csub(shoup_mul(submod(up[16 * e], *w, q), pinv_i, pinv_s, q), q);
+                if (ap) r = addmod(r, ap[16 * e], q);
+                if (PERM && cp) {
+                    r = addmod(r, cp[(t << 8) + 16 * e + j], q);
+                } else if (cp) {
+                    for (int z = 0; z < A.nz; z++) {
+                        const int src = galois_src((t << 8) + 16 * e + j, A.galois[A.rot0 + z * A.rot_inc], A.logN, 1);
+                        if (!HANN_CHECK_INDEX(src, N)) continue;
+                        r = addmod(r, cp[z * A.c0_z + src], q);
+                    }
+                }
+                if (PERM) *w = r;
+                else o[(t << 8) + 16 * e + j] = r;
+            }
+        }
+        if (PERM) {
+            const int r = A.rot0 + (int)item * A.rot_inc;
+            const unsigned k = A.galois[r], kinv = A.galois[(A.n - r) % A.n];
+            const int tt = galois_src(t << 8, kinv, A.logN, 1) >> 8;  // the chunk of the result that reads this one
+            const LaneSource ls((tt << 8) + j, k, A.logN);
+            const bool inside = HANN_CHECK_INDEX((ls.base >> 8) - t, 1);
+            const u64* sr = sb + ((ls.base & 15) << 4);  // logical position 16 a + b at word 16 a + (b ^ a), a the word's low nibble
+            __syncwarp(hmask);
+#pragma unroll 8
+            for (int e = 0; e < 16; e++)
+                if (inside) o[(tt << 8) + 16 * e + j] = sr[ls.high(e) ^ (ls.base & 15)];
+        }
+    }
+}
+
+template <int IB, int T>
+void launch_apply(hann_ctx* c, const ApplyArgs& A) {
+    // sixteen lanes per digit, whole warps
+    const int threads = (IB * A.L * 16 + 31) / 32 * 32;
+    const size_t smem = (size_t)4096 + (2 * A.L + (size_t)threads / 16 + 2 * IB) * 2048;
+    cudaFuncSetAttribute(k_ks_apply<IB, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    KProf kp(c, KC_KS_INNER);
+    k_ks_apply<IB, T><<<dim3(c->N >> 8, A.L + 1, (unsigned)((A.items + IB - 1) / IB)), threads, smem, c->stream>>>(A);
+}
+
+}  // namespace
+
+bool ks_fused_available(const hann_ctx* c) { return c->logN >= 10 && c->ntt_tau; }
+
+// digits: output of launch_ks_lift for the nz * items polynomials of L limbs; own (optional): the polynomials themselves, in which
+// case the digits were lifted without their own modulus.  Leaves u[item][2][L+1][N] (see ApplyArgs), the input of the ModDown lift.
+int launch_ks_apply(hann_ctx* c, const u64* digits, const u64* own, int64_t own_it, int64_t own_z, int64_t items, int nz, int rot0, int rot_zinc, u64* u) {
+    if (items <= 0 || nz <= 0) return HANN_OK;
+    ApplyArgs A = {};
+    A.digits = digits;
+    A.n_tgt = own ? c->L : c->L + 1;
+    A.own = own;
+    A.own_it = own_it;
+    A.own_z = own_z;
+    A.keytab = c->keytab_dev;
+    A.galois = c->galois_dev;
+    A.rot0 = rot0;
+    A.rot_zinc = rot_zinc;
+    A.nz = nz;
+    A.items = items;
+    A.u = u;
+    A.N = c->N;
+    A.logN = c->logN;
+    A.L = c->L;
+    A.tw_fwd_f64 = c->tw_fwd_f64;
+    A.tw_fwd_int = c->tw_fwd;
+    A.tw_inv_f64 = c->tw_inv_f64;
+    A.tw_inv_int = c->tw_inv;
+    A.lt = c->lt_dev;
+    // items per CTA: their digits fill at most sixteen half-warps, and the eight-product sums allow several items up to eight
+    // primes only; key words and table entries are read once for all of them
+    if (items >= 4 && c->L <= 4) launch_apply<4, 256>(c, A);
+    else if (items >= 2 && c->L <= 4) launch_apply<2, 128>(c, A);
+    else if (items >= 2 && c->L <= 8) launch_apply<2, 256>(c, A);
+    else if (c->L <= 4) launch_apply<1, 64>(c, A);
+    else launch_apply<1, 256>(c, A);
+    return check_launch(c, "ks_apply");
+}
+
+// lifted: output of launch_ks_lift for the special-prime limbs of u.  perm_items: the automorphism is still to be applied, that of
+// item `it` being rotation rot0 + it * rot_inc (otherwise rotation rot0 + z * rot_inc belongs to the c0 term z < nz).
+int launch_ks_finish(hann_ctx* c, const u64* u, const u64* lifted, int64_t items, bool perm_items, int rot0, int rot_inc, int nz, const u64* c0,
+                     int64_t c0_it, int64_t c0_z, const u64* add, int64_t add_it, u64* out0, u64* out1, int64_t out_it) {
+    if (items <= 0) return HANN_OK;
+    FinishArgs A = {};
+    A.lifted = lifted;
+    A.u = u;
+    A.add = add;
+    A.add_it = add_it;
+    A.c0 = c0;
+    A.c0_it = c0_it;
+    A.c0_z = c0_z;
+    A.rot0 = rot0;
+    A.rot_inc = rot_inc;
+    A.nz = nz;
+    A.out0 = out0;
+    A.out1 = out1;
+    A.out_it = out_it;
+    A.galois = c->galois_dev;
+    A.items = items;
+    A.N = c->N;
+    A.logN = c->logN;
+    A.L = c->L;
+    A.n = c->n;
+    A.tw_fwd_f64 = c->tw_fwd_f64;
+    A.tw_fwd_int = c->tw_fwd;
+    A.lt = c->lt_dev;
+    // up to sixteen half-warps per CTA, which then walk further polynomials under the staged tables while the grid fills the
+    // machine twice over
+    const int hws = (int)(2 * items < 16 ? 2 * items : 16), threads = 16 * hws;
+    const size_t smem = 4096 + (size_t)hws * 2048;
+    const long long per = (long long)(c->N >> 8) * c->L, groups = (2 * items + hws - 1) / hws;
+    long long gz = (2 * 148 * 3 + per - 1) / per;
+    if (gz > groups) gz = groups;
+    const dim3 grid(c->N >> 8, c->L, (unsigned)gz);
+    KProf kp(c, KC_MODDOWN_COMBINE);
+    if (perm_items) k_ks_finish<true><<<grid, threads, smem, c->stream>>>(A);
+    else k_ks_finish<false><<<grid, threads, smem, c->stream>>>(A);
+    return check_launch(c, "ks_finish");
+}
+
+HANN_DEBUG_DEFINE_BIND(debug_bind_ksfused)

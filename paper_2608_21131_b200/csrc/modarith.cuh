@@ -23,8 +23,15 @@ struct LimbConst {
     u64 pinv_s;
     u64 pmod;    // p mod q               (ciphertext primes only)
     u64 half;    // floor(q / 2): residues above it lift to negative integers
+    double qd;        // q, floor(q / 2) and fl(1 / q) in binary64
+    double halfd;
+    double qinv;
+    double c51_bal;   // 2^51 mod q as a balanced integer (moduli below 2^50: the high word of an exact sum counts 2^51)
+    double c51_q;     // fl(c51_bal / q)
     double ninv_bal;  // N^{-1} mod q as a balanced integer (binary64 transform path)
     double ninv_q;    // fl(ninv_bal / q)
+    double pinv_bal;  // p^{-1} mod q as a balanced integer, ciphertext primes only
+    double pinv_q;    // fl(pinv_bal / q)
 };
 
 #define HANN_MAXL1 16  // up to 15 ciphertext primes + the special prime (limb numbers travel in 4-bit fields)

@@ -57,6 +57,9 @@ struct NttArgs {
     // of from `data` (nullptr: in place)
     const u64* src;
     long long src_gstride;
+    // src_per > 0: group g is read from src + (g / src_per) * src_zstride + (g % src_per) * src_gstride
+    int src_per;
+    long long src_zstride;
     u64 pos4, limb4;  // 4-bit fields: position within the period and limb of selection k (at most 16 selections)
     // forward pass B (bulk-copy kernel) of polynomials that are fixed by X -> 1/X and stored as their first N/2 transform
     // values only: the grid covers the first half of the chunks (stride is then N/2 or more)
@@ -400,15 +403,19 @@ __global__ void __launch_bounds__(256, 3) k_ntt_inv_b8t(NttArgs A, int groups, i
     const int yg0 = blockIdx.z, ystep = gridDim.z;
     u64* gbase = A.data + (((long long)yg0 * kTP + t) * A.period + pos) * A.stride + ((size_t)chunk0 << 8);
     // source of the copies: the same words, or a separately laid out input (group stride src_gstride)
-    const u64* sbase = A.src ? A.src + ((long long)yg0 * kTP + t) * A.src_gstride + (long long)pos * A.stride + ((size_t)chunk0 << 8) : gbase;
-    const long long stile_stride = A.src ? (long long)kTP * A.src_gstride : (long long)kTP * A.period * A.stride;
+    const u64* sbase = A.src ? A.src + (long long)pos * A.stride + ((size_t)chunk0 << 8) : gbase;
+    auto source = [&](int i) {
+        if (!A.src) return sbase + (long long)i * ystep * tile_stride;
+        const int g = (yg0 + i * ystep) * kTP + t;
+        return sbase + (A.src_per > 0 ? (g / A.src_per) * A.src_zstride + (g % A.src_per) * A.src_gstride : g * A.src_gstride);
+    };
     const int my_tiles = yg0 < ntiles ? (ntiles - yg0 + ystep - 1) / ystep : 0;
     auto tile_valid = [&](int i) { return i < my_tiles && (long long)(yg0 + (long long)i * ystep) * kTP + t < groups; };
     if (lane == 0) {
         for (int i = 0; i < 2; i++)
             if (tile_valid(i)) {
                 mbar_expect_tx(bar0 + 8 * i, 4096);
-                bulk_load(buf0 + 4096 * i, sbase + (long long)i * ystep * stile_stride, 4096, bar0 + 8 * i);
+                bulk_load(buf0 + 4096 * i, source(i), 4096, bar0 + 8 * i);
             }
     }
     for (int i = threadIdx.x; i < kTK * 256; i += 256) {
@@ -434,25 +441,36 @@ __global__ void __launch_bounds__(256, 3) k_ntt_inv_b8t(NttArgs A, int groups, i
             return;
         }
         u64* sb = wbuf + s * 512 + ch * 256;
+        u64* go = gbase + (long long)i * ystep * tile_stride + ((size_t)ch << 8);
         typename AR::T x[16];
 #pragma unroll
         for (int e = 0; e < 16; e++) x[e] = ar.inv_input(sb[16 * e + j]);  // logical positions 16 j + e
         __syncwarp();
-        inv_round_f<4>(ar, x, [=](int st, int il) { return tcc[((16 - (16 >> st) + il + 1) << 4) + j]; });
+        if constexpr (AR::kUnroll) {
+            inv_round_f<4>(ar, x, [=](int st, int il) { return tcc[((16 - (16 >> st) + il + 1) << 4) + j]; });
 #pragma unroll
-        for (int e = 0; e < 16; e++) sb[16 * j + (e ^ j)] = ar.to_mid(x[e]);
-        __syncwarp();
+            for (int e = 0; e < 16; e++) sb[16 * j + (e ^ j)] = ar.to_mid(x[e]);
+            __syncwarp();
 #pragma unroll
-        for (int e = 0; e < 16; e++) x[e] = ar.from_mid(sb[16 * e + (j ^ e)]);  // logical positions j + 16 e
-        inv_round_f<4>(ar, x, [=](int st, int il) { return tcc[16 - (16 >> st) + il]; });
-        u64* go = gbase + (long long)i * ystep * tile_stride + ((size_t)ch << 8);
+            for (int e = 0; e < 16; e++) x[e] = ar.from_mid(sb[16 * e + (j ^ e)]);  // logical positions j + 16 e
+            inv_round_f<4>(ar, x, [=](int st, int il) { return tcc[16 - (16 >> st) + il]; });
 #pragma unroll
-        for (int e = 0; e < 16; e++) go[j + 16 * e] = ar.to_mid(x[e]);
+            for (int e = 0; e < 16; e++) go[j + 16 * e] = ar.to_mid(x[e]);
+        } else {  // in place at the words of the exchange, rolled (see fwd_round4_smem)
+#pragma unroll
+            for (int e = 0; e < 16; e++) sb[16 * j + (e ^ j)] = x[e];
+            inv_round4_staged(ar, [=](int e) { return sb + 16 * j + (e ^ j); }, tcc + 16, 16, j);
+            __syncwarp();
+            const auto second = [=](int e) { return sb + 16 * e + (j ^ e); };
+            inv_round4_staged(ar, second, tcc, 1, 0);
+#pragma unroll
+            for (int e = 0; e < 16; e++) go[j + 16 * e] = *second(e);
+        }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
         if (lane == 0 && tile_valid(i + 2)) {
             mbar_expect_tx(bar0 + 8 * s, 4096);
-            bulk_load(buf0 + 4096 * s, sbase + (long long)(i + 2) * ystep * stile_stride, 4096, bar0 + 8 * s);
+            bulk_load(buf0 + 4096 * s, source(i + 2), 4096, bar0 + 8 * s);
         }
     }
 }
@@ -590,6 +608,7 @@ struct LiftArgs {
     u64 src_limb4;        // limb of source polynomial sp = nibble (sp % src_period)
     u64* dst;             // target polynomial (sp, ti) at dst + (sp * n_tgt + ti) * N, in forward pass-A output format
     int n_tgt, tgt_limb0;
+    int skip_own;         // target ti of a source of limb sl is limb ti (ti < sl) or ti + 1: its own modulus is left out
     int logN;
     const void *tw_inv_int, *tw_inv_f64, *tw_fwd_int, *tw_fwd_f64;
     const LimbConst* lt;
@@ -781,7 +800,7 @@ __device__ __forceinline__ void lift_targets(const LiftArgs& A, int sl, long lon
     // a launch too small to fill the machine is cut along the targets as well: gridDim.z CTAs repeat the inverse rounds and
     // share out the targets, which shortens the chain one CTA runs
     for (int ti = blockIdx.z; ti < A.n_tgt; ti += gridDim.z) {
-        const int tl = A.tgt_limb0 + ti;
+        const int tl = A.tgt_limb0 + ti + (A.skip_own && ti >= sl ? 1 : 0);
         const LimbConst* tlc = A.lt + tl;
         const u64 q = tlc->q;
         u64* dbase = A.dst + (sp * A.n_tgt + ti) * (long long)N + c0;
@@ -954,7 +973,7 @@ void launch_fwd_class(hann_ctx* c, const NttArgs& A, int groups, bool skip_a, bo
 template <class AR>
 void launch_inv_class(hann_ctx* c, const NttArgs& A, int groups, bool skip_a) {
     if (A.b == 8 && A.a > 0 && A.tau && ((c->N >> 8) % kTK) == 0 && ((uintptr_t)A.data & 15) == 0 && (A.stride & 1) == 0 &&
-        ((uintptr_t)A.src & 15) == 0 && (A.src_gstride & 1) == 0) {
+        ((uintptr_t)A.src & 15) == 0 && (A.src_gstride & 1) == 0 && (A.src_zstride & 1) == 0) {
         KProf kp(c, KC_NTT_INV_B);
         const size_t smem = (size_t)kTK * 256 * 16 + (size_t)kTP * 2 * 512 * 8 + (size_t)kTP * 2 * 8;
         cudaFuncSetAttribute(k_ntt_inv_b8t<AR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -984,7 +1003,7 @@ void launch_inv_class(hann_ctx* c, const NttArgs& A, int groups, bool skip_a) {
 // npoly polynomials, `stride` words apart, polynomial p using modulus lm.limb[p % lm.period]; npoly must be a multiple of
 // the period.  One set of launches per arithmetic class present in the period.
 int launch_ntt(hann_ctx* c, u64* data, int64_t npoly, int64_t stride, const LimbMap& lm, bool inverse, bool skip_a = false,
-               const u64* src = nullptr, int64_t src_gstride = 0, bool half = false) {
+               const u64* src = nullptr, int64_t src_gstride = 0, bool half = false, int64_t src_per = 0, int64_t src_zstride = 0) {
     if (npoly <= 0) return HANN_OK;
     if (npoly % lm.period) {
         c->err = "transform batch is not a whole number of limb periods";
@@ -1002,6 +1021,8 @@ int launch_ntt(hann_ctx* c, u64* data, int64_t npoly, int64_t stride, const Limb
     A.tau = c->ntt_tau;
     A.src = src;
     A.src_gstride = src_gstride;
+    A.src_per = (int)src_per;
+    A.src_zstride = src_zstride;
     A.period = lm.period;
     A.half = half ? 1 : 0;
     if (half) {
@@ -1033,6 +1054,10 @@ int launch_ntt(hann_ctx* c, u64* data, int64_t npoly, int64_t stride, const Limb
         NttArgs& X = Ac[cls];
         if (!X.nsel) continue;
         const int64_t gmax = 65535 / (mixed ? Ac[0].nsel + Ac[2].nsel : X.nsel);
+        if (src_per > 0 && groups_total > gmax) {
+            c->err = "gathered transform batch too large";
+            return HANN_EINVAL;
+        }
         for (int64_t g0 = 0; g0 < groups_total; g0 += gmax) {
             const int groups = (int)std::min<int64_t>(gmax, groups_total - g0);
             X.data = data + g0 * lm.period * stride;
@@ -1156,7 +1181,7 @@ static int lift_zsplit(long ctas, int n_tgt) {
 // After inverse pass B' of the nsrc source polynomials (launch_ntt_inv_pass_b): finish their inverse transforms, lift the
 // coefficients (centred) into the n_tgt moduli tgt_limb0 .. and run pass A of the target transforms.  The caller finishes
 // with launch_ntt_fwd_pass_b over the targets.
-int launch_ks_lift(hann_ctx* c, u64* src, int64_t src_stride, int64_t nsrc, const LimbMap& src_lm, u64* dst, int n_tgt, int tgt_limb0) {
+int launch_ks_lift(hann_ctx* c, u64* src, int64_t src_stride, int64_t nsrc, const LimbMap& src_lm, u64* dst, int n_tgt, int tgt_limb0, bool skip_own) {
     if (nsrc <= 0) return HANN_OK;
     LiftArgs A;
     A.src = src;
@@ -1167,6 +1192,7 @@ int launch_ks_lift(hann_ctx* c, u64* src, int64_t src_stride, int64_t nsrc, cons
     A.dst = dst;
     A.n_tgt = n_tgt;
     A.tgt_limb0 = tgt_limb0;
+    A.skip_own = skip_own ? 1 : 0;
     A.logN = c->logN;
     A.tw_inv_int = c->tw_inv;
     A.tw_inv_f64 = c->tw_inv_f64;
@@ -1203,10 +1229,11 @@ bool ntt_inv_pass_b_gathers(const hann_ctx* c, const void* src, const void* dst)
 }
 
 // The same with the input read from elsewhere: group g (lm.period polynomials, `stride` words apart) starts at
-// src + g * src_gstride; the output goes to data as above.  Only where ntt_inv_pass_b_gathers(c) holds and both pointers are
+// src + g * src_gstride (src_per > 0: at src + (g / src_per) * src_zstride + (g % src_per) * src_gstride); the output goes to data as above.  Only where ntt_inv_pass_b_gathers(c) holds and both pointers are
 // 16-byte aligned (the bulk-copy kernel); the caller copies and uses launch_ntt_inv_pass_b otherwise.
-int launch_ntt_inv_pass_b_from(hann_ctx* c, const u64* src, int64_t src_gstride, u64* data, int64_t npoly, int64_t stride, const LimbMap& lm) {
-    return launch_ntt(c, data, npoly, stride, lm, true, true, src, src_gstride);
+int launch_ntt_inv_pass_b_from(hann_ctx* c, const u64* src, int64_t src_gstride, u64* data, int64_t npoly, int64_t stride, const LimbMap& lm,
+                               int64_t src_per, int64_t src_zstride) {
+    return launch_ntt(c, data, npoly, stride, lm, true, true, src, src_gstride, false, src_per, src_zstride);
 }
 
 int launch_wait_selftest(hann_ctx* c, unsigned long long limit_ns, unsigned long long* waited_ns_dev) {

@@ -18,11 +18,12 @@ struct ArithF64 {
     double q, qinv, half;
     long long qi;
     static constexpr int kMinBlocks = HANN_F64_MINBLOCKS;
+    static constexpr bool kUnroll = true;
     static constexpr double kRound = 6755399441055744.0;  // 1.5 * 2^52: fl(v + kRound) - kRound = rint(v) for |v| < 2^51
     static constexpr double kTwo52 = 4503599627370496.0;
     TW ninv;
     __device__ __forceinline__ ArithF64(const LimbConst* lc)
-        : q((double)lc->q), qinv(1.0 / (double)lc->q), half((double)lc->half), qi((long long)lc->q), ninv(make_double2(lc->ninv_bal, lc->ninv_q)) {}
+        : q(lc->qd), qinv(lc->qinv), half(lc->halfd), qi((long long)lc->q), ninv(make_double2(lc->ninv_bal, lc->ninv_q)) {}
     // x - round(x/q) q; the quotient (at most 8 in magnitude) is rounded by adding 1.5 * 2^52
     __device__ __forceinline__ T reduce(T x) const {
         return __fma_rn(-__dsub_rn(__fma_rn(x, qinv, kRound), kRound), q, x);
@@ -40,6 +41,11 @@ struct ArithF64 {
         const double l = __fma_rn(y, w.x, -h);
         const double c = __dsub_rn(__fma_rn(y, w.y, kRound), kRound);
         return __dadd_rn(__fma_rn(-c, q, h), l);
+    }
+    // the value of an exact two-word sum (acc2_fma, at most eight products) modulo q, below 1.25 q in magnitude: the high word is
+    // 2^51 times an integer of at most 2q, the low word an integer of at most 2^53
+    __device__ __forceinline__ T acc2_value(double ah, double al, TW c51) const {
+        return __dadd_rn(mulmod_small(__dmul_rn(__dsub_rn(ah, kAcc2Start), 0x1p-51), c51), reduce(al));
     }
     // integers below 2^52 <-> binary64 through the mantissa of 2^52 + v (one add and one logic operation)
     __device__ __forceinline__ T from_canonical(u64 v) const {
@@ -86,6 +92,7 @@ struct ArithInt {
     typedef ulonglong2 TW;
     u64 q, q2;
     static constexpr int kMinBlocks = HANN_NTT_MINBLOCKS;
+    static constexpr bool kUnroll = false;
     TW ninv;
     __device__ __forceinline__ ArithInt(const LimbConst* lc) : q(lc->q), q2(2 * lc->q), ninv(make_ulonglong2(lc->ninv, lc->ninv_s)) {}
     __device__ __forceinline__ T from_canonical(u64 v) const { return v; }
@@ -223,6 +230,45 @@ __device__ __forceinline__ void inv_round4_smem(const AR& ar, const WORD& word, 
         const unsigned b = it < 4 ? 4 * base + k : base;
         u64 x0 = *word(e0), x1 = *word(e0 + st), x2 = *word(e0 + 2 * st), x3 = *word(e0 + 3 * st);
         const typename AR::TW w = tw[b], wa = tw[2 * b], wb = tw[2 * b + 1];
+        ar.inv(x0, x1, wa);
+        ar.inv(x2, x3, wb);
+        ar.inv(x0, x2, w);
+        ar.inv(x1, x3, w);
+        *word(e0) = x0;
+        *word(e0 + st) = x1;
+        *word(e0 + 2 * st) = x2;
+        *word(e0 + 3 * st) = x3;
+    }
+}
+
+// the same rounds with a staged table: entry il of stage s of the round at tc[((1 << s) - 1 + il) * step + off] (forward),
+// tc[(16 - (16 >> s) + il) * step + off] (inverse)
+template <class AR, class WORD>
+__device__ __forceinline__ void fwd_round4_staged(const AR& ar, const WORD& word, const typename AR::TW* tc, int step, int off) {
+#pragma unroll 1
+    for (int it = 0; it < 8; it++) {
+        const int k = it & 3, e0 = it < 4 ? k : 4 * k, st = it < 4 ? 4 : 1;
+        const int a = it < 4 ? 0 : 3 + k, b = it < 4 ? 1 : 7 + 2 * k;
+        u64 x0 = *word(e0), x1 = *word(e0 + st), x2 = *word(e0 + 2 * st), x3 = *word(e0 + 3 * st);
+        const typename AR::TW w = tc[a * step + off], wa = tc[b * step + off], wb = tc[(b + 1) * step + off];
+        ar.fwd(x0, x2, w);
+        ar.fwd(x1, x3, w);
+        ar.fwd(x0, x1, wa);
+        ar.fwd(x2, x3, wb);
+        *word(e0) = x0;
+        *word(e0 + st) = x1;
+        *word(e0 + 2 * st) = x2;
+        *word(e0 + 3 * st) = x3;
+    }
+}
+template <class AR, class WORD>
+__device__ __forceinline__ void inv_round4_staged(const AR& ar, const WORD& word, const typename AR::TW* tc, int step, int off) {
+#pragma unroll 1
+    for (int it = 0; it < 8; it++) {
+        const int k = it & 3, e0 = it < 4 ? 4 * k : k, st = it < 4 ? 1 : 4;
+        const int a = it < 4 ? 2 * k : 12, b = it < 4 ? 8 + k : 14;
+        u64 x0 = *word(e0), x1 = *word(e0 + st), x2 = *word(e0 + 2 * st), x3 = *word(e0 + 3 * st);
+        const typename AR::TW w = tc[b * step + off], wa = tc[a * step + off], wb = tc[(a + 1) * step + off];
         ar.inv(x0, x1, wa);
         ar.inv(x2, x3, wb);
         ar.inv(x0, x2, w);

@@ -1,0 +1,70 @@
+"""The key-switch kernels (lift, digit product with the sum over rotations, final combination) on residues drawn directly, at the
+edges of their dispatch: one to nine digits, one to five blocks, moduli of every arithmetic class side by side, neighbouring moduli
+of very different size, residues at the ends of their range, and buffers that are only 8-byte aligned.  Exact against the oracle."""
+import numpy as np
+import pytest
+
+from oracle.oracle import find_primes
+from paper_2608_21131_b200 import synth
+from tests.helpers import make_oracle
+
+pytestmark = pytest.mark.gpu
+
+
+def edge_residues(seed, q, N, lead):
+    a = synth.uniform_residues(seed, 1, list(q), N, lead=lead)
+    for i, m in enumerate(q):
+        a[..., i, 0:6] = (0, 1, m - 1, m // 2, m // 2 + 1, m // 2 - 1)
+        a[0, ..., i, :] = m - 1 if lead[0] > 1 else a[0, ..., i, :]
+    return a
+
+
+@pytest.mark.parametrize(
+    "logN,bits,pbits,nb",
+    [
+        (10, (50,), 60, 3),                     # one digit, whose only modulus is its own
+        (10, (30, 30), 31, 5),                  # the special prime below 2^50 as well
+        (11, (50, 40, 30), 60, 2),              # source moduli far above the target's: the coefficient is folded first
+        (12, (50,) * 4, 60, 4),                 # four items per CTA, one round
+        (12, (50,) * 4, 60, 5),                 # and a remainder
+        (11, (58, 54, 45, 45, 45), 62, 3),      # every arithmetic class, two items per CTA
+        (10, (45,) * 9, 60, 2),                 # more than eight digits: two exact sums per position
+        (13, (50,) * 4, 60, 1),
+        (15, (50, 50), 60, 2),                  # second lift round of three stages
+    ],
+)
+def test_rotate_sum_on_edge_residues(logN, bits, pbits, nb):
+    import torch
+
+    from paper_2608_21131_b200 import binding as b
+
+    q = []
+    for w in bits:
+        q.append(next(x for x in find_primes(w, logN + 1, len(bits)) if x not in q))
+    p = next(x for x in find_primes(pbits, logN + 1, len(bits) + 1) if x not in q)
+    R, B = 16, 4
+    ps = synth.ParamSet("edge", logN, tuple(q), p, 20, R, B, 0)
+    G, N, L = ps.G, ps.N, ps.L
+    rots = [1, 2, 3] + [g * B for g in range(1, G)]
+    c, o = b.Context(ps), make_oracle(ps)
+    km = synth.key_material(ps, logN, rots=rots)
+    evk = {r: o.evk_gen(km.s, r, km.evk_a[i], km.evk_e[i]) for i, r in enumerate(rots)}
+    c.load_keys(np.stack([evk[r] for r in rots]), rots)
+    inner = edge_residues(7, q, N, (nb * G, 2))
+    dev = c.import_(b.KIND_CT, inner, nb * G)
+    ws = c.workspace(nb)
+    giant = np.stack([evk[g * B] for g in range(1, G)])
+    inner = inner.reshape(nb, G, 2, L, N)
+    want = np.stack([o.rotate_sum(inner[i], evk[B]) for i in range(nb)])
+    want_lazy = np.stack([o.rotate_sum_lazy(inner[i], giant) for i in range(nb)])
+    odd = c.alloc(dev.numel() * 8 + 8)[1:]
+    odd.copy_(dev)
+    for src in (dev, odd):
+        assert np.array_equal(c.export(b.KIND_CT, c.rotate_sum(src, nb, ws), nb), want)
+        assert np.array_equal(c.export(b.KIND_CT, c.rotate_sum_lazy(src, nb, ws), nb), want_lazy)
+    # the hoisted rotations: three keys, one digit set
+    baby = c.query_prepare(dev[: 2 * L * N], ws)
+    got = c.export(b.KIND_CT, baby, B)
+    for r in (1, 2, 3):
+        assert np.array_equal(got[r], o.rotate(inner[0, 0], r, evk[r])), r
+    torch.cuda.synchronize()
