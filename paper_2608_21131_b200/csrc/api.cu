@@ -356,12 +356,10 @@ extern "C" int hann_ctx_create(const hann_params* prm, hann_ctx** out) {
     // encode tables
     const int nh = std::max(n / 2, 1);
     std::vector<double2> T(nh), U(n);
-    c->hU_re.resize(n); c->hU_im.resize(n); c->h_uidx.resize(n);
     for (int t = 0; t < nh; t++) { double cs, sn; hm::unit_root(t, n, &cs, &sn); T[t] = make_double2(cs, -sn + 0.0); }
     for (int k = 0; k < n; k++) {
         double cs, sn; hm::unit_root(k, 2L * N, &cs, &sn);
         U[k] = make_double2(cs, -sn + 0.0);
-        c->hU_re[k] = U[k].x; c->hU_im[k] = U[k].y;
     }
     std::vector<int32_t> jinv(n);
     std::vector<unsigned> gal(n);
@@ -369,7 +367,6 @@ extern "C" int hann_ctx_create(const hann_params* prm, hann_ctx** out) {
         long g = 1;
         for (int j = 0; j < n; j++) {
             gal[j] = (unsigned)g;
-            c->h_uidx[j] = (int32_t)((g - 1) / 4);
             jinv[(g - 1) / 4] = j;
             g = (g * 5) % (2L * N);
         }
@@ -1004,46 +1001,40 @@ extern "C" int hann_encrypt_query(hann_ctx* c, const int8_t* s, const float* q, 
     return HANN_OK;
 }
 
-// count ciphertexts of nl limbs each, ct [count][2][nl][N] canonical, plaintext scale 1 / inv_scale
-static int decrypt_impl(hann_ctx* c, const int8_t* s, const uint64_t* ct, int64_t count, int nl, long double inv_scale,
-                        double* scores, double* imag_or_null) {
+// count ciphertexts of nl limbs each, ct [count][2][nl][N] canonical, plaintext scale 2^-exp2 / mult, in pieces of up to eight
+// ciphertexts
+static int decrypt_impl(hann_ctx* c, const int8_t* s, const uint64_t* ct, int64_t count, int nl, u64 mult, int exp2, double* scores,
+                        double* imag_or_null) {
     const int N = c->N, n = c->n;
     DeviceGuard dg(c->device);
-    const int64_t LN = (int64_t)nl * N;
-    RET(ensure_scratch(c, 4 * LN * 8 + align256(N) + kSlack));
+    const int64_t LN = (int64_t)nl * N, piece = std::max<int64_t>(1, std::min<int64_t>(count, 8));
+    RET(ensure_scratch(c, (LN + piece * (2 * LN + N + 2 * n)) * 8 + align256(N) + kSlack));
     Arena ar{(char*)c->scratch, 0, c->scratch_bytes};
     u64* shat = ar.take<u64>(LN);
-    u64* CT = ar.take<u64>(2 * LN);
-    u64* MU = ar.take<u64>(LN);
+    u64* C0 = ar.take<u64>(piece * LN);
+    u64* C1 = ar.take<u64>(piece * LN);
+    double2* buf = ar.take<double2>(piece * n);
+    double* re = ar.take<double>(piece * n);
+    double* im = ar.take<double>(piece * n);
     int8_t* s8 = ar.take<int8_t>(N);
     const LimbMap lm = limbmap_first(nl);
     CK(cudaMemcpyAsync(s8, s, N, cudaMemcpyHostToDevice, c->stream));
     RET(launch_lift_i8(c, s8, nl, shat));
     RET(launch_ntt_fwd(c, shat, nl, N, lm));
-    std::vector<u64> mu(LN);
-    std::vector<long double> real(N);
-    std::vector<double> re(n), im(n);
-    for (int64_t i = 0; i < count; i++) {
-        CK(cudaMemcpyAsync(CT, ct + i * 2 * LN, 2 * LN * 8, cudaMemcpyDefault, c->stream));
-        RET(launch_ntt_fwd(c, CT, 2 * nl, N, lm));
-        RET(launch_mul(c, CT + LN, shat, nl, MU, nl, lm));   // c1 * s
-        RET(launch_add(c, MU, CT, MU, nl, lm));              // + c0
-        RET(launch_ntt_inv(c, MU, nl, N, lm));
-        CK(cudaMemcpyAsync(mu.data(), MU, LN * 8, cudaMemcpyDeviceToHost, c->stream));
+    for (int64_t i0 = 0; i0 < count; i0 += piece) {
+        const int64_t np = std::min(piece, count - i0);
+        for (int64_t i = 0; i < np; i++) {
+            const uint64_t* src = ct + (i0 + i) * 2 * LN;
+            CK(cudaMemcpyAsync(C1 + i * LN, src + LN, LN * 8, cudaMemcpyDefault, c->stream));
+            CK(cudaMemcpyAsync(C0 + i * LN, src, LN * 8, cudaMemcpyDefault, c->stream));
+        }
+        RET(launch_ntt_fwd(c, C1, np * nl, N, lm));
+        RET(launch_mul(c, C1, shat, nl, C1, np * nl, lm));  // c1 * s; c0 is added in the coefficient domain
+        RET(launch_ntt_inv(c, C1, np * nl, N, lm));
+        RET(launch_decode(c, C0, C1, np, nl, mult, exp2, buf, re, imag_or_null ? im : nullptr));
+        CK(cudaMemcpyAsync(scores + i0 * n, re, (size_t)np * n * 8, cudaMemcpyDeviceToHost, c->stream));
+        if (imag_or_null) CK(cudaMemcpyAsync(imag_or_null + i0 * n, im, (size_t)np * n * 8, cudaMemcpyDeviceToHost, c->stream));
         RET(sync_and_check(c));
-        hm::crt_to_real(mu.data(), nl, N, c->mod, real.data());
-        // slots: a_k = (mu_k + i mu_{k+n}) conj(U[k]);  z_j * scale = sum_k a_k exp(+2 pi i u_j k / n)
-        for (int k = 0; k < n; k++) {
-            const double mr = (double)(real[k] * inv_scale), mi = (double)(real[k + n] * inv_scale);
-            const double ur = c->hU_re[k], ui = -c->hU_im[k];
-            re[k] = mr * ur - mi * ui;
-            im[k] = mr * ui + mi * ur;
-        }
-        hm::fft_inplace(re.data(), im.data(), n, c->logN - 1, +1);
-        for (int j = 0; j < n; j++) {
-            scores[i * n + j] = re[c->h_uidx[j]];
-            if (imag_or_null) imag_or_null[i * n + j] = im[c->h_uidx[j]];
-        }
     }
     return HANN_OK;
 }
@@ -1052,7 +1043,7 @@ extern "C" int hann_decrypt_scores(hann_ctx* c, const int8_t* s, const uint64_t*
                                    double* scores, double* imag_or_null) {
     if (!c) return HANN_EINVAL;
     if (!s || !ct || !scores || count < 0) return fail(c, HANN_EINVAL, "hann_decrypt_scores: bad argument");
-    return decrypt_impl(c, s, ct, count, c->L, ldexpl(1.0L, -log_scale_out), scores, imag_or_null);
+    return decrypt_impl(c, s, ct, count, c->L, 1, -log_scale_out, scores, imag_or_null);
 }
 
 extern "C" int hann_decrypt_compact(hann_ctx* c, const int8_t* s, const uint64_t* ct, int64_t count, int limbs, int rescaled,
@@ -1060,9 +1051,7 @@ extern "C" int hann_decrypt_compact(hann_ctx* c, const int8_t* s, const uint64_t
     if (!c) return HANN_EINVAL;
     if (!s || !ct || !scores || count < 0) return fail(c, HANN_EINVAL, "hann_decrypt_compact: bad argument");
     if (limbs < 1 || limbs > c->L - (rescaled ? 1 : 0)) return fail(c, HANN_ESHAPE, "hann_decrypt_compact: limb count out of range");
-    long double inv_scale = ldexpl(1.0L, -log_scale_in);
-    if (rescaled) inv_scale *= (long double)c->mod[c->L - 1];
-    return decrypt_impl(c, s, ct, count, limbs, inv_scale, scores, imag_or_null);
+    return decrypt_impl(c, s, ct, count, limbs, rescaled ? c->mod[c->L - 1] : 1, -log_scale_in, scores, imag_or_null);
 }
 
 // ================================================================================================ server side

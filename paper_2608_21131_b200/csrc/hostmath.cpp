@@ -1,5 +1,5 @@
-// Host-side mathematics of the library: parameter validation, roots of unity, table values, and the client's
-// CRT reconstruction and slot decoding.  None of this is on the per-query device path.
+// Host-side mathematics of the library: parameter validation, roots of unity, table values and the seeded generators.  None of this
+// is on the per-query device path.
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -118,115 +118,6 @@ void unit_root(long t, long den, double* c, double* s) {
     }
     *c += 0.0;  // turn -0.0 into +0.0
     *s += 0.0;
-}
-
-// ---- CRT -------------------------------------------------------------------------------------------------
-// Garner's mixed-radix digits, then Horner evaluation in multi-word integers, centring against Q/2 and
-// conversion to long double.
-
-namespace {
-struct Big {
-    u64 w[HANN_MAXL1 + 1];
-    int n;
-};
-void big_zero(Big& b, int n) {
-    b.n = n;
-    memset(b.w, 0, sizeof(b.w));
-}
-void big_mul_add(Big& b, u64 m, u64 a) {  // b = b*m + a
-    u128 carry = a;
-    for (int i = 0; i < b.n; i++) {
-        u128 t = (u128)b.w[i] * m + carry;
-        b.w[i] = (u64)t;
-        carry = t >> 64;
-    }
-}
-int big_cmp(const Big& a, const Big& b) {
-    for (int i = a.n - 1; i >= 0; i--)
-        if (a.w[i] != b.w[i]) return a.w[i] < b.w[i] ? -1 : 1;
-    return 0;
-}
-void big_sub(Big& a, const Big& b) {  // a -= b (a >= b)
-    u64 borrow = 0;
-    for (int i = 0; i < a.n; i++) {
-        u64 bi = b.w[i], ai = a.w[i];
-        u64 d = ai - bi - borrow;
-        borrow = (ai < bi || (ai == bi && borrow)) ? 1 : 0;
-        a.w[i] = d;
-    }
-}
-void big_half(Big& a) {
-    for (int i = 0; i < a.n; i++) a.w[i] = (a.w[i] >> 1) | (i + 1 < a.n ? a.w[i + 1] << 63 : 0);
-}
-long double big_to_ld(const Big& a) {
-    long double v = 0;
-    for (int i = a.n - 1; i >= 0; i--) v = v * 18446744073709551616.0L + (long double)a.w[i];
-    return v;
-}
-}  // namespace
-
-void crt_to_real(const u64* res, int L, int N, const u64* q, long double* out) {
-    // inv[i][k] = q_k^{-1} mod q_i for k < i
-    std::vector<u64> inv((size_t)L * L, 0);
-    for (int i = 0; i < L; i++)
-        for (int k = 0; k < i; k++) inv[(size_t)i * L + k] = invmod(q[k] % q[i], q[i]);
-    Big Q, halfQ;
-    big_zero(Q, L + 1);
-    Q.w[0] = 1;
-    for (int i = 0; i < L; i++) big_mul_add(Q, q[i], 0);
-    halfQ = Q;
-    big_half(halfQ);
-    for (int x = 0; x < N; x++) {
-        u64 v[HANN_MAXL1];
-        for (int i = 0; i < L; i++) {
-            // v_i = (((r_i - v_0) / q_0 - v_1) / q_1 - ...) mod q_i
-            u64 t = res[(size_t)i * N + x] % q[i];
-            for (int k = 0; k < i; k++) {
-                u64 vk = v[k] % q[i];
-                t = t >= vk ? t - vk : t + q[i] - vk;
-                t = mulmod(t, inv[(size_t)i * L + k], q[i]);
-            }
-            v[i] = t;
-        }
-        Big X;
-        big_zero(X, L + 1);
-        for (int i = L - 1; i >= 0; i--) big_mul_add(X, q[i], v[i]);  // X = v_0 + q_0 (v_1 + q_1 (v_2 + ...))
-        if (big_cmp(X, halfQ) > 0) {
-            Big D = Q;
-            big_sub(D, X);
-            out[x] = -big_to_ld(D);
-        } else {
-            out[x] = big_to_ld(X);
-        }
-    }
-}
-
-// plain radix-2 complex FFT (decode only; its result is compared within a tolerance, never bit for bit)
-void fft_inplace(double* re, double* im, int n, int logn, int sign) {
-    for (int i = 0; i < n; i++) {
-        int j = bitrev(i, logn);
-        if (i < j) {
-            std::swap(re[i], re[j]);
-            std::swap(im[i], im[j]);
-        }
-    }
-    for (int len = 2; len <= n; len <<= 1) {
-        std::vector<double> wr(len / 2), wi(len / 2);
-        for (int t = 0; t < len / 2; t++) {
-            const double ang = 2.0 * M_PI * t / len;
-            wr[t] = std::cos(ang);
-            wi[t] = sign * std::sin(ang);
-        }
-        for (int k0 = 0; k0 < n; k0 += len)
-            for (int t = 0; t < len / 2; t++) {
-                int a = k0 + t, b = a + len / 2;
-                double yr = re[b] * wr[t] - im[b] * wi[t], yi = re[b] * wi[t] + im[b] * wr[t];
-                re[b] = re[a] - yr;
-                im[b] = im[a] - yi;
-                re[a] += yr;
-                im[a] += yi;
-            }
-    }
 }
 
 static u64 mix64(u64 x) {

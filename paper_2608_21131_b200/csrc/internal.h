@@ -59,9 +59,6 @@ struct hann_ctx {
     int32_t* jinv = nullptr;   // [n]   slot j feeding FFT input position pos: jinv[pos] = j with u_j = brev(pos), u_j = (5^j mod 2N - 1)/4
     unsigned* galois_dev = nullptr;  // [n] 5^r mod 2N
     std::vector<unsigned> h_galois;
-    // host copies used by decode
-    std::vector<double> hU_re, hU_im;
-    std::vector<int32_t> h_uidx;
     // evaluation keys by rotation: device buffers [L][2][L+1][N], transformed and permuted by the inverse
     // automorphism so that the key-switch inner product reads keys and digits contiguously
     std::vector<u64*> keytab_host;
@@ -125,9 +122,6 @@ u64 find_psi(u64 q, int N);
 u64 shoup(u64 w, u64 q);  // floor(w * 2^64 / q)
 int bitrev(int x, int bits);
 void unit_root(long t, long den, double* c, double* s);  // exp(2 pi i t/den), correctly rounded
-// residues [L][N] -> centred integers in (-Q/2, Q/2] as long double
-void crt_to_real(const u64* res, int L, int N, const u64* q, long double* out);
-void fft_inplace(double* re, double* im, int n, int logn, int sign);
 u64 hash64(u64 seed, u64 stream, u64 ctr);  // the 64-bit counter hash of the seeded calls (see hann_expand_uniform)
 void seeded_ternary(u64 seed, u64 stream, int N, int8_t* s);                       // uniform on {-1, 0, 1}
 void seeded_gaussian(u64 seed, u64 stream, u64 ctr0, long count, double sigma, int8_t* e);  // rounded Gaussian (Box-Muller)
@@ -219,7 +213,8 @@ LimbMap limbmap_first(int nlimbs);  // period nlimbs: limbs 0..nlimbs-1
 // helpers of the client half
 int launch_lift_i8(hann_ctx* c, const int8_t* v, int nlimbs, u64* out);
 int launch_mul(hann_ctx* c, const u64* a, const u64* b, int bperiod, u64* out, int64_t npoly, const LimbMap& lm);
-int launch_add(hann_ctx* c, const u64* a, const u64* b, u64* out, int64_t npoly, const LimbMap& lm);
+// decode.cu: decrypted polynomials c0 + prod (coefficient domain) -> slots
+int launch_decode(hann_ctx* c, const u64* c0, const u64* prod, int64_t count, int L, u64 mult, int exp2, double2* buf, double* re, double* im);
 int launch_evk_finish(hann_ctx* c, const u64* as_coeff, const int8_t* e, const int8_t* sprime, u64* b_out);
 int launch_encrypt_finish(hann_ctx* c, const u64* as_coeff, const int8_t* e, const u64* m, u64* c0_out);
 // a[L][N] = counter hash of (seed, stream, l*N + x) mod q_l (coefficient domain, canonical)

@@ -427,16 +427,6 @@ __global__ void __launch_bounds__(kThreads) k_mul(const u64* __restrict__ a, con
     }
 }
 
-// out[p][x] = a[p][x] + b[p][x] mod limb(p)
-__global__ void __launch_bounds__(kThreads) k_add(const u64* __restrict__ a, const u64* __restrict__ b,
-                                                  u64* __restrict__ out, long long npoly, int N, LimbMap lm, LimbTable lt) {
-    const long long total = npoly * N;
-    for (long long idx = (long long)blockIdx.x * kThreads + threadIdx.x; idx < total; idx += (long long)gridDim.x * kThreads) {
-        const long long p = idx / N;
-        out[idx] = addmod(a[idx], b[idx], lt.c[lm.limb[p % lm.period]].q);
-    }
-}
-
 // evaluation key finish, coefficient domain: b[j][i][x] = -as[j][i][x] + e[j][x] + (i == j ? (p mod q_j) * s'[x] : 0)
 __global__ void __launch_bounds__(kThreads) k_evk_finish(const u64* __restrict__ as, const int8_t* __restrict__ e,
                                                          const int8_t* __restrict__ sprime, u64* __restrict__ b_out,
@@ -837,14 +827,6 @@ int launch_mul(hann_ctx* c, const u64* a, const u64* b, int bperiod, u64* out, i
         k_mul<<<grid_for(npoly * c->N), kThreads, 0, c->stream>>>(a, b, bperiod, out, npoly, c->N, lm, c->lt);
     }
     return check_launch(c, "mul");
-}
-
-int launch_add(hann_ctx* c, const u64* a, const u64* b, u64* out, int64_t npoly, const LimbMap& lm) {
-    {
-        KProf kp(c, KC_OTHER);
-        k_add<<<grid_for(npoly * c->N), kThreads, 0, c->stream>>>(a, b, out, npoly, c->N, lm, c->lt);
-    }
-    return check_launch(c, "add");
 }
 
 int launch_evk_finish(hann_ctx* c, const u64* as_coeff, const int8_t* e, const int8_t* sprime, u64* b_out) {

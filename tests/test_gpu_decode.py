@@ -1,0 +1,62 @@
+"""hann_decrypt_scores / hann_decrypt_compact on ciphertexts that are plaintexts (c1 = 0) of chosen integers: the CRT has to give every
+centred integer exactly, rounded to binary64 once, for every chain length and for integers at the ends of their range; the slots are
+compared with a binary64 FFT of the exactly rounded coefficients."""
+import random
+
+import numpy as np
+import pytest
+
+from oracle.oracle import find_primes
+from paper_2608_21131_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def slots(coeffs, logN):
+    """sum over k of m_k zeta_j^k at the canonical slots, from n complex numbers (m_k + i m_{k+n}) exp(i pi k / N)"""
+    n, N = 1 << (logN - 1), 1 << logN
+    a = (coeffs[:n] + 1j * coeffs[n:]) * np.exp(1j * np.pi * np.arange(n) / N)
+    u, g = [], 1
+    for _ in range(n):
+        u.append((g - 1) // 4)
+        g = g * 5 % (2 * N)
+    return (n * np.fft.ifft(a))[u]
+
+
+@pytest.mark.parametrize("logN,bits,count", [(4, (50,), 1), (5, (62, 61), 3), (9, (50, 45, 40), 9), (10, (50,) * 4, 17), (9, (58, 45, 45, 45, 45), 2),
+                                             (11, (45,) * 9, 2), (10, (61,) * 15, 1)])
+def test_decoded_slots_of_chosen_integers(logN, bits, count):
+    from paper_2608_21131_b200 import binding as b
+
+    q = []
+    for w in bits:
+        q.append(next(x for x in find_primes(w, logN + 1, 16) if x not in q))
+    p = next(x for x in find_primes(60, logN + 1, 16) if x not in q)
+    ps = synth.ParamSet("dec", logN, tuple(q), p, 20, 4, 2, 0)
+    c = b.Context(ps)
+    N, L = ps.N, ps.L
+    s = synth.key_material(ps, 1, rots=[]).s
+    rng = random.Random(logN * 100 + L)
+    for limbs, rescaled in [(L, False)] + ([(max(1, L - 1), True)] if L > 1 else []):
+        Q = 1
+        for x in q[:limbs]:
+            Q *= x
+        ct = np.zeros((count, 2, limbs, N), dtype=np.uint64)
+        mult, log_scale = (q[-1] if rescaled else 1), Q.bit_length()
+        exact = np.zeros((count, N))
+        for i in range(count):
+            # the ends of the range, small integers, numbers halfway between two binary64, then uniform ones of every size
+            m = [Q // 2, -(Q // 2), 0, 1, -1, (1 << 53) + 1, -(1 << 53) - 1, 3 << 52]
+            m += [rng.randrange(-(Q // 2), Q // 2 + 1) >> rng.randrange(0, Q.bit_length()) for _ in range(N - len(m))]
+            m = [(x + Q // 2) % Q - Q // 2 for x in m]
+            for l in range(limbs):
+                ct[i, 0, l] = [x % q[l] for x in m]
+            exact[i] = [x * mult / (1 << log_scale) for x in m]  # a quotient of integers is rounded once
+        if rescaled:
+            got, imag = c.decrypt_compact(s, ct, True, log_scale_in=log_scale, want_imag=True)
+        else:
+            got, imag = c.decrypt_scores(s, ct, log_scale_out=log_scale, want_imag=True)
+        for i in range(count):
+            want = slots(exact[i], logN)
+            # logN - 1 butterfly stages and the twist, each a rounding or two of relative size 2^-53, on either side
+            assert np.linalg.norm(got[i] + 1j * imag[i] - want) <= 8 * logN * 2.0 ** -53 * np.linalg.norm(want)
