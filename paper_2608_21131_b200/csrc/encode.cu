@@ -10,6 +10,9 @@
 // Two kernels: pass 1 runs the stages that stay inside contiguous chunks of S1 = 2^b1 points (the input gather
 // z_j -> position brev(u_j) is folded into its loads); pass 2 runs the remaining stages on column tiles of the
 // (n/S1) x S1 matrix view, then twists, rounds, reduces modulo every ciphertext prime and writes residues.
+#include <algorithm>
+#include <cstring>
+
 #include "internal.h"
 #include "debugcheck.cuh"
 
@@ -209,6 +212,7 @@ struct FusedArgs {
     long long out_stride;
     const double2* tw;   // forward transform twiddles, binary64 format, [L+1][N]
     const LimbConst* lt;
+    int half_hi;         // high word of the smallest floor(q / 2): a coefficient whose high word lies below it needs no reduction
 };
 
 __device__ __forceinline__ void dit(double2& x, double2& y, double2 w) {
@@ -497,6 +501,228 @@ __global__ void __launch_bounds__(256, HANN_X_MINBLOCKS) k_encode_x(FusedArgs A)
     }
 }
 
+// ---- real slot vectors at half the FFT ---------------------------------------------------------------------------------
+//
+// The FFT of a real sequence is Hermitian, X_{n-k} = conj(X_k), bit for bit: the twiddle table is symmetric to the last bit and
+// separately rounded products commute with conjugation.  So every sub-transform is kept as its first half (frequencies 0 .. S/2),
+// a stage combines only those, and products by the exact table entries 1 and -i are moves.  Kernel W8H leaves 128 complex words
+// per chunk of 256 points (word 0: the two real frequencies 0 and 128); kernel H runs the strided stages on columns 1 .. 128
+// (and 0) only, and takes the coefficients of column 256 - c from those of column c: with m_k + i m_{k+n} the rounded words of
+// frequency k, m_{n-k} = -m_{k+n} and m_{2n-k} = -m_k.
+//
+// Per block of 128 plaintexts (N = 2^16, L = 4), inside a level of seven blocks: k_fft_w8 / k_encode_x<4, 4, true> 31 and 95 us, these
+// 24 and 81 us; the FP64 pipe and the latency of the gather bound them.  Below five stages in pass A (N = 2^12) kernel H has
+// half the CTAs and lost (15 against 10 us for 128 plaintexts of the toy ring): those rings keep the other pair.
+
+__global__ void __launch_bounds__(128, 5) k_fft_w8h(FusedArgs A) {
+    __shared__ double2 tc[256];
+    __shared__ double2 sm[8 * 153];                 // [plaintext][frequency 0..8][sub-transform 0..15], 17 words per frequency
+    float* sin_ = (float*)(sm + 8 * 153) - 8 * 272;  // gathered inputs, as in k_fft_w8
+    const int n = 1 << A.logn;
+    const int P0 = blockIdx.y * 8;
+    const int g = (A.p_first + P0) / A.B, b0 = (A.p_first + P0) % A.B;
+    const int chunk = blockIdx.x;
+    for (int i = threadIdx.x; i < 255; i += 128) {
+        const int s = 32 - __clz(i + 1);
+        const int h = 1 << (s - 1), t = i - (h - 1);
+        tc[i] = A.T[(long long)t << (A.logn - s)];
+    }
+#pragma unroll
+    for (int i = 0; i < 16; i++) {
+        const int idx = threadIdx.x + 128 * i, p = idx >> 3, pl = idx & 7;
+        const int jj = A.jinv[(chunk << 8) + p];
+        int row = jj - g * A.B;
+        if (row < 0) row += n;
+        const int col = (jj + b0 + pl) % A.R;
+        sin_[pl * 272 + p + (p >> 4)] = (row < A.rows_in_block && col < A.dim) ? A.rows[(long long)row * A.dim + col] : 0.0f;
+    }
+    __syncthreads();
+    {
+        // stages 1 .. 4: the sub-transform of sixteen real numbers, frequencies 0 .. 8
+        const int pl = threadIdx.x >> 4, j = threadIdx.x & 15;
+        double re[16], im[16];
+#pragma unroll
+        for (int e = 0; e < 16; e++) re[e] = (double)sin_[pl * 272 + 17 * j + e];
+#pragma unroll
+        for (int s = 0; s < 4; s++) {
+            const int h = 1 << s;
+#pragma unroll
+            for (int b = 0; b < 16; b += 2 * h) {
+                const double e0 = re[b], o0 = re[b + h];
+                re[b] = __dadd_rn(e0, o0);
+                re[b + h] = __dsub_rn(e0, o0);
+#pragma unroll
+                for (int t = 1; 2 * t < h; t++) {
+                    const double2 v = cmul_rn(make_double2(re[b + h + t], im[b + h + t]), tc[h - 1 + t]);
+                    const double er = re[b + t], ei = im[b + t];
+                    re[b + t] = __dadd_rn(er, v.x);
+                    im[b + t] = __dadd_rn(ei, v.y);
+                    re[b + h - t] = __dsub_rn(er, v.x);
+                    im[b + h - t] = -__dsub_rn(ei, v.y);
+                }
+                if (h >= 2) im[b + h / 2] = -re[b + h + h / 2];
+            }
+        }
+        im[0] = im[8] = 0.0;
+        double2* d = sm + pl * 153 + j;
+        __syncthreads();  // every thread has read its gathered inputs: the tile may be overwritten
+#pragma unroll
+        for (int t = 0; t <= 8; t++) d[17 * t] = make_double2(re[t], im[t]);
+    }
+    __syncthreads();
+    // stages 5 .. 8 on frequencies 0 .. 8 of the sixteen sub-transforms
+    if (threadIdx.x < 72) {
+        const int pl = threadIdx.x / 9, t = threadIdx.x % 9;
+        double2 x[16];
+#pragma unroll
+        for (int e = 0; e < 16; e++) x[e] = sm[pl * 153 + 17 * t + e];
+#pragma unroll
+        for (int s = 0; s < 4; s++) {
+            const int span = 1 << s;
+#pragma unroll
+            for (int e = 0; e < 16; e++)
+                if (!(e & span)) dit(x[e], x[e + span], tc[16 * span - 1 + t + 16 * (e & (span - 1))]);
+        }
+        double2* o = A.buf + (long long)(P0 + pl) * (n >> 1) + ((long long)chunk << 7);
+        if (t == 0) x[0].y = x[8].x;
+#pragma unroll
+        for (int e = 0; e < 8; e++) {
+            o[t + 16 * e] = x[e];
+            if (t != 0 && t != 8) o[16 - t + 16 * e] = make_double2(x[15 - e].x, -x[15 - e].y);
+        }
+    }
+}
+
+// R1 = 4; a = 4 + R2, R2 >= 1.  A CTA is 128 threads on CW = 128 >> R2 columns c = first .. first + CW - 1 of 1 .. 128 and their mirror
+// images; CTA blockIdx.x = 2^R2 takes column 0 of CW plaintexts.  A thread holds the coefficients of eight rows of a column,
+// runs the first transform round for the column and for its mirror image, and one second round.
+template <int R2>
+__global__ void __launch_bounds__(128, 5) k_encode_h(FusedArgs A, int count) {
+    extern __shared__ u64 smx[];
+    constexpr int a = 4 + R2, G1 = 1 << R2, logCW = 7 - R2, CW = 1 << logCW, NT = 1 << a;
+    const int n = 1 << A.logn;
+    const bool special = blockIdx.x == G1;
+    if (special && (blockIdx.y & (CW - 1))) return;
+    const int ci = threadIdx.x & (CW - 1), g = threadIdx.x >> logCW;
+    const int c0 = special ? 0 : 1 + (blockIdx.x << logCW);
+    // plaintext and column of a CTA column
+    const auto plaintext = [&](int cc) { return special ? (int)blockIdx.y + cc : (int)blockIdx.y; };
+    const auto column = [&](int cc) { return special ? 0 : c0 + cc; };
+    const auto word = [&](int row, int cc) -> double2 {
+        const int P = plaintext(cc), c = column(cc);
+        if (P >= count) return make_double2(0.0, 0.0);
+        const double2 v = A.buf[(long long)P * (n >> 1) + ((long long)row << 7) + (c & 127)];
+        return c == 0 ? make_double2(v.x, 0.0) : c == 128 ? make_double2(v.y, 0.0) : v;
+    };
+    double2* smc = (double2*)smx;  // [8 G1 rows][CW]
+    double2* twc = (double2*)(smx + 2048);
+    {
+        constexpr int E = 1 << R2;
+#pragma unroll
+        for (int w = threadIdx.x; w < 8 * CW; w += 128) {
+            const int cc = w & (CW - 1), gg = w >> logCW, c = column(cc);
+            double2 x[E];
+#pragma unroll
+            for (int e = 0; e < E; e++) x[e] = word((gg << R2) + e, cc);
+#pragma unroll
+            for (int t = 0; t < R2; t++) {
+                const int span = 1 << t;
+#pragma unroll
+                for (int e = 0; e < E; e++)
+                    if (!(e & span)) dit(x[e], x[e + span], A.T[(long long)((e & (span - 1)) * 256 + c) << (a - 2 - t)]);
+            }
+#pragma unroll
+            for (int e = 0; e < E; e++) smc[(((gg << R2) + e) << logCW) + cc] = x[e];
+        }
+    }
+    for (int i = threadIdx.x; i < A.L * NT; i += 128) {
+        const int l = i / NT, e = i % NT;
+        if (e) twc[i] = A.tw[((size_t)l << (A.logn + 1)) + e];
+    }
+    __syncthreads();
+    // last FFT round (three stages) on rows g + G1 e, then twist, scale, round
+    double m[16];  // m[e], m[e + 8]: rounded real and imaginary part of row g + G1 e
+    const int c = column(ci);
+    {
+        double2 x[8];
+#pragma unroll
+        for (int e = 0; e < 8; e++) x[e] = smc[((g + G1 * e) << logCW) + ci];
+#pragma unroll
+        for (int u = 0; u < 3; u++) {
+            const int span = 1 << u, t = R2 + u;
+#pragma unroll
+            for (int e = 0; e < 8; e++)
+                if (!(e & span)) dit(x[e], x[e + span], A.T[(long long)((g + G1 * (e & (span - 1))) * 256 + c) << (a - 2 - t)]);
+        }
+#pragma unroll
+        for (int e = 0; e < 8; e++) {
+            const double2 cc = cmul_rn(x[e], A.U[(g + G1 * e) * 256 + c]);
+            m[e] = rint(__dmul_rn(cc.x, A.scale));
+            m[e + 8] = rint(__dmul_rn(cc.y, A.scale));
+        }
+    }
+    // coefficients below half the smallest prime (the case of rows of moderate norm) enter the transforms as they are
+    int top = 0;
+#pragma unroll
+    for (int e = 0; e < 16; e++) top = max(top, __double2hiint(m[e]) & 0x7fffffff);
+    const bool small = top < A.half_hi;
+    const bool mirror = !special && c != 128;
+    // tile word of (row, column): columns 0 .. CW - 1 direct, CW .. 2 CW - 1 mirror images; odd rows swap halves of sixteen
+    const auto tile = [&](int row, int cc) -> u64& { return smx[(row << (logCW + 1)) + (cc ^ ((row & 1) << 3))]; };
+    for (int l = 0; l < A.L; l++) {
+        const ArithF64 ar(A.lt + l);
+        const double2* tw = twc + l * NT;
+        const double2 w1 = tw[1];
+        __syncthreads();  // the twiddle cache is filled, the FFT tile read (first limb) / the exchange tile is free again
+        {
+            double x[8];
+#pragma unroll
+            for (int e = 0; e < 8; e++)
+                x[e] = small ? __dadd_rn(m[e], ar.mulmod_small(m[e + 8], w1)) : __dadd_rn(ar.reduce(m[e]), ar.mulmod_small(ar.reduce(m[e + 8]), w1));
+            fwd_round<3, ArithF64, 3>(ar, x, tw, 2u);
+#pragma unroll
+            for (int e = 0; e < 8; e++) tile(g + G1 * e, ci) = ar.to_exch(x[e]);
+        }
+        if (mirror) {
+            // rows G1 - 1 - g + G1 e of column 256 - c: row r' = 8 G1 - 1 - r
+            double x[8];
+#pragma unroll
+            for (int e = 0; e < 8; e++) {
+                const double mr = -m[15 - e], mi = -m[7 - e];
+                x[e] = small ? __dadd_rn(mr, ar.mulmod_small(mi, w1)) : __dadd_rn(ar.reduce(mr), ar.mulmod_small(ar.reduce(mi), w1));
+            }
+            fwd_round<3, ArithF64, 3>(ar, x, tw, 2u);
+#pragma unroll
+            for (int e = 0; e < 8; e++) tile(G1 - 1 - g + G1 * e, CW + ci) = ar.to_exch(x[e]);
+        }
+        __syncthreads();
+        // second round: 8 groups of 2^R2 rows x 2 CW columns
+#pragma unroll
+        for (int w = threadIdx.x; w < 16 * CW; w += 128) {
+            const int cc = w & (2 * CW - 1), gg = w >> (logCW + 1), cs = cc & (CW - 1), cl = column(cs);
+            const bool mir = cc >= CW;
+            if (plaintext(cs) >= count || (mir && (special || cl == 128))) continue;
+            u64* base = A.out + ((long long)plaintext(cs) * A.L + l) * A.out_stride + (mir ? 256 - cl : cl);
+            double x[1 << R2];
+#pragma unroll
+            for (int e = 0; e < (1 << R2); e++) x[e] = ar.from_mid(tile((gg << R2) + e, cc));
+            fwd_round<R2, ArithF64, 1>(ar, x, tw, (unsigned)(16 + gg));
+#pragma unroll
+            for (int e = 0; e < (1 << R2); e++) base[(size_t)((gg << R2) + e) * 256] = ar.to_mid(x[e]);
+        }
+    }
+}
+
+typedef void (*KernH)(FusedArgs, int);
+KernH pick_h(int a) {
+    switch (a) {
+        case 5: return k_encode_h<1>;
+        case 6: return k_encode_h<2>;
+        case 7: return k_encode_h<3>;
+        default: return k_encode_h<4>;
+    }
+}
+
 typedef void (*KernX)(FusedArgs);
 template <bool SYM>
 KernX pick_x_t(int a) {
@@ -547,6 +773,22 @@ int launch_encode_rows_fused(hann_ctx* c, const float* rows, int64_t rows_in_blo
     A.lt = c->lt_dev;
     const int n = c->n, a = c->logN - 8;
     const int chunks = n >> 8;  // >= 1 because logN >= 9
+    if (sym && a >= 5 && c->B % 8 == 0 && count % 8 == 0 && p_first % 8 == 0) {
+        double half = 0x1p52;
+        for (int l = 0; l < c->L; l++) half = std::min(half, (double)(c->mod[l] / 2));
+        long long bits;
+        memcpy(&bits, &half, 8);
+        A.half_hi = (int)(bits >> 32);
+        {
+            KProf kp(c, KC_FFT_A);
+            k_fft_w8h<<<dim3(chunks, count / 8), 128, 0, c->stream>>>(A);
+        }
+        KProf kp(c, KC_FFT_B);
+        const size_t smem = 16384 + (size_t)c->L * (1 << a) * 16;
+        if (smem > 48 * 1024) cudaFuncSetAttribute(pick_h(a), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        pick_h(a)<<<dim3((1 << (a - 4)) + 1, count), 128, smem, c->stream>>>(A, count);
+        return check_launch(c, "encode_half");
+    }
     if (c->B % 8 == 0 && count % 8 == 0 && p_first % 8 == 0) {
         KProf kp(c, KC_FFT_A);
         k_fft_w8<<<dim3(chunks, count / 8), 128, 0, c->stream>>>(A);

@@ -1,0 +1,41 @@
+"""hann_encode_candidates against the oracle's encoding, exactly, over the rings and plaintext counts at which its kernels change: pass A of
+four to eight stages, fewer plaintexts than columns of a CTA, rows small enough to skip the reduction of their coefficients and rows that
+are not, ragged blocks and padded dimensions, baby-step counts that are and are not multiples of eight."""
+import numpy as np
+import pytest
+
+from oracle.oracle import find_primes
+from paper_2608_21131_b200 import synth
+from tests.helpers import make_oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("logN,R,B,bits,norm,dim,short", [
+    (12, 8, 8, (50, 50), 1.0, 8, 0),           # four stages: full transforms of the slots
+    (13, 8, 8, (50, 40), 1.0, 8, 1),           # five; eight plaintexts, sixty-four columns a CTA
+    (13, 16, 8, (30, 30, 30), 1.0, 11, 700),   # coefficients above half the 30-bit primes
+    (14, 16, 16, (50,), 1.0, 16, 4000),
+    (14, 16, 8, (50, 50), 600.0, 13, 5),       # some coefficients of 2^49 and more, others below
+    (15, 8, 8, (50, 45), 1.0, 8, 16000),
+    (16, 8, 8, (50, 50), 1.0, 7, 3),
+    (16, 8, 8, (50,), 3000.0, 8, 0),
+    (14, 16, 4, (50,), 1.0, 12, 9),            # baby steps not a multiple of eight
+])
+def test_encoded_candidates_equal_the_oracle(logN, R, B, bits, norm, dim, short):
+    import torch
+
+    from paper_2608_21131_b200 import binding as b
+
+    q = []
+    for w in bits:
+        q.append(next(x for x in find_primes(w, logN + 1, len(bits)) if x not in q))
+    ps = synth.ParamSet("enc", logN, tuple(q), next(x for x in find_primes(60, logN + 1, 8) if x not in q), 40, R, B, 0)
+    c, o = b.Context(ps), make_oracle(ps)
+    rng = np.random.default_rng(logN * 7 + R)
+    rows = (norm * synth.normalise(rng.standard_normal((ps.n - short, dim)))).astype(np.float32)
+    full = np.zeros((ps.n, R), dtype=np.float32)
+    full[: rows.shape[0], :dim] = rows
+    want = o.encode_block(full).reshape(R, ps.L, ps.N)
+    pt = c.encode_candidates(torch.from_numpy(rows).to(c.device), c.workspace(1))
+    assert np.array_equal(c.export(b.KIND_PT, pt, R).reshape(R, ps.L, ps.N), want)
