@@ -122,15 +122,17 @@ struct Timer {
 };
 
 int64_t ks_item_words(const hann_ctx* c) {
-    // per item: c1 coefficients, digits, u, lifted, one temporary ciphertext
+    // per item: c1 coefficients, digits (without those modulo their own prime where the fused kernels run), u, lifted, one
+    // temporary ciphertext
     const int64_t L = c->L, N = c->N;
-    return L * N + L * (L + 1) * N + 2 * (L + 1) * N + 2 * L * N + 2 * L * N;
+    return L * N + L * (ks_fused_available(c) ? L : L + 1) * N + 2 * (L + 1) * N + 2 * L * N + 2 * L * N;
 }
 
-// words of workspace the lazy rotate-and-sum needs per block of a round: G-1 terms (c1 coefficients, digits, key product)
-// and one ModDown (special-prime limb of the sum, its lift)
+// words of workspace the lazy rotate-and-sum needs per block of a round: G-1 terms (c1 coefficients, digits, and their key products
+// unless the fused kernels sum them), the summed product and one ModDown
 int64_t lazy_block_words(const hann_ctx* c) {
     const int64_t L = c->L, N = c->N, G1 = c->G - 1;
+    if (ks_fused_available(c)) return G1 * (L * N + L * L * N) + 2 * (L + 1) * N + 2 * L * N;
     return G1 * (L * N + L * (L + 1) * N + 2 * (L + 1) * N) + 2 * N + 2 * L * N;
 }
 
@@ -140,6 +142,12 @@ int64_t prepare_words(const hann_ctx* c) {
 }
 
 constexpr int64_t kSlack = 16 * 256;  // room for the alignment of a dozen sub-buffers
+
+// items per round when `total` items go through in rounds of at most `most`: as few rounds, as even as they can be
+int64_t balanced(int64_t most, int64_t total) {
+    const int64_t rounds = (total + most - 1) / most;
+    return (total + rounds - 1) / rounds;
+}
 
 // the four sub-buffers of ONE key switch (hann_keyswitch, hann_keyswitch_static): input copy, digits, u, lifted
 struct KsBuffers {
@@ -1220,11 +1228,11 @@ extern "C" int hann_score_level_ctdb(hann_ctx* c, const void* baby_dev, const vo
     int64_t ch = ((int64_t)ws_bytes - kSlack) / per;
     if (ch < 1) return fail(c, HANN_EWORKSPACE, "hann_score_level_ctdb: workspace too small");
     const int64_t items = n_blocks * G;
-    ch = std::min<int64_t>(std::min<int64_t>(ch, items), 8 * G);
+    ch = balanced(std::min<int64_t>(ch, 8 * G), items);
     Arena ar{(char*)ws, 0, (int64_t)ws_bytes, c};
     u64* d = ar.take<u64>(ch * 3 * LN);
     u64* c1c = ar.take<u64>(ch * LN);
-    u64* digits = ar.take<u64>(ch * L * L1N);
+    u64* digits = ar.take<u64>(ch * L * (ks_fused_available(c) ? LN : L1N));
     u64* u = ar.take<u64>(ch * 2 * L1N);
     u64* lifted = ar.take<u64>(ch * 2 * LN);
     if (!d || !c1c || !digits || !u || !lifted) return fail(c, HANN_EWORKSPACE, "hann_score_level_ctdb: workspace too small");
@@ -1263,11 +1271,11 @@ extern "C" int hann_multiply(hann_ctx* c, const void* a_dev, const void* b_dev, 
     const int64_t per = (3 * LN + ks_item_words(c)) * 8;
     int64_t ch = ((int64_t)ws_bytes - kSlack) / per;
     if (ch < 1) return fail(c, HANN_EWORKSPACE, "hann_multiply: workspace too small");
-    ch = std::min<int64_t>(std::min<int64_t>(ch, count), 32);
+    ch = balanced(std::min<int64_t>(ch, 32), count);
     Arena ar{(char*)ws, 0, (int64_t)ws_bytes, c};
     u64* d = ar.take<u64>(ch * 3 * LN);
     u64* c1c = ar.take<u64>(ch * LN);
-    u64* digits = ar.take<u64>(ch * L * L1N);
+    u64* digits = ar.take<u64>(ch * L * (ks_fused_available(c) ? LN : L1N));
     u64* u = ar.take<u64>(ch * 2 * L1N);
     u64* lifted = ar.take<u64>(ch * 2 * LN);
     if (!d || !c1c || !digits || !u || !lifted) return fail(c, HANN_EWORKSPACE, "hann_multiply: workspace too small");
@@ -1312,10 +1320,10 @@ extern "C" int hann_rotate_sum(hann_ctx* c, const void* inner_dev, int64_t n_blo
     auto run_range = [&](int64_t b_lo, int64_t b_hi, char* wsp, int64_t wsp_bytes) -> int {
         int64_t ch = (wsp_bytes - kSlack) / (ks_item_words(c) * 8);
         if (ch < 1) return fail(c, HANN_EWORKSPACE, "hann_rotate_sum: workspace too small");
-        ch = std::min<int64_t>(std::min<int64_t>(ch, b_hi - b_lo), 8);
+        ch = balanced(std::min<int64_t>(ch, 8), b_hi - b_lo);
         Arena ar{wsp, 0, wsp_bytes, c};
         u64* c1c = ar.take<u64>(ch * LN);
-        u64* digits = ar.take<u64>(ch * L * L1N);
+        u64* digits = ar.take<u64>(ch * L * (fused ? LN : L1N));
         u64* u = ar.take<u64>(ch * 2 * L1N);
         u64* lifted = ar.take<u64>(ch * 2 * LN);
         u64* tmp = ar.take<u64>(ch * ctw);
@@ -1344,10 +1352,15 @@ extern "C" int hann_rotate_sum(hann_ctx* c, const void* inner_dev, int64_t n_blo
         }
         return HANN_OK;
     };
-    // Blocks are independent: up to four ranges run side by side on the context's stream and the helper streams, each in
-    // its own part of the workspace, which keeps the machine busy through the many small launches of a key switch.
-    // (One lane while the per-launch profile is on, so that its kernel times do not overlap.)
+    // Blocks are independent: two ranges run side by side on the context's stream and a helper stream, each in its own part of
+    // the workspace, so that the short launches of a key switch overlap.  Rings of 2^10 points and more do that above 2^17 points or
+    // sixteen blocks: below, one round of all blocks fills the machine better (us of a level in one / two / four ranges: four
+    // blocks of 2^15 850 / 880 / 892, eight 1373 / 1347 / 1391; three of 2^12 327 / 361 / 387, sixteen 844 / 845 / 979, twenty-nine
+    // 1629 / 1373 / 1884; two of 2^16 1106 / 1114 / 1111, three 1335 / 1321 / 1353).
+    // (One lane while the per-launch profile is on, so that its kernel times do not overlap; with guards on always two, so that
+    // they cover both carvings.)
     int lanes = (int)std::min<int64_t>(c->max_lanes, n_blocks);
+    if (fused) lanes = n_blocks * c->N <= (1 << 17) && n_blocks <= 16 && !c->canaries ? 1 : std::min(lanes, 2);
     if (c->stream == c->aux_stream || c->kprof) lanes = 1;
     while (lanes > 1 && (((int64_t)ws_bytes / lanes) & ~(int64_t)255) < ks_item_words(c) * 8 + kSlack) lanes--;
     if (lanes <= 1) return run_range(0, n_blocks, (char*)ws, (int64_t)ws_bytes);
@@ -1399,13 +1412,13 @@ extern "C" int hann_rotate_sum_lazy(hann_ctx* c, const void* inner_dev, int64_t 
     auto run_range = [&](int64_t b_lo, int64_t b_hi, char* wsp, int64_t wsp_bytes) -> int {
         int64_t ch = (wsp_bytes - kSlack) / (lazy_block_words(c) * 8);
         if (ch < 1) return fail(c, HANN_EWORKSPACE, "hann_rotate_sum_lazy: workspace too small");
-        ch = std::min<int64_t>(std::min<int64_t>(ch, b_hi - b_lo), 16);
+        ch = balanced(std::min<int64_t>(ch, 16), b_hi - b_lo);
         Arena ar{wsp, 0, wsp_bytes, c};
         const int64_t items_max = ch * (G - 1);
         u64* c1c = ar.take<u64>(items_max * LN);
-        u64* digits = ar.take<u64>(items_max * L * L1N);
-        u64* u = ar.take<u64>(items_max * 2 * L1N);
-        u64* up = ar.take<u64>(ch * 2 * N);
+        u64* digits = ar.take<u64>(items_max * L * (fused ? LN : L1N));
+        u64* u = ar.take<u64>((fused ? ch : items_max) * 2 * L1N);
+        u64* up = fused ? u : ar.take<u64>(ch * 2 * N);
         u64* lifted = ar.take<u64>(ch * 2 * LN);
         if (!c1c || !digits || !u || !up || !lifted) return fail(c, HANN_EWORKSPACE, "hann_rotate_sum_lazy: workspace too small");
         for (int64_t b0 = b_lo; b0 < b_hi; b0 += ch) {

@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(kThreads) k_fft_a(EncArgs A) {
         if (A.rows) {
             int row = j - g * A.B;
             if (row < 0) row += n;
-            int col = (j + b) % A.R;
+            int col = (j + b) & (A.R - 1);  // R divides a power of two
             v = (row < A.rows_in_block && col < A.dim) ? (double)A.rows[(long long)row * A.dim + col] : 0.0;
         } else {
             v = A.z[(long long)P * n + j];
@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(128) k_fft_w(FusedArgs A) {
             const int jj = A.jinv[pos0 + e];
             int row = jj - g * A.B;
             if (row < 0) row += n;
-            const int col = (jj + b) % A.R;
+            const int col = (jj + b) & (A.R - 1);  // R divides a power of two
             const double v = (row < A.rows_in_block && col < A.dim) ? (double)A.rows[(long long)row * A.dim + col] : 0.0;
             x[e] = make_double2(v, 0.0);
         }
@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(128, 5) k_fft_w8(FusedArgs A) {
         const int jj = A.jinv[(chunk << 8) + p];
         int row = jj - g * A.B;
         if (row < 0) row += n;
-        const int col = (jj + b0 + pl) % A.R;
+        const int col = (jj + b0 + pl) & (A.R - 1);  // R divides a power of two
         sin_[pl * 272 + p + (p >> 4)] = (row < A.rows_in_block && col < A.dim) ? A.rows[(long long)row * A.dim + col] : 0.0f;
     }
     __syncthreads();
@@ -533,7 +533,7 @@ __global__ void __launch_bounds__(128, 5) k_fft_w8h(FusedArgs A) {
         const int jj = A.jinv[(chunk << 8) + p];
         int row = jj - g * A.B;
         if (row < 0) row += n;
-        const int col = (jj + b0 + pl) % A.R;
+        const int col = (jj + b0 + pl) & (A.R - 1);  // R divides a power of two
         sin_[pl * 272 + p + (p >> 4)] = (row < A.rows_in_block && col < A.dim) ? A.rows[(long long)row * A.dim + col] : 0.0f;
     }
     __syncthreads();
