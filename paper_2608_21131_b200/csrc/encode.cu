@@ -294,6 +294,7 @@ __global__ void __launch_bounds__(128, 5) k_fft_w8(FusedArgs A) {
     const int P0 = blockIdx.y * 8;
     const int g = (A.p_first + P0) / A.B, b0 = (A.p_first + P0) % A.B;
     const int chunk = blockIdx.x;
+    chain_wait();
     for (int i = threadIdx.x; i < 255; i += 128) {
         const int s = 32 - __clz(i + 1);
         const int h = 1 << (s - 1), t = i - (h - 1);
@@ -365,6 +366,7 @@ __global__ void __launch_bounds__(256, HANN_X_MINBLOCKS) k_encode_x(FusedArgs A)
     const int c0 = blockIdx.x << 4;
     const double2* in = A.buf + (long long)P * n + c0;
     double2* smc = (double2*)smx;  // [rows_fft][16]
+    chain_wait();
     if (R2 > 0) {
         // FFT round of R2 stages: rows gg*2^R2 + e, spans 1 .. 2^(R2-1) rows
         constexpr int E = 1 << (R2 == 0 ? 1 : R2);
@@ -527,6 +529,7 @@ __global__ void __launch_bounds__(128, 5) k_fft_w8h(FusedArgs A) {
         const int h = 1 << (s - 1), t = i - (h - 1);
         tc[i] = A.T[(long long)t << (A.logn - s)];
     }
+    chain_wait();
 #pragma unroll
     for (int i = 0; i < 16; i++) {
         const int idx = threadIdx.x + 128 * i, p = idx >> 3, pl = idx & 7;
@@ -602,6 +605,7 @@ __global__ void __launch_bounds__(128, 5) k_encode_h(FusedArgs A, int count) {
     constexpr int a = 4 + R2, G1 = 1 << R2, logCW = 7 - R2, CW = 1 << logCW, NT = 1 << a;
     const int n = 1 << A.logn;
     const bool special = blockIdx.x == G1;
+    chain_wait();
     if (special && (blockIdx.y & (CW - 1))) return;
     const int ci = threadIdx.x & (CW - 1), g = threadIdx.x >> logCW;
     const int c0 = special ? 0 : 1 + (blockIdx.x << logCW);
@@ -781,17 +785,17 @@ int launch_encode_rows_fused(hann_ctx* c, const float* rows, int64_t rows_in_blo
         A.half_hi = (int)(bits >> 32);
         {
             KProf kp(c, KC_FFT_A);
-            k_fft_w8h<<<dim3(chunks, count / 8), 128, 0, c->stream>>>(A);
+            launch_chain(c, k_fft_w8h, dim3(chunks, count / 8), 128, 0, A);
         }
         KProf kp(c, KC_FFT_B);
         const size_t smem = 16384 + (size_t)c->L * (1 << a) * 16;
         if (smem > 48 * 1024) cudaFuncSetAttribute(pick_h(a), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        pick_h(a)<<<dim3((1 << (a - 4)) + 1, count), 128, smem, c->stream>>>(A, count);
+        launch_chain(c, pick_h(a), dim3((1 << (a - 4)) + 1, count), 128, smem, A, count);
         return check_launch(c, "encode_half");
     }
     if (c->B % 8 == 0 && count % 8 == 0 && p_first % 8 == 0) {
         KProf kp(c, KC_FFT_A);
-        k_fft_w8<<<dim3(chunks, count / 8), 128, 0, c->stream>>>(A);
+        launch_chain(c, k_fft_w8, dim3(chunks, count / 8), 128, 0, A);
     } else if (chunks % kWChunks == 0) {
         KProf kp(c, KC_FFT_A);
         k_fft_w<<<dim3(chunks / kWChunks, count), 128, 0, c->stream>>>(A);
@@ -820,7 +824,7 @@ int launch_encode_rows_fused(hann_ctx* c, const float* rows, int64_t rows_in_blo
         KProf kp(c, KC_FFT_B);
         const int threads = a >= 8 ? 256 : (a == 7 ? 128 : 64);  // 16 columns x 2^R2 row groups, at least two warps
         if (smem > 48 * 1024) cudaFuncSetAttribute(pick_x(a, sym), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        pick_x(a, sym)<<<dim3(16, count), threads, smem, c->stream>>>(A);
+        launch_chain(c, pick_x(a, sym), dim3(16, count), threads, smem, A);
     }
     return check_launch(c, "encode_fused");
 }

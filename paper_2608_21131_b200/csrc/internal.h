@@ -112,6 +112,30 @@ struct KProf {
     }
 };
 
+// Programmatic dependent launch of the kernels of a chain, which are a few microseconds each on small levels: such a kernel is set up
+// while the one before it in the stream still runs, and waits in chain_wait -- called by every thread, before its first access to
+// anything an earlier kernel of the stream wrote and before its first store -- until that one has completed and its stores are
+// visible.  No kernel lets its successor start early (griddepcontrol.launch_dependents): the waiting CTAs then hold slots that other
+// streams and the kernel's own tail need.  Us of a pass, plain launches / these / these with an early start: toy level 322 / 228 /
+// 241, coarse 773 / 763 / 802, projection 1055 / 976 / 1074, eight queries 5661 / 5626 / 5768, membership 8892 / 8438 / 8591.
+#ifdef __CUDACC__
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <class... KA, class... A>
+void launch_chain(hann_ctx* c, void (*kern)(KA...), dim3 grid, int threads, size_t smem, A&&... args) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = c->stream;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kern, KA(args)...);
+}
+#endif
+
 // ---- host mathematics (hostmath.cpp)
 namespace hm {
 u64 mulmod(u64 a, u64 b, u64 q);

@@ -47,6 +47,7 @@ __global__ void __launch_bounds__(kThreads) k_ks_inner(const u64* __restrict__ d
                                                        const u64* const* __restrict__ keytab, int rot0, int rot_inc,
                                                        u64* __restrict__ u, int N, int L, long long nitems,
                                                        LimbTable lt, int f64) {
+    chain_wait();
     const long long L1N = (long long)(L + 1) * N;
     const long long total = nitems * L1N;
     for (long long idx = (long long)blockIdx.x * kThreads + threadIdx.x; idx < total; idx += (long long)gridDim.x * kThreads) {
@@ -217,6 +218,7 @@ __global__ void __launch_bounds__(128) k_ks_inner_stream(const u64* __restrict__
     u += (long long)blockIdx.z * nitems * 2 * L1N;
     const long long it0 = (long long)blockIdx.y * items_per_cta;
     const long long it1 = it0 + items_per_cta < nitems ? it0 + items_per_cta : nitems;
+    chain_wait();
     if (it0 >= it1) return;
     // a CTA lies inside one limb, so the choice is uniform
     if (lc.q < (1ULL << 50) && f64) ks_inner_body<LL, KEYS_STREAM, 3>(digits, digit_stride, keytab, rot0, rot_inc, u, L1N, pos, it0, it1, lc);
@@ -533,6 +535,7 @@ struct LinearArgs {
 // b_period > 0: b has only b_period words (one ciphertext) and is used for every ciphertext of a.
 __global__ void __launch_bounds__(kThreads) k_linear(const u64* __restrict__ a, const u64* __restrict__ b, u64* __restrict__ out,
                                                      long long npoly, int limbs, int N, long long b_period, LinearArgs la, LimbTable lt) {
+    chain_wait();
     const long long total = npoly * limbs * N;
     for (long long idx = (long long)blockIdx.x * kThreads + threadIdx.x; idx < total; idx += (long long)gridDim.x * kThreads) {
         const int l = (int)((idx / N) % limbs);
@@ -552,6 +555,7 @@ __global__ void __launch_bounds__(kThreads) k_linear(const u64* __restrict__ a, 
 // in the transform domain
 __global__ void __launch_bounds__(kThreads) k_mul_ct(const u64* __restrict__ a, const u64* __restrict__ b, u64* __restrict__ d,
                                                      long long count, int limbs, int N, LimbTable lt) {
+    chain_wait();
     const long long LN = (long long)limbs * N, total = count * LN;
     for (long long idx = (long long)blockIdx.x * kThreads + threadIdx.x; idx < total; idx += (long long)gridDim.x * kThreads) {
         const long long i = idx / LN, pos = idx % LN;
@@ -593,7 +597,7 @@ int check_launch(hann_ctx* c, const char* what) {
 int launch_mul_ct(hann_ctx* c, const u64* a, const u64* b, int64_t count, u64* d) {
     {
         KProf kp(c, KC_MAC);
-        k_mul_ct<<<grid_for(count * c->L * c->N), kThreads, 0, c->stream>>>(a, b, d, count, c->L, c->N, c->lt);
+        launch_chain(c, k_mul_ct, dim3(grid_for(count * c->L * c->N)), kThreads, 0, a, b, d, count, c->L, c->N, c->lt);
     }
     return check_launch(c, "mul_ct");
 }
@@ -609,7 +613,7 @@ int launch_linear(hann_ctx* c, const u64* a, long long ma, const u64* b, long lo
     }
     {
         KProf kp(c, KC_OTHER);
-        k_linear<<<grid_for(npoly * c->L * c->N), kThreads, 0, c->stream>>>(a, b, out, npoly, c->L, c->N, b_period, la, c->lt);
+        launch_chain(c, k_linear, dim3(grid_for(npoly * c->L * c->N)), kThreads, 0, a, b, out, npoly, c->L, c->N, b_period, la, c->lt);
     }
     return check_launch(c, "linear");
 }
@@ -642,12 +646,8 @@ void launch_ks_inner_stream(hann_ctx* c, const u64* digits, int64_t digit_stride
     const int per = (int)((nitems + split - 1) / split);
     split = (int)((nitems + per - 1) / per);
     KProf kp(c, digit_stride == 0 && nitems > 1 ? KC_KS_INNER_KEYS : KC_KS_INNER);  // streamed keys timed on their own
-    if (digit_stride == 0)
-        k_ks_inner_stream<LL, true><<<dim3(tiles, split, nz), 128, 0, c->stream>>>(digits, 0, c->keytab_dev, rot0, rot_inc, u, c->N, nitems,
-                                                                                per, c->lt_dev, rot_zinc, c->mac_f64);
-    else
-        k_ks_inner_stream<LL, false><<<dim3(tiles, split, nz), 128, 0, c->stream>>>(digits, digit_stride, c->keytab_dev, rot0, rot_inc, u,
-                                                                                 c->N, nitems, per, c->lt_dev, rot_zinc, c->mac_f64);
+    launch_chain(c, digit_stride == 0 ? k_ks_inner_stream<LL, true> : k_ks_inner_stream<LL, false>, dim3(tiles, split, nz), 128, 0, digits,
+                 digit_stride, c->keytab_dev, rot0, rot_inc, u, c->N, nitems, per, c->lt_dev, rot_zinc, c->mac_f64);
 }
 
 int launch_ks_inner(hann_ctx* c, const u64* digits, int64_t digit_stride, int rot0, int rot_inc, int64_t nitems, u64* u) {
@@ -664,8 +664,7 @@ int launch_ks_inner(hann_ctx* c, const u64* digits, int64_t digit_stride, int ro
     }
     {
         KProf kp(c, KC_KS_INNER);
-        k_ks_inner<<<grid_for(nitems * (c->L + 1) * c->N), kThreads, 0, c->stream>>>(digits, digit_stride, c->keytab_dev, rot0, rot_inc, u,
-                                                                                   c->N, c->L, nitems, c->lt, c->mac_f64);
+        launch_chain(c, k_ks_inner, dim3(grid_for(nitems * (c->L + 1) * c->N)), kThreads, 0, digits, digit_stride, c->keytab_dev, rot0, rot_inc, u, c->N, c->L, nitems, c->lt, c->mac_f64);
     }
     return check_launch(c, "ks_inner");
 }
@@ -749,6 +748,7 @@ int launch_moddown_combine(hann_ctx* c, const u64* u, const u64* lifted, int64_t
 // lifted[poly][i][x] = centred lift of t[poly][x] (residue mod q_{L-1}, coefficient domain) reduced mod q_i, i < keep
 __global__ void __launch_bounds__(kThreads) k_rescale_lift(const u64* __restrict__ t, u64* __restrict__ lifted, int N, int L,
                                                            int keep, long long npoly, LimbTable lt) {
+    chain_wait();
     const long long total = npoly * N;
     const u64 ql = lt.c[L - 1].q, half = lt.c[L - 1].half;
     for (long long idx = (long long)blockIdx.x * kThreads + threadIdx.x; idx < total; idx += (long long)gridDim.x * kThreads) {
@@ -772,6 +772,7 @@ struct RescaleConst {
 __global__ void __launch_bounds__(kThreads) k_rescale_combine(const u64* __restrict__ src, const u64* __restrict__ lifted,
                                                               u64* __restrict__ out, int N, int L, int keep, long long npoly,
                                                               LimbTable lt, RescaleConst rc) {
+    chain_wait();
     const long long total = npoly * keep * N;
     for (long long idx = (long long)blockIdx.x * kThreads + threadIdx.x; idx < total; idx += (long long)gridDim.x * kThreads) {
         const int x = (int)(idx % N);
@@ -786,7 +787,7 @@ __global__ void __launch_bounds__(kThreads) k_rescale_combine(const u64* __restr
 int launch_rescale_lift(hann_ctx* c, const u64* t, int64_t npoly, int keep, u64* lifted) {
     {
         KProf kp(c, KC_OTHER);
-        k_rescale_lift<<<grid_for(npoly * c->N), kThreads, 0, c->stream>>>(t, lifted, c->N, c->L, keep, npoly, c->lt);
+        launch_chain(c, k_rescale_lift, dim3(grid_for(npoly * c->N)), kThreads, 0, t, lifted, c->N, c->L, keep, npoly, c->lt);
     }
     return check_launch(c, "rescale_lift");
 }
@@ -800,7 +801,7 @@ int launch_rescale_combine(hann_ctx* c, const u64* src, const u64* lifted, int64
     }
     {
         KProf kp(c, KC_OTHER);
-        k_rescale_combine<<<grid_for(npoly * keep * c->N), kThreads, 0, c->stream>>>(src, lifted, out, c->N, c->L, keep, npoly, c->lt, rc);
+        launch_chain(c, k_rescale_combine, dim3(grid_for(npoly * keep * c->N)), kThreads, 0, src, lifted, out, c->N, c->L, keep, npoly, c->lt, rc);
     }
     return check_launch(c, "rescale_combine");
 }
@@ -851,6 +852,7 @@ int launch_rlk_finish(hann_ctx* c, const u64* as_coeff, const int8_t* e, const u
 namespace {
 __global__ void __launch_bounds__(kThreads) k_copy2d(u64* __restrict__ dst, long long dst_pitch, const u64* __restrict__ src,
                                                      long long src_pitch, long long width, long long rows) {
+    chain_wait();
     const long long total = rows * width;
     for (long long idx = (long long)blockIdx.x * kThreads + threadIdx.x; idx < total; idx += (long long)gridDim.x * kThreads) {
         const long long r = idx / width, x = idx % width;
@@ -860,7 +862,7 @@ __global__ void __launch_bounds__(kThreads) k_copy2d(u64* __restrict__ dst, long
 }  // namespace
 int launch_copy2d(hann_ctx* c, u64* dst, int64_t dst_pitch, const u64* src, int64_t src_pitch, int64_t width, int64_t rows) {
     if (width <= 0 || rows <= 0) return HANN_OK;
-    k_copy2d<<<grid_for(width * rows), kThreads, 0, c->stream>>>(dst, dst_pitch, src, src_pitch, width, rows);
+    launch_chain(c, k_copy2d, dim3(grid_for(width * rows)), kThreads, 0, dst, dst_pitch, src, src_pitch, width, rows);
     return check_launch(c, "copy2d");
 }
 

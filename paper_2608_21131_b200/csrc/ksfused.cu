@@ -132,17 +132,18 @@ __global__ void __launch_bounds__(T, 640 / T) k_ks_apply(ApplyArgs A) {
                            : A.digits + (((z * A.items + it0 + it) * L + dj) * A.n_tgt + (A.n_tgt > L || i < dj ? i : i - 1)) * N;
         p += (sc << 8);
         if (z) __syncthreads();  // the products of the previous rotation have been taken
-        double x[16];  // binary64 or integer words alike
-        if (valid) {
-#pragma unroll
-            for (int e = 0; e < 16; e++) x[e] = __longlong_as_double((long long)p[j + 16 * e]);
-        }
         stage_keys(ks, A.keytab[A.rot0 + z * A.rot_zinc] + (long long)i * N + (sc << 8), L1N, L);
         if (staged != sc) {
             if (f64) stage_twiddles(tc, (const double2*)A.tw_fwd_f64 + ((size_t)i << A.logN), m0 + sc);
             else stage_twiddles((ulonglong2*)tc, (const ulonglong2*)A.tw_fwd_int + ((size_t)i << A.logN), m0 + sc);
         }
         staged = sc;
+        if (z == 0) chain_wait();
+        double x[16];  // binary64 or integer words alike
+        if (valid) {
+#pragma unroll
+            for (int e = 0; e < 16; e++) x[e] = __longlong_as_double((long long)p[j + 16 * e]);
+        }
         __syncthreads();
         if (valid && own) {  // canonical words of the transform itself
 #pragma unroll
@@ -312,6 +313,7 @@ __global__ void __launch_bounds__(256, 3) k_ks_finish(FinishArgs A) {
     const u64 pinv_i = lc->pinv, pinv_s = lc->pinv_s;
     if (f64) stage_twiddles(tc, (const double2*)A.tw_fwd_f64 + ((size_t)i << A.logN), m0 + t);
     else stage_twiddles((ulonglong2*)tc, (const ulonglong2*)A.tw_fwd_int + ((size_t)i << A.logN), m0 + t);
+    chain_wait();
     __syncthreads();
     const long long units = 2 * A.items, ustep = (long long)gridDim.z * (blockDim.x >> 4);
     for (long long v = (long long)blockIdx.z * (blockDim.x >> 4) + hw; v < units; v += ustep) {
@@ -411,7 +413,7 @@ void launch_apply(hann_ctx* c, const ApplyArgs& A) {
     const size_t smem = (size_t)4096 + (2 * A.L + (size_t)threads / 16 + 2 * IB) * 2048;
     cudaFuncSetAttribute(k_ks_apply<IB, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     KProf kp(c, KC_KS_INNER);
-    k_ks_apply<IB, T><<<dim3(c->N >> 8, A.L + 1, (unsigned)((A.items + IB - 1) / IB)), threads, smem, c->stream>>>(A);
+    launch_chain(c, k_ks_apply<IB, T>, dim3(c->N >> 8, A.L + 1, (unsigned)((A.items + IB - 1) / IB)), threads, smem, A);
 }
 
 }  // namespace
@@ -490,8 +492,7 @@ int launch_ks_finish(hann_ctx* c, const u64* u, const u64* lifted, int64_t items
     if (gz > groups) gz = groups;
     const dim3 grid(c->N >> 8, c->L, (unsigned)gz);
     KProf kp(c, KC_MODDOWN_COMBINE);
-    if (perm_items) k_ks_finish<true><<<grid, threads, smem, c->stream>>>(A);
-    else k_ks_finish<false><<<grid, threads, smem, c->stream>>>(A);
+    launch_chain(c, perm_items ? k_ks_finish<true> : k_ks_finish<false>, grid, threads, smem, A);
     return check_launch(c, "ks_finish");
 }
 

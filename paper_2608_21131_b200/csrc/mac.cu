@@ -243,6 +243,7 @@ __global__ void __launch_bounds__(32 * NG) k_mac_ct_stream(const u64* __restrict
     const long long pos0 = (long long)blockIdx.x * 32;
     const int lane = threadIdx.x & 31, wg = threadIdx.x >> 5;
     const LimbConst* lc = lt + pos0 / N;
+    chain_wait();
     unsigned w0[BB][2], w1[BB][2];
     double wd[BB][2];
     const double qd = (double)lc->q, halfd = (double)lc->half;
@@ -397,11 +398,15 @@ __global__ void __launch_bounds__(32 * NG) k_mac_bulk(const u64* __restrict__ ba
     const long long posv[2] = {(long long)limb * N + t0 + lane, (long long)limb * N + (N - 1 - t0 - lane)};
     const long long bg0 = (long long)blockIdx.y * bg_per_cta;
     const long long bg1 = bg0 + bg_per_cta < n_bg ? bg0 + bg_per_cta : n_bg;
-    if (bg0 >= bg1) return;
+    if (bg0 >= bg1) {
+        chain_wait();
+        return;
+    }
     const int npairs = (int)(bg1 - bg0);
     const unsigned bar0 = smem_addr(&bars[wg][0]), ring0 = smem_addr(&ring[wg][0][0][0]);
     const int row0 = (int)(bg0 * B + wg * BB);  // first plaintext row of this warp's pair 0; pair i starts B rows further
     if (threadIdx.x == 0) s_abort = 0;
+    chain_wait();
     if (lane == 0) {
         for (int st = 0; st < kMacStages; st++) mbar_init(bar0 + 8 * st, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -629,7 +634,7 @@ void launch_mac_stream(hann_ctx* c, const u64* baby, int64_t baby_stride, const 
         if (((uintptr_t)pt & 15) == 0 && n_bg * (NG * BB) < (1LL << 31) && plaintext_map(pt, Ln, n_bg * (NG * BB), BB, &map)) {
             auto go = [&](auto kern, size_t smem) {
                 if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                kern<<<dim3(tiles, split), 32 * NG, smem, c->stream>>>(baby, map, inner, c->N, c->L, n_bg, per, c->lt_dev, c->kflag);
+                launch_chain(c, kern, dim3(tiles, split), 32 * NG, smem, baby, map, inner, c->N, c->L, n_bg, per, c->lt_dev, c->kflag);
             };
             if (!c->mac_f64) go(k_mac_bulk<NG, BB, 0>, mac_bulk_smem<NG, BB, 0>());
             else if (big_primes) go(k_mac_bulk<NG, BB, 2>, mac_bulk_smem<NG, BB, 2>());
@@ -734,7 +739,7 @@ int launch_mac_ct(hann_ctx* c, const u64* baby, const u64* ctdb, int64_t n_bg, u
         split = (int)((n_bg + per - 1) / per);
         KProf kp(c, KC_MAC);
         const dim3 grid(tiles, split);
-        auto go = [&](auto kern, int threads) { kern<<<grid, threads, 0, c->stream>>>(baby, ctdb, inner3, c->N, c->L, n_bg, per, c->lt_dev); };
+        auto go = [&](auto kern, int threads) { launch_chain(c, kern, grid, threads, 0, baby, ctdb, inner3, c->N, c->L, n_bg, per, c->lt_dev); };
         if (c->mac_f64) {
             switch (c->B) {
                 case 4: go(k_mac_ct_stream<4, 1, true>, 128); break;

@@ -120,6 +120,7 @@ __global__ void __launch_bounds__(kThreads, AR::kMinBlocks) k_ntt_fwd_a(NttArgs 
     const Sel sel = select(A);
     const AR ar(A.lt + sel.limb);
     u64* base = A.data + sel.poly * A.stride + ((long long)blockIdx.x << A.logC);
+    chain_wait();
     fwd_a_body<R1, R2>(A, ar, base, (const typename AR::TW*)A.tw + ((size_t)sel.limb << A.logN), sm);
 }
 
@@ -300,6 +301,7 @@ __device__ __forceinline__ void fwd_b8t_body(const NttArgs& A, int groups, int* 
     const int my_tiles = yg0 < ntiles ? (ntiles - yg0 + ystep - 1) / ystep : 0;
     // tile i of this warp is valid when its polynomial exists (only the last tile can be ragged)
     auto tile_valid = [&](int i) { return i < my_tiles && (long long)(yg0 + (long long)i * ystep) * kTP + t < groups; };
+    chain_wait();
     if (lane == 0) {
         for (int i = 0; i < 2; i++)
             if (tile_valid(i)) {
@@ -411,6 +413,7 @@ __global__ void __launch_bounds__(256, 3) k_ntt_inv_b8t(NttArgs A, int groups, i
     };
     const int my_tiles = yg0 < ntiles ? (ntiles - yg0 + ystep - 1) / ystep : 0;
     auto tile_valid = [&](int i) { return i < my_tiles && (long long)(yg0 + (long long)i * ystep) * kTP + t < groups; };
+    chain_wait();
     if (lane == 0) {
         for (int i = 0; i < 2; i++)
             if (tile_valid(i)) {
@@ -583,6 +586,7 @@ __global__ void __launch_bounds__(kThreads, AR::kMinBlocks) k_ntt_inv_a(NttArgs 
     const Sel sel = select(A);
     const AR ar(A.lt + sel.limb);
     u64* base = A.data + sel.poly * A.stride + ((long long)blockIdx.x << A.logC);
+    chain_wait();
     inv_a_body<R1, R2>(A, ar, base, (const typename AR::TW*)A.tw + ((size_t)sel.limb << A.logN), sm);
 }
 
@@ -830,6 +834,7 @@ __global__ void __launch_bounds__(kLiftThreads, HANN_LIFT_MINBLOCKS) k_ks_lift(L
     const int sl = (int)((A.src_limb4 >> (4 * (sp % A.src_period))) & 15);
     const LimbConst* slc = A.lt + sl;
     const u64* sbase = A.src + sp * A.src_stride + c0;
+    chain_wait();
     u64* vs = sm + threadIdx.x;                        // [2^R1][128]: the thread's centred coefficients
     u64* tile = sm + (kLiftThreads << R1);             // exchange tile
     if (slc->q < (1ULL << 50)) {
@@ -929,21 +934,21 @@ void launch_fwd_b8t_mixed(hann_ctx* c, const NttArgs& Af, const NttArgs& Ai, int
     KProf kp(c, KC_NTT_FWD_B);
     cudaFuncSetAttribute(k_ntt_fwd_b8t_mixed, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kB8tSmem);
     const int ranges = (c->N >> 8) / kTK, ntiles = (groups + kTP - 1) / kTP, nsel = Af.nsel + Ai.nsel;
-    k_ntt_fwd_b8t_mixed<<<dim3(ranges, nsel, b8t_zsplit(ranges * nsel, ntiles)), 256, kB8tSmem, c->stream>>>(Af, Ai, groups, c->kflag);
+    launch_chain(c, k_ntt_fwd_b8t_mixed, dim3(ranges, nsel, b8t_zsplit(ranges * nsel, ntiles)), 256, kB8tSmem, Af, Ai, groups, c->kflag);
 }
 
 template <class AR>
 void launch_fwd_class(hann_ctx* c, const NttArgs& A, int groups, bool skip_a, bool skip_b = false) {
     if (A.a > 0 && !skip_a) {
         KProf kp(c, KC_NTT_FWD_A);
-        pick_fwd_a<AR>(A.a)<<<dim3(1 << (A.b - A.logC), groups * A.nsel), kThreads, smem_a(A), c->stream>>>(A);
+        launch_chain(c, pick_fwd_a<AR>(A.a), dim3(1 << (A.b - A.logC), groups * A.nsel), kThreads, smem_a(A), A);
     }
     if (skip_b) return;
     KProf kp(c, KC_NTT_FWD_B);
     if (b8t_eligible(c, A)) {
         cudaFuncSetAttribute(k_ntt_fwd_b8t<AR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kB8tSmem);
         const int ranges = ((c->N >> 8) / kTK) >> (A.half ? 1 : 0), ntiles = (groups + kTP - 1) / kTP;
-        k_ntt_fwd_b8t<AR><<<dim3(ranges, A.nsel, b8t_zsplit(ranges * A.nsel, ntiles)), 256, kB8tSmem, c->stream>>>(A, groups, c->kflag);
+        launch_chain(c, k_ntt_fwd_b8t<AR>, dim3(ranges, A.nsel, b8t_zsplit(ranges * A.nsel, ntiles)), 256, kB8tSmem, A, groups, c->kflag);
         return;
     }
     if (A.b == 8 && A.a > 0 && A.tau && ((c->N >> 8) % kBK) == 0) {
@@ -989,14 +994,14 @@ void launch_inv_class(hann_ctx* c, const NttArgs& A, int groups, bool skip_a) {
                 zs = z;
             }
         }
-        k_ntt_inv_b8t<AR><<<dim3(ranges, A.nsel, zs), 256, smem, c->stream>>>(A, groups, c->kflag);
+        launch_chain(c, k_ntt_inv_b8t<AR>, dim3(ranges, A.nsel, zs), 256, smem, A, groups, c->kflag);
     } else {
         KProf kp(c, KC_NTT_INV_B);
         pick_inv_b<AR>(A.b)<<<dim3((c->N >> A.b) / A.K, groups * A.nsel), kThreads, smem_b(A), c->stream>>>(A, A.a == 0 ? 1 : 0);
     }
     if (A.a > 0 && !skip_a) {
         KProf kp(c, KC_NTT_INV_A);
-        pick_inv_a<AR>(A.a)<<<dim3(1 << (A.b - A.logC), groups * A.nsel), kThreads, smem_a(A), c->stream>>>(A);
+        launch_chain(c, pick_inv_a<AR>(A.a), dim3(1 << (A.b - A.logC), groups * A.nsel), kThreads, smem_a(A), A);
     }
 }
 
@@ -1210,7 +1215,7 @@ int launch_ks_lift(hann_ctx* c, u64* src, int64_t src_stride, int64_t nsrc, cons
         Ap.src_limb4 = 0;
         for (int i = 0; i < src_lm.period && i < 16; i++) Ap.src_limb4 |= (u64)src_lm.limb[(s0 + i) % src_lm.period] << (4 * i);
         KProf kp(c, KC_LIFT_DIGITS);
-        pick_lift(a)<<<dim3(tiles, ns, lift_zsplit((long)tiles * ns, n_tgt)), kLiftThreads, smem, c->stream>>>(Ap);
+        launch_chain(c, pick_lift(a), dim3(tiles, ns, lift_zsplit((long)tiles * ns, n_tgt)), kLiftThreads, smem, Ap);
     }
     return check_launch(c, "ks_lift");
 }

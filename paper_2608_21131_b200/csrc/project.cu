@@ -52,6 +52,7 @@ __global__ void __launch_bounds__(kThreads) k_mask_combine(const u64* __restrict
                                                            const u64* __restrict__ rot_h, const u64* __restrict__ lo,
                                                            const u64* __restrict__ hi, u64* __restrict__ cyc, int Bn, int N, int L,
                                                            LimbTable lt) {
+    chain_wait();
     const long long LN = (long long)L * N, ctw = 2 * LN, total = (long long)Bn * ctw;
     const int n = N >> 1;
     for (long long idx = (long long)blockIdx.x * kThreads + threadIdx.x; idx < total; idx += (long long)gridDim.x * kThreads) {
@@ -89,8 +90,7 @@ int launch_window_masks(hann_ctx* c, int b, double* lo, double* hi) {
 int launch_mask_combine(hann_ctx* c, const u64* ct, const u64* rot_a, const u64* rot_h, const u64* lo, const u64* hi, u64* cyc) {
     {
         KProf kp(c, KC_OTHER);
-        k_mask_combine<<<grid_for((int64_t)c->B * 2 * c->L * c->N, 148 * 32), kThreads, 0, c->stream>>>(ct, rot_a, rot_h, lo, hi, cyc,
-                                                                                                      c->B, c->N, c->L, c->lt);
+        launch_chain(c, k_mask_combine, dim3(grid_for((int64_t)c->B * 2 * c->L * c->N, 148 * 32)), kThreads, 0, ct, rot_a, rot_h, lo, hi, cyc, c->B, c->N, c->L, c->lt);
     }
     return check_launch(c, "mask_combine");
 }
