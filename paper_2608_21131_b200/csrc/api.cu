@@ -337,11 +337,17 @@ extern "C" int hann_ctx_create(const hann_params* prm, hann_ctx** out) {
             lc.pmod = prm->p % q;
             lc.pinv = hm::invmod(lc.pmod, q);
             lc.pinv_s = hm::shoup(lc.pinv, q);
+            lc.linv = i + 1 < L ? hm::invmod(prm->q[L - 1] % q, q) : 0;
+            lc.linv_s = hm::shoup(lc.linv, q);
+            lc.linv_bal = lc.linv > q / 2 ? -(double)(q - lc.linv) : (double)lc.linv;
+            lc.linv_q = lc.linv_bal / (double)q;
             lc.pinv_bal = lc.pinv > q / 2 ? -(double)(q - lc.pinv) : (double)lc.pinv;
             lc.pinv_q = lc.pinv_bal / (double)q;
         } else {
             lc.pmod = 0; lc.pinv = 0; lc.pinv_s = 0;
             lc.pinv_bal = lc.pinv_q = 0;
+            lc.linv = lc.linv_s = 0;
+            lc.linv_bal = lc.linv_q = 0;
         }
         const u64 psi = hm::find_psi(q, N), ipsi = hm::invmod(psi, q);
         pw[0] = ipw[0] = 1;
@@ -814,6 +820,19 @@ extern "C" int hann_compact_scores(hann_ctx* c, const void* score_ct_dev, int64_
     if (!t || !lifted) return fail(c, HANN_EWORKSPACE, "hann_compact_scores: workspace too small");
     for (int64_t p0 = 0; p0 < npoly; p0 += ch) {
         const int64_t np = std::min(ch, npoly - p0);
+        const u64* last = src + (p0 * L + (L - 1)) * N;
+        if (ks_fused_available(c)) {
+            // a ModDown by the last ciphertext prime: its limb back to coefficients, lifted into the others, and combined
+            if (ntt_inv_pass_b_gathers(c, last, t)) {
+                RET(launch_ntt_inv_pass_b_from(c, last, (int64_t)L * N, t, np, N, limbmap_single(L - 1)));
+            } else {
+                RET(launch_copy2d(c, t, N, last, (int64_t)L * N, N, np));
+                RET(launch_ntt_inv_pass_b(c, t, np, N, limbmap_single(L - 1)));
+            }
+            RET(launch_ks_lift(c, t, N, np, limbmap_single(L - 1), lifted, keep, 0));
+            RET(launch_rescale_finish(c, src + p0 * L * N, lifted, np, keep, out + p0 * keep * N));
+            continue;
+        }
         CK(cudaMemcpy2DAsync(t, (size_t)N * 8, src + (p0 * L + (L - 1)) * N, (size_t)L * N * 8, (size_t)N * 8, (size_t)np,
                              cudaMemcpyDeviceToDevice, c->stream));
         RET(launch_ntt_inv(c, t, np, N, limbmap_single(L - 1)));

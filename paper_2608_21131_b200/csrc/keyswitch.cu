@@ -2,8 +2,11 @@
 // switching (digit lift, inner product with the evaluation key, ModDown), the automorphism gather, the output
 // compaction, and the small helpers of the client half.  All polynomials are [.][limb][N] arrays of 64-bit residues in
 // [0, q).
+#include <algorithm>
+
 #include "internal.h"
 #include "debugcheck.cuh"
+#include "nttcore.cuh"
 
 namespace {
 
@@ -14,6 +17,14 @@ inline int grid_for(int64_t work, int per_block = kThreads, int cap = 148 * 16) 
     if (g > cap) g = cap;
     if (g < 1) g = 1;
     return (int)g;
+}
+
+// rows of N words each: up to eight CTAs per SM, a row (or part of one) per blockIdx.y
+inline dim3 row_grid(const hann_ctx* c, int rows) {
+    const int gy = rows < 4096 ? rows : 4096;
+    int gx = (148 * 8 + gy - 1) / gy;
+    if (gx > (c->N + kThreads - 1) / kThreads) gx = (c->N + kThreads - 1) / kThreads;
+    return dim3(gx, gy);
 }
 
 // ------------------------------------------------------------------------------------------ key switching
@@ -530,41 +541,62 @@ __global__ void __launch_bounds__(kThreads) k_encrypt_finish(const u64* __restri
 // the additions, negations, integer multiples and added constants of a leveled circuit, in the transform domain (a constant
 // polynomial transforms to its constant in every position).  Ciphertexts of `limbs` limbs: polynomial pairs.
 struct LinearArgs {
-    u64 ma[HANN_MAXL1], mb[HANN_MAXL1], k[HANN_MAXL1];
+    u64 ma[HANN_MAXL1], ma_s[HANN_MAXL1], mb[HANN_MAXL1], mb_s[HANN_MAXL1], k[HANN_MAXL1];  // with their Shoup companions
 };
 // b_period > 0: b has only b_period words (one ciphertext) and is used for every ciphertext of a.
+// A row of blocks per limb polynomial (no division by the run-time sizes per word).
 __global__ void __launch_bounds__(kThreads) k_linear(const u64* __restrict__ a, const u64* __restrict__ b, u64* __restrict__ out,
-                                                     long long npoly, int limbs, int N, long long b_period, LinearArgs la, LimbTable lt) {
+                                                     int rows, int limbs, int N, int b_rows, LinearArgs la, LimbTable lt) {
     chain_wait();
-    const long long total = npoly * limbs * N;
-    for (long long idx = (long long)blockIdx.x * kThreads + threadIdx.x; idx < total; idx += (long long)gridDim.x * kThreads) {
-        const int l = (int)((idx / N) % limbs);
-        const long long poly = idx / ((long long)limbs * N);
+    for (int y = blockIdx.y; y < rows; y += gridDim.y) {
+        const int l = y % limbs;
         const LimbConst& lc = lt.c[l];
-        u64 v = la.ma[l] == 1 ? a[idx] : mulmod(a[idx], la.ma[l], lc);
-        if (b) {
-            const u64 bv = b[b_period > 0 ? idx % b_period : idx];
-            v = addmod(v, la.mb[l] == 1 ? bv : mulmod(bv, la.mb[l], lc), lc.q);
+        const u64 q = lc.q, ma = la.ma[l], mas = la.ma_s[l], mb = la.mb[l], mbs = la.mb_s[l], k = (y / limbs) & 1 ? 0 : la.k[l];
+        const u64 *ar = a + (long long)y * N, *br = b ? b + (long long)(b_rows > 0 ? y % b_rows : y) * N : nullptr;
+        u64* o = out + (long long)y * N;
+#pragma unroll 4
+        for (int x = blockIdx.x * kThreads + threadIdx.x; x < N; x += gridDim.x * kThreads) {
+            u64 v = ma == 1 ? ar[x] : csub(shoup_mul(ar[x], ma, mas, q), q);
+            if (br) v = addmod(v, mb == 1 ? br[x] : csub(shoup_mul(br[x], mb, mbs, q), q), q);
+            o[x] = addmod(v, k, q);
         }
-        if ((poly & 1) == 0 && la.k[l]) v = addmod(v, la.k[l], lc.q);
-        out[idx] = v;
     }
 }
 
 // degree-2 product of `count` independent ciphertext pairs: d[i] = (a0 b0, a0 b1 + a1 b0, a1 b1), all [.][limbs][N], elementwise
 // in the transform domain
+// Moduli below 2^50: the products as exact two-word sums on the FP64 pipe (acc2_fma) instead of four 128-bit reductions.
 __global__ void __launch_bounds__(kThreads) k_mul_ct(const u64* __restrict__ a, const u64* __restrict__ b, u64* __restrict__ d,
-                                                     long long count, int limbs, int N, LimbTable lt) {
+                                                     int rows, int limbs, int N, LimbTable lt) {
+    const long long LN = (long long)limbs * N;
     chain_wait();
-    const long long LN = (long long)limbs * N, total = count * LN;
-    for (long long idx = (long long)blockIdx.x * kThreads + threadIdx.x; idx < total; idx += (long long)gridDim.x * kThreads) {
-        const long long i = idx / LN, pos = idx % LN;
-        const LimbConst& lc = lt.c[(int)(pos / N)];
-        const u64 a0 = a[i * 2 * LN + pos], a1 = a[i * 2 * LN + LN + pos], b0 = b[i * 2 * LN + pos], b1 = b[i * 2 * LN + LN + pos];
-        u64* o = d + i * 3 * LN + pos;
-        o[0] = mulmod(a0, b0, lc);
-        o[LN] = addmod(mulmod(a0, b1, lc), mulmod(a1, b0, lc), lc.q);
-        o[2 * LN] = mulmod(a1, b1, lc);
+    for (int y = blockIdx.y; y < rows; y += gridDim.y) {
+        const int i = y / limbs, l = y % limbs;
+        const LimbConst& lc = lt.c[l];
+        const long long ro = i * 2 * LN + (long long)l * N, wo = i * 3 * LN + (long long)l * N;
+        if (lc.q < (1ULL << 50)) {
+            const ArithF64 ar(&lc);
+            const double2 c51 = make_double2(lc.c51_bal, lc.c51_q);
+#pragma unroll 2
+            for (int x = blockIdx.x * kThreads + threadIdx.x; x < N; x += gridDim.x * kThreads) {
+                const double a0 = residue_to_f64(a[ro + x]), a1 = residue_to_f64(a[ro + LN + x]);
+                const double b0 = residue_to_balanced_f64(b[ro + x], ar.q, ar.half), b1 = residue_to_balanced_f64(b[ro + LN + x], ar.q, ar.half);
+                double h[3] = {kAcc2Start, kAcc2Start, kAcc2Start}, lo[3] = {0, 0, 0};
+                acc2_fma(h[0], lo[0], a0, b0);
+                acc2_fma(h[1], lo[1], a0, b1);
+                acc2_fma(h[1], lo[1], a1, b0);
+                acc2_fma(h[2], lo[2], a1, b1);
+#pragma unroll
+                for (int k = 0; k < 3; k++) d[wo + k * LN + x] = ar.to_canonical(ar.acc2_value(h[k], lo[k], c51));
+            }
+            continue;
+        }
+        for (int x = blockIdx.x * kThreads + threadIdx.x; x < N; x += gridDim.x * kThreads) {
+            const u64 a0 = a[ro + x], a1 = a[ro + LN + x], b0 = b[ro + x], b1 = b[ro + LN + x];
+            d[wo + x] = mulmod(a0, b0, lc);
+            d[wo + LN + x] = addmod(mulmod(a0, b1, lc), mulmod(a1, b0, lc), lc.q);
+            d[wo + 2 * LN + x] = mulmod(a1, b1, lc);
+        }
     }
 }
 
@@ -597,7 +629,8 @@ int check_launch(hann_ctx* c, const char* what) {
 int launch_mul_ct(hann_ctx* c, const u64* a, const u64* b, int64_t count, u64* d) {
     {
         KProf kp(c, KC_MAC);
-        launch_chain(c, k_mul_ct, dim3(grid_for(count * c->L * c->N)), kThreads, 0, a, b, d, count, c->L, c->N, c->lt);
+        const int rows = (int)(count * c->L);
+        launch_chain(c, k_mul_ct, row_grid(c, rows), kThreads, 0, a, b, d, rows, c->L, c->N, c->lt);
     }
     return check_launch(c, "mul_ct");
 }
@@ -610,10 +643,13 @@ int launch_linear(hann_ctx* c, const u64* a, long long ma, const u64* b, long lo
         la.ma[l] = residue(ma, c->mod[l]);
         la.mb[l] = residue(mb, c->mod[l]);
         la.k[l] = residue(k, c->mod[l]);
+        la.ma_s[l] = hm::shoup(la.ma[l], c->mod[l]);
+        la.mb_s[l] = hm::shoup(la.mb[l], c->mod[l]);
     }
     {
         KProf kp(c, KC_OTHER);
-        launch_chain(c, k_linear, dim3(grid_for(npoly * c->L * c->N)), kThreads, 0, a, b, out, npoly, c->L, c->N, b_period, la, c->lt);
+        const int rows = (int)(npoly * c->L);
+        launch_chain(c, k_linear, row_grid(c, rows), kThreads, 0, a, b, out, rows, c->L, c->N, (int)(b_period / c->N), la, c->lt);
     }
     return check_launch(c, "linear");
 }
@@ -850,19 +886,29 @@ int launch_rlk_finish(hann_ctx* c, const u64* as_coeff, const int8_t* e, const u
 // buffers may be scheduled on a copy engine behind queued host transfers, which would stall the compute stream of
 // hann_score_level_host until all of a level's rows have arrived
 namespace {
-__global__ void __launch_bounds__(kThreads) k_copy2d(u64* __restrict__ dst, long long dst_pitch, const u64* __restrict__ src,
-                                                     long long src_pitch, long long width, long long rows) {
+template <class V>
+__global__ void __launch_bounds__(kThreads) k_copy2d(V* __restrict__ dst, long long dst_pitch, const V* __restrict__ src, long long src_pitch,
+                                                     long long width, long long rows) {
     chain_wait();
-    const long long total = rows * width;
-    for (long long idx = (long long)blockIdx.x * kThreads + threadIdx.x; idx < total; idx += (long long)gridDim.x * kThreads) {
-        const long long r = idx / width, x = idx % width;
-        dst[r * dst_pitch + x] = src[r * src_pitch + x];
+    for (long long r = blockIdx.y; r < rows; r += gridDim.y) {
+#pragma unroll 4
+        for (long long x = (long long)blockIdx.x * kThreads + threadIdx.x; x < width; x += (long long)gridDim.x * kThreads)
+            dst[r * dst_pitch + x] = src[r * src_pitch + x];
     }
 }
 }  // namespace
 int launch_copy2d(hann_ctx* c, u64* dst, int64_t dst_pitch, const u64* src, int64_t src_pitch, int64_t width, int64_t rows) {
     if (width <= 0 || rows <= 0) return HANN_OK;
-    launch_chain(c, k_copy2d, dim3(grid_for(width * rows)), kThreads, 0, dst, dst_pitch, src, src_pitch, width, rows);
+    const auto grid = [&](int64_t w) {
+        const int64_t gy = std::min<int64_t>(rows, 4096), gx = std::min<int64_t>((w + kThreads - 1) / kThreads, std::max<int64_t>(1, 148 * 8 / gy));
+        return dim3((unsigned)gx, (unsigned)gy);
+    };
+    // sixteen bytes at a time where both sides allow it
+    if (!(((uintptr_t)dst | (uintptr_t)src) & 15) && !((dst_pitch | src_pitch | width) & 1))
+        launch_chain(c, k_copy2d<ulonglong2>, grid(width / 2), kThreads, 0, (ulonglong2*)dst, dst_pitch / 2, (const ulonglong2*)src, src_pitch / 2,
+                     width / 2, rows);
+    else
+        launch_chain(c, k_copy2d<u64>, grid(width), kThreads, 0, dst, dst_pitch, src, src_pitch, width, rows);
     return check_launch(c, "copy2d");
 }
 

@@ -272,8 +272,11 @@ __global__ void __launch_bounds__(T, 640 / T) k_ks_apply(ApplyArgs A) {
 }
 
 struct FinishArgs {
-    const u64* lifted;  // [item][2][L][N], pass-A format
-    const u64* u;       // [item][2][L+1][N]
+    const u64* lifted;  // [item][2][limbs][N], pass-A format
+    const u64* u;       // [item][2] polynomials u_poly words apart; u_mid: binary64 words of limbs below 2^50 (see ApplyArgs)
+    long long u_poly;
+    int u_mid, limbs;   // limbs of the result
+    int last;           // 1: divided by the chain's last prime instead of the special prime
     const u64* add;     // optional: add + item * add_it + component * L N, in the order of the result
     long long add_it;
     const u64* c0;      // optional, first component only: the sum over z of phi_z(c0 + item * c0_it + z * c0_z)
@@ -282,13 +285,13 @@ struct FinishArgs {
     u64 *out0, *out1;
     long long out_it;
     const unsigned* galois;
-    long long items;
-    int N, logN, L, n;
+    long long units;    // polynomials: two per item
+    int N, logN, n;
     const void *tw_fwd_f64, *tw_fwd_int;
     const LimbConst* lt;
 };
 
-// out[item][c][i] = (u - lifted) p^{-1} + add + phi(c0), modulus i = blockIdx.y, chunk blockIdx.x, a half-warp per (item, component):
+// out[item][c][i] = (u - lifted) d^{-1} + add + phi(c0), d the special prime or the chain's last, modulus i = blockIdx.y, chunk blockIdx.x, a half-warp per (item, component):
 // pass B of the lifted ModDown polynomials with the combination behind its last round.
 // PERM: u, lifted and c0 are still in the order before the automorphism, which differs from item to item (hoisted rotations); the
 // finished words are permuted in shared memory and stored to the item's own chunk of the result.
@@ -298,8 +301,8 @@ struct FinishArgs {
 template <bool PERM>
 __global__ void __launch_bounds__(256, 3) k_ks_finish(FinishArgs A) {
     extern __shared__ __align__(16) u64 sm[];
-    const int L = A.L, N = A.N, t = blockIdx.x, i = blockIdx.y;
-    const long long LN = (long long)L * N, L1N = LN + N;
+    const int N = A.N, t = blockIdx.x, i = blockIdx.y;
+    const long long LN = (long long)A.limbs * N;
     double2* tc = (double2*)sm;
     const int hw = threadIdx.x >> 4, j = threadIdx.x & 15;
     const unsigned hmask = 0xFFFFu << (threadIdx.x & 16);
@@ -309,18 +312,18 @@ __global__ void __launch_bounds__(256, 3) k_ks_finish(FinishArgs A) {
     const unsigned m0 = (unsigned)(N >> 8);
     const bool f64 = q < (1ULL << 50);
     const ArithF64 ar(lc);
-    const double2 pinv = make_double2(lc->pinv_bal, lc->pinv_q);
-    const u64 pinv_i = lc->pinv, pinv_s = lc->pinv_s;
+    const double2 pinv = A.last ? make_double2(lc->linv_bal, lc->linv_q) : make_double2(lc->pinv_bal, lc->pinv_q);
+    const u64 pinv_i = A.last ? lc->linv : lc->pinv, pinv_s = A.last ? lc->linv_s : lc->pinv_s;
     if (f64) stage_twiddles(tc, (const double2*)A.tw_fwd_f64 + ((size_t)i << A.logN), m0 + t);
     else stage_twiddles((ulonglong2*)tc, (const ulonglong2*)A.tw_fwd_int + ((size_t)i << A.logN), m0 + t);
     chain_wait();
     __syncthreads();
-    const long long units = 2 * A.items, ustep = (long long)gridDim.z * (blockDim.x >> 4);
+    const long long units = A.units, ustep = (long long)gridDim.z * (blockDim.x >> 4);
     for (long long v = (long long)blockIdx.z * (blockDim.x >> 4) + hw; v < units; v += ustep) {
         const long long item = v >> 1;
         const int c = (int)(v & 1);
-        const u64* p = A.lifted + (v * L + i) * N + (t << 8);
-        const u64* up = A.u + v * L1N + (long long)i * N + (t << 8) + j;
+        const u64* p = A.lifted + (v * A.limbs + i) * N + (t << 8);
+        const u64* up = A.u + v * A.u_poly + (long long)i * N + (t << 8) + j;
         const u64* ap = A.add ? A.add + item * A.add_it + c * LN + (long long)i * N + (t << 8) + j : nullptr;
         const u64* cp = A.c0 && c == 0 ? A.c0 + item * A.c0_it + (long long)i * N : nullptr;
         u64* o = (c == 0 ? A.out0 : A.out1) + item * A.out_it + (long long)i * N;
@@ -339,7 +342,7 @@ __global__ void __launch_bounds__(256, 3) k_ks_finish(FinishArgs A) {
 #pragma unroll
                 for (int e = 0; e < 8; e++) {
                     const u64 v = up[16 * (e0 + e)];
-                    uw[e] = PERM ? ar.from_canonical(v) : ar.from_mid(v);
+                    uw[e] = A.u_mid ? ar.from_mid(v) : ar.from_canonical(v);
                 }
 #pragma unroll
                 for (int e = 0; e < 8; e++) a[e] = ap ? ar.from_canonical(ap[16 * (e0 + e)]) : 0.0;
@@ -406,6 +409,26 @@ __global__ void __launch_bounds__(256, 3) k_ks_finish(FinishArgs A) {
     }
 }
 
+int run_finish(hann_ctx* c, FinishArgs& A, bool perm_items) {
+    A.galois = c->galois_dev;
+    A.N = c->N;
+    A.logN = c->logN;
+    A.n = c->n;
+    A.tw_fwd_f64 = c->tw_fwd_f64;
+    A.tw_fwd_int = c->tw_fwd;
+    A.lt = c->lt_dev;
+    // up to sixteen half-warps per CTA, which then walk further polynomials under the staged tables while the grid fills the
+    // machine twice over
+    const int hws = (int)(A.units < 16 ? A.units : 16), threads = (16 * hws + 31) / 32 * 32;
+    const size_t smem = 4096 + (size_t)threads / 16 * 2048;
+    const long long per = (long long)(c->N >> 8) * A.limbs, groups = (A.units + threads / 16 - 1) / (threads / 16);
+    long long gz = (2 * 148 * 3 + per - 1) / per;
+    if (gz > groups) gz = groups;
+    KProf kp(c, KC_MODDOWN_COMBINE);
+    launch_chain(c, perm_items ? k_ks_finish<true> : k_ks_finish<false>, dim3(c->N >> 8, A.limbs, (unsigned)gz), threads, smem, A);
+    return check_launch(c, "ks_finish");
+}
+
 template <int IB, int T>
 void launch_apply(hann_ctx* c, const ApplyArgs& A) {
     // sixteen lanes per digit, whole warps
@@ -463,6 +486,9 @@ int launch_ks_finish(hann_ctx* c, const u64* u, const u64* lifted, int64_t items
     FinishArgs A = {};
     A.lifted = lifted;
     A.u = u;
+    A.u_poly = (long long)(c->L + 1) * c->N;
+    A.u_mid = perm_items ? 0 : 1;
+    A.limbs = c->L;
     A.add = add;
     A.add_it = add_it;
     A.c0 = c0;
@@ -474,26 +500,25 @@ int launch_ks_finish(hann_ctx* c, const u64* u, const u64* lifted, int64_t items
     A.out0 = out0;
     A.out1 = out1;
     A.out_it = out_it;
-    A.galois = c->galois_dev;
-    A.items = items;
-    A.N = c->N;
-    A.logN = c->logN;
-    A.L = c->L;
-    A.n = c->n;
-    A.tw_fwd_f64 = c->tw_fwd_f64;
-    A.tw_fwd_int = c->tw_fwd;
-    A.lt = c->lt_dev;
-    // up to sixteen half-warps per CTA, which then walk further polynomials under the staged tables while the grid fills the
-    // machine twice over
-    const int hws = (int)(2 * items < 16 ? 2 * items : 16), threads = 16 * hws;
-    const size_t smem = 4096 + (size_t)hws * 2048;
-    const long long per = (long long)(c->N >> 8) * c->L, groups = (2 * items + hws - 1) / hws;
-    long long gz = (2 * 148 * 3 + per - 1) / per;
-    if (gz > groups) gz = groups;
-    const dim3 grid(c->N >> 8, c->L, (unsigned)gz);
-    KProf kp(c, KC_MODDOWN_COMBINE);
-    launch_chain(c, perm_items ? k_ks_finish<true> : k_ks_finish<false>, grid, threads, smem, A);
-    return check_launch(c, "ks_finish");
+    A.units = 2 * items;
+    return run_finish(c, A, perm_items);
+}
+
+// out[poly][i] = (src[poly][i] - lifted[poly][i]) q_{L-1}^{-1}, i < keep; src polynomials have L limbs.  One launch in place of pass B
+// and a combination, and the lift in place of an inverse pass A, a lift and a pass A.
+int launch_rescale_finish(hann_ctx* c, const u64* src, const u64* lifted, int64_t npoly, int keep, u64* out) {
+    if (npoly <= 0) return HANN_OK;
+    FinishArgs A = {};
+    A.lifted = lifted;
+    A.u = src;
+    A.u_poly = (long long)c->L * c->N;
+    A.limbs = keep;
+    A.last = 1;
+    A.out0 = out;
+    A.out1 = out + (int64_t)keep * c->N;
+    A.out_it = 2 * (int64_t)keep * c->N;
+    A.units = npoly;
+    return run_finish(c, A, false);
 }
 
 HANN_DEBUG_DEFINE_BIND(debug_bind_ksfused)

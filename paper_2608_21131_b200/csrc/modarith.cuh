@@ -32,6 +32,10 @@ struct LimbConst {
     double ninv_q;    // fl(ninv_bal / q)
     double pinv_bal;  // p^{-1} mod q as a balanced integer, ciphertext primes only
     double pinv_q;    // fl(pinv_bal / q)
+    u64 linv;         // the inverse of the chain's last prime mod q in the same forms (the primes before it only)
+    u64 linv_s;
+    double linv_bal;
+    double linv_q;
 };
 
 #define HANN_MAXL1 16  // up to 15 ciphertext primes + the special prime (limb numbers travel in 4-bit fields)
