@@ -7,6 +7,7 @@
 
 #include "internal.h"
 #include "bulkcopy.cuh"
+#include "nttcore.cuh"
 
 namespace {
 
@@ -42,6 +43,19 @@ __global__ void __launch_bounds__(kThreads) k_mac(const u64* __restrict__ baby, 
     }
 }
 
+// residue of the sum of NG <= 8 partial sums of at most 1.25 q each (ArithF64::acc2_value): the total may reach 10 q, so the second
+// half is added to the reduced first
+template <int NG, class F>
+__device__ __forceinline__ u64 sum_values(const ArithF64& ar, const F& value) {
+    double t = value(0);
+#pragma unroll
+    for (int g = 1; g < NG; g++) {
+        if (g == 4) t = ar.reduce(t);
+        t = __dadd_rn(t, value(g));
+    }
+    return ar.to_canonical(t);
+}
+
 // Streaming kernel for moduli below 2^50 (the HBM-bound case the path is sized for).  A CTA owns 32 consecutive
 // positions of one limb.  Its NG warps split the B baby steps among them: warp w keeps the baby-step words of steps
 // w*BB .. w*BB+BB-1 (both ciphertext components) for its lane's position in REGISTERS for the CTA's whole life, and
@@ -63,7 +77,9 @@ __global__ void __launch_bounds__(32 * NG) k_mac_stream(const u64* __restrict__ 
                                                         const LimbConst* __restrict__ lt) {
     constexpr int B = NG * BB;
     constexpr int NV = 2 * NQ;  // (query, side): side 0 is position t, side 1 its mirror image N - 1 - t
-    constexpr int PS = F64 ? 2 : 3;  // words per partial sum: (high, low) of the binary64 sums, or the three Karatsuba sums
+    // words per partial sum: the reduced binary64 sum, two words where the chain has primes of 2^50 and more (F64 == 2), or the
+    // three Karatsuba sums
+    constexpr int PS = F64 == 1 ? 1 : F64 ? 2 : 3;
     static_assert(F64 == 0 || BB <= 8, "the two-word binary64 sum holds eight products");
     // two buffers (a warp may write the next pair's partial sums while others still add up this pair's) where they fit the
     // static shared memory, one and a second barrier per pair otherwise
@@ -81,6 +97,8 @@ __global__ void __launch_bounds__(32 * NG) k_mac_stream(const u64* __restrict__ 
     double wd[NV][BB][2];
     const double qd = (double)lc->q, halfd = (double)lc->half;
     const bool big = F64 == 2 && lc->q >= (1ULL << 50);  // see k_mac_bulk
+    const ArithF64 ar(lc);
+    const double2 c51 = make_double2(lc->c51_bal, lc->c51_q);
 #pragma unroll
     for (int v = 0; v < NV; v++)
 #pragma unroll
@@ -146,8 +164,7 @@ __global__ void __launch_bounds__(32 * NG) k_mac_stream(const u64* __restrict__ 
             for (int v = 0; v < NV; v++)
 #pragma unroll
                 for (int c = 0; c < 2; c++) {
-                    buf[wg][(v * 2 + c) * PS + 0][lane] = (u64)acc2_high(ah[v][c]);
-                    buf[wg][(v * 2 + c) * PS + 1][lane] = (u64)acc2_low(al[v][c]);
+                    buf[wg][(v * 2 + c) * PS][lane] = (u64)__double_as_longlong(ar.acc2_value(ah[v][c], al[v][c], c51));
                 }
         } else {
             u64 p00[NV][2], p11[NV][2], pm[NV][2];
@@ -190,13 +207,7 @@ __global__ void __launch_bounds__(32 * NG) k_mac_stream(const u64* __restrict__ 
                 }
                 r = reduce128(hi, lo, *lc);
             } else if (F64) {
-                long long m = 0, sl = 0;
-#pragma unroll
-                for (int g = 0; g < NG; g++) {
-                    m += (long long)buf[g][vc * PS + 0][lane];
-                    sl += (long long)buf[g][vc * PS + 1][lane];
-                }
-                r = acc2_reduce(m, sl, *lc);
+                r = sum_values<NG>(ar, [&](int g) { return __longlong_as_double((long long)buf[g][vc * PS][lane]); });
             } else {
                 u64 s00 = 0, sm = 0, s11 = 0;
 #pragma unroll
@@ -366,17 +377,20 @@ __global__ void __launch_bounds__(32 * NG) k_mac_ct_stream(const u64* __restrict
 // into registers, so an SM keeps about four times as much in flight and the registers of the prefetch
 // are free.  Completion is signalled on per-buffer mbarriers; waits are bounded, and a warp whose wait runs out raises the
 // context's kernel flag and lets the whole CTA leave at its next barrier.
-constexpr int kMacStages = 4;
+// (three stages: four are the same within 0.3 %, five cost 2 %, six 6 % of the kernel: the shared memory is worth more as L1)
+constexpr int kMacStages = 3;
 
 // partial sums per thread that cross the warps: four sums of three words (integer multiplier) or of two (FP64 pipe)
 template <int NG, int BB, int F64>
 constexpr size_t mac_bulk_smem() {
-    return (size_t)NG * kMacStages * BB * 256 + (size_t)2 * NG * (F64 ? 8 : 12) * 256 + (size_t)NG * kMacStages * 8 + 16;
+    return (size_t)NG * kMacStages * BB * 256 + (size_t)2 * NG * (F64 == 1 ? 4 : F64 ? 8 : 12) * 256 + (size_t)NG * kMacStages * 8 + 16;
 }
 
 // F64 != 0: the products are summed exactly in pairs of binary64 words on the FP64 pipe (acc2_fma: four operations per
-// product on a pipe of more than twice the multiplier's throughput, and two words of partial sum per thread instead of
-// three); 0: on the integer multiplier as in k_mac_stream.  Same integers either way, hence the same residues.
+// product on a pipe of more than twice the multiplier's throughput); every warp reduces its own eight products to one binary64 word
+// (acc2_value), which is what crosses the warps.  0: on the integer multiplier as in k_mac_stream.  Same integers either way, hence
+// the same residues.  Bound: HBM (31 blocks of N = 2^16: 4.9 GB in 0.99 ms, 75 % of the measured copy bandwidth); with both words
+// crossing the warps and a 128-bit integer reduction per output it was 1.10 ms, and 272 instead of 237 us on seven blocks.
 template <int NG, int BB, int F64>
 __global__ void __launch_bounds__(32 * NG) k_mac_bulk(const u64* __restrict__ baby, const __grid_constant__ CUtensorMap pt_map,
                                                       u64* __restrict__ inner, int N, int L, long long n_bg, int bg_per_cta,
@@ -384,7 +398,7 @@ __global__ void __launch_bounds__(32 * NG) k_mac_bulk(const u64* __restrict__ ba
     constexpr int B = NG * BB;
     extern __shared__ __align__(128) u64 smem_mac[];
     u64(*ring)[kMacStages][BB][32] = (u64(*)[kMacStages][BB][32])smem_mac;                        // [NG]
-    constexpr int PS = F64 ? 2 : 3, PW = 4 * PS;  // words per partial sum, per thread
+    constexpr int PS = F64 == 1 ? 1 : F64 ? 2 : 3, PW = 4 * PS;  // words per partial sum (as in k_mac_stream), per thread
     u64(*part)[NG][PW][32] = (u64(*)[NG][PW][32])(smem_mac + (size_t)NG * kMacStages * BB * 32);  // [2]
     u64(*bars)[kMacStages] = (u64(*)[kMacStages])(smem_mac + (size_t)NG * kMacStages * BB * 32 + (size_t)2 * NG * PW * 32);  // [NG]
     int& s_abort = *(int*)(&bars[NG][0]);
@@ -423,6 +437,8 @@ __global__ void __launch_bounds__(32 * NG) k_mac_bulk(const u64* __restrict__ ba
     // F64 == 2: the chain has primes in [2^50, 2^60); their limbs (uniform over a CTA) take 128-bit integer sums, the words
     // kept as they are
     const bool big = F64 == 2 && lc->q >= (1ULL << 50);
+    const ArithF64 ar(lc);
+    const double2 c51 = make_double2(lc->c51_bal, lc->c51_q);
 #pragma unroll
     for (int v = 0; v < 2; v++)
 #pragma unroll
@@ -485,8 +501,7 @@ __global__ void __launch_bounds__(32 * NG) k_mac_bulk(const u64* __restrict__ ba
             for (int v = 0; v < 2; v++)
 #pragma unroll
                 for (int c = 0; c < 2; c++) {
-                    buf[wg][(v * 2 + c) * PS + 0][lane] = (u64)acc2_high(ah[v][c]);
-                    buf[wg][(v * 2 + c) * PS + 1][lane] = (u64)acc2_low(al[v][c]);
+                    buf[wg][(v * 2 + c) * PS][lane] = (u64)__double_as_longlong(ar.acc2_value(ah[v][c], al[v][c], c51));
                 }
         } else {
             u64 p00[2][2] = {{0, 0}, {0, 0}}, p11[2][2] = {{0, 0}, {0, 0}}, pm[2][2] = {{0, 0}, {0, 0}};
@@ -529,13 +544,7 @@ __global__ void __launch_bounds__(32 * NG) k_mac_bulk(const u64* __restrict__ ba
                 }
                 r = reduce128(hi, lo, *lc);
             } else if (F64) {
-                long long m = 0, sl = 0;
-#pragma unroll
-                for (int g = 0; g < NG; g++) {
-                    m += (long long)buf[g][vc * PS + 0][lane];
-                    sl += (long long)buf[g][vc * PS + 1][lane];
-                }
-                r = acc2_reduce(m, sl, *lc);
+                r = sum_values<NG>(ar, [&](int g) { return __longlong_as_double((long long)buf[g][vc * PS][lane]); });
             } else {
                 u64 s00 = 0, sm = 0, s11 = 0;
 #pragma unroll
