@@ -677,10 +677,20 @@ void launch_ks_inner_stream(hann_ctx* c, const u64* digits, int64_t digit_stride
                             int nz = 1, int rot_zinc = 0) {
     const long long L1N = (long long)(LL + 1) * c->N;
     const int tiles = (int)(L1N / 128);
-    int split = 1;
-    while ((long long)tiles * split * nz < 148 * 8 && split < nitems) split *= 2;
-    const int per = (int)((nitems + split - 1) / split);
-    split = (int)((nitems + per - 1) / per);
+    // CTAs that share out the items of a tile: smallest (waves x items of a CTA), ties to fewer.  72 registers: seven CTAs per SM; a
+    // CTA of 31 keys takes long enough for an almost empty third wave to cost a sixth of the launch (155 -> 148 us, at N = 2^15 91 -> 76).
+    const long long slots = 148 * 7;
+    int per = (int)nitems;
+    long long best = -1;
+    for (int sp = 1; sp <= nitems && sp <= 64; sp++) {
+        const int p = (int)((nitems + sp - 1) / sp);
+        const long long cost = (((long long)tiles * sp * nz + slots - 1) / slots) * (4 * p + 1);  // the stationary words: a quarter item
+        if (best < 0 || cost < best) {
+            best = cost;
+            per = p;
+        }
+    }
+    const int split = (int)((nitems + per - 1) / per);
     KProf kp(c, digit_stride == 0 && nitems > 1 ? KC_KS_INNER_KEYS : KC_KS_INNER);  // streamed keys timed on their own
     launch_chain(c, digit_stride == 0 ? k_ks_inner_stream<LL, true> : k_ks_inner_stream<LL, false>, dim3(tiles, split, nz), 128, 0, digits,
                  digit_stride, c->keytab_dev, rot0, rot_inc, u, c->N, nitems, per, c->lt_dev, rot_zinc, c->mac_f64);
