@@ -144,18 +144,16 @@ def build_workload(config, rows_override=None, logn=16, baby=None):
 
 # DRAM bytes (read + write) per unit of work of the transform kernels, from the ncu captures summarised under profiles/
 # (small case: one block of 32,768 rows; traffic grows in proportion to the units): pass B of a half-size plaintext
-# transform, pass B of a full key-switch transform, the fused FFT tail + pass A per plaintext
-NCU_DRAM_BYTES = {"pass_b_plaintext_poly": 212.4e6 / 512, "pass_b_full_poly": 490.4e6 / 512, "fft_b_plaintext": 153.6e6 / 128}
+# transform, pass B of a full key-switch transform
+NCU_DRAM_BYTES = {"pass_b_plaintext_poly": 212.4e6 / 512, "pass_b_full_poly": 490.4e6 / 512}
 
 
 def ncu_traffic_per_step(kernel, ctx, n_blocks):
     """DRAM traffic of one step of a kernel class, scaled from the ncu captures (None where none was taken)"""
     L, B, G, R = ctx.L, ctx.B, ctx.G, ctx.R
     if kernel == "ntt_fwd_b":
-        ks_polys = (L * (L + 1) + (B - 1) * 2 * L) + (G - 1) * n_blocks * (L * (L + 1) + 2 * L)
-        return n_blocks * R * L * NCU_DRAM_BYTES["pass_b_plaintext_poly"] + ks_polys * NCU_DRAM_BYTES["pass_b_full_poly"]
-    if kernel == "fft_b":
-        return n_blocks * R * NCU_DRAM_BYTES["fft_b_plaintext"]
+        # (the digits of the query; those of the rotate-and-sum are transformed inside the key product)
+        return n_blocks * R * L * NCU_DRAM_BYTES["pass_b_plaintext_poly"] + L * (L + 1) * NCU_DRAM_BYTES["pass_b_full_poly"]
     return None
 
 
@@ -197,6 +195,32 @@ def algorithmic_work(ctx, n_blocks, n_rows):
         "fft_a": ("hbm", n_blocks * R * (n * 16) + n_rows * R * 4, n_blocks * R),
         "fft_b": ("alu", n_blocks * R * ((a - 1) * (n // 2) * 10 + L * pass_a_half), n_blocks * R),
     }
+
+
+def kernel_work(ctx, n_blocks, n_rows, lazy):
+    """algorithmic_work as the kernels share it out: pass B of the rotate-and-sum's digits runs inside the key product (class
+    ks_inner) and that of the ModDown inside the combination, a digit modulo its own prime is not transformed, the special
+    prime's inverse pass B' of the rotate-and-sum belongs to the key product, and the FFT of the real slot vectors is half size."""
+    w = algorithmic_work(ctx, n_blocks, n_rows)
+    L, N, B, G, R = ctx.L, ctx.N, ctx.B, ctx.G, ctx.R
+    n, logN = ctx.n, ctx.logN
+    b = min(logN, 8)
+    a = logN - b
+    W = 8 * N
+    items = (G - 1) * n_blocks
+    moddowns = n_blocks if lazy else items
+    pt_polys, digits, inv_polys = n_blocks * R * L, L * (L + 1), L + (B - 1) * 2 + items * L
+    lift = [(L, L + 1), ((B - 1) * 2, L), (items * L, L), (moddowns * 2, L)]
+    pass_a_half = (N // 2) * 7 + (a - 1) * (N // 4) * 8
+    w["ntt_fwd_b"] = ("alu", (pt_polys * (N // 4) + digits * (N // 2)) * b * 8, pt_polys + digits)
+    w["ntt_inv_b"] = ("alu", inv_polys * (N // 2) * b * 8, inv_polys)
+    w["lift_digits"] = ("alu", sum(src * (1 + tgt) * a * (N // 2) * 8 for src, tgt in lift), sum(src for src, _ in lift))
+    w["ks_inner"] = ("hbm", (G - 1) * L * 2 * (L + 1) * W + items * (L * L + L) * W + moddowns * 2 * (L + 1) * W, items)
+    w["fft_a"] = ("hbm", n_blocks * R * (n * 8) + n_rows * R * 4, n_blocks * R)
+    w["fft_b"] = ("alu", n_blocks * R * ((a - 1) * (n // 4) * 10 + L * pass_a_half), n_blocks * R)
+    algorithmic_work.transform_bytes = {"ntt_fwd_b": pt_polys * W + digits * 2 * W, "ntt_inv_b": inv_polys * 2 * W,
+                                        "fft_b": n_blocks * R * (n * 8 + L * (W // 2))}
+    return w
 
 
 def run_ours(args):
@@ -368,7 +392,7 @@ def run_ours(args):
     # arithmetic ceilings measured on this device by the library's own probe kernels: register-resident binary64 modular
     # butterflies (no memory traffic) and 32 x 32 -> 64 multiply-adds
     bfly_peak, madd_peak = ctx.probe_rates()
-    work = algorithmic_work(ctx, nb, n_rows)
+    work = kernel_work(ctx, nb, n_rows, args.giant != "horner")
     dom = max((k for k in kernels if k in work), key=lambda k: kernels[k]["ms_per_step"])
     bound, amount, units = work[dom]
     dom_s = kernels[dom]["ms_per_step"] * 1e-3
