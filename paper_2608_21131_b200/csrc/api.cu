@@ -1877,7 +1877,7 @@ extern "C" int hann_score_level_host(hann_ctx* c, const uint64_t* ct_host, const
     // of blocks: a group is scored (multiply-accumulate, rotate-and-sum, inverse transform of its score ciphertexts) on
     // one of two scoring streams while the following groups are still uploaded and encoded, and its scores go home on
     // the download stream beside all that.  Only the last group's scoring and download follow the last upload.  (One
-    // group: everything on the context's stream, the rotate-and-sum on its four lanes.)
+    // group: everything on the context's stream, the rotate-and-sum in its own lanes.)
     const int ng = p.ng;
     while ((int64_t)c->blk_ev.size() < p.nblk) {
         cudaEvent_t e;
