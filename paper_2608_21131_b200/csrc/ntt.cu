@@ -53,12 +53,12 @@ struct NttArgs {
     // limb[]): all positions whose modulus falls in the launch's arithmetic class
     int period, nsel;
     int tau;  // chunks of 256 positions are stored with their low nibbles swapped (see galois_src)
-    // inverse pass B' only (bulk-copy kernel): read group g, position pos from src + g * src_gstride + pos * stride instead
-    // of from `data` (nullptr: in place)
+    // inverse pass B' only (bulk-copy kernel; nullptr: in place): group g of the launch, group h = src_g0 + g of the batch, is read
+    // from src + h * src_gstride, or (src_per > 0) from src + (h / src_per) * src_zstride + (h % src_per) * src_gstride, position
+    // pos of the group pos * stride words further
     const u64* src;
     long long src_gstride;
-    // src_per > 0: group g is read from src + (g / src_per) * src_zstride + (g % src_per) * src_gstride
-    int src_per;
+    int src_per, src_g0;
     long long src_zstride;
     u64 pos4, limb4;  // 4-bit fields: position within the period and limb of selection k (at most 16 selections)
     // forward pass B (bulk-copy kernel) of polynomials that are fixed by X -> 1/X and stored as their first N/2 transform
@@ -408,7 +408,7 @@ __global__ void __launch_bounds__(256, 3) k_ntt_inv_b8t(NttArgs A, int groups, i
     const u64* sbase = A.src ? A.src + (long long)pos * A.stride + ((size_t)chunk0 << 8) : gbase;
     auto source = [&](int i) {
         if (!A.src) return sbase + (long long)i * ystep * tile_stride;
-        const int g = (yg0 + i * ystep) * kTP + t;
+        const int g = A.src_g0 + (yg0 + i * ystep) * kTP + t;
         return sbase + (A.src_per > 0 ? (g / A.src_per) * A.src_zstride + (g % A.src_per) * A.src_gstride : g * A.src_gstride);
     };
     const int my_tiles = yg0 < ntiles ? (ntiles - yg0 + ystep - 1) / ystep : 0;
@@ -1027,6 +1027,7 @@ int launch_ntt(hann_ctx* c, u64* data, int64_t npoly, int64_t stride, const Limb
     A.src = src;
     A.src_gstride = src_gstride;
     A.src_per = (int)src_per;
+    A.src_g0 = 0;
     A.src_zstride = src_zstride;
     A.period = lm.period;
     A.half = half ? 1 : 0;
@@ -1059,14 +1060,10 @@ int launch_ntt(hann_ctx* c, u64* data, int64_t npoly, int64_t stride, const Limb
         NttArgs& X = Ac[cls];
         if (!X.nsel) continue;
         const int64_t gmax = 65535 / (mixed ? Ac[0].nsel + Ac[2].nsel : X.nsel);
-        if (src_per > 0 && groups_total > gmax) {
-            c->err = "gathered transform batch too large";
-            return HANN_EINVAL;
-        }
         for (int64_t g0 = 0; g0 < groups_total; g0 += gmax) {
             const int groups = (int)std::min<int64_t>(gmax, groups_total - g0);
             X.data = data + g0 * lm.period * stride;
-            if (src) X.src = src + g0 * src_gstride;
+            if (src) X.src_g0 = (int)g0;
             const bool merge = mixed && b8t_eligible(c, X);
             if (!inverse) {
                 if (cls == 0) launch_fwd_class<ArithF64>(c, X, groups, skip_a, merge);

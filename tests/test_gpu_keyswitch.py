@@ -68,3 +68,26 @@ def test_rotate_sum_on_edge_residues(logN, bits, pbits, nb):
     for r in (1, 2, 3):
         assert np.array_equal(got[r], o.rotate(inner[0, 0], r, evk[r])), r
     torch.cuda.synchronize()
+
+
+def test_lazy_round_of_many_giant_steps():
+    """15 blocks x 511 giant steps in one round: 7,665 polynomials of nine limbs, more than one launch covers (65535 / 9).  A large
+    workspace only means larger rounds: the same bits as with rounds of one block"""
+    import torch
+
+    from paper_2608_21131_b200 import binding as b
+
+    logN, L, nb = 10, 9, 15
+    q = find_primes(45, logN + 1, L)
+    ps = synth.ParamSet("many", logN, tuple(q), find_primes(60, logN + 1, 1)[0], 20, 512, 1, 0)
+    c = b.Context(ps)
+    c.set_tuning(b.TUNE_LAZY_LANES, 1)
+    keys = synth.uniform_residues(3, 2, q + [ps.p], ps.N, lead=(5, L, 2))
+    for r in range(1, ps.G):
+        c.load_keys(keys[r % 5][None], [r])
+    inner = torch.randint(0, min(q), (nb * c.sizeof(b.SIZE_INNER) // 8,), dtype=torch.int64, device=c.device,
+                          generator=torch.Generator(c.device).manual_seed(4))
+    one = c.rotate_sum_lazy(inner, nb, c.workspace(1))
+    all_ = c.rotate_sum_lazy(inner, nb, c.alloc((nb + 1) * c.workspace_bytes(1)))
+    c.sync()
+    assert torch.equal(one, all_)
