@@ -118,6 +118,13 @@ struct KProf {
 // visible.  No kernel lets its successor start early (griddepcontrol.launch_dependents): the waiting CTAs then hold slots that other
 // streams and the kernel's own tail need.  Us of a pass, plain launches / these / these with an early start: toy level 322 / 228 /
 // 241, coarse 773 / 763 / 802, projection 1055 / 976 / 1074, eight queries 5661 / 5626 / 5768, membership 8892 / 8438 / 8591.
+//
+// What such a kernel may load before chain_wait, or through a parameter declared `const ... __restrict__` (which promises memory that
+// nobody writes while the kernel is resident, so that the compiler may load it early and past the coherent caches): the context's
+// tables only.  Everything that a kernel or copy of the stream can have written comes through unqualified pointers after the wait.
+// The evaluation keys, which k_ks_apply fetches before the wait, are such data too; there it is enough that the kernel always follows
+// k_ks_lift, none of whose CTAs ends before its own wait is over: when k_ks_apply starts, all that was enqueued before the lift is
+// complete and visible.
 #ifdef __CUDACC__
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <class... KA, class... A>

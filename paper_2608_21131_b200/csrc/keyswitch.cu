@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(kThreads) k_lift_digits(const u64* __restrict_
 // u[item][comp][i][x] = sum_j digits[item_d][j][i][x] * key[j][comp][i][x] mod modulus i.
 // digit_stride = 0 shares one digit set among all items (hoisted rotations of one ciphertext); the key of item
 // `it` is keytab[rot0 + it*rot_inc].
-__global__ void __launch_bounds__(kThreads) k_ks_inner(const u64* __restrict__ digits, long long digit_stride,
+__global__ void __launch_bounds__(kThreads) k_ks_inner(const u64* digits, long long digit_stride,
                                                        const u64* const* __restrict__ keytab, int rot0, int rot_inc,
                                                        u64* __restrict__ u, int N, int L, long long nitems,
                                                        LimbTable lt, int f64) {
@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(kThreads) k_ks_inner(const u64* __restrict__ d
 // 30-bit halves, 4 products (sums of 2 LL <= 8 products of 60 bits fit 64 bits); MODE 2: anything else, 128-bit
 // accumulation.
 template <int LL, bool KEYS_STREAM, int MODE>
-__device__ __forceinline__ void ks_inner_body(const u64* __restrict__ digits, long long digit_stride, const u64* const* __restrict__ keytab,
+__device__ __forceinline__ void ks_inner_body(const u64* digits, long long digit_stride, const u64* const* __restrict__ keytab,
                                               int rot0, int rot_inc, u64* __restrict__ u, long long L1N, long long pos, long long it0,
                                               long long it1, const LimbConst& lc) {
     constexpr int NS = KEYS_STREAM ? 2 * LL : LL;   // streamed words per item
@@ -217,7 +217,7 @@ __device__ __forceinline__ void ks_inner_body(const u64* __restrict__ digits, lo
 // blockIdx.z selects one of several independent batches of `nitems` items laid out one after the other (digits and u), batch
 // z using rotation rot0 + z * rot_zinc: the giant steps of the lazy rotate-and-sum, each under its own key
 template <int LL, bool KEYS_STREAM>
-__global__ void __launch_bounds__(128) k_ks_inner_stream(const u64* __restrict__ digits, long long digit_stride,
+__global__ void __launch_bounds__(128) k_ks_inner_stream(const u64* digits, long long digit_stride,
                                                          const u64* const* __restrict__ keytab, int rot0, int rot_inc,
                                                          u64* __restrict__ u, int N, long long nitems, int items_per_cta,
                                                          const LimbConst* __restrict__ lt, int rot_zinc, int f64) {
@@ -545,7 +545,7 @@ struct LinearArgs {
 };
 // b_period > 0: b has only b_period words (one ciphertext) and is used for every ciphertext of a.
 // A row of blocks per limb polynomial (no division by the run-time sizes per word).
-__global__ void __launch_bounds__(kThreads) k_linear(const u64* __restrict__ a, const u64* __restrict__ b, u64* __restrict__ out,
+__global__ void __launch_bounds__(kThreads) k_linear(const u64* a, const u64* b, u64* __restrict__ out,
                                                      int rows, int limbs, int N, int b_rows, LinearArgs la, LimbTable lt) {
     chain_wait();
     for (int y = blockIdx.y; y < rows; y += gridDim.y) {
@@ -566,7 +566,7 @@ __global__ void __launch_bounds__(kThreads) k_linear(const u64* __restrict__ a, 
 // degree-2 product of `count` independent ciphertext pairs: d[i] = (a0 b0, a0 b1 + a1 b0, a1 b1), all [.][limbs][N], elementwise
 // in the transform domain
 // Moduli below 2^50: the products as exact two-word sums on the FP64 pipe (acc2_fma) instead of four 128-bit reductions.
-__global__ void __launch_bounds__(kThreads) k_mul_ct(const u64* __restrict__ a, const u64* __restrict__ b, u64* __restrict__ d,
+__global__ void __launch_bounds__(kThreads) k_mul_ct(const u64* a, const u64* b, u64* __restrict__ d,
                                                      int rows, int limbs, int N, LimbTable lt) {
     const long long LN = (long long)limbs * N;
     chain_wait();
@@ -792,7 +792,7 @@ int launch_moddown_combine(hann_ctx* c, const u64* u, const u64* lifted, int64_t
 
 // ---- output compaction: rescale by the last ciphertext prime ---------------------------------------------------------
 // lifted[poly][i][x] = centred lift of t[poly][x] (residue mod q_{L-1}, coefficient domain) reduced mod q_i, i < keep
-__global__ void __launch_bounds__(kThreads) k_rescale_lift(const u64* __restrict__ t, u64* __restrict__ lifted, int N, int L,
+__global__ void __launch_bounds__(kThreads) k_rescale_lift(const u64* t, u64* __restrict__ lifted, int N, int L,
                                                            int keep, long long npoly, LimbTable lt) {
     chain_wait();
     const long long total = npoly * N;
@@ -815,7 +815,7 @@ struct RescaleConst {
 };
 
 // out[poly][i][x] = (src[poly][i][x] - lifted[poly][i][x]) * q_{L-1}^{-1} mod q_i; src polynomials have L limbs, out keep
-__global__ void __launch_bounds__(kThreads) k_rescale_combine(const u64* __restrict__ src, const u64* __restrict__ lifted,
+__global__ void __launch_bounds__(kThreads) k_rescale_combine(const u64* src, const u64* lifted,
                                                               u64* __restrict__ out, int N, int L, int keep, long long npoly,
                                                               LimbTable lt, RescaleConst rc) {
     chain_wait();
@@ -897,7 +897,7 @@ int launch_rlk_finish(hann_ctx* c, const u64* as_coeff, const int8_t* e, const u
 // hann_score_level_host until all of a level's rows have arrived
 namespace {
 template <class V>
-__global__ void __launch_bounds__(kThreads) k_copy2d(V* __restrict__ dst, long long dst_pitch, const V* __restrict__ src, long long src_pitch,
+__global__ void __launch_bounds__(kThreads) k_copy2d(V* __restrict__ dst, long long dst_pitch, const V* src, long long src_pitch,
                                                      long long width, long long rows) {
     chain_wait();
     for (long long r = blockIdx.y; r < rows; r += gridDim.y) {

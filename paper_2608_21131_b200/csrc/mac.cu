@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(32 * NG) k_mac_stream(const u64* __restrict__ 
 // database ciphertext streamed past them one after the other: x_h * y_c adds to d_{h+c}, so the three degree-2 sums share
 // one set of Karatsuba accumulators and every database word is read once.
 template <int NG, int BB, bool F64>
-__global__ void __launch_bounds__(32 * NG) k_mac_ct_stream(const u64* __restrict__ baby, const u64* __restrict__ ctdb,
+__global__ void __launch_bounds__(32 * NG) k_mac_ct_stream(const u64* baby, const u64* ctdb,
                                                            u64* __restrict__ inner3, int N, int L, long long n_bg, int bg_per_cta,
                                                            const LimbConst* __restrict__ lt) {
     constexpr int B = NG * BB;
@@ -392,7 +392,7 @@ constexpr size_t mac_bulk_smem() {
 // the same residues.  Bound: HBM (31 blocks of N = 2^16: 4.9 GB in 0.99 ms, 75 % of the measured copy bandwidth); with both words
 // crossing the warps and a 128-bit integer reduction per output it was 1.10 ms, and 272 instead of 237 us on seven blocks.
 template <int NG, int BB, int F64>
-__global__ void __launch_bounds__(32 * NG) k_mac_bulk(const u64* __restrict__ baby, const __grid_constant__ CUtensorMap pt_map,
+__global__ void __launch_bounds__(32 * NG) k_mac_bulk(const u64* baby, const __grid_constant__ CUtensorMap pt_map,
                                                       u64* __restrict__ inner, int N, int L, long long n_bg, int bg_per_cta,
                                                       const LimbConst* __restrict__ lt, int* kflag) {
     constexpr int B = NG * BB;

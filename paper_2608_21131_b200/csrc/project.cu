@@ -48,9 +48,9 @@ __global__ void __launch_bounds__(kThreads) k_window_masks(int R, int b, int n, 
 // cyc[b][comp][l][t] = lo[b][l][t'] * A_b[comp][l][t] + hi[b][l][t'] * H_b[comp][l][t]   (transform domain, elementwise)
 // A_0 = ct and no H_0 (hi_0 = 0); A_b = rot_a[b-1], H_b = rot_h[b-1] for b >= 1.  The masks are stored as the first N/2
 // transform values of a real slot vector's encoding: position t >= N/2 mirrors position N - 1 - t.
-__global__ void __launch_bounds__(kThreads) k_mask_combine(const u64* __restrict__ ct, const u64* __restrict__ rot_a,
-                                                           const u64* __restrict__ rot_h, const u64* __restrict__ lo,
-                                                           const u64* __restrict__ hi, u64* __restrict__ cyc, int Bn, int N, int L,
+__global__ void __launch_bounds__(kThreads) k_mask_combine(const u64* ct, const u64* rot_a,
+                                                           const u64* rot_h, const u64* lo,
+                                                           const u64* hi, u64* __restrict__ cyc, int Bn, int N, int L,
                                                            LimbTable lt) {
     chain_wait();
     const long long LN = (long long)L * N, ctw = 2 * LN, total = (long long)Bn * ctw;
