@@ -429,7 +429,7 @@ extern "C" int hann_ctx_create(const hann_params* prm, hann_ctx** out) {
         ok = cudaStreamCreateWithFlags(&c->score_stream[i], cudaStreamNonBlocking) == cudaSuccess &&
              cudaEventCreateWithFlags(&c->score_join[i], cudaEventDisableTiming) == cudaSuccess;
     if (ok) ok = cudaEventCreateWithFlags(&c->prep_done, cudaEventDisableTiming) == cudaSuccess;
-    if (ok) ok = ntt_configure(c) == HANN_OK;
+    if (ok) ok = ntt_configure(c) == HANN_OK && ks_fused_configure() == HANN_OK && encode_configure() == HANN_OK;
     // a -DHANN_DEBUG build: the range checks of the kernels report through this context's error word
     if (ok) ok = debug_bind_keyswitch(c->kflag) == 0 && debug_bind_project(c->kflag) == 0 && debug_bind_encode(c->kflag) == 0 && debug_bind_ksfused(c->kflag) == 0;
     if (ok) {

@@ -745,6 +745,25 @@ KernX pick_x(int a, bool sym) { return sym && a >= 2 ? pick_x_t<true>(a) : pick_
 
 }  // namespace
 
+namespace {
+// kernel H: exchange tile, then L x 2^a twiddle pairs
+constexpr size_t encode_h_smem(int a, int L) { return 16384 + (size_t)L * (1 << a) * 16; }
+// kernel X: exchange tile (FFT: 2^(a-1) x 16 complex = transform: 2^a x 16 words) when a > 4, then L x 2^a twiddle pairs
+constexpr size_t encode_x_smem(int a, int L) { return (a > 4 ? (size_t)(1 << a) * 16 * 8 : 0) + (size_t)L * (1 << a) * 16; }
+}  // namespace
+
+// Dynamic shared memory of the instances that may need more than the default 48 KiB, for the longest chain: the limit belongs to the
+// kernel and the device, so it is the same for contexts of every chain length.
+int encode_configure() {
+    static_assert(encode_h_smem(7, HANN_MAX_PRIMES) <= 48 * 1024 && encode_x_smem(7, HANN_MAX_PRIMES) <= 48 * 1024, "only rings of 2^16 points need it");
+    if (cudaFuncSetAttribute(pick_h(8), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)encode_h_smem(8, HANN_MAX_PRIMES)) != cudaSuccess)
+        return HANN_ECUDA;
+    for (bool sym : {false, true})
+        if (cudaFuncSetAttribute(pick_x(8, sym), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)encode_x_smem(8, HANN_MAX_PRIMES)) != cudaSuccess)
+            return HANN_ECUDA;
+    return HANN_OK;
+}
+
 bool encode_fused_available(const hann_ctx* c) {
     if (c->logN < 9) return false;
     for (int l = 0; l < c->L; l++)
@@ -788,9 +807,7 @@ int launch_encode_rows_fused(hann_ctx* c, const float* rows, int64_t rows_in_blo
             launch_chain(c, k_fft_w8h, dim3(chunks, count / 8), 128, 0, A);
         }
         KProf kp(c, KC_FFT_B);
-        const size_t smem = 16384 + (size_t)c->L * (1 << a) * 16;
-        if (smem > 48 * 1024) cudaFuncSetAttribute(pick_h(a), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        launch_chain(c, pick_h(a), dim3((1 << (a - 4)) + 1, count), 128, smem, A, count);
+        launch_chain(c, pick_h(a), dim3((1 << (a - 4)) + 1, count), 128, encode_h_smem(a, c->L), A, count);
         return check_launch(c, "encode_half");
     }
     if (c->B % 8 == 0 && count % 8 == 0 && p_first % 8 == 0) {
@@ -819,12 +836,9 @@ int launch_encode_rows_fused(hann_ctx* c, const float* rows, int64_t rows_in_blo
         k_fft_a<<<dim3(chunks / E.K1, count), kThreads, (size_t)E.K1 * 256 * sizeof(double2), c->stream>>>(E);
     }
     {
-        // exchange tile (FFT: 2^(a-1) x 16 complex = transform: 2^a x 16 words) when a > 4, then L x 2^a twiddle pairs
-        const size_t smem = (a > 4 ? (size_t)(1 << a) * 16 * 8 : 0) + (size_t)c->L * (1 << a) * 16;
         KProf kp(c, KC_FFT_B);
         const int threads = a >= 8 ? 256 : (a == 7 ? 128 : 64);  // 16 columns x 2^R2 row groups, at least two warps
-        if (smem > 48 * 1024) cudaFuncSetAttribute(pick_x(a, sym), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        launch_chain(c, pick_x(a, sym), dim3(16, count), threads, smem, A);
+        launch_chain(c, pick_x(a, sym), dim3(16, count), threads, encode_x_smem(a, c->L), A);
     }
     return check_launch(c, "encode_fused");
 }

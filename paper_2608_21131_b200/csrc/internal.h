@@ -195,6 +195,7 @@ int launch_wait_selftest(hann_ctx* c, unsigned long long limit_ns, unsigned long
 int launch_ks_lift(hann_ctx* c, u64* src, int64_t src_stride, int64_t nsrc, const LimbMap& src_lm, u64* dst, int n_tgt, int tgt_limb0, bool skip_own = false);
 // encode a block and run pass A of the transforms in one kernel when the parameters allow it (returns false if not)
 bool encode_fused_available(const hann_ctx* c);
+int encode_configure();  // once per context, its device current
 int launch_encode_rows_fused(hann_ctx* c, const float* rows, int64_t rows_in_block, int dim, int p_first, int count, u64* out,
                              int64_t out_stride, void* ws, bool sym);
 LimbMap limbmap_q(const hann_ctx* c);   // period L: limbs 0..L-1
@@ -224,6 +225,7 @@ int launch_ks_inner(hann_ctx* c, const u64* digits, int64_t digit_stride, int ro
 int launch_moddown_lift(hann_ctx* c, const u64* u, int64_t npoly, u64* lifted);
 // fused key switch of rings of 2^10 points and more (ksfused.cu)
 bool ks_fused_available(const hann_ctx* c);
+int ks_fused_configure();  // once per context, its device current
 int launch_ks_apply(hann_ctx* c, const u64* digits, const u64* own, int64_t own_it, int64_t own_z, int64_t items, int nz, int rot0, int rot_zinc, u64* u);
 int launch_ks_finish(hann_ctx* c, const u64* u, const u64* lifted, int64_t items, bool perm_items, int rot0, int rot_inc, int nz, const u64* c0,
                      int64_t c0_it, int64_t c0_z, const u64* add, int64_t add_it, u64* out0, u64* out1, int64_t out_it);

@@ -429,17 +429,29 @@ int run_finish(hann_ctx* c, FinishArgs& A, bool perm_items) {
     return check_launch(c, "ks_finish");
 }
 
+// sixteen lanes per digit, whole warps
+constexpr int apply_threads(int IB, int L) { return (IB * L * 16 + 31) / 32 * 32; }
+constexpr size_t apply_smem(int IB, int L) { return 4096 + (size_t)(2 * L + apply_threads(IB, L) / 16 + 2 * IB) * 2048; }
+
 template <int IB, int T>
 void launch_apply(hann_ctx* c, const ApplyArgs& A) {
-    // sixteen lanes per digit, whole warps
-    const int threads = (IB * A.L * 16 + 31) / 32 * 32;
-    const size_t smem = (size_t)4096 + (2 * A.L + (size_t)threads / 16 + 2 * IB) * 2048;
-    cudaFuncSetAttribute(k_ks_apply<IB, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     KProf kp(c, KC_KS_INNER);
-    launch_chain(c, k_ks_apply<IB, T>, dim3(c->N >> 8, A.L + 1, (unsigned)((A.items + IB - 1) / IB)), threads, smem, A);
+    launch_chain(c, k_ks_apply<IB, T>, dim3(c->N >> 8, A.L + 1, (unsigned)((A.items + IB - 1) / IB)), apply_threads(IB, A.L), apply_smem(IB, A.L), A);
 }
 
 }  // namespace
+
+// Dynamic shared memory of the instances that may need more than the default 48 KiB, for the longest chain launch_ks_apply sends to
+// each.  The limit belongs to the kernel and the device, not to a context: it is the same for every context, so that contexts of
+// different chain lengths do not take it from one another.
+int ks_fused_configure() {
+    static_assert(apply_smem(2, 4) <= 48 * 1024 && apply_smem(1, 4) <= 48 * 1024, "the other instances need no opt-in");
+    if (cudaFuncSetAttribute(k_ks_apply<4, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apply_smem(4, 4)) != cudaSuccess) return HANN_ECUDA;
+    if (cudaFuncSetAttribute(k_ks_apply<2, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apply_smem(2, 8)) != cudaSuccess) return HANN_ECUDA;
+    if (cudaFuncSetAttribute(k_ks_apply<1, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apply_smem(1, HANN_MAX_PRIMES)) != cudaSuccess)
+        return HANN_ECUDA;
+    return HANN_OK;
+}
 
 bool ks_fused_available(const hann_ctx* c) { return c->logN >= 10 && c->ntt_tau; }
 

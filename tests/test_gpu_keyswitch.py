@@ -91,3 +91,50 @@ def test_lazy_round_of_many_giant_steps():
     all_ = c.rotate_sum_lazy(inner, nb, c.alloc((nb + 1) * c.workspace_bytes(1)))
     c.sync()
     assert torch.equal(one, all_)
+
+
+def test_contexts_of_different_chains_on_two_threads():
+    """a call of a five-prime and one of a fifteen-prime context use the same kernel instance with different amounts of shared memory;
+    driven by two threads at once, neither takes its limit from the other"""
+    import threading
+
+    import torch
+
+    from paper_2608_21131_b200 import binding as b
+
+    logN, calls = 10, 150
+    q = find_primes(45, logN + 1, 15)
+    p = find_primes(60, logN + 1, 1)[0]
+
+    class Worker(threading.Thread):
+        def __init__(self, L):
+            super().__init__()
+            self.ps = synth.ParamSet("chain", logN, tuple(q[:L]), p, 20, 64, 1, 0)
+            self.stream = torch.cuda.Stream()
+            self.c = c = b.Context(self.ps, stream=self.stream)
+            c.load_keys(synth.uniform_residues(L, 2, q[:L] + [p], self.ps.N, lead=(1, L, 2)), [1])
+            self.inner = torch.randint(0, min(q), (c.sizeof(b.SIZE_INNER) // 8,), dtype=torch.int64, device=c.device,
+                                       generator=torch.Generator(c.device).manual_seed(L))
+            self.ws, self.score = c.workspace(1), c.alloc(c.sizeof(b.SIZE_CT))
+            torch.cuda.synchronize()
+            self.want = c.rotate_sum(self.inner, 1, self.ws)
+            c.sync()
+            self.error = None
+
+        def run(self):
+            try:
+                for _ in range(calls):  # 63 giant steps each
+                    self.c.rotate_sum(self.inner, 1, self.ws, self.score)
+                self.c.sync()
+            except b.HannError as e:
+                self.error = e
+
+    workers = [Worker(5), Worker(15)]
+    for w in workers:
+        w.start()
+    for w in workers:
+        w.join()
+    torch.cuda.synchronize()
+    for w in workers:
+        assert w.error is None, w.error
+        assert torch.equal(w.score, w.want)
