@@ -26,6 +26,11 @@
  *     steady state: while the per-launch profile (hann_kernel_profile) is on, every launch takes a CUDA event pair
  *     from a pool that grows on demand; and hann_score_level_host creates one event per block and per block group
  *     the first time it sees a level of that size (later calls of the same or a smaller size create nothing).
+ *   - The exchange and client calls (hann_import, hann_export*, key generation, encryption, decryption) stage their data in device
+ *     memory of the context: allocated at the first call that needs it, grown when a later one needs more, kept until
+ *     hann_ctx_destroy, never used by the server-side calls.  Its size is that of the largest call so far: 64 polynomials of L
+ *     limbs for hann_import (kind PT) and hann_export, (2 L + 1)(L + 1) polynomials of one limb for key generation, at most
+ *     64 MiB (and no less than one ciphertext) for decryption.
  *   - Canonical exchange layout (the only layout with a meaning outside the library): coefficient
  *     domain, natural coefficient order, residues in [0, q_i), uint64, index order [poly][limb][coeff];
  *     a ciphertext is 2 polynomials (c0, c1) of L limbs.  The internal device layout (transform domain,

@@ -1029,13 +1029,18 @@ extern "C" int hann_encrypt_query(hann_ctx* c, const int8_t* s, const float* q, 
 }
 
 // count ciphertexts of nl limbs each, ct [count][2][nl][N] canonical, plaintext scale 2^-exp2 / mult, in pieces of up to eight
-// ciphertexts
+// ciphertexts, as many as kDecryptScratch holds (one of N = 2^16 and four primes takes 5 MiB, of fifteen 17 MiB) and the device still
+// has memory for: one at a time works wherever one ciphertext fits
+constexpr int64_t kDecryptScratch = 64 << 20;
 static int decrypt_impl(hann_ctx* c, const int8_t* s, const uint64_t* ct, int64_t count, int nl, u64 mult, int exp2, double* scores,
                         double* imag_or_null) {
     const int N = c->N, n = c->n;
     DeviceGuard dg(c->device);
-    const int64_t LN = (int64_t)nl * N, piece = std::max<int64_t>(1, std::min<int64_t>(count, 8));
-    RET(ensure_scratch(c, (LN + piece * (2 * LN + N + 2 * n)) * 8 + align256(N) + kSlack));
+    const int64_t LN = (int64_t)nl * N, per = (2 * LN + N + 2 * n) * 8, rest = LN * 8 + align256(N) + kSlack;
+    int64_t piece = std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(count, 8), (kDecryptScratch - rest) / per));
+    int rc = ensure_scratch(c, rest + piece * per);
+    while (rc == HANN_ENOMEM && piece > 1) rc = ensure_scratch(c, rest + (piece /= 2) * per);
+    RET(rc);
     Arena ar{(char*)c->scratch, 0, c->scratch_bytes};
     u64* shat = ar.take<u64>(LN);
     u64* C0 = ar.take<u64>(piece * LN);

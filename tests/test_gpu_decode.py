@@ -60,3 +60,23 @@ def test_decoded_slots_of_chosen_integers(logN, bits, count):
             want = slots(exact[i], logN)
             # logN - 1 butterfly stages and the twist, each a rounding or two of relative size 2^-53, on either side
             assert np.linalg.norm(got[i] + 1j * imag[i] - want) <= 8 * logN * 2.0 ** -53 * np.linalg.norm(want)
+
+
+def test_scratch_of_a_decryption_is_bounded():
+    """eight ciphertexts of fifteen primes at N = 2^16 go through in pieces: the context's device memory grows by no more than the 64 MiB
+    that the header gives, and every ciphertext decrypts to the bits it has on its own"""
+    import torch
+
+    from paper_2608_21131_b200 import binding as b
+
+    q = find_primes(45, 17, 15)
+    ps = synth.ParamSet("deep", 16, tuple(q), find_primes(60, 17, 1)[0], 20, 4, 2, 0)
+    c = b.Context(ps)
+    s = synth.key_material(ps, 1, rots=[]).s
+    ct = np.random.default_rng(5).integers(0, min(q), size=(8, 2, ps.L, ps.N), dtype=np.uint64)
+    alone = [c.decrypt_scores(s, ct[i:i + 1], log_scale_out=640, want_imag=True) for i in range(8)]
+    free = torch.cuda.mem_get_info()[0]
+    got, imag = c.decrypt_scores(s, ct, log_scale_out=640, want_imag=True)
+    assert free - torch.cuda.mem_get_info()[0] <= 64 << 20
+    for i in range(8):
+        assert np.array_equal(got[i], alone[i][0][0]) and np.array_equal(imag[i], alone[i][1][0])
