@@ -176,8 +176,8 @@ int hann_kernel_times(hann_ctx *ctx, double *ms, uint64_t *launches);
  *     and records the source line in the context's error word, which the next synchronising call reports as HANN_ECUDA
  *     ("index range check failed ... source line N").  A release build has no such code.
  *   - hann_debug_canaries(ctx, 1) (any build) makes every server-side call put a 256-byte guard behind each sub-buffer it
- *     carves from the caller's workspace (the slack in hann_workspace_bytes covers them), filled with a pattern on the
- *     spot; hann_debug_verify(ctx, &checked, &damaged) checks all guards carved since the last verify, reports how many
+ *     carves from the caller's workspace (the slack in hann_workspace_bytes and hann_level_host_bytes covers them), filled
+ *     with a pattern on the spot; hann_debug_verify(ctx, &checked, &damaged) checks all guards carved since the last verify, reports how many
  *     there were and how many a kernel overwrote (HANN_ECUDA if any, naming the first one), and forgets them.  Call it
  *     while the workspaces of those calls are still allocated.  A later call that carves the same workspace retires the
  *     guards its own sub-buffers cover (they are overwritten legitimately), so verify after the call you want checked. */

@@ -1381,10 +1381,9 @@ extern "C" int hann_rotate_sum(hann_ctx* c, const void* inner_dev, int64_t n_blo
     // sixteen blocks: below, one round of all blocks fills the machine better (us of a level in one / two / four ranges: four
     // blocks of 2^15 850 / 880 / 892, eight 1373 / 1347 / 1391; three of 2^12 327 / 361 / 387, sixteen 844 / 845 / 979, twenty-nine
     // 1629 / 1373 / 1884; two of 2^16 1106 / 1114 / 1111, three 1335 / 1321 / 1353).
-    // (One lane while the per-launch profile is on, so that its kernel times do not overlap; with guards on always two, so that
-    // they cover both carvings.)
+    // (One lane while the per-launch profile is on, so that its kernel times do not overlap.)
     int lanes = (int)std::min<int64_t>(c->max_lanes, n_blocks);
-    if (fused) lanes = n_blocks * c->N <= (1 << 17) && n_blocks <= 16 && !c->canaries ? 1 : std::min(lanes, 2);
+    if (fused) lanes = n_blocks * c->N <= (1 << 17) && n_blocks <= 16 ? 1 : std::min(lanes, 2);
     if (c->stream == c->aux_stream || c->kprof) lanes = 1;
     while (lanes > 1 && (((int64_t)ws_bytes / lanes) & ~(int64_t)255) < ks_item_words(c) * 8 + kSlack) lanes--;
     if (lanes <= 1) return run_range(0, n_blocks, (char*)ws, (int64_t)ws_bytes);
@@ -1855,7 +1854,7 @@ LevelPlan plan_level(const hann_ctx* c, int64_t n_rows, int dim) {
 
 extern "C" int64_t hann_level_host_bytes(const hann_ctx* c, int64_t n_rows) {
     if (!c || n_rows < 0) return HANN_EINVAL;
-    return plan_level(c, n_rows, c->R).total;
+    return plan_level(c, n_rows, c->R).total + kSlack;  // the slack is for the guards of hann_debug_canaries
 }
 
 extern "C" int hann_score_level_host(hann_ctx* c, const uint64_t* ct_host, const float* rows_host, int64_t n_rows, int dim,
@@ -1867,16 +1866,17 @@ extern "C" int hann_score_level_host(hann_ctx* c, const uint64_t* ct_host, const
     const LevelPlan p = plan_level(c, n_rows, dim);
     if ((int64_t)ws_bytes < p.total) return fail(c, HANN_EWORKSPACE, "hann_score_level_host: workspace too small");
     DeviceGuard dg(c->device);
-    char* b = (char*)ws_dev;
-    u64* ct = (u64*)b; b += p.ct;
-    u64* baby = (u64*)b; b += p.baby;
-    float* rows = (float*)b; b += p.rows;
-    u64* pt = (u64*)b; b += p.pt;
-    u64* inner = (u64*)b; b += p.inner;
-    u64* score = (u64*)b; b += p.score;
-    u64* stage = (u64*)b; b += p.stage;
-    void* ws = b; b += p.ws;
-    char* ws_score[2] = {b, b + p.ws_score};
+    Arena ar{(char*)ws_dev, 0, (int64_t)ws_bytes, (int64_t)ws_bytes >= p.total + kSlack ? c : nullptr};
+    u64* ct = (u64*)ar.take<char>(p.ct);
+    u64* baby = (u64*)ar.take<char>(p.baby);
+    float* rows = (float*)ar.take<char>(p.rows);
+    u64* pt = (u64*)ar.take<char>(p.pt);
+    u64* inner = (u64*)ar.take<char>(p.inner);
+    u64* score = (u64*)ar.take<char>(p.score);
+    u64* stage = (u64*)ar.take<char>(p.stage);
+    void* ws = ar.take<char>(p.ws);
+    char* ws_score[2] = {nullptr, nullptr};
+    for (int i = 0; i < 2 && p.ng > 1; i++) ws_score[i] = ar.take<char>(p.ws_score);
     // The query goes up first, then the rows block by block on the upload stream; the helper stream prepares the baby
     // rotations; the context's stream encodes each block as soon as its rows have arrived.  The level is cut into groups
     // of blocks: a group is scored (multiply-accumulate, rotate-and-sum, inverse transform of its score ciphertexts) on

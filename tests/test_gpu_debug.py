@@ -68,6 +68,27 @@ def test_workspace_guards_survive_a_level(logN, R, B, L, big, n_rows):
     assert g.debug_verify() == (0, 0)       # switched off: nothing is carved with guards any more
 
 
+@pytest.mark.parametrize("nb,lanes", [(3, 1), (17, 2)])
+def test_guards_are_carved_as_without_them(nb, lanes):
+    """the rotate-and-sum of up to sixteen blocks of a small ring runs in one range, that of more in two, each with five sub-buffers of
+    its own: the guarded call takes the same ranges as the unguarded one, and every guard survives"""
+    import torch
+
+    from paper_2608_21131_b200 import binding as b
+
+    ps = synth.small_params(10, 16, 4, L=2)
+    g = Pair(ps, key_seed=2).g
+    inner = torch.randint(0, min(ps.q), (nb * g.sizeof(b.SIZE_INNER) // 8,), dtype=torch.int64, device=g.device,
+                          generator=torch.Generator(g.device).manual_seed(nb))
+    ws = g.workspace(nb)
+    plain = g.rotate_sum(inner, nb, ws)
+    g.debug_canaries(True)
+    guarded = g.rotate_sum(inner, nb, ws)
+    assert g.debug_verify() == (5 * lanes, 0)
+    g.debug_canaries(False)
+    assert torch.equal(plain, guarded)
+
+
 def test_a_damaged_guard_is_reported():
     """the verify kernel does notice an overwritten guard: the test itself overwrites one word of a guard (a host-side
     copy into the caller's own workspace: no kernel misbehaves), verify reports exactly one damaged guard, and the context
