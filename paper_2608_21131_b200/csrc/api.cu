@@ -234,17 +234,19 @@ int ks_digits_to_lifted(hann_ctx* c, u64* c1c, int64_t items, u64* digits, int64
 }
 
 // The same round on rings of 2^10 points and more (ksfused.cu), with the sum over nz rotations taken before the ModDown: polynomial
-// (z, item) to switch lies at src + item * src_it + z * src_z (transform domain, L limbs; left as it is unless it is c1c itself, which
-// the inverse pass overwrites: then nz = 1) and goes under the key of rotation rot0 + z * rot_zinc.  The automorphism is applied to
-// the sums, so what is left to the caller is launch_ks_finish.  Buffers, in words: c1c nz * items * LN, digits nz * items * L * L1N,
-// u items * 2 L1N, lifted items * 2 LN.
+// (z, item) to switch lies at src + item * src_it + z * src_z (transform domain, L limbs; left as it is) and goes under the key of
+// rotation rot0 + z * rot_zinc.  The automorphism is applied to the sums, so what is left to the caller is launch_ks_finish.  Buffers,
+// in words: c1c nz * items * LN, digits nz * items * L * LN, u items * 2 L1N, lifted items * 2 LN.
+// src == c1c, one polynomial (nz = items = 1) only: the inverse pass overwrites it, so its digits are lifted to their own modulus as
+// well, and the digits take L * L1N words (carve_keyswitch).
 int ks_round_fused(hann_ctx* c, const u64* src, int64_t src_it, int64_t src_z, int64_t items, int nz, int rot0, int rot_zinc, u64* c1c, u64* digits,
                    u64* u, u64* lifted) {
     const int L = c->L, N = c->N;
     const int64_t LN = (int64_t)L * N, L1N = (int64_t)(L + 1) * N;
     const bool in_place = src == c1c;
+    if (in_place && (nz != 1 || items != 1)) return fail(c, HANN_EINVAL, "a key-switch round in place takes one polynomial");
     if (in_place) {
-        RET(launch_ntt_inv_pass_b(c, c1c, items * L, N, limbmap_q(c)));
+        RET(launch_ntt_inv_pass_b(c, c1c, L, N, limbmap_q(c)));
     } else if (ntt_inv_pass_b_gathers(c, src, c1c) && ((src_it | src_z) & 1) == 0) {
         RET(launch_ntt_inv_pass_b_from(c, src, src_it, c1c, nz * items * L, N, limbmap_q(c), items, src_z));
     } else {
