@@ -1457,24 +1457,9 @@ extern "C" int hann_rotate_sum_lazy(hann_ctx* c, const void* inner_dev, int64_t 
                 continue;
             }
             // c1 of term (g, blk), still in the transform domain, into c1c[(g - 1) * nb + blk]
-            bool all_fused = lift;
-            for (int g = 1; g < G; g++) {
-                const u64* src = inner + (b0 * G + g) * ctw + LN;
-                u64* dst = c1c + (int64_t)(g - 1) * nb * LN;
-                const bool gathers = lift && ntt_inv_pass_b_gathers(c, src, dst);
-                all_fused = all_fused && gathers;
-                if (gathers) RET(launch_ntt_inv_pass_b_from(c, src, (int64_t)G * ctw, dst, nb * L, N, limbmap_q(c)));
-                else RET(launch_copy2d(c, dst, LN, src, (int64_t)G * ctw, LN, nb));
-            }
+            for (int g = 1; g < G; g++) RET(launch_copy2d(c, c1c + (int64_t)(g - 1) * nb * LN, LN, in0 + g * ctw + LN, (int64_t)G * ctw, LN, nb));
             if (lift) {
-                if (!all_fused) {
-                    // the terms whose inverse pass ran while gathering are finished; the copied ones still need it
-                    for (int g = 1; g < G; g++) {
-                        const u64* src = inner + (b0 * G + g) * ctw + LN;
-                        u64* dst = c1c + (int64_t)(g - 1) * nb * LN;
-                        if (!ntt_inv_pass_b_gathers(c, src, dst)) RET(launch_ntt_inv_pass_b(c, dst, nb * L, N, limbmap_q(c)));
-                    }
-                }
+                RET(launch_ntt_inv_pass_b(c, c1c, items * L, N, limbmap_q(c)));
                 RET(launch_ks_lift(c, c1c, N, items * L, limbmap_q(c), digits, L + 1, 0));
                 RET(launch_ntt_fwd_pass_b(c, digits, items * L * (L + 1), N, limbmap_qp(c)));
             } else {
@@ -1495,7 +1480,7 @@ extern "C" int hann_rotate_sum_lazy(hann_ctx* c, const void* inner_dev, int64_t 
                 RET(launch_lift_p(c, up, nb * 2, lifted));
                 RET(launch_ntt_fwd(c, lifted, nb * 2 * L, N, limbmap_q(c)));
             }
-            RET(launch_giant_combine(c, u, lifted, inner + b0 * G * ctw, nb, score + b0 * ctw));
+            RET(launch_giant_combine(c, u, lifted, in0, nb, score + b0 * ctw));
         }
         return HANN_OK;
     };
