@@ -41,7 +41,7 @@ struct hann_ctx {
     cudaEvent_t score_join[2] = {nullptr, nullptr};
     cudaEvent_t prep_done = nullptr;
     std::vector<cudaEvent_t> enc_ev;
-    int max_lanes = 4;  // block ranges hann_rotate_sum runs side by side
+    int max_lanes = 4;  // at most this many block ranges of hann_rotate_sum run side by side (rings of 2^10 points and more: one or two)
     u64 mod[HANN_MAXL1] = {};  // q_0..q_{L-1}, p
     LimbTable lt = {};
     LimbConst* lt_dev = nullptr;  // device copy of lt.c (the transform kernels read it from memory)

@@ -105,11 +105,11 @@ __global__ void __launch_bounds__(kThreads) k_ks_inner(const u64* digits, long l
 // and loops over the items.  When the items share one digit set and differ by key (the hoisted baby rotations:
 // KEYS_STREAM), the L digit words stay in registers and the 2L key words of each item stream past them; when the
 // items share the key (rotate-and-sum over blocks), the key words stay and the digit words stream.  The streamed
-// words of the next item are in flight while the current item is multiplied.  Moduli below 2^50 use the carry-free
-// 25-bit Karatsuba products of the multiply-accumulate kernel; the special prime uses 128-bit accumulation.
+// words of the next item are in flight while the current item is multiplied.  Rings of 2^10 points and more use the first
+// form alone: there the second one's work, and the sum over the giant steps, is k_ks_apply's (ksfused.cu).
 // MODE 0: moduli below 2^50, 25-bit halves, Karatsuba (3 products); MODE 1: moduli below 2^60 (the special prime),
 // 30-bit halves, 4 products (sums of 2 LL <= 8 products of 60 bits fit 64 bits); MODE 2: anything else, 128-bit
-// accumulation.
+// accumulation; MODE 3 (default): moduli below 2^50, exact two-word sums on the FP64 pipe.
 template <int LL, bool KEYS_STREAM, int MODE>
 __device__ __forceinline__ void ks_inner_body(const u64* digits, long long digit_stride, const u64* const* __restrict__ keytab,
                                               int rot0, int rot_inc, u64* __restrict__ u, long long L1N, long long pos, long long it0,
@@ -215,7 +215,7 @@ __device__ __forceinline__ void ks_inner_body(const u64* digits, long long digit
 }
 
 // blockIdx.z selects one of several independent batches of `nitems` items laid out one after the other (digits and u), batch
-// z using rotation rot0 + z * rot_zinc: the giant steps of the lazy rotate-and-sum, each under its own key
+// z using rotation rot0 + z * rot_zinc: the giant steps of the lazy rotate-and-sum on rings below 2^10 points, each under its own key
 template <int LL, bool KEYS_STREAM>
 __global__ void __launch_bounds__(128) k_ks_inner_stream(const u64* digits, long long digit_stride,
                                                          const u64* const* __restrict__ keytab, int rot0, int rot_inc,
@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(kThreads) k_moddown_combine(
     }
 }
 
-// The same combine for rings of at least 256 points, without scattered global reads.  In bit-reversed order the
+// The same combine for rings of 256 and 512 points (larger ones: k_ks_finish), without scattered global reads.  In bit-reversed order the
 // automorphism maps every aligned chunk of 256 positions onto another aligned chunk (the top 8 bits of a position are
 // the low 8 bits of its evaluation index, which an affine map modulo 2^logN keeps together), so a CTA loads the source
 // chunk of u, lifted and c0 contiguously into shared memory and permutes there.

@@ -480,8 +480,15 @@ int launch_ks_apply(hann_ctx* c, const u64* digits, const u64* own, int64_t own_
     A.tw_inv_f64 = c->tw_inv_f64;
     A.tw_inv_int = c->tw_inv;
     A.lt = c->lt_dev;
-    // items per CTA: their digits fill at most sixteen half-warps, and the eight-product sums allow several items up to eight
-    // primes only; key words and table entries are read once for all of them
+    // Items per CTA: their digits fill at most sixteen half-warps, and the eight-product sums allow several items up to eight
+    // primes only; key words and table entries are read once for all of them.  Us of a launch with one / two / four items per CTA
+    // (the absent items of a ragged last CTA cost their products all the same):
+    //   N = 2^16, L = 4, one rotation:    1 item 22 / 24 / 38, 2: 37 / 31 / 42, 3: 54 / 48 / 50, 4: 69 / 52 / 52, 5: 85 / 70 / 86, 8: 131 / 100 / 98
+    //             three rotations:        1 item 52 / 65 / 100, 2: 92 / 73 / 106, 4: 173 / 129 / 130, 5: 212 / 177 / 215, 16: 646 / 468 / 472
+    //   N = 2^15, L = 4, one rotation:    1 item 18 / 19 / 22, 2: 23 / 21 / 23, 4: 43 / 33 / 28, 8: 77 / 57 / 51, 16: 140 / 105 / 96
+    //   N = 2^12, L = 2, seven rotations: 1 item 78 / 68 / 62, 16: 86 / 88 / 83
+    //   N = 2^15, L = 8, one rotation:    1 item 24 / 32, 2: 45 / 42, 3: 64 / 70, 4: 82 / 77, 16: 292 / 281
+    // Four lose to two where they leave half of the last CTA empty (five and six items of four primes: 86 against 70 us).
     if (items >= 4 && c->L <= 4) launch_apply<4, 256>(c, A);
     else if (items >= 2 && c->L <= 4) launch_apply<2, 128>(c, A);
     else if (items >= 2 && c->L <= 8) launch_apply<2, 256>(c, A);

@@ -380,7 +380,8 @@ __global__ void __launch_bounds__(32 * NG) k_mac_ct_stream(const u64* baby, cons
 // (three stages: four are the same within 0.3 %, five cost 2 %, six 6 % of the kernel: the shared memory is worth more as L1)
 constexpr int kMacStages = 3;
 
-// partial sums per thread that cross the warps: four sums of three words (integer multiplier) or of two (FP64 pipe)
+// partial sums per thread that cross the warps: four sums of three words (integer multiplier), of one (FP64 pipe) or of two (the
+// same on a chain with primes of 2^50 and more, whose limbs cross as 128-bit sums)
 template <int NG, int BB, int F64>
 constexpr size_t mac_bulk_smem() {
     return (size_t)NG * kMacStages * BB * 256 + (size_t)2 * NG * (F64 == 1 ? 4 : F64 ? 8 : 12) * 256 + (size_t)NG * kMacStages * 8 + 16;

@@ -603,7 +603,8 @@ __global__ void __launch_bounds__(kThreads, AR::kMinBlocks) k_ntt_inv_a(NttArgs 
 // them, and its bound is the latency of that chain unless enough of them run side by side.  A binary64 coefficient enters a
 // binary64 target as it is; only the 60-bit special prime costs integer work, and its rounds are rolled (fwd_round4_smem).
 // Sum of the launches of a pass, against CTAs of 256 threads with the coefficients in registers and a Barrett reduction per
-// target: 493 -> 382 us (seven blocks, N = 2^16, L = 4), 5.18 -> 2.89 ms (membership circuit, N = 2^15, L = 12).
+// target: 493 -> 382 us (seven blocks, N = 2^16, L = 4), 5.18 -> 2.89 ms (membership circuit, N = 2^15, L = 12); 281 us on the seven
+// blocks since the rotate-and-sum leaves out the digits modulo their own prime (skip_own).
 
 struct LiftArgs {
     u64* src;             // source polynomials after inverse pass B' (private format of their modulus)
