@@ -248,7 +248,7 @@ int ks_round_fused(hann_ctx* c, const u64* src, int64_t src_it, int64_t src_z, i
     if (in_place) {
         RET(launch_ntt_inv_pass_b(c, c1c, L, N, limbmap_q(c)));
     } else if (ntt_inv_pass_b_gathers(c, src, c1c) && ((src_it | src_z) & 1) == 0) {
-        RET(launch_ntt_inv_pass_b_from(c, src, src_it, c1c, nz * items * L, N, limbmap_q(c), items, src_z));
+        RET(launch_ntt_inv_pass_b_from(c, src, src_it, c1c, nz * items * L, N, limbmap_q(c), nz > 1 ? items : 0, src_z));
     } else {
         for (int z = 0; z < nz; z++) RET(launch_copy2d(c, c1c + z * items * LN, LN, src + z * src_z, src_it, LN, items));
         RET(launch_ntt_inv_pass_b(c, c1c, nz * items * L, N, limbmap_q(c)));

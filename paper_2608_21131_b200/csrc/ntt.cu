@@ -58,7 +58,7 @@ struct NttArgs {
     // pos of the group pos * stride words further
     const u64* src;
     long long src_gstride;
-    int src_per, src_g0;
+    unsigned src_per, src_g0;
     long long src_zstride;
     u64 pos4, limb4;  // 4-bit fields: position within the period and limb of selection k (at most 16 selections)
     // forward pass B (bulk-copy kernel) of polynomials that are fixed by X -> 1/X and stored as their first N/2 transform
@@ -408,8 +408,10 @@ __global__ void __launch_bounds__(256, 3) k_ntt_inv_b8t(NttArgs A, int groups, i
     const u64* sbase = A.src ? A.src + (long long)pos * A.stride + ((size_t)chunk0 << 8) : gbase;
     auto source = [&](int i) {
         if (!A.src) return sbase + (long long)i * ystep * tile_stride;
-        const int g = A.src_g0 + (yg0 + i * ystep) * kTP + t;
-        return sbase + (A.src_per > 0 ? (g / A.src_per) * A.src_zstride + (g % A.src_per) * A.src_gstride : g * A.src_gstride);
+        const unsigned g = A.src_g0 + (yg0 + i * ystep) * kTP + t;
+        if (A.src_per == 0) return sbase + g * A.src_gstride;  // the division is a chain in front of the first copy
+        const unsigned z = g / A.src_per;
+        return sbase + z * A.src_zstride + (g - z * A.src_per) * A.src_gstride;
     };
     const int my_tiles = yg0 < ntiles ? (ntiles - yg0 + ystep - 1) / ystep : 0;
     auto tile_valid = [&](int i) { return i < my_tiles && (long long)(yg0 + (long long)i * ystep) * kTP + t < groups; };
@@ -1027,7 +1029,7 @@ int launch_ntt(hann_ctx* c, u64* data, int64_t npoly, int64_t stride, const Limb
     A.tau = c->ntt_tau;
     A.src = src;
     A.src_gstride = src_gstride;
-    A.src_per = (int)src_per;
+    A.src_per = (unsigned)src_per;
     A.src_g0 = 0;
     A.src_zstride = src_zstride;
     A.period = lm.period;
@@ -1064,7 +1066,7 @@ int launch_ntt(hann_ctx* c, u64* data, int64_t npoly, int64_t stride, const Limb
         for (int64_t g0 = 0; g0 < groups_total; g0 += gmax) {
             const int groups = (int)std::min<int64_t>(gmax, groups_total - g0);
             X.data = data + g0 * lm.period * stride;
-            if (src) X.src_g0 = (int)g0;
+            if (src) X.src_g0 = (unsigned)g0;
             const bool merge = mixed && b8t_eligible(c, X);
             if (!inverse) {
                 if (cls == 0) launch_fwd_class<ArithF64>(c, X, groups, skip_a, merge);
