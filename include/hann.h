@@ -244,7 +244,8 @@ int hann_decrypt_compact(hann_ctx *ctx, const int8_t *s, const uint64_t *ct, int
 
 /* Upload evaluation keys (canonical layout as produced by hann_keygen_from_samples; `evk` may be a host or a
  * device pointer) into the context, replacing keys with the same rotation.  Allocates device memory owned by the
- * context.  Needed later: rotations 1..B-1 for hann_query_prepare, rotation B for hann_rotate_sum. */
+ * context: 2 L (L + 1) polynomials of one limb per key, and 6 L more where the key switch has auxiliary primes (rings of 2^10 points
+ * and more, three ciphertext primes below 2^50 and a special prime in [2^50, 2^61)); as much again while the call runs.  Needed later: rotations 1..B-1 for hann_query_prepare, rotation B for hann_rotate_sum. */
 int hann_load_keys(hann_ctx *ctx, const uint64_t *evk, int n_rot, const int32_t *rot);
 
 /* Once per query (Sec. 3.1 Detail: the baby steps of the diagonal method; Sec. 3.4: the rotated query is computed

@@ -128,6 +128,9 @@ int64_t ks_item_words(const hann_ctx* c) {
     return L * N + L * (ks_fused_available(c) ? L : L + 1) * N + 2 * (L + 1) * N + 2 * L * N + 2 * L * N;
 }
 
+// limbs of the product u of a key-switch round (ks_round_fused) whose polynomials are not switched in place
+int ks_u_limbs(const hann_ctx* c) { return c->L + (c->aux ? kAux : 1); }
+
 // words of workspace the lazy rotate-and-sum needs per block of a round: G-1 terms (c1 coefficients, digits, and their key products
 // unless the fused kernels sum them), the summed product and one ModDown
 int64_t lazy_block_words(const hann_ctx* c) {
@@ -147,6 +150,24 @@ constexpr int64_t kSlack = 16 * 256;  // room for the alignment of a dozen sub-b
 int64_t balanced(int64_t most, int64_t total) {
     const int64_t rounds = (total + most - 1) / most;
     return (total + rounds - 1) / rounds;
+}
+
+// the sub-buffers of a key-switch round (ks_round_fused, or ks_digits_to_lifted on smaller rings) on nz * items polynomials.  With
+// auxiliary primes u has two more limbs and a digit one target less, so a round needs no more words than ks_item_words and
+// lazy_block_words count, except on a chain of three primes: where the arena ends there, the lifted polynomials (carved last) take
+// the place of the digits, which k_ks_apply was the last to read.
+struct RoundBuffers {
+    u64 *c1c, *digits, *u, *lifted;
+};
+bool carve_round(const hann_ctx* c, Arena& ar, int64_t items, int64_t nz, RoundBuffers& b) {
+    const int64_t L = c->L, N = c->N, digits = L * (ks_fused_available(c) ? (c->aux ? L - 1 : L) : L + 1) * N;
+    const int64_t u = 2 * (ks_fused_available(c) ? ks_u_limbs(c) : L + 1) * N;
+    b.c1c = ar.take<u64>(nz * items * L * N);
+    b.digits = ar.take<u64>(nz * items * digits);
+    b.u = ar.take<u64>(items * u);
+    b.lifted = ar.take<u64>(items * 2 * L * N);
+    if (!b.lifted && c->aux && L == 3) b.lifted = b.digits;
+    return b.c1c && b.digits && b.u && b.lifted;
 }
 
 // the four sub-buffers of ONE key switch (hann_keyswitch, hann_keyswitch_static): input copy, digits, u, lifted
@@ -235,10 +256,10 @@ int ks_digits_to_lifted(hann_ctx* c, u64* c1c, int64_t items, u64* digits, int64
 
 // The same round on rings of 2^10 points and more (ksfused.cu), with the sum over nz rotations taken before the ModDown: polynomial
 // (z, item) to switch lies at src + item * src_it + z * src_z (transform domain, L limbs; left as it is) and goes under the key of
-// rotation rot0 + z * rot_zinc.  The automorphism is applied to the sums, so what is left to the caller is launch_ks_finish.  Buffers,
-// in words: c1c nz * items * LN, digits nz * items * L * LN, u items * 2 L1N, lifted items * 2 LN.
+// rotation rot0 + z * rot_zinc.  The automorphism is applied to the sums, so what is left to the caller is launch_ks_finish.  Buffers
+// as carve_round leaves them.
 // src == c1c, one polynomial (nz = items = 1) only: the inverse pass overwrites it, so its digits are lifted to their own modulus as
-// well, and the digits take L * L1N words (carve_keyswitch).
+// well, the product modulo the special prime takes no auxiliary primes, and the digits take L * L1N words (carve_keyswitch).
 int ks_round_fused(hann_ctx* c, const u64* src, int64_t src_it, int64_t src_z, int64_t items, int nz, int rot0, int rot_zinc, u64* c1c, u64* digits,
                    u64* u, u64* lifted) {
     const int L = c->L, N = c->N;
@@ -254,9 +275,11 @@ int ks_round_fused(hann_ctx* c, const u64* src, int64_t src_it, int64_t src_z, i
         RET(launch_ntt_inv_pass_b(c, c1c, nz * items * L, N, limbmap_q(c)));
     }
     // a digit's transform modulo its own prime is the polynomial that came in, where that still exists
-    RET(launch_ks_lift(c, c1c, N, nz * items * L, limbmap_q(c), digits, in_place ? L + 1 : L, 0, !in_place));
+    const bool aux = c->aux && !in_place;
+    RET(launch_ks_lift(c, c1c, N, nz * items * L, limbmap_q(c), digits, in_place ? L + 1 : aux ? L - 1 : L, 0, !in_place));
     RET(launch_ks_apply(c, digits, in_place ? nullptr : src, src_it, src_z, items, nz, rot0, rot_zinc, u));
-    RET(launch_ks_lift(c, u + LN, L1N, items * 2, limbmap_single(L), lifted, L, 0));
+    if (aux) RET(launch_ks_lift_aux(c, u + LN, LN + kAux * (int64_t)N, items * 2, lifted));
+    else RET(launch_ks_lift(c, u + LN, L1N, items * 2, limbmap_single(L), lifted, L, 0));
     return HANN_OK;
 }
 
@@ -272,6 +295,41 @@ int64_t keyswitch_ws_bytes(const hann_ctx* c) {
     ar.base = (char*)256;  // any non-null base: the carving only does pointer arithmetic
     carve_keyswitch(c, ar, kb);
     return ar.off;
+}
+
+// Auxiliary primes of the key switch (AuxCrt): the three largest ciphertext primes below 2^50, on rings whose key switch is fused,
+// with a special prime in [2^50, 2^61) (a smaller one has transforms on the FP64 pipe itself), if every sum of key products a call
+// takes before its ModDown -- up to G - 1 rotations of L digits, |digit| < q_j / 2, |key| < p / 2 -- stays below a quarter of their
+// product.
+static void choose_aux(hann_ctx* c) {
+    if (!ks_fused_available(c) || c->mod[c->L] < (1ULL << 50) || c->mod[c->L] >= (1ULL << 61)) return;
+    std::vector<int> small;
+    for (int i = 0; i < c->L; i++)
+        if (c->mod[i] < (1ULL << 50)) small.push_back(i);
+    if (small.size() < kAux) return;
+    std::stable_sort(small.begin(), small.end(), [&](int a, int b) { return c->mod[a] > c->mod[b]; });
+    const u64 qa = c->mod[small[0]], qb = c->mod[small[1]], qc = c->mod[small[2]], p = c->mod[c->L];
+    if (qa / 2 >= qc) return;  // the digits of the recombination stay below four times the modulus they meet
+    double digits = 0;
+    for (int i = 0; i < c->L; i++) digits += (double)c->mod[i] / 2;
+    const double terms = (double)c->N * std::max(c->G - 1, 1);
+    if (log2(digits) + log2((double)p / 2) + log2(terms) + 2.01 > log2((double)qa) + log2((double)qb) + log2((double)qc)) return;
+    AuxCrt& X = c->crt;
+    for (int k = 0; k < kAux; k++) X.limb[k] = (signed char)small[k];
+    auto inverse = [](u64 v, u64 q) {
+        const u64 w = hm::invmod(v % q, q);
+        const double b = w > q / 2 ? -(double)(q - w) : (double)w;
+        return make_double2(b, b / (double)q);
+    };
+    X.ab = inverse(qa, qb);
+    X.ac = inverse(qa, qc);
+    X.bc = inverse(qb, qc);
+    X.c1 = qa % p;
+    X.c2 = hm::mulmod(qa % p, qb % p, p);
+    X.c1s = hm::shoup(X.c1, p);
+    X.c2s = hm::shoup(X.c2, p);
+    X.off = 2 * p - hm::mulmod((1ULL << 50) % p, (X.c1 + X.c2) % p, p);
+    c->aux = true;
 }
 
 // ================================================================================================ context
@@ -369,6 +427,7 @@ extern "C" int hann_ctx_create(const hann_params* prm, hann_ctx** out) {
             twi64[o] = iwb; twi64[o + 1] = iwb / (double)q;
         }
     }
+    choose_aux(c);
     // encode tables
     const int nh = std::max(n / 2, 1);
     std::vector<double2> T(nh), U(n);
@@ -1097,13 +1156,16 @@ extern "C" int hann_load_keys(hann_ctx* c, const uint64_t* evk, int n_rot, const
     for (int i = 0; i < n_rot; i++)
         if (rot[i] < 0 || rot[i] >= c->n) return fail(c, HANN_ESHAPE, "hann_load_keys: rotation out of range");
     DeviceGuard dg(c->device);
-    const int64_t keyw = (int64_t)L * 2 * (L + 1) * N;
-    RET(ensure_scratch(c, keyw * 8));
+    const int64_t keyw = (int64_t)L * 2 * (L + 1) * N, auxw = c->aux ? (int64_t)L * 2 * kAux * N : 0;
+    RET(ensure_scratch(c, (keyw + auxw) * 8));
+    LimbMap lm_aux;
+    lm_aux.period = kAux;
+    for (int k = 0; k < kAux; k++) lm_aux.limb[k] = c->crt.limb[k];
     for (int i = 0; i < n_rot; i++) {
         const int r = rot[i];
         if (!c->keytab_host[r]) {
             u64* buf = nullptr;
-            if (cudaMalloc(&buf, keyw * 8) != cudaSuccess) {
+            if (cudaMalloc(&buf, (keyw + auxw) * 8) != cudaSuccess) {
                 cudaGetLastError();
                 return fail(c, HANN_ENOMEM, "hann_load_keys: device allocation failed");
             }
@@ -1111,13 +1173,17 @@ extern "C" int hann_load_keys(hann_ctx* c, const uint64_t* evk, int n_rot, const
         }
         u64* tmp = (u64*)c->scratch;
         CK(cudaMemcpyAsync(tmp, evk + (int64_t)i * keyw, keyw * 8, cudaMemcpyDefault, c->stream));
+        if (c->aux) {
+            RET(launch_key_aux(c, tmp, tmp + keyw));
+            RET(launch_ntt_fwd(c, tmp + keyw, (int64_t)L * 2 * kAux, N, lm_aux));
+        }
         RET(launch_ntt_fwd(c, tmp, (int64_t)L * 2 * (L + 1), N, limbmap_qp(c)));
         // store phi_k^{-1}(key): the inner product then runs on unpermuted digits and the automorphism is applied
         // once, to its much smaller result
         const unsigned k = c->h_galois[r];
         const unsigned kinv = c->h_galois[(c->n - r) % c->n];  // 5^{-r} = 5^{n-r} (5 has order n modulo 2N)
         (void)k;
-        RET(launch_permute(c, tmp, c->keytab_host[r], (int64_t)L * 2 * (L + 1), kinv));
+        RET(launch_permute(c, tmp, c->keytab_host[r], (keyw + auxw) / N, kinv));
         RET(sync_and_check(c));
     }
     CK(cudaMemcpy(c->keytab_dev, c->keytab_host.data(), c->keytab_host.size() * sizeof(u64*), cudaMemcpyHostToDevice));
@@ -1142,7 +1208,7 @@ static int rotate_hoisted(hann_ctx* c, const char* who, const u64* ct, int rot0,
     // one digit set, count keys: item i uses rotation rot0 + i
     const bool fin = ks_fused_available(c);
     RET(ks_digits_to_lifted(c, c1c, 1, digits, 0, rot0, 1, count, u, lifted, ct + LN, 2 * LN, fin));
-    if (fin) RET(launch_ks_finish(c, u, lifted, count, true, rot0, 1, 1, ct, 0, 0, nullptr, 0, out, out + LN, ctw));
+    if (fin) RET(launch_ks_finish(c, u, L + 1, lifted, count, true, rot0, 1, 1, ct, 0, 0, nullptr, 0, out, out + LN, ctw));
     else RET(launch_moddown_combine(c, u, lifted, count, rot0, 1, ct, 0, nullptr, 0, out, out + LN, ctw));
     return HANN_OK;
 }
@@ -1257,11 +1323,8 @@ extern "C" int hann_score_level_ctdb(hann_ctx* c, const void* baby_dev, const vo
     ch = balanced(std::min<int64_t>(ch, 8 * G), items);
     Arena ar{(char*)ws, 0, (int64_t)ws_bytes, c};
     u64* d = ar.take<u64>(ch * 3 * LN);
-    u64* c1c = ar.take<u64>(ch * LN);
-    u64* digits = ar.take<u64>(ch * L * (ks_fused_available(c) ? LN : L1N));
-    u64* u = ar.take<u64>(ch * 2 * L1N);
-    u64* lifted = ar.take<u64>(ch * 2 * LN);
-    if (!d || !c1c || !digits || !u || !lifted) return fail(c, HANN_EWORKSPACE, "hann_score_level_ctdb: workspace too small");
+    RoundBuffers rb;
+    if (!d || !carve_round(c, ar, ch, 1, rb)) return fail(c, HANN_EWORKSPACE, "hann_score_level_ctdb: workspace too small");
     const u64* ctdb = (const u64*)ctdb_dev;
     u64* inner = (u64*)inner_dev;
     for (int64_t i0 = 0; i0 < items; i0 += ch) {
@@ -1270,13 +1333,13 @@ extern "C" int hann_score_level_ctdb(hann_ctx* c, const void* baby_dev, const vo
         // relinearise: (d0 + ks0, d1 + ks1) with (ks0, ks1) the key switch of d2 under the key of s^2 ("rotation 0": no
         // automorphism)
         if (ks_fused_available(c)) {
-            RET(ks_round_fused(c, d + 2 * LN, 3 * LN, 0, ni, 1, 0, 0, c1c, digits, u, lifted));
-            RET(launch_ks_finish(c, u, lifted, ni, false, 0, 0, 1, nullptr, 0, 0, d, 3 * LN, inner + i0 * ctw, inner + i0 * ctw + LN, ctw));
+            RET(ks_round_fused(c, d + 2 * LN, 3 * LN, 0, ni, 1, 0, 0, rb.c1c, rb.digits, rb.u, rb.lifted));
+            RET(launch_ks_finish(c, rb.u, ks_u_limbs(c), rb.lifted, ni, false, 0, 0, 1, nullptr, 0, 0, d, 3 * LN, inner + i0 * ctw, inner + i0 * ctw + LN, ctw));
             continue;
         }
-        RET(launch_copy2d(c, c1c, LN, d + 2 * LN, 3 * LN, LN, ni));
-        RET(ks_digits_to_lifted(c, c1c, ni, digits, (int64_t)L * L1N, 0, 0, ni, u, lifted));
-        RET(launch_moddown_combine(c, u, lifted, ni, 0, 0, nullptr, 0, d, 3 * LN, inner + i0 * ctw, inner + i0 * ctw + LN, ctw));
+        RET(launch_copy2d(c, rb.c1c, LN, d + 2 * LN, 3 * LN, LN, ni));
+        RET(ks_digits_to_lifted(c, rb.c1c, ni, rb.digits, (int64_t)L * L1N, 0, 0, ni, rb.u, rb.lifted));
+        RET(launch_moddown_combine(c, rb.u, rb.lifted, ni, 0, 0, nullptr, 0, d, 3 * LN, inner + i0 * ctw, inner + i0 * ctw + LN, ctw));
     }
     return HANN_OK;
 }
@@ -1300,11 +1363,8 @@ extern "C" int hann_multiply(hann_ctx* c, const void* a_dev, const void* b_dev, 
     ch = balanced(std::min<int64_t>(ch, 32), count);
     Arena ar{(char*)ws, 0, (int64_t)ws_bytes, c};
     u64* d = ar.take<u64>(ch * 3 * LN);
-    u64* c1c = ar.take<u64>(ch * LN);
-    u64* digits = ar.take<u64>(ch * L * (ks_fused_available(c) ? LN : L1N));
-    u64* u = ar.take<u64>(ch * 2 * L1N);
-    u64* lifted = ar.take<u64>(ch * 2 * LN);
-    if (!d || !c1c || !digits || !u || !lifted) return fail(c, HANN_EWORKSPACE, "hann_multiply: workspace too small");
+    RoundBuffers rb;
+    if (!d || !carve_round(c, ar, ch, 1, rb)) return fail(c, HANN_EWORKSPACE, "hann_multiply: workspace too small");
     const u64 *a = (const u64*)a_dev, *b = (const u64*)b_dev;
     u64* out = (u64*)out_dev;
     for (int64_t i0 = 0; i0 < count; i0 += ch) {
@@ -1312,13 +1372,13 @@ extern "C" int hann_multiply(hann_ctx* c, const void* a_dev, const void* b_dev, 
         RET(launch_mul_ct(c, a + i0 * ctw, b + i0 * ctw, ni, d));
         // relinearise: (d0 + ks0, d1 + ks1), (ks0, ks1) the key switch of d2 under the key of s^2 ("rotation 0")
         if (ks_fused_available(c)) {
-            RET(ks_round_fused(c, d + 2 * LN, 3 * LN, 0, ni, 1, 0, 0, c1c, digits, u, lifted));
-            RET(launch_ks_finish(c, u, lifted, ni, false, 0, 0, 1, nullptr, 0, 0, d, 3 * LN, out + i0 * ctw, out + i0 * ctw + LN, ctw));
+            RET(ks_round_fused(c, d + 2 * LN, 3 * LN, 0, ni, 1, 0, 0, rb.c1c, rb.digits, rb.u, rb.lifted));
+            RET(launch_ks_finish(c, rb.u, ks_u_limbs(c), rb.lifted, ni, false, 0, 0, 1, nullptr, 0, 0, d, 3 * LN, out + i0 * ctw, out + i0 * ctw + LN, ctw));
             continue;
         }
-        RET(launch_copy2d(c, c1c, LN, d + 2 * LN, 3 * LN, LN, ni));
-        RET(ks_digits_to_lifted(c, c1c, ni, digits, (int64_t)L * L1N, 0, 0, ni, u, lifted));
-        RET(launch_moddown_combine(c, u, lifted, ni, 0, 0, nullptr, 0, d, 3 * LN, out + i0 * ctw, out + i0 * ctw + LN, ctw));
+        RET(launch_copy2d(c, rb.c1c, LN, d + 2 * LN, 3 * LN, LN, ni));
+        RET(ks_digits_to_lifted(c, rb.c1c, ni, rb.digits, (int64_t)L * L1N, 0, 0, ni, rb.u, rb.lifted));
+        RET(launch_moddown_combine(c, rb.u, rb.lifted, ni, 0, 0, nullptr, 0, d, 3 * LN, out + i0 * ctw, out + i0 * ctw + LN, ctw));
     }
     return HANN_OK;
 }
@@ -1348,12 +1408,9 @@ extern "C" int hann_rotate_sum(hann_ctx* c, const void* inner_dev, int64_t n_blo
         if (ch < 1) return fail(c, HANN_EWORKSPACE, "hann_rotate_sum: workspace too small");
         ch = balanced(std::min<int64_t>(ch, 8), b_hi - b_lo);
         Arena ar{wsp, 0, wsp_bytes, c};
-        u64* c1c = ar.take<u64>(ch * LN);
-        u64* digits = ar.take<u64>(ch * L * (fused ? LN : L1N));
-        u64* u = ar.take<u64>(ch * 2 * L1N);
-        u64* lifted = ar.take<u64>(ch * 2 * LN);
+        RoundBuffers rb;
         u64* tmp = ar.take<u64>(ch * ctw);
-        if (!c1c || !digits || !u || !lifted || !tmp) return fail(c, HANN_EWORKSPACE, "hann_rotate_sum: workspace too small");
+        if (!tmp || !carve_round(c, ar, ch, 1, rb)) return fail(c, HANN_EWORKSPACE, "hann_rotate_sum: workspace too small");
         for (int64_t b0 = b_lo; b0 < b_hi; b0 += ch) {
             const int64_t nb = std::min(ch, b_hi - b0);
             const u64* old = inner + (b0 * G + (G - 1)) * ctw;  // acc = inner[G-1]
@@ -1362,15 +1419,15 @@ extern "C" int hann_rotate_sum(hann_ctx* c, const void* inner_dev, int64_t n_blo
                 u64* out = (g % 2 == 0) ? score + b0 * ctw : tmp;
                 // c1 of every accumulator, still in the transform domain; the key-switch round takes it from there
                 if (fused) {
-                    RET(ks_round_fused(c, old + LN, old_stride, 0, nb, 1, B, 0, c1c, digits, u, lifted));
-                    RET(launch_ks_finish(c, u, lifted, nb, false, B, 0, 1, old, old_stride, 0, inner + (b0 * G + g) * ctw, (int64_t)G * ctw, out,
+                    RET(ks_round_fused(c, old + LN, old_stride, 0, nb, 1, B, 0, rb.c1c, rb.digits, rb.u, rb.lifted));
+                    RET(launch_ks_finish(c, rb.u, ks_u_limbs(c), rb.lifted, nb, false, B, 0, 1, old, old_stride, 0, inner + (b0 * G + g) * ctw, (int64_t)G * ctw, out,
                                          out + LN, ctw));
                     old = out;
                     old_stride = ctw;
                     continue;
                 }
-                RET(ks_digits_to_lifted(c, c1c, nb, digits, (int64_t)L * L1N, B, 0, nb, u, lifted, old + LN, old_stride));
-                RET(launch_moddown_combine(c, u, lifted, nb, B, 0, old, old_stride, inner + (b0 * G + g) * ctw, (int64_t)G * ctw, out,
+                RET(ks_digits_to_lifted(c, rb.c1c, nb, rb.digits, (int64_t)L * L1N, B, 0, nb, rb.u, rb.lifted, old + LN, old_stride));
+                RET(launch_moddown_combine(c, rb.u, rb.lifted, nb, B, 0, old, old_stride, inner + (b0 * G + g) * ctw, (int64_t)G * ctw, out,
                                            out + LN, ctw));
                 old = out;
                 old_stride = ctw;
@@ -1440,19 +1497,27 @@ extern "C" int hann_rotate_sum_lazy(hann_ctx* c, const void* inner_dev, int64_t 
         ch = balanced(std::min<int64_t>(ch, 16), b_hi - b_lo);
         Arena ar{wsp, 0, wsp_bytes, c};
         const int64_t items_max = ch * (G - 1);
-        u64* c1c = ar.take<u64>(items_max * LN);
-        u64* digits = ar.take<u64>(items_max * L * (fused ? LN : L1N));
-        u64* u = ar.take<u64>((fused ? ch : items_max) * 2 * L1N);
-        u64* up = fused ? u : ar.take<u64>(ch * 2 * N);
-        u64* lifted = ar.take<u64>(ch * 2 * LN);
-        if (!c1c || !digits || !u || !up || !lifted) return fail(c, HANN_EWORKSPACE, "hann_rotate_sum_lazy: workspace too small");
+        RoundBuffers rb = {};
+        u64 *c1c = nullptr, *digits = nullptr, *u = nullptr, *up = nullptr, *lifted = nullptr;
+        bool carved;
+        if (fused) {
+            carved = carve_round(c, ar, ch, G - 1, rb);
+        } else {
+            c1c = ar.take<u64>(items_max * LN);
+            digits = ar.take<u64>(items_max * L * L1N);
+            u = ar.take<u64>(items_max * 2 * L1N);
+            up = ar.take<u64>(ch * 2 * N);
+            lifted = ar.take<u64>(ch * 2 * LN);
+            carved = c1c && digits && u && up && lifted;
+        }
+        if (!carved) return fail(c, HANN_EWORKSPACE, "hann_rotate_sum_lazy: workspace too small");
         for (int64_t b0 = b_lo; b0 < b_hi; b0 += ch) {
             const int64_t nb = std::min(ch, b_hi - b0), items = nb * (G - 1);
             const u64* in0 = inner + b0 * G * ctw;
             if (fused) {
                 // all giant steps summed under their own keys and automorphisms before one ModDown per block
-                RET(ks_round_fused(c, in0 + ctw + LN, (int64_t)G * ctw, ctw, nb, G - 1, B, B, c1c, digits, u, lifted));
-                RET(launch_ks_finish(c, u, lifted, nb, false, B, B, G - 1, in0 + ctw, (int64_t)G * ctw, ctw, in0, (int64_t)G * ctw, score + b0 * ctw,
+                RET(ks_round_fused(c, in0 + ctw + LN, (int64_t)G * ctw, ctw, nb, G - 1, B, B, rb.c1c, rb.digits, rb.u, rb.lifted));
+                RET(launch_ks_finish(c, rb.u, ks_u_limbs(c), rb.lifted, nb, false, B, B, G - 1, in0 + ctw, (int64_t)G * ctw, ctw, in0, (int64_t)G * ctw, score + b0 * ctw,
                                      score + b0 * ctw + LN, ctw));
                 continue;
             }
@@ -1629,20 +1694,20 @@ extern "C" int hann_fold(hann_ctx* c, void* ct_dev, int stride, int steps, void*
     DeviceGuard dg(c->device);
     Timer tm(c, 3);
     Arena ar{(char*)ws, 0, (int64_t)ws_bytes, c};
-    KsBuffers kb;
+    RoundBuffers rb;
     u64* tmp = ar.take<u64>(ctw);
-    if (!tmp || !carve_keyswitch(c, ar, kb)) return fail(c, HANN_EWORKSPACE, "hann_fold: workspace too small");
+    if (!tmp || !carve_round(c, ar, 1, 1, rb)) return fail(c, HANN_EWORKSPACE, "hann_fold: workspace too small");
     u64* cur = (u64*)ct_dev;
     u64* nxt = tmp;
     for (int t = 0; t < steps; t++) {
         const int r = stride << t;
         // nxt = cur + rot_r(cur): the Horner step of the rotate-and-sum with the ciphertext itself as the addend
         if (ks_fused_available(c)) {
-            RET(ks_round_fused(c, cur + LN, ctw, 0, 1, 1, r, 0, kb.c1c, kb.digits, kb.u, kb.lifted));
-            RET(launch_ks_finish(c, kb.u, kb.lifted, 1, false, r, 0, 1, cur, ctw, 0, cur, ctw, nxt, nxt + LN, ctw));
+            RET(ks_round_fused(c, cur + LN, ctw, 0, 1, 1, r, 0, rb.c1c, rb.digits, rb.u, rb.lifted));
+            RET(launch_ks_finish(c, rb.u, ks_u_limbs(c), rb.lifted, 1, false, r, 0, 1, cur, ctw, 0, cur, ctw, nxt, nxt + LN, ctw));
         } else {
-            RET(ks_digits_to_lifted(c, kb.c1c, 1, kb.digits, (int64_t)L * L1N, r, 0, 1, kb.u, kb.lifted, cur + LN, ctw));
-            RET(launch_moddown_combine(c, kb.u, kb.lifted, 1, r, 0, cur, ctw, cur, ctw, nxt, nxt + LN, ctw));
+            RET(ks_digits_to_lifted(c, rb.c1c, 1, rb.digits, (int64_t)L * L1N, r, 0, 1, rb.u, rb.lifted, cur + LN, ctw));
+            RET(launch_moddown_combine(c, rb.u, rb.lifted, 1, r, 0, cur, ctw, cur, ctw, nxt, nxt + LN, ctw));
         }
         std::swap(cur, nxt);
     }
@@ -1720,7 +1785,7 @@ extern "C" int hann_keyswitch(hann_ctx* c, int rot, const void* poly_dev, void* 
     RET(launch_permute(c, (const u64*)poly_dev, c1c, L, kinv));
     if (ks_fused_available(c)) {
         RET(ks_round_fused(c, c1c, (int64_t)L * c->N, 0, 1, 1, rot, 0, c1c, digits, u, lifted));
-        return launch_ks_finish(c, u, lifted, 1, false, 0, 0, 1, nullptr, 0, 0, nullptr, 0, (u64*)ks0_dev, (u64*)ks1_dev, 0);
+        return launch_ks_finish(c, u, L + 1, lifted, 1, false, 0, 0, 1, nullptr, 0, 0, nullptr, 0, (u64*)ks0_dev, (u64*)ks1_dev, 0);
     }
     RET(ks_digits_to_lifted(c, c1c, 1, digits, 0, rot, 0, 1, u, lifted));
     RET(launch_moddown_combine(c, u, lifted, 1, rot, 0, nullptr, 0, nullptr, 0, (u64*)ks0_dev, (u64*)ks1_dev, 0));

@@ -16,6 +16,17 @@ enum {
     KC_MODDOWN_LIFT, KC_MODDOWN_COMBINE, KC_PERMUTE, KC_OTHER, KC_KS_INNER_KEYS, KC_COUNT
 };
 
+// Auxiliary primes of the key switch: the product with a key modulo the special prime p is an integer below a quarter of the product of
+// three ciphertext primes q_a, q_b, q_c below 2^50, so it is computed modulo those -- whose transforms run on the FP64 pipe and of which
+// the digits are transforms already -- and taken modulo p afterwards (see k_ks_lift_aux in ntt.cu for the recombination).
+struct AuxCrt {
+    signed char limb[4];  // a, b, c
+    double2 ab, ac, bc;   // q_a^{-1} mod q_b, q_a^{-1} mod q_c, q_b^{-1} mod q_c as (balanced, fl(. / modulus))
+    u64 c1, c1s, c2, c2s;  // q_a and q_a q_b modulo p with their Shoup companions
+    u64 off;               // -2^50 (c1 + c2) modulo p, in [p, 2p)
+};
+constexpr int kAux = 3;
+
 struct hann_ctx {
     hann_params prm;
     int logN = 0, N = 0, n = 0, L = 0, R = 0, B = 0, G = 0;
@@ -43,6 +54,8 @@ struct hann_ctx {
     std::vector<cudaEvent_t> enc_ev;
     int max_lanes = 4;  // at most this many block ranges of hann_rotate_sum run side by side (rings of 2^10 points and more: one or two)
     u64 mod[HANN_MAXL1] = {};  // q_0..q_{L-1}, p
+    bool aux = false;          // key switches take the products modulo p through auxiliary primes
+    AuxCrt crt = {};
     LimbTable lt = {};
     LimbConst* lt_dev = nullptr;  // device copy of lt.c (the transform kernels read it from memory)
     // word raised by a kernel that gave up a bounded wait: mapped page-locked host memory (kflag is its device address), read
@@ -60,7 +73,8 @@ struct hann_ctx {
     unsigned* galois_dev = nullptr;  // [n] 5^r mod 2N
     std::vector<unsigned> h_galois;
     // evaluation keys by rotation: device buffers [L][2][L+1][N], transformed and permuted by the inverse
-    // automorphism so that the key-switch inner product reads keys and digits contiguously
+    // automorphism so that the key-switch inner product reads keys and digits contiguously; with auxiliary primes followed by
+    // [L][2][3][N], the residues modulo p lifted (centred) to those primes
     std::vector<u64*> keytab_host;
     u64** keytab_dev = nullptr;  // [n] device copy of keytab_host
     // growable device scratch of the exchange and client calls (never used by the server-side scoring calls)
@@ -193,6 +207,7 @@ int launch_ntt_inv_pass_b_from(hann_ctx* c, const u64* src, int64_t src_gstride,
 bool ks_lift_available(const hann_ctx* c);
 int launch_wait_selftest(hann_ctx* c, unsigned long long limit_ns, unsigned long long* waited_ns_dev);
 int launch_ks_lift(hann_ctx* c, u64* src, int64_t src_stride, int64_t nsrc, const LimbMap& src_lm, u64* dst, int n_tgt, int tgt_limb0, bool skip_own = false);
+int launch_ks_lift_aux(hann_ctx* c, const u64* src, int64_t src_stride, int64_t nsrc, u64* dst);
 // encode a block and run pass A of the transforms in one kernel when the parameters allow it (returns false if not)
 bool encode_fused_available(const hann_ctx* c);
 int encode_configure();  // once per context, its device current
@@ -227,7 +242,7 @@ int launch_moddown_lift(hann_ctx* c, const u64* u, int64_t npoly, u64* lifted);
 bool ks_fused_available(const hann_ctx* c);
 int ks_fused_configure();  // once per context, its device current
 int launch_ks_apply(hann_ctx* c, const u64* digits, const u64* own, int64_t own_it, int64_t own_z, int64_t items, int nz, int rot0, int rot_zinc, u64* u);
-int launch_ks_finish(hann_ctx* c, const u64* u, const u64* lifted, int64_t items, bool perm_items, int rot0, int rot_inc, int nz, const u64* c0,
+int launch_ks_finish(hann_ctx* c, const u64* u, int u_limbs, const u64* lifted, int64_t items, bool perm_items, int rot0, int rot_inc, int nz, const u64* c0,
                      int64_t c0_it, int64_t c0_z, const u64* add, int64_t add_it, u64* out0, u64* out1, int64_t out_it);
 int launch_rescale_finish(hann_ctx* c, const u64* src, const u64* lifted, int64_t npoly, int keep, u64* out);
 // lazy giant steps (items laid out giant step after giant step, see keyswitch.cu)
@@ -239,6 +254,7 @@ int launch_moddown_combine(hann_ctx* c, const u64* u, const u64* lifted, int64_t
                            int64_t c0_stride, const u64* addend, int64_t addend_stride, u64* out0, u64* out1,
                            int64_t out_stride);
 int launch_permute(hann_ctx* c, const u64* src, u64* dst, int64_t npoly, unsigned k);
+int launch_key_aux(hann_ctx* c, const u64* key, u64* out);
 // output compaction: centred lift of coefficient-domain residues mod q_{L-1} into limbs 0..keep-1; (src - lifted) / q_{L-1}
 int launch_rescale_lift(hann_ctx* c, const u64* t, int64_t npoly, int keep, u64* lifted);
 int launch_rescale_combine(hann_ctx* c, const u64* src, const u64* lifted, int64_t npoly, int keep, u64* out);

@@ -352,6 +352,25 @@ __global__ void __launch_bounds__(kThreads) k_giant_sum_p(const u64* __restrict_
     }
 }
 
+// out[j][comp][k][x] = centred lift of key[j][comp][limb L][x] (residue mod p, coefficient domain) mod auxiliary prime k
+__global__ void __launch_bounds__(kThreads) k_key_aux(const u64* __restrict__ key, u64* __restrict__ out, int N, int L, AuxCrt X, LimbTable lt) {
+    const long long total = 2LL * L * N;
+    const u64 p = lt.c[L].q, half = lt.c[L].half;
+    for (long long idx = (long long)blockIdx.x * kThreads + threadIdx.x; idx < total; idx += (long long)gridDim.x * kThreads) {
+        const long long poly = idx / N;
+        const int x = (int)(idx % N);
+        const u64 v = key[(poly * (L + 1) + L) * N + x];
+        const bool neg = v > half;
+        const u64 mag = neg ? p - v : v;
+#pragma unroll
+        for (int k = 0; k < kAux; k++) {
+            const LimbConst& lc = lt.c[(int)X.limb[k]];
+            const u64 r = barrett64(mag, lc);
+            out[(poly * kAux + k) * N + x] = (neg && r) ? lc.q - r : r;
+        }
+    }
+}
+
 // lifted[poly][i][x] = centred lift of up[poly][x] (residue mod p, coefficient domain, polynomials N words apart) mod q_i
 __global__ void __launch_bounds__(kThreads) k_lift_p(const u64* __restrict__ up, u64* __restrict__ lifted, int N, int L, long long npoly,
                                                      LimbTable lt) {
@@ -743,6 +762,14 @@ int launch_giant_sum_p(hann_ctx* c, const u64* u, int64_t nblk, u64* up) {
                                                                            c->ntt_tau, c->lt);
     }
     return check_launch(c, "giant_sum_p");
+}
+
+int launch_key_aux(hann_ctx* c, const u64* key, u64* out) {
+    {
+        KProf kp(c, KC_MODDOWN_LIFT);
+        k_key_aux<<<grid_for((int64_t)2 * c->L * c->N), kThreads, 0, c->stream>>>(key, out, c->N, c->L, c->crt, c->lt);
+    }
+    return check_launch(c, "key_aux");
 }
 
 int launch_lift_p(hann_ctx* c, const u64* up, int64_t npoly, u64* lifted) {

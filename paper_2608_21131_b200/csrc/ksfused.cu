@@ -43,11 +43,11 @@ __device__ __forceinline__ void stage_twiddles(TW* __restrict__ tc, const TW* __
     }
 }
 
-// 16-byte asynchronous copies of the 2 L key chunks (256 words each, L1N words apart) of a modulus into shared memory
-__device__ __forceinline__ void stage_keys(u64* __restrict__ ks, const u64* __restrict__ key, long long L1N, int L) {
+// 16-byte asynchronous copies of the 2 L key chunks (256 words each, KN words apart) of a modulus into shared memory
+__device__ __forceinline__ void stage_keys(u64* __restrict__ ks, const u64* __restrict__ key, long long KN, int L) {
     const unsigned dst = (unsigned)__cvta_generic_to_shared(ks);
     for (int v = threadIdx.x; v < 2 * L * 128; v += blockDim.x) {
-        const u64* src = key + (long long)(v >> 7) * L1N + (v & 127) * 2;
+        const u64* src = key + (long long)(v >> 7) * KN + (v & 127) * 2;
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + v * 16), "l"(src) : "memory");
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
@@ -78,22 +78,26 @@ __device__ __forceinline__ void chunk_forward_int(const AR& ar, const ulonglong2
 
 struct ApplyArgs {
     const u64* digits;  // pass-A output of digit (z, item, j) for modulus i: ((z * items + item) * L + j) * n_tgt + target of i
-    int n_tgt;          // L + 1 targets per digit, or L: a digit's own modulus is left out and read from `own`
+    int n_tgt;          // targets per digit: L + 1; or one less, a digit's own modulus being left out and read from `own`; with
+                        // auxiliary primes none for the special prime either
+    int nx;             // 1, or the number of auxiliary primes that stand for the special prime
+    u64 aux4;           // their limbs in 4-bit fields, behind them the other limbs
+    long long aux_key;  // and the offset of their words in a key
     const u64* own;     // the polynomials being switched, transform domain: own + item * own_it + z * own_z + j * N (or null)
     long long own_it, own_z;
     const u64* const* keytab;
     const unsigned* galois;
     int rot0, rot_zinc, nz;  // rotation of z
     long long items;
-    u64* u;  // [item][2][L+1][N]: limbs below L canonical (below 2^50: balanced binary64 integers), the special prime's after its
-             // inverse pass B' (private format)
+    u64* u;  // [item][2][L+nx][N]: limbs below L canonical (below 2^50: balanced binary64 integers), the special prime's (or the
+             // auxiliary primes') after inverse pass B' (private format)
     int N, logN, L;
     const void *tw_fwd_f64, *tw_fwd_int, *tw_inv_f64, *tw_inv_int;
     const LimbConst* lt;
 };
 
-// u[item][c][i] = sum over z of phi_z( sum_j digit(z, item, j) * key_z[j][c] )  modulo i, for chunk blockIdx.x of the result, modulus
-// i = L - blockIdx.y (the special prime, which has the longest chain, first) and IB items.  A half-warp transforms one digit's
+// u[item][c][i] = sum over z of phi_z( sum_j digit(z, item, j) * key_z[j][c] )  modulo i, for chunk blockIdx.x of the result, a modulus
+// per blockIdx.y (the special prime or the auxiliary ones, which have the longest chain, first) and IB items.  A half-warp transforms one digit's
 // chunk; then every thread multiplies positions of all items with key words it loads once.
 //
 // Bound: issue slots and FP64 pipe together (ncu, two items x three z at N = 2^16, L = 4: FP64 27 %, issue 51 %, 96 registers and 20
@@ -102,15 +106,25 @@ struct ApplyArgs {
 // memory they sat in the chain.  The sums are reduced on the FP64 pipe: the 128-bit integer reduction was as long as the products.
 // Against pass B, key product and permuted sum as kernels of their own (seven blocks, three giant steps, N = 2^16, L = 4):
 // 513 -> 390 us with the finish kernel below, and four of twenty digit transforms less in the lift.
-template <int IB, int T>
+//
+// SHARE (with auxiliary primes): the CTA of an auxiliary prime takes the products with the key modulo that prime as well, instead of a
+// CTA of their own that transforms the same digits again; both key sets and sums then wait in shared memory.  At four items per CTA that
+// is 100 KiB, two CTAs per SM as without: 31 blocks of three rotations 1163 -> 840 us.  At one and two items it leaves three
+// CTAs in place of five and lost (95 -> 108 us for two).
+template <int IB, int T, bool SHARE>
 __global__ void __launch_bounds__(T, 640 / T) k_ks_apply(ApplyArgs A) {
     extern __shared__ __align__(16) u64 sm[];
-    const int L = A.L, N = A.N, t = blockIdx.x, i = L - (int)blockIdx.y;
-    const long long L1N = (long long)(L + 1) * N;
+    const int L = A.L, N = A.N, t = blockIdx.x, y = blockIdx.y;
+    const bool last = y < A.nx, aux = last && A.nx > 1;
+    const int i = SHARE || aux ? (int)(A.aux4 >> (4 * y)) & 15 : last ? L : y - A.nx;
+    const int sets = aux ? 2 : 1;  // SHARE: key sets, 0 the modulus' own, 1 the auxiliary one
+    const long long UN = (long long)(L + A.nx) * N;
     double2* tc = (double2*)sm;                  // [256]
-    u64* ks = sm + 512;                          // [L][2][256] key words
+    u64* ks = sm + 512;                          // [L][2][256] key words of a set, those of the second behind the sums
     u64* buf = ks + (size_t)L * 512;             // [IB * L][256] digits
-    u64* acc = buf + (size_t)IB * L * 256;       // [IB][2][256] sums
+    u64* acc = buf + (size_t)IB * L * 256;       // [IB][2][256] sums of a set
+    // words from the first set's buffers to the second's
+    const int ks2 = SHARE ? L * 512 + IB * (L * 256 + 512) : 0, acc2 = SHARE ? IB * 512 + L * 512 : 0;
     const long long it0 = (long long)blockIdx.z * IB;
     const int nit = A.items - it0 < IB ? (int)(A.items - it0) : IB;
     const int hw = threadIdx.x >> 4, j = threadIdx.x & 15;
@@ -129,10 +143,12 @@ __global__ void __launch_bounds__(T, 640 / T) k_ks_apply(ApplyArgs A) {
         const unsigned k = A.galois[A.rot0 + z * A.rot_zinc];
         const int sc = k == 1u ? t : galois_src(t << 8, k, A.logN, 1) >> 8;
         const u64* p = own ? A.own + (it0 + it) * A.own_it + z * A.own_z + (long long)i * N
-                           : A.digits + (((z * A.items + it0 + it) * L + dj) * A.n_tgt + (A.n_tgt > L || i < dj ? i : i - 1)) * N;
+                           : A.digits + (((z * A.items + it0 + it) * L + dj) * A.n_tgt + (!A.own || i < dj ? i : i - 1)) * N;
         p += (sc << 8);
         if (z) __syncthreads();  // the products of the previous rotation have been taken
-        stage_keys(ks, A.keytab[A.rot0 + z * A.rot_zinc] + (long long)i * N + (sc << 8), L1N, L);
+        const u64* key = A.keytab[A.rot0 + z * A.rot_zinc] + (sc << 8);
+        if (SHARE || !aux) stage_keys(ks, key + (long long)i * N, (long long)(L + 1) * N, L);
+        if (aux) stage_keys(ks + ks2, key + A.aux_key + (long long)y * N, (long long)kAux * N, L);
         if (staged != sc) {
             if (f64) stage_twiddles(tc, (const double2*)A.tw_fwd_f64 + ((size_t)i << A.logN), m0 + sc);
             else stage_twiddles((ulonglong2*)tc, (const ulonglong2*)A.tw_fwd_int + ((size_t)i << A.logN), m0 + sc);
@@ -170,10 +186,10 @@ __global__ void __launch_bounds__(T, 640 / T) k_ks_apply(ApplyArgs A) {
                 if (!HANN_CHECK_INDEX((src >> 8) - sc, 1)) continue;
                 s = src & 255;
             }
-            const u64* kp = ks + s;
             const u64* xp = buf + swz(s);
-            u64* ac = acc + swz(m);
-            if (f64) {
+            if (f64) for (int st = 0; st < (SHARE ? sets : 1); st++) {
+                const u64* kp = ks + (SHARE && st ? ks2 : 0) + s;
+                u64* ac = acc + (SHARE && st ? acc2 : 0) + swz(m);
                 // exact sums of at most eight products in two binary64 words (acc2_fma), reduced on the FP64 pipe; chains of more
                 // than eight primes run one item per CTA and add up several such sums
                 double r[IB][2];
@@ -209,6 +225,8 @@ __global__ void __launch_bounds__(T, 640 / T) k_ks_apply(ApplyArgs A) {
                     ac[b * 512 + 256] = (u64)__double_as_longlong(r[b][1]);
                 }
             } else {
+                const u64* kp = ks + s;
+                u64* ac = acc + swz(m);
                 u64 hi[IB][2], lo[IB][2];
 #pragma unroll
                 for (int b = 0; b < IB; b++) hi[b][0] = hi[b][1] = lo[b][0] = lo[b][1] = 0;
@@ -233,17 +251,17 @@ __global__ void __launch_bounds__(T, 640 / T) k_ks_apply(ApplyArgs A) {
             }
         }
     }
-    u64* out = A.u + it0 * 2 * L1N + (long long)i * N + (t << 8);
-    if (i < L) {  // every thread stores the sums it made
+    u64* out = A.u + it0 * 2 * UN + (t << 8);
+    if (!last || (SHARE && aux)) {  // every thread stores the sums it made
         for (int m = threadIdx.x; m < 256; m += blockDim.x)
-            for (int v = 0; v < 2 * nit; v++) out[v * L1N + m] = acc[v * 256 + swz(m)];
-        return;
+            for (int v = 0; v < 2 * nit; v++) out[v * UN + (long long)i * N + m] = acc[v * 256 + swz(m)];
     }
-    // the special prime's sums go straight into the inverse pass B' of their chunk
+    if (!last) return;
+    // those modulo the special prime or with the auxiliary key set go straight into the inverse pass B' of their chunk
     __syncthreads();
     for (int v = hw; v < 2 * nit; v += blockDim.x >> 4) {
-        u64* sv = acc + v * 256;
-        u64* o = out + v * L1N;
+        u64* sv = acc + acc2 + v * 256;
+        u64* o = out + v * UN + (long long)(L + (aux ? y : 0)) * N;
         if (f64) {
             const double2* tw = (const double2*)A.tw_inv_f64 + ((size_t)i << A.logN);
             double x[16];
@@ -431,12 +449,15 @@ int run_finish(hann_ctx* c, FinishArgs& A, bool perm_items) {
 
 // sixteen lanes per digit, whole warps
 constexpr int apply_threads(int IB, int L) { return (IB * L * 16 + 31) / 32 * 32; }
-constexpr size_t apply_smem(int IB, int L) { return 4096 + (size_t)(2 * L + apply_threads(IB, L) / 16 + 2 * IB) * 2048; }
+constexpr size_t apply_smem(int IB, int L, bool share = false) {
+    return 4096 + (size_t)((share ? 2 : 1) * (2 * L + 2 * IB) + apply_threads(IB, L) / 16) * 2048;
+}
 
-template <int IB, int T>
+template <int IB, int T, bool SHARE = false>
 void launch_apply(hann_ctx* c, const ApplyArgs& A) {
     KProf kp(c, KC_KS_INNER);
-    launch_chain(c, k_ks_apply<IB, T>, dim3(c->N >> 8, A.L + 1, (unsigned)((A.items + IB - 1) / IB)), apply_threads(IB, A.L), apply_smem(IB, A.L), A);
+    launch_chain(c, k_ks_apply<IB, T, SHARE>, dim3(c->N >> 8, SHARE ? A.L : A.L + A.nx, (unsigned)((A.items + IB - 1) / IB)), apply_threads(IB, A.L),
+                 apply_smem(IB, A.L, SHARE), A);
 }
 
 }  // namespace
@@ -446,9 +467,10 @@ void launch_apply(hann_ctx* c, const ApplyArgs& A) {
 // different chain lengths do not take it from one another.
 int ks_fused_configure() {
     static_assert(apply_smem(2, 4) <= 48 * 1024 && apply_smem(1, 4) <= 48 * 1024, "the other instances need no opt-in");
-    if (cudaFuncSetAttribute(k_ks_apply<4, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apply_smem(4, 4)) != cudaSuccess) return HANN_ECUDA;
-    if (cudaFuncSetAttribute(k_ks_apply<2, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apply_smem(2, 8)) != cudaSuccess) return HANN_ECUDA;
-    if (cudaFuncSetAttribute(k_ks_apply<1, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apply_smem(1, HANN_MAX_PRIMES)) != cudaSuccess)
+    if (cudaFuncSetAttribute(k_ks_apply<4, 256, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apply_smem(4, 4)) != cudaSuccess) return HANN_ECUDA;
+    if (cudaFuncSetAttribute(k_ks_apply<4, 256, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apply_smem(4, 4, true)) != cudaSuccess) return HANN_ECUDA;
+    if (cudaFuncSetAttribute(k_ks_apply<2, 256, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apply_smem(2, 8)) != cudaSuccess) return HANN_ECUDA;
+    if (cudaFuncSetAttribute(k_ks_apply<1, 256, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apply_smem(1, HANN_MAX_PRIMES)) != cudaSuccess)
         return HANN_ECUDA;
     return HANN_OK;
 }
@@ -456,12 +478,19 @@ int ks_fused_configure() {
 bool ks_fused_available(const hann_ctx* c) { return c->logN >= 10 && c->ntt_tau; }
 
 // digits: output of launch_ks_lift for the nz * items polynomials of L limbs; own (optional): the polynomials themselves, in which
-// case the digits were lifted without their own modulus.  Leaves u[item][2][L+1][N] (see ApplyArgs), the input of the ModDown lift.
+// case the digits were lifted without their own modulus (and, where the context has auxiliary primes, without the special prime).
+// Leaves u[item][2][L + nx][N] (see ApplyArgs), the input of the ModDown lift.
 int launch_ks_apply(hann_ctx* c, const u64* digits, const u64* own, int64_t own_it, int64_t own_z, int64_t items, int nz, int rot0, int rot_zinc, u64* u) {
     if (items <= 0 || nz <= 0) return HANN_OK;
     ApplyArgs A = {};
     A.digits = digits;
-    A.n_tgt = own ? c->L : c->L + 1;
+    const bool aux = c->aux && own;
+    A.nx = aux ? kAux : 1;
+    for (int k = 0; k < kAux; k++) A.aux4 |= (u64)c->crt.limb[k] << (4 * k);
+    for (int l = 0, k = kAux; aux && l < c->L; l++)
+        if (l != c->crt.limb[0] && l != c->crt.limb[1] && l != c->crt.limb[2]) A.aux4 |= (u64)l << (4 * k++);
+    A.aux_key = (long long)c->L * 2 * (c->L + 1) * c->N;
+    A.n_tgt = aux ? c->L - 1 : own ? c->L : c->L + 1;
     A.own = own;
     A.own_it = own_it;
     A.own_z = own_z;
@@ -489,7 +518,8 @@ int launch_ks_apply(hann_ctx* c, const u64* digits, const u64* own, int64_t own_
     //   N = 2^12, L = 2, seven rotations: 1 item 78 / 68 / 62, 16: 86 / 88 / 83
     //   N = 2^15, L = 8, one rotation:    1 item 24 / 32, 2: 45 / 42, 3: 64 / 70, 4: 82 / 77, 16: 292 / 281
     // Four lose to two where they leave half of the last CTA empty (five and six items of four primes: 86 against 70 us).
-    if (items >= 4 && c->L <= 4) launch_apply<4, 256>(c, A);
+    if (items >= 4 && c->L <= 4 && aux) launch_apply<4, 256, true>(c, A);
+    else if (items >= 4 && c->L <= 4) launch_apply<4, 256>(c, A);
     else if (items >= 2 && c->L <= 4) launch_apply<2, 128>(c, A);
     else if (items >= 2 && c->L <= 8) launch_apply<2, 256>(c, A);
     else if (c->L <= 4) launch_apply<1, 64>(c, A);
@@ -497,15 +527,15 @@ int launch_ks_apply(hann_ctx* c, const u64* digits, const u64* own, int64_t own_
     return check_launch(c, "ks_apply");
 }
 
-// lifted: output of launch_ks_lift for the special-prime limbs of u.  perm_items: the automorphism is still to be applied, that of
+// lifted: output of launch_ks_lift (launch_ks_lift_aux) for the special-prime (auxiliary) limbs of u, whose polynomials have u_limbs limbs.  perm_items: the automorphism is still to be applied, that of
 // item `it` being rotation rot0 + it * rot_inc (otherwise rotation rot0 + z * rot_inc belongs to the c0 term z < nz).
-int launch_ks_finish(hann_ctx* c, const u64* u, const u64* lifted, int64_t items, bool perm_items, int rot0, int rot_inc, int nz, const u64* c0,
+int launch_ks_finish(hann_ctx* c, const u64* u, int u_limbs, const u64* lifted, int64_t items, bool perm_items, int rot0, int rot_inc, int nz, const u64* c0,
                      int64_t c0_it, int64_t c0_z, const u64* add, int64_t add_it, u64* out0, u64* out1, int64_t out_it) {
     if (items <= 0) return HANN_OK;
     FinishArgs A = {};
     A.lifted = lifted;
     A.u = u;
-    A.u_poly = (long long)(c->L + 1) * c->N;
+    A.u_poly = (long long)u_limbs * c->N;
     A.u_mid = perm_items ? 0 : 1;
     A.limbs = c->L;
     A.add = add;

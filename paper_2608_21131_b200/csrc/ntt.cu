@@ -609,7 +609,7 @@ __global__ void __launch_bounds__(kThreads, AR::kMinBlocks) k_ntt_inv_a(NttArgs 
 // blocks since the rotate-and-sum leaves out the digits modulo their own prime (skip_own).
 
 struct LiftArgs {
-    u64* src;             // source polynomials after inverse pass B' (private format of their modulus)
+    const u64* src;       // source polynomials after inverse pass B' (private format of their modulus)
     long long src_stride;
     int src_period;
     u64 src_limb4;        // limb of source polynomial sp = nibble (sp % src_period)
@@ -633,6 +633,12 @@ __device__ __forceinline__ int lift_word(int row, int c) {
     return (row << logC) + c + (R2 == 4 ? (row >> 4) << 3 : 0);
 }
 
+// the 128 threads that work on a tile: a CTA of its own (k_ks_lift) or one of the four groups of a larger one, with a barrier of their own
+struct LiftGroup {
+    int id, barrier;
+    __device__ __forceinline__ void sync() const { asm volatile("bar.sync %0, %1;" ::"r"(barrier), "n"(kLiftThreads) : "memory"); }
+};
+
 // the centred coefficients of a source polynomial: balanced binary64 integers (class 0) or signed integers (class 2)
 __device__ __forceinline__ u64 lift_centred(const ArithF64& ar, double x, const LimbConst*) {
     return (u64)__double_as_longlong(ar.reduce(ar.mulmod(ar.reduce(x), ar.ninv)));
@@ -644,12 +650,12 @@ __device__ __forceinline__ u64 lift_centred(const ArithInt<false>& ar, u64 x, co
 
 template <int R1, int R2, class AR>
 __device__ __forceinline__ void lift_inverse(const AR ar, const LimbConst* lc, const typename AR::TW* __restrict__ tw,
-                                             const u64* __restrict__ base, u64* __restrict__ sm, u64* __restrict__ vs, int g, int c) {
+                                             const u64* base, u64* sm, u64* vs, int step, int g, int c, const LiftGroup th) {
     constexpr int G1 = 1 << R2, G2 = 1 << R1, logC = 7 - R2, C = 1 << logC;
     constexpr int RR2 = R2 == 0 ? 1 : R2;
     if (R2 != 0) {
 #pragma unroll
-        for (int w = threadIdx.x; w < (G2 << logC); w += kLiftThreads) {
+        for (int w = th.id; w < (G2 << logC); w += kLiftThreads) {
             const int cc = w & (C - 1), gg = w >> logC;
             typename AR::T x[1 << RR2];
 #pragma unroll
@@ -658,20 +664,20 @@ __device__ __forceinline__ void lift_inverse(const AR ar, const LimbConst* lc, c
 #pragma unroll
             for (int e = 0; e < (1 << RR2); e++) sm[lift_word<R2>((gg << RR2) + e, cc)] = ar.to_mid(x[e]);
         }
-        __syncthreads();
+        th.sync();
     }
     typename AR::T x[1 << R1];
 #pragma unroll
     for (int e = 0; e < (1 << R1); e++) x[e] = ar.from_mid(R2 == 0 ? base[(size_t)(g + G1 * e) * 256 + c] : sm[lift_word<R2>(g + G1 * e, c)]);
     inv_round<R1>(ar, x, tw, 1u);
 #pragma unroll
-    for (int e = 0; e < (1 << R1); e++) vs[e * kLiftThreads] = lift_centred(ar, x[e], lc);
+    for (int e = 0; e < (1 << R1); e++) vs[e * step] = lift_centred(ar, x[e], lc);
 }
 
 // the same for the integer class, its rounds of four stages in place in the exchange tile (see fwd_round4_smem)
 template <int R1, int R2>
 __device__ __forceinline__ void lift_inverse_int(const ArithInt<false> ar, const LimbConst* lc, const ulonglong2* __restrict__ tw,
-                                                 const u64* __restrict__ base, u64* __restrict__ sm, u64* __restrict__ vs, int g, int c) {
+                                                 const u64* __restrict__ base, u64* __restrict__ sm, u64* __restrict__ vs, int g, int c, const LiftGroup th) {
     if constexpr (R1 == 4) {
         constexpr int G1 = 1 << R2, logC = 7 - R2, C = 1 << logC;
         if constexpr (R2 == 4) {
@@ -681,7 +687,7 @@ __device__ __forceinline__ void lift_inverse_int(const ArithInt<false> ar, const
             inv_round4_smem(ar, word, tw, (unsigned)(16 + g));
         } else if constexpr (R2 > 0) {
 #pragma unroll 1
-            for (int w = threadIdx.x; w < (16 << logC); w += kLiftThreads) {
+            for (int w = th.id; w < (16 << logC); w += kLiftThreads) {
                 const int cc = w & (C - 1), gg = w >> logC;
                 u64 x[1 << R2];
 #pragma unroll
@@ -694,13 +700,13 @@ __device__ __forceinline__ void lift_inverse_int(const ArithInt<false> ar, const
 #pragma unroll 4
             for (int e = 0; e < 16; e++) sm[lift_word<R2>(e, c)] = base[(size_t)e * 256 + c];
         }
-        if (R2 != 0) __syncthreads();
+        if (R2 != 0) th.sync();
         const auto word = [=](int e) { return sm + lift_word<R2>(g + G1 * e, c); };
         inv_round4_smem(ar, word, tw, 1u);
 #pragma unroll 2
         for (int e = 0; e < 16; e++) vs[e * kLiftThreads] = lift_centred(ar, *word(e), lc);
     } else {
-        lift_inverse<R1, R2>(ar, lc, tw, base, sm, vs, g, c);
+        lift_inverse<R1, R2>(ar, lc, tw, base, sm, vs, kLiftThreads, g, c, th);
     }
 }
 
@@ -733,7 +739,7 @@ struct Lifted {
 
 template <int R1, int R2, class AR, class LIFT>
 __device__ __forceinline__ void lift_forward(const AR ar, const LimbConst* lc, const LIFT lift, const typename AR::TW* __restrict__ tw,
-                                             u64* __restrict__ base, u64* __restrict__ sm, const u64* __restrict__ vs, int g, int c) {
+                                             u64* __restrict__ base, u64* __restrict__ sm, const u64* __restrict__ vs, int g, int c, const LiftGroup th) {
     constexpr int G1 = 1 << R2, G2 = 1 << R1, logC = 7 - R2, C = 1 << logC;
     constexpr int RR2 = R2 == 0 ? 1 : R2;
     {
@@ -748,9 +754,9 @@ __device__ __forceinline__ void lift_forward(const AR ar, const LimbConst* lc, c
         }
     }
     if (R2 != 0) {
-        __syncthreads();
+        th.sync();
 #pragma unroll
-        for (int w = threadIdx.x; w < (G2 << logC); w += kLiftThreads) {
+        for (int w = th.id; w < (G2 << logC); w += kLiftThreads) {
             const int cc = w & (C - 1), gg = w >> logC;
             typename AR::T x[1 << RR2];
 #pragma unroll
@@ -759,21 +765,21 @@ __device__ __forceinline__ void lift_forward(const AR ar, const LimbConst* lc, c
 #pragma unroll
             for (int e = 0; e < (1 << RR2); e++) base[(size_t)((gg << RR2) + e) * 256 + cc] = ar.to_mid(x[e]);
         }
-        __syncthreads();  // the exchange tile is free for the next target
+        th.sync();  // the exchange tile is free for the next target
     }
 }
 
 // integer targets, their rounds of four stages in place in the exchange tile
 template <int R1, int R2, class AR, class LIFT>
 __device__ __forceinline__ void lift_forward_int(const AR ar, const LimbConst* lc, const LIFT lift, const ulonglong2* __restrict__ tw,
-                                                 u64* __restrict__ base, u64* __restrict__ sm, const u64* __restrict__ vs, int g, int c) {
+                                                 u64* __restrict__ base, u64* __restrict__ sm, const u64* __restrict__ vs, int g, int c, const LiftGroup th) {
     if constexpr (R1 == 4) {
         constexpr int G1 = 1 << R2, logC = 7 - R2, C = 1 << logC;
         const auto first = [=](int e) { return sm + lift_word<R2>(g + G1 * e, c); };
 #pragma unroll 2
         for (int e = 0; e < 16; e++) *first(e) = lift(ar, vs[e * kLiftThreads], lc);
         fwd_round4_smem(ar, first, tw, 1u);
-        if (R2 != 0) __syncthreads();
+        if (R2 != 0) th.sync();
         if constexpr (R2 == 4) {
             const auto second = [=](int e) { return sm + lift_word<R2>((g << 4) + e, c); };
             fwd_round4_smem(ar, second, tw, (unsigned)(16 + g));
@@ -781,7 +787,7 @@ __device__ __forceinline__ void lift_forward_int(const AR ar, const LimbConst* l
             for (int e = 0; e < 16; e++) base[(size_t)((g << 4) + e) * 256 + c] = *second(e);
         } else if constexpr (R2 > 0) {
 #pragma unroll 1
-            for (int w = threadIdx.x; w < (16 << logC); w += kLiftThreads) {
+            for (int w = th.id; w < (16 << logC); w += kLiftThreads) {
                 const int cc = w & (C - 1), gg = w >> logC;
                 u64 x[1 << R2];
 #pragma unroll
@@ -794,19 +800,18 @@ __device__ __forceinline__ void lift_forward_int(const AR ar, const LimbConst* l
 #pragma unroll 4
             for (int e = 0; e < 16; e++) base[(size_t)e * 256 + c] = *first(e);
         }
-        if (R2 != 0) __syncthreads();  // the exchange tile is free for the next target
+        if (R2 != 0) th.sync();  // the exchange tile is free for the next target
     } else {
-        lift_forward<R1, R2>(ar, lc, lift, tw, base, sm, vs, g, c);
+        lift_forward<R1, R2>(ar, lc, lift, tw, base, sm, vs, g, c, th);
     }
 }
 
 template <int R1, int R2, int SRC>
-__device__ __forceinline__ void lift_targets(const LiftArgs& A, int sl, long long sp, int c0, u64* sm, const u64* vs, int g, int c) {
+__device__ __forceinline__ void lift_targets(const LiftArgs& A, int sl, long long sp, int c0, u64* sm, const u64* vs, int g, int c, const LiftGroup th,
+                                             int first, int step) {
     const int N = 1 << A.logN;
     const u64 src_q = A.lt[sl].q;
-    // a launch too small to fill the machine is cut along the targets as well: gridDim.z CTAs repeat the inverse rounds and
-    // share out the targets, which shortens the chain one CTA runs
-    for (int ti = blockIdx.z; ti < A.n_tgt; ti += gridDim.z) {
+    for (int ti = first; ti < A.n_tgt; ti += step) {
         const int tl = A.tgt_limb0 + ti + (A.skip_own && ti >= sl ? 1 : 0);
         const LimbConst* tlc = A.lt + tl;
         const u64 q = tlc->q;
@@ -816,13 +821,13 @@ __device__ __forceinline__ void lift_targets(const LiftArgs& A, int sl, long lon
         lift.fold = src_q > q + (q >> 5);
         if (q < (1ULL << 50)) {
             const ArithF64 ar(tlc);
-            lift_forward<R1, R2>(ar, tlc, lift, (const double2*)A.tw_fwd_f64 + ((size_t)tl << A.logN), dbase, sm, vs, g, c);
+            lift_forward<R1, R2>(ar, tlc, lift, (const double2*)A.tw_fwd_f64 + ((size_t)tl << A.logN), dbase, sm, vs, g, c, th);
         } else if (q < (1ULL << 57)) {
             const ArithInt<true> ar(tlc);
-            lift_forward_int<R1, R2>(ar, tlc, lift, (const ulonglong2*)A.tw_fwd_int + ((size_t)tl << A.logN), dbase, sm, vs, g, c);
+            lift_forward_int<R1, R2>(ar, tlc, lift, (const ulonglong2*)A.tw_fwd_int + ((size_t)tl << A.logN), dbase, sm, vs, g, c, th);
         } else {
             const ArithInt<false> ar(tlc);
-            lift_forward_int<R1, R2>(ar, tlc, lift, (const ulonglong2*)A.tw_fwd_int + ((size_t)tl << A.logN), dbase, sm, vs, g, c);
+            lift_forward_int<R1, R2>(ar, tlc, lift, (const ulonglong2*)A.tw_fwd_int + ((size_t)tl << A.logN), dbase, sm, vs, g, c, th);
         }
     }
 }
@@ -837,19 +842,90 @@ __global__ void __launch_bounds__(kLiftThreads, HANN_LIFT_MINBLOCKS) k_ks_lift(L
     const int sl = (int)((A.src_limb4 >> (4 * (sp % A.src_period))) & 15);
     const LimbConst* slc = A.lt + sl;
     const u64* sbase = A.src + sp * A.src_stride + c0;
+    const LiftGroup th{(int)threadIdx.x, 1};
     chain_wait();
     u64* vs = sm + threadIdx.x;                        // [2^R1][128]: the thread's centred coefficients
     u64* tile = sm + (kLiftThreads << R1);             // exchange tile
+    // a launch too small to fill the machine is cut along the targets as well: gridDim.z CTAs repeat the inverse rounds and
+    // share out the targets, which shortens the chain one CTA runs
     if (slc->q < (1ULL << 50)) {
         const ArithF64 ar(slc);
-        lift_inverse<R1, R2>(ar, slc, (const double2*)A.tw_inv_f64 + ((size_t)sl << A.logN), sbase, tile, vs, g, c);
+        lift_inverse<R1, R2>(ar, slc, (const double2*)A.tw_inv_f64 + ((size_t)sl << A.logN), sbase, tile, vs, kLiftThreads, g, c, th);
         if (R2 != 0) __syncthreads();  // every thread is done with the exchange tile of the inverse rounds
-        lift_targets<R1, R2, 0>(A, sl, sp, c0, tile, vs, g, c);
+        lift_targets<R1, R2, 0>(A, sl, sp, c0, tile, vs, g, c, th, blockIdx.z, gridDim.z);
     } else {
         const ArithInt<false> ar(slc);
-        lift_inverse_int<R1, R2>(ar, slc, (const ulonglong2*)A.tw_inv_int + ((size_t)sl << A.logN), sbase, tile, vs, g, c);
+        lift_inverse_int<R1, R2>(ar, slc, (const ulonglong2*)A.tw_inv_int + ((size_t)sl << A.logN), sbase, tile, vs, g, c, th);
         if (R2 != 0) __syncthreads();
-        lift_targets<R1, R2, 2>(A, sl, sp, c0, tile, vs, g, c);
+        lift_targets<R1, R2, 2>(A, sl, sp, c0, tile, vs, g, c, th, blockIdx.z, gridDim.z);
+    }
+}
+
+// ModDown of a product held modulo the three auxiliary primes (AuxCrt): the inverse tails of its three polynomials, every coefficient
+// put together and taken modulo the special prime p, then the lift into the ciphertext primes and their pass A as above.  With
+// balanced residues x_a, x_b, x_c the integer is x_a + q_a (v1 + q_b v2), v1 = (x_b - x_a) / q_a modulo q_b and
+// v2 = ((x_c - x_a) / q_a - v1) / q_b modulo q_c, balanced: it is below a quarter of q_a q_b q_c (choose_aux checks that), so a
+// digit that misses its balanced range by a rounding changes nothing.  The two products modulo p take v + 2^50, which is not negative.
+//
+// A CTA is four groups of 128 threads on a tile: three groups run the inverse tails side by side, all put the coefficients together, and
+// every group takes targets of its own, so that the chain of rounds is no longer than that of one inverse and one target.
+//
+// The integer transforms modulo the 60-bit special prime were half of the digit lift's instructions (240 of 498 a source word, 46 for a
+// target on the FP64 pipe).  Without them the digits of six items take 33 us in place of 49 (N = 2^16, L = 4); this launch takes as long as
+// the one inverse transform on the integer pipe (as one group with the three inverses in sequence: 32 against 12 us for four products).
+template <int R1, int R2>
+__global__ void __launch_bounds__(4 * kLiftThreads, 1) k_ks_lift_aux(LiftArgs A, const __grid_constant__ AuxCrt X, int L) {
+    extern __shared__ u64 sm[];
+    constexpr int logC = 7 - R2, C = 1 << logC, G1 = 1 << R2, step = (G1 << logC) + (R2 == 4 ? 8 : 0), tile_words = (kLiftThreads << R1) + (R2 == 4 ? 128 : 0);
+    const long long sp = blockIdx.y;
+    const int c0 = blockIdx.x << logC, k = threadIdx.x >> 7;
+    const LiftGroup th{(int)threadIdx.x & (kLiftThreads - 1), 1 + k};
+    const int c = th.id & (C - 1), g = th.id >> logC;
+    u64* vs = sm + th.id;                              // [2^R1][128]: the centred coefficients modulo p
+    u64* tiles = sm + (kLiftThreads << R1);            // an exchange tile per group
+    const u64* own = tiles + lift_word<R2>(g, c);      // the words of a thread's place in the last inverse round, `step` apart
+    const LimbConst* plc = A.lt + L;
+    const ArithF64 ab(A.lt + X.limb[1]), ac(A.lt + X.limb[2]);
+    chain_wait();
+    if (k < kAux) {
+        const int l = X.limb[k];
+        const ArithF64 ar(A.lt + l);
+        u64* tile = tiles + k * tile_words;
+        lift_inverse<R1, R2>(ar, nullptr, (const double2*)A.tw_inv_f64 + ((size_t)l << A.logN), A.src + sp * A.src_stride + ((size_t)k << A.logN) + c0, tile,
+                             tile + lift_word<R2>(g, c), step, g, c, th);
+    }
+    __syncthreads();
+    const u64 p = plc->q;
+#pragma unroll 2
+    for (int e = k; e < (1 << R1); e += 4) {
+        const double xa = __longlong_as_double((long long)own[e * step]), xb = __longlong_as_double((long long)own[tile_words + e * step]);
+        const double xc = __longlong_as_double((long long)own[2 * tile_words + e * step]);
+        const double v1 = ab.reduce(ab.mulmod_small(__dsub_rn(xb, xa), X.ab));
+        const double v2 = ac.reduce(ac.mulmod_small(__dsub_rn(ac.mulmod_small(__dsub_rn(xc, xa), X.ac), v1), X.bc));
+        const auto whole = [](double v) { return __double_as_longlong(__dadd_rn(v, ArithF64::kRound)) - 0x4338000000000000LL; };
+        // below 2p + 2p + 2p + 2^49
+        u64 r = shoup_mul((u64)(whole(v1) + (1LL << 50)), X.c1, X.c1s, p) + shoup_mul((u64)(whole(v2) + (1LL << 50)), X.c2, X.c2s, p) +
+                (X.off + (u64)whole(xa));
+        r = csub(r, 4 * p);
+        r = csub(r, 2 * p);
+        r = csub(r, p);
+        vs[e * kLiftThreads] = r > plc->half ? r - p : r;
+    }
+    __syncthreads();
+    lift_targets<R1, R2, 2>(A, L, sp, c0, tiles + k * tile_words, vs, g, c, th, blockIdx.z * 4 + k, gridDim.z * 4);
+}
+
+typedef void (*KernLiftAux)(LiftArgs, AuxCrt, int);
+KernLiftAux pick_lift_aux(int a) {
+    switch (a) {
+        case 1: return k_ks_lift_aux<1, 0>;
+        case 2: return k_ks_lift_aux<2, 0>;
+        case 3: return k_ks_lift_aux<3, 0>;
+        case 4: return k_ks_lift_aux<4, 0>;
+        case 5: return k_ks_lift_aux<4, 1>;
+        case 6: return k_ks_lift_aux<4, 2>;
+        case 7: return k_ks_lift_aux<4, 3>;
+        default: return k_ks_lift_aux<4, 4>;
     }
 }
 
@@ -1167,14 +1243,13 @@ int launch_ntt_inv(hann_ctx* c, u64* data, int64_t npoly, int64_t stride, const 
 
 bool ks_lift_available(const hann_ctx* c) { return c->logN >= 9; }
 
-// CTAs that share out the targets of a tile: smallest (waves x rounds of a CTA, the inverse rounds counting as one target),
+// CTAs that share out the targets of a tile: smallest (waves x rounds of a CTA, the inverse rounds counting as `inverse` targets),
 // ties to fewer CTAs
-static int lift_zsplit(long ctas, int n_tgt) {
-    const long slots = 148 * HANN_LIFT_MINBLOCKS;
+static int lift_zsplit(long ctas, int n_tgt, int inverse = 1, long slots = 148 * HANN_LIFT_MINBLOCKS) {
     int zs = 1;
     long best = -1;
     for (int z = 1; z <= n_tgt; z++) {
-        const long cost = ((ctas * z + slots - 1) / slots) * (1 + (n_tgt + z - 1) / z);
+        const long cost = ((ctas * z + slots - 1) / slots) * (inverse + (n_tgt + z - 1) / z);
         if (best < 0 || cost < best) {
             best = cost;
             zs = z;
@@ -1183,27 +1258,29 @@ static int lift_zsplit(long ctas, int n_tgt) {
     return zs;
 }
 
-// After inverse pass B' of the nsrc source polynomials (launch_ntt_inv_pass_b): finish their inverse transforms, lift the
-// coefficients (centred) into the n_tgt moduli tgt_limb0 .. and run pass A of the target transforms.  The caller finishes
-// with launch_ntt_fwd_pass_b over the targets.
-int launch_ks_lift(hann_ctx* c, u64* src, int64_t src_stride, int64_t nsrc, const LimbMap& src_lm, u64* dst, int n_tgt, int tgt_limb0, bool skip_own) {
-    if (nsrc <= 0) return HANN_OK;
-    LiftArgs A;
-    A.src = src;
+static LiftArgs lift_args(const hann_ctx* c, int64_t src_stride, int n_tgt) {
+    LiftArgs A = {};
     A.src_stride = src_stride;
-    A.src_period = src_lm.period;
-    A.src_limb4 = 0;
-    for (int i = 0; i < src_lm.period && i < 16; i++) A.src_limb4 |= (u64)src_lm.limb[i] << (4 * i);
-    A.dst = dst;
+    A.src_period = 1;
     A.n_tgt = n_tgt;
-    A.tgt_limb0 = tgt_limb0;
-    A.skip_own = skip_own ? 1 : 0;
     A.logN = c->logN;
     A.tw_inv_int = c->tw_inv;
     A.tw_inv_f64 = c->tw_inv_f64;
     A.tw_fwd_int = c->tw_fwd;
     A.tw_fwd_f64 = c->tw_fwd_f64;
     A.lt = c->lt_dev;
+    return A;
+}
+
+// After inverse pass B' of the nsrc source polynomials (launch_ntt_inv_pass_b): finish their inverse transforms, lift the
+// coefficients (centred) into the n_tgt moduli tgt_limb0 .. and run pass A of the target transforms.  The caller finishes
+// with launch_ntt_fwd_pass_b over the targets.
+int launch_ks_lift(hann_ctx* c, u64* src, int64_t src_stride, int64_t nsrc, const LimbMap& src_lm, u64* dst, int n_tgt, int tgt_limb0, bool skip_own) {
+    if (nsrc <= 0) return HANN_OK;
+    LiftArgs A = lift_args(c, src_stride, n_tgt);
+    A.src_period = src_lm.period;
+    A.tgt_limb0 = tgt_limb0;
+    A.skip_own = skip_own ? 1 : 0;
     const int a = c->logN - 8, R1 = a < 4 ? a : 4, R2 = a - R1, tiles = 256 >> (7 - R2);
     const size_t smem = (size_t)8 * (2 * (kLiftThreads << R1) + (R2 == 4 ? 128 : 0));
     for (int64_t s0 = 0; s0 < nsrc; s0 += 65535) {
@@ -1218,6 +1295,24 @@ int launch_ks_lift(hann_ctx* c, u64* src, int64_t src_stride, int64_t nsrc, cons
         launch_chain(c, pick_lift(a), dim3(tiles, ns, lift_zsplit((long)tiles * ns, n_tgt)), kLiftThreads, smem, Ap);
     }
     return check_launch(c, "ks_lift");
+}
+
+static constexpr size_t lift_aux_smem(int R1, int R2) { return (size_t)8 * (5 * (kLiftThreads << R1) + (R2 == 4 ? 4 * 128 : 0)); }
+
+// The same for nsrc products held modulo the auxiliary primes (kAux polynomials of N words each at src + i * src_stride), into the L
+// ciphertext primes.
+int launch_ks_lift_aux(hann_ctx* c, const u64* src, int64_t src_stride, int64_t nsrc, u64* dst) {
+    if (nsrc <= 0) return HANN_OK;
+    const int a = c->logN - 8, R1 = a < 4 ? a : 4, R2 = a - R1, tiles = 256 >> (7 - R2);
+    for (int64_t s0 = 0; s0 < nsrc; s0 += 65535) {
+        const int ns = (int)std::min<int64_t>(65535, nsrc - s0);
+        LiftArgs A = lift_args(c, src_stride, c->L);
+        A.src = src + s0 * src_stride;
+        A.dst = dst + s0 * c->L * (int64_t)c->N;
+        KProf kp(c, KC_LIFT_DIGITS);
+        launch_chain(c, pick_lift_aux(a), dim3(tiles, ns, lift_zsplit((long)tiles * ns, (c->L + 3) / 4, 2, 148)), 4 * kLiftThreads, lift_aux_smem(R1, R2), A, c->crt, c->L);
+    }
+    return check_launch(c, "ks_lift_aux");
 }
 
 int launch_ntt_inv_pass_b(hann_ctx* c, u64* data, int64_t npoly, int64_t stride, const LimbMap& lm) {
@@ -1248,7 +1343,9 @@ int launch_wait_selftest(hann_ctx* c, unsigned long long limit_ns, unsigned long
 
 int ntt_configure(hann_ctx* c) {
     // every configuration stays below the 48 KiB default of dynamic shared memory (pass A: 2^8 rows x 16 columns x 8 B
-    // = 32 KiB; pass B: 16 chunks x 272 words x 8 B = 34 KiB), so nothing to opt in to
+    // = 32 KiB; pass B: 16 chunks x 272 words x 8 B = 34 KiB), except k_ks_lift_aux
     (void)c;
+    for (int a = 4; a <= 8; a++)
+        if (cudaFuncSetAttribute(pick_lift_aux(a), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lift_aux_smem(4, a - 4)) != cudaSuccess) return HANN_ECUDA;
     return HANN_OK;
 }

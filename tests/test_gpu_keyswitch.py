@@ -70,6 +70,23 @@ def test_rotate_sum_on_edge_residues(logN, bits, pbits, nb):
     torch.cuda.synchronize()
 
 
+@pytest.mark.parametrize(
+    "logN,bits,pbits,nb",
+    [
+        (10, (50,) * 3, 60, 3),            # three primes: all auxiliary, the lifted polynomials in the place of the digits
+        (11, (58, 46, 45, 46), 60, 3),     # a prime of 2^50 and more between them, the digits of which are longer
+        (12, (50, 50, 50, 40), 60, 2),     # a ciphertext prime far below the auxiliary ones
+        (10, (50,) * 4, 61, 2),            # the largest special prime they stand for
+        (10, (50,) * 4, 51, 5),            # and the smallest
+        (10, (50, 50, 48), 60, 2),         # primes of too different size, and too few of them: the special prime itself
+        (10, (50, 50, 58), 60, 2),
+        (14, (50,) * 4, 60, 1),            # second lift round of two stages
+    ],
+)
+def test_rotate_sum_through_auxiliary_primes(logN, bits, pbits, nb):
+    test_rotate_sum_on_edge_residues(logN, bits, pbits, nb)
+
+
 def test_lazy_round_of_many_giant_steps():
     """15 blocks x 511 giant steps in one round: 7,665 polynomials of nine limbs, more than one launch covers (65535 / 9).  A large
     workspace only means larger rounds: the same bits as with rounds of one block"""
