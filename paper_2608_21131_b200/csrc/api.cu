@@ -261,12 +261,14 @@ int ks_digits_to_lifted(hann_ctx* c, u64* c1c, int64_t items, u64* digits, int64
 // src == c1c, one polynomial (nz = items = 1) only: the inverse pass overwrites it, so its digits are lifted to their own modulus as
 // well, the product modulo the special prime takes no auxiliary primes, and the digits take L * L1N words (carve_keyswitch).
 int ks_round_fused(hann_ctx* c, const u64* src, int64_t src_it, int64_t src_z, int64_t items, int nz, int rot0, int rot_zinc, u64* c1c, u64* digits,
-                   u64* u, u64* lifted) {
+                   u64* u, u64* lifted, bool inverted = false) {
     const int L = c->L, N = c->N;
     const int64_t LN = (int64_t)L * N, L1N = (int64_t)(L + 1) * N;
     const bool in_place = src == c1c;
     if (in_place && (nz != 1 || items != 1)) return fail(c, HANN_EINVAL, "a key-switch round in place takes one polynomial");
-    if (in_place) {
+    if (inverted) {
+        // c1c holds the polynomials after their inverse pass B' already (launch_ks_finish of the key switch before)
+    } else if (in_place) {
         RET(launch_ntt_inv_pass_b(c, c1c, L, N, limbmap_q(c)));
     } else if (ntt_inv_pass_b_gathers(c, src, c1c) && ((src_it | src_z) & 1) == 0) {
         RET(launch_ntt_inv_pass_b_from(c, src, src_it, c1c, nz * items * L, N, limbmap_q(c), nz > 1 ? items : 0, src_z));
@@ -1419,9 +1421,9 @@ extern "C" int hann_rotate_sum(hann_ctx* c, const void* inner_dev, int64_t n_blo
                 u64* out = (g % 2 == 0) ? score + b0 * ctw : tmp;
                 // c1 of every accumulator, still in the transform domain; the key-switch round takes it from there
                 if (fused) {
-                    RET(ks_round_fused(c, old + LN, old_stride, 0, nb, 1, B, 0, rb.c1c, rb.digits, rb.u, rb.lifted));
+                    RET(ks_round_fused(c, old + LN, old_stride, 0, nb, 1, B, 0, rb.c1c, rb.digits, rb.u, rb.lifted, g < G - 2));
                     RET(launch_ks_finish(c, rb.u, ks_u_limbs(c), rb.lifted, nb, false, B, 0, 1, old, old_stride, 0, inner + (b0 * G + g) * ctw, (int64_t)G * ctw, out,
-                                         out + LN, ctw));
+                                         out + LN, ctw, g > 0 ? rb.c1c : nullptr));
                     old = out;
                     old_stride = ctw;
                     continue;
@@ -1703,8 +1705,9 @@ extern "C" int hann_fold(hann_ctx* c, void* ct_dev, int stride, int steps, void*
         const int r = stride << t;
         // nxt = cur + rot_r(cur): the Horner step of the rotate-and-sum with the ciphertext itself as the addend
         if (ks_fused_available(c)) {
-            RET(ks_round_fused(c, cur + LN, ctw, 0, 1, 1, r, 0, rb.c1c, rb.digits, rb.u, rb.lifted));
-            RET(launch_ks_finish(c, rb.u, ks_u_limbs(c), rb.lifted, 1, false, r, 0, 1, cur, ctw, 0, cur, ctw, nxt, nxt + LN, ctw));
+            RET(ks_round_fused(c, cur + LN, ctw, 0, 1, 1, r, 0, rb.c1c, rb.digits, rb.u, rb.lifted, t > 0));
+            RET(launch_ks_finish(c, rb.u, ks_u_limbs(c), rb.lifted, 1, false, r, 0, 1, cur, ctw, 0, cur, ctw, nxt, nxt + LN, ctw,
+                                 t + 1 < steps ? rb.c1c : nullptr));
         } else {
             RET(ks_digits_to_lifted(c, rb.c1c, 1, rb.digits, (int64_t)L * L1N, r, 0, 1, rb.u, rb.lifted, cur + LN, ctw));
             RET(launch_moddown_combine(c, rb.u, rb.lifted, 1, r, 0, cur, ctw, cur, ctw, nxt, nxt + LN, ctw));

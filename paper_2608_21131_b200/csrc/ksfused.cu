@@ -76,6 +76,51 @@ __device__ __forceinline__ void chunk_forward_int(const AR& ar, const ulonglong2
     for (int e = 0; e < 16; e++) *second(e) = ar.to_canonical(*second(e));
 }
 
+// the inverse table's entries of a chunk (cbase = 2^a + chunk number) in the order of the two inverse rounds: entry 16 (r + 1) + j,
+// r = 16 - (16 >> st) + il, for stage st of the first, entries 0..14 (r) for the second
+template <class TW>
+__device__ __forceinline__ void stage_inverse_twiddles(TW* __restrict__ tc, const TW* __restrict__ tw, unsigned cbase) {
+#pragma unroll 4
+    for (int e = threadIdx.x; e < 256; e += blockDim.x) {
+        const int r = e < 16 ? e : (e >> 4) - 1, s = r < 8 ? 0 : r < 12 ? 1 : r < 14 ? 2 : 3, il = r - (16 - (16 >> s));
+        const unsigned idx = ((e < 16 ? cbase : (cbase << 4) + (e & 15)) << (3 - s)) + il;
+        if (r < 15) tc[e] = tw[idx];
+    }
+}
+
+// inverse pass B' of a chunk (cbase = 2^a + chunk number) by sixteen lanes, lane j holding its logical positions 16 j + e at the words
+// sv[16 j + (e ^ j)] (balanced binary64 integers, or residues in [0, 2q)); the chunk in the private format at o.  STAGED: tw is what
+// stage_inverse_twiddles left, otherwise the table of the modulus
+template <bool STAGED>
+__device__ __forceinline__ void chunk_inverse(const ArithF64& ar, const double2* __restrict__ tw, unsigned cbase, u64* sv, u64* o, int j, unsigned hmask) {
+    double x[16];
+#pragma unroll
+    for (int e = 0; e < 16; e++) x[e] = ar.from_mid(sv[16 * j + (e ^ j)]);
+    if (STAGED) inv_round_f<4>(ar, x, [=](int st, int il) { return tw[((16 - (16 >> st) + il + 1) << 4) + j]; });
+    else inv_round<4>(ar, x, tw, (cbase << 4) + j);
+#pragma unroll
+    for (int e = 0; e < 16; e++) sv[16 * j + (e ^ j)] = ar.to_mid(x[e]);
+    __syncwarp(hmask);
+#pragma unroll
+    for (int e = 0; e < 16; e++) x[e] = ar.from_mid(sv[16 * e + (j ^ e)]);
+    if (STAGED) inv_round_f<4>(ar, x, [=](int st, int il) { return tw[16 - (16 >> st) + il]; });
+    else inv_round<4>(ar, x, tw, cbase);
+#pragma unroll
+    for (int e = 0; e < 16; e++) o[j + 16 * e] = ar.to_mid(x[e]);
+}
+template <bool STAGED>
+__device__ __forceinline__ void chunk_inverse(const ArithInt<false>& ar, const ulonglong2* __restrict__ tw, unsigned cbase, u64* sv, u64* o, int j, unsigned hmask) {
+    const auto first = [=](int e) { return sv + 16 * j + (e ^ j); };
+    const auto second = [=](int e) { return sv + 16 * e + (j ^ e); };
+    if (STAGED) inv_round4_staged(ar, first, tw + 16, 16, j);
+    else inv_round4_smem(ar, first, tw, (cbase << 4) + j);
+    __syncwarp(hmask);
+    if (STAGED) inv_round4_staged(ar, second, tw, 1, 0);
+    else inv_round4_smem(ar, second, tw, cbase);
+#pragma unroll 8
+    for (int e = 0; e < 16; e++) o[j + 16 * e] = *second(e);
+}
+
 struct ApplyArgs {
     const u64* digits;  // pass-A output of digit (z, item, j) for modulus i: ((z * items + item) * L + j) * n_tgt + target of i
     int n_tgt;          // targets per digit: L + 1; or one less, a digit's own modulus being left out and read from `own`; with
@@ -119,8 +164,11 @@ __global__ void __launch_bounds__(T, 640 / T) k_ks_apply(ApplyArgs A) {
     const int i = SHARE || aux ? (int)(A.aux4 >> (4 * y)) & 15 : last ? L : y - A.nx;
     const int sets = aux ? 2 : 1;  // SHARE: key sets, 0 the modulus' own, 1 the auxiliary one
     const long long UN = (long long)(L + A.nx) * N;
-    double2* tc = (double2*)sm;                  // [256]
-    u64* ks = sm + 512;                          // [L][2][256] key words of a set, those of the second behind the sums
+    // (the inverse table is staged where enough threads share that: a launch of CTAs of 64 threads was 7 % slower with it, one of 256
+    // 10 % faster)
+    constexpr bool INV = T >= 256;
+    double2* tc = (double2*)sm;                  // [256] forward, INV: [256] inverse
+    u64* ks = sm + (INV ? 1024 : 512);           // [L][2][256] key words of a set, those of the second behind the sums
     u64* buf = ks + (size_t)L * 512;             // [IB * L][256] digits
     u64* acc = buf + (size_t)IB * L * 256;       // [IB][2][256] sums of a set
     // words from the first set's buffers to the second's
@@ -154,6 +202,10 @@ __global__ void __launch_bounds__(T, 640 / T) k_ks_apply(ApplyArgs A) {
             else stage_twiddles((ulonglong2*)tc, (const ulonglong2*)A.tw_fwd_int + ((size_t)i << A.logN), m0 + sc);
         }
         staged = sc;
+        if (INV && z == 0 && last) {
+            if (f64) stage_inverse_twiddles(tc + 256, (const double2*)A.tw_inv_f64 + ((size_t)i << A.logN), m0 + t);
+            else stage_inverse_twiddles((ulonglong2*)tc + 256, (const ulonglong2*)A.tw_inv_int + ((size_t)i << A.logN), m0 + t);
+        }
         if (z == 0) chain_wait();
         double x[16];  // binary64 or integer words alike
         if (valid) {
@@ -262,30 +314,10 @@ __global__ void __launch_bounds__(T, 640 / T) k_ks_apply(ApplyArgs A) {
     for (int v = hw; v < 2 * nit; v += blockDim.x >> 4) {
         u64* sv = acc + acc2 + v * 256;
         u64* o = out + v * UN + (long long)(L + (aux ? y : 0)) * N;
-        if (f64) {
-            const double2* tw = (const double2*)A.tw_inv_f64 + ((size_t)i << A.logN);
-            double x[16];
-#pragma unroll
-            for (int e = 0; e < 16; e++) x[e] = ar.from_mid(sv[16 * j + (e ^ j)]);
-            inv_round<4>(ar, x, tw, ((m0 + t) << 4) + j);
-#pragma unroll
-            for (int e = 0; e < 16; e++) sv[16 * j + (e ^ j)] = ar.to_mid(x[e]);
-            __syncwarp(hmask);
-#pragma unroll
-            for (int e = 0; e < 16; e++) x[e] = ar.from_mid(sv[16 * e + (j ^ e)]);
-            inv_round<4>(ar, x, tw, m0 + t);
-#pragma unroll
-            for (int e = 0; e < 16; e++) o[j + 16 * e] = ar.to_mid(x[e]);
-        } else {
-            const ArithInt<false> ar(lc);
-            const ulonglong2* tw = (const ulonglong2*)A.tw_inv_int + ((size_t)i << A.logN);
-            inv_round4_smem(ar, [=](int e) { return sv + 16 * j + (e ^ j); }, tw, ((m0 + t) << 4) + j);
-            __syncwarp(hmask);
-            const auto second = [=](int e) { return sv + 16 * e + (j ^ e); };
-            inv_round4_smem(ar, second, tw, m0 + t);
-#pragma unroll 8
-            for (int e = 0; e < 16; e++) o[j + 16 * e] = *second(e);
-        }
+        const double2* twf = INV ? tc + 256 : (const double2*)A.tw_inv_f64 + ((size_t)i << A.logN);
+        const ulonglong2* twi = INV ? (const ulonglong2*)tc + 256 : (const ulonglong2*)A.tw_inv_int + ((size_t)i << A.logN);
+        if (f64) chunk_inverse<INV>(ar, twf, m0 + t, sv, o, j, hmask);
+        else chunk_inverse<INV>(ArithInt<false>(lc), twi, m0 + t, sv, o, j, hmask);
     }
 }
 
@@ -302,10 +334,11 @@ struct FinishArgs {
     int rot0, rot_inc, nz;  // rotation of z; with PERM, of the item
     u64 *out0, *out1;
     long long out_it;
+    u64* next;          // NEXT: inverse pass B' of the second component, [item][limbs][N] (private format)
     const unsigned* galois;
     long long units;    // polynomials: two per item
     int N, logN, n;
-    const void *tw_fwd_f64, *tw_fwd_int;
+    const void *tw_fwd_f64, *tw_fwd_int, *tw_inv_f64, *tw_inv_int;
     const LimbConst* lt;
 };
 
@@ -313,10 +346,12 @@ struct FinishArgs {
 // pass B of the lifted ModDown polynomials with the combination behind its last round.
 // PERM: u, lifted and c0 are still in the order before the automorphism, which differs from item to item (hoisted rotations); the
 // finished words are permuted in shared memory and stored to the item's own chunk of the result.
+// NEXT: the result's second component is what the next key switch decomposes, and the half-warp that made a chunk of it runs the
+// chunk's inverse pass B' as well: a launch and two passes over the polynomial less for every step of a chain of key switches.
 //
 // 31 rotations at N = 2^16, L = 4: 170 us (pass B and the combination as two kernels) -> 103 us; the integer reductions of the
 // combination and a 16-fold unrolled tail (instruction fetch) cost most of that on the way.
-template <bool PERM>
+template <bool PERM, bool NEXT>
 __global__ void __launch_bounds__(256, 3) k_ks_finish(FinishArgs A) {
     extern __shared__ __align__(16) u64 sm[];
     const int N = A.N, t = blockIdx.x, i = blockIdx.y;
@@ -337,7 +372,9 @@ __global__ void __launch_bounds__(256, 3) k_ks_finish(FinishArgs A) {
     chain_wait();
     __syncthreads();
     const long long units = A.units, ustep = (long long)gridDim.z * (blockDim.x >> 4);
-    for (long long v = (long long)blockIdx.z * (blockDim.x >> 4) + hw; v < units; v += ustep) {
+    for (long long k = (long long)blockIdx.z * (blockDim.x >> 4) + hw; k < units; k += ustep) {
+        // (NEXT: second components after all first ones, so that the half-warps of a warp do the same)
+        const long long items = units >> 1, v = !NEXT ? k : k < items ? 2 * k : 2 * (k - items) + 1;
         const long long item = v >> 1;
         const int c = (int)(v & 1);
         const u64* p = A.lifted + (v * A.limbs + i) * N + (t << 8);
@@ -384,7 +421,12 @@ __global__ void __launch_bounds__(256, 3) k_ks_finish(FinishArgs A) {
                     // |u - reduce(x)| <= 1.5 q, the product lies below 0.7 q, the added words below 5 q
                     u64* w = sb + 16 * j + ((e0 + e) ^ j);
                     const double y = ar.mulmod_small(__dsub_rn(uw[e], __longlong_as_double((long long)*w)), pinv);
-                    const u64 r = ar.to_canonical(__dadd_rn(y, a[e]));
+                    double v = __dadd_rn(y, a[e]);
+                    if (NEXT) {
+                        v = ar.reduce(v);
+                        *w = (u64)__double_as_longlong(v);
+                    }
+                    const u64 r = ar.to_canonical(v);
                     if (PERM) *w = r;
                     else o[(t << 8) + 16 * (e0 + e) + j] = r;
                 }
@@ -408,9 +450,14 @@ __global__ void __launch_bounds__(256, 3) k_ks_finish(FinishArgs A) {
                         r = addmod(r, cp[z * A.c0_z + src], q);
                     }
                 }
-                if (PERM) *w = r;
-                else o[(t << 8) + 16 * e + j] = r;
+                if (PERM || NEXT) *w = r;
+                if (!PERM) o[(t << 8) + 16 * e + j] = r;
             }
+        }
+        if (NEXT && c == 1) {
+            u64* nx = A.next + item * LN + (long long)i * N + (t << 8);
+            if (f64) chunk_inverse<false>(ar, (const double2*)A.tw_inv_f64 + ((size_t)i << A.logN), m0 + t, sb, nx, j, hmask);
+            else chunk_inverse<false>(ArithInt<false>(lc), (const ulonglong2*)A.tw_inv_int + ((size_t)i << A.logN), m0 + t, sb, nx, j, hmask);
         }
         if (PERM) {
             const int r = A.rot0 + (int)item * A.rot_inc;
@@ -434,6 +481,8 @@ int run_finish(hann_ctx* c, FinishArgs& A, bool perm_items) {
     A.n = c->n;
     A.tw_fwd_f64 = c->tw_fwd_f64;
     A.tw_fwd_int = c->tw_fwd;
+    A.tw_inv_f64 = c->tw_inv_f64;
+    A.tw_inv_int = c->tw_inv;
     A.lt = c->lt_dev;
     // up to sixteen half-warps per CTA, which then walk further polynomials under the staged tables while the grid fills the
     // machine twice over
@@ -443,21 +492,21 @@ int run_finish(hann_ctx* c, FinishArgs& A, bool perm_items) {
     long long gz = (2 * 148 * 3 + per - 1) / per;
     if (gz > groups) gz = groups;
     KProf kp(c, KC_MODDOWN_COMBINE);
-    launch_chain(c, perm_items ? k_ks_finish<true> : k_ks_finish<false>, dim3(c->N >> 8, A.limbs, (unsigned)gz), threads, smem, A);
+    launch_chain(c, perm_items ? k_ks_finish<true, false> : A.next ? k_ks_finish<false, true> : k_ks_finish<false, false>, dim3(c->N >> 8, A.limbs, (unsigned)gz), threads, smem, A);
     return check_launch(c, "ks_finish");
 }
 
 // sixteen lanes per digit, whole warps
 constexpr int apply_threads(int IB, int L) { return (IB * L * 16 + 31) / 32 * 32; }
-constexpr size_t apply_smem(int IB, int L, bool share = false) {
-    return 4096 + (size_t)((share ? 2 : 1) * (2 * L + 2 * IB) + apply_threads(IB, L) / 16) * 2048;
+constexpr size_t apply_smem(int IB, int L, bool share = false, bool inv = true) {
+    return (inv ? 8192 : 4096) + (size_t)((share ? 2 : 1) * (2 * L + 2 * IB) + apply_threads(IB, L) / 16) * 2048;
 }
 
 template <int IB, int T, bool SHARE = false>
 void launch_apply(hann_ctx* c, const ApplyArgs& A) {
     KProf kp(c, KC_KS_INNER);
     launch_chain(c, k_ks_apply<IB, T, SHARE>, dim3(c->N >> 8, SHARE ? A.L : A.L + A.nx, (unsigned)((A.items + IB - 1) / IB)), apply_threads(IB, A.L),
-                 apply_smem(IB, A.L, SHARE), A);
+                 apply_smem(IB, A.L, SHARE, T >= 256), A);
 }
 
 }  // namespace
@@ -466,7 +515,7 @@ void launch_apply(hann_ctx* c, const ApplyArgs& A) {
 // each.  The limit belongs to the kernel and the device, not to a context: it is the same for every context, so that contexts of
 // different chain lengths do not take it from one another.
 int ks_fused_configure() {
-    static_assert(apply_smem(2, 4) <= 48 * 1024 && apply_smem(1, 4) <= 48 * 1024, "the other instances need no opt-in");
+    static_assert(apply_smem(2, 4, false, false) <= 48 * 1024 && apply_smem(1, 4, false, false) <= 48 * 1024, "the other instances need no opt-in");
     if (cudaFuncSetAttribute(k_ks_apply<4, 256, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apply_smem(4, 4)) != cudaSuccess) return HANN_ECUDA;
     if (cudaFuncSetAttribute(k_ks_apply<4, 256, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apply_smem(4, 4, true)) != cudaSuccess) return HANN_ECUDA;
     if (cudaFuncSetAttribute(k_ks_apply<2, 256, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apply_smem(2, 8)) != cudaSuccess) return HANN_ECUDA;
@@ -528,9 +577,10 @@ int launch_ks_apply(hann_ctx* c, const u64* digits, const u64* own, int64_t own_
 }
 
 // lifted: output of launch_ks_lift (launch_ks_lift_aux) for the special-prime (auxiliary) limbs of u, whose polynomials have u_limbs limbs.  perm_items: the automorphism is still to be applied, that of
-// item `it` being rotation rot0 + it * rot_inc (otherwise rotation rot0 + z * rot_inc belongs to the c0 term z < nz).
+// item `it` being rotation rot0 + it * rot_inc (otherwise rotation rot0 + z * rot_inc belongs to the c0 term z < nz).  next (optional, not
+// with perm_items): the second components after their inverse pass B', [item][L][N], for a key switch that follows.
 int launch_ks_finish(hann_ctx* c, const u64* u, int u_limbs, const u64* lifted, int64_t items, bool perm_items, int rot0, int rot_inc, int nz, const u64* c0,
-                     int64_t c0_it, int64_t c0_z, const u64* add, int64_t add_it, u64* out0, u64* out1, int64_t out_it) {
+                     int64_t c0_it, int64_t c0_z, const u64* add, int64_t add_it, u64* out0, u64* out1, int64_t out_it, u64* next) {
     if (items <= 0) return HANN_OK;
     FinishArgs A = {};
     A.lifted = lifted;
@@ -549,6 +599,7 @@ int launch_ks_finish(hann_ctx* c, const u64* u, int u_limbs, const u64* lifted, 
     A.out0 = out0;
     A.out1 = out1;
     A.out_it = out_it;
+    A.next = next;
     A.units = 2 * items;
     return run_finish(c, A, perm_items);
 }

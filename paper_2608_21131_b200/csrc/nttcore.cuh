@@ -200,84 +200,69 @@ __device__ __forceinline__ void inv_round_f(const AR& ar, typename AR::T (&x)[1 
 }
 
 // A round of FOUR stages of the integer classes on sixteen words that stay in shared memory, four at a time: two stages per
-// quad, eight quads in a rolled loop.  Unrolled like the binary64 rounds, an integer round is about a thousand instructions that
-// a warp runs through once, and a launch of few CTAs then spends most of its time fetching them (ncu: "no instruction" was ten
-// of thirteen stall cycles of a two-polynomial ModDown lift).  word(e): address of word e; tw: the table entries of the round,
-// base as in fwd_round / inv_round.
+// quad, eight quads in two rolled loops, the first (forward) or second (inverse) of which has one set of twiddles.  Unrolled like the
+// binary64 rounds, an integer round is about a thousand instructions that a warp runs through once, and a launch of few CTAs then
+// spends most of its time fetching them (ncu: "no instruction" was ten of thirteen stall cycles of a two-polynomial ModDown lift).
+// word(e): address of word e; tw(s, il): entry of group il of stage s of the round.
+template <class AR, class WORD>
+__device__ __forceinline__ void fwd_quad(const AR& ar, const WORD& word, int e0, int st, typename AR::TW w, typename AR::TW wa, typename AR::TW wb) {
+    u64 x0 = *word(e0), x1 = *word(e0 + st), x2 = *word(e0 + 2 * st), x3 = *word(e0 + 3 * st);
+    ar.fwd(x0, x2, w);
+    ar.fwd(x1, x3, w);
+    ar.fwd(x0, x1, wa);
+    ar.fwd(x2, x3, wb);
+    *word(e0) = x0;
+    *word(e0 + st) = x1;
+    *word(e0 + 2 * st) = x2;
+    *word(e0 + 3 * st) = x3;
+}
+template <class AR, class WORD>
+__device__ __forceinline__ void inv_quad(const AR& ar, const WORD& word, int e0, int st, typename AR::TW wa, typename AR::TW wb, typename AR::TW w) {
+    u64 x0 = *word(e0), x1 = *word(e0 + st), x2 = *word(e0 + 2 * st), x3 = *word(e0 + 3 * st);
+    ar.inv(x0, x1, wa);
+    ar.inv(x2, x3, wb);
+    ar.inv(x0, x2, w);
+    ar.inv(x1, x3, w);
+    *word(e0) = x0;
+    *word(e0 + st) = x1;
+    *word(e0 + 2 * st) = x2;
+    *word(e0 + 3 * st) = x3;
+}
+template <class AR, class WORD, class TWF>
+__device__ __forceinline__ void fwd_round4_quads(const AR& ar, const WORD& word, const TWF& tw) {
+    const typename AR::TW w = tw(0, 0), wa = tw(1, 0), wb = tw(1, 1);
+#pragma unroll 1
+    for (int k = 0; k < 4; k++) fwd_quad(ar, word, k, 4, w, wa, wb);
+#pragma unroll 1
+    for (int k = 0; k < 4; k++) fwd_quad(ar, word, 4 * k, 1, tw(2, k), tw(3, 2 * k), tw(3, 2 * k + 1));
+}
+template <class AR, class WORD, class TWF>
+__device__ __forceinline__ void inv_round4_quads(const AR& ar, const WORD& word, const TWF& tw) {
+#pragma unroll 1
+    for (int k = 0; k < 4; k++) inv_quad(ar, word, 4 * k, 1, tw(0, 2 * k), tw(0, 2 * k + 1), tw(1, k));
+    const typename AR::TW wa = tw(2, 0), wb = tw(2, 1), w = tw(3, 0);
+#pragma unroll 1
+    for (int k = 0; k < 4; k++) inv_quad(ar, word, k, 4, wa, wb, w);
+}
+
+// the table entries of a round, base as in fwd_round / inv_round
 template <class AR, class WORD>
 __device__ __forceinline__ void fwd_round4_smem(const AR& ar, const WORD& word, const typename AR::TW* __restrict__ tw, unsigned base) {
-#pragma unroll 1
-    for (int it = 0; it < 8; it++) {
-        const int k = it & 3, e0 = it < 4 ? k : 4 * k, st = it < 4 ? 4 : 1;
-        const unsigned b = it < 4 ? base : 4 * base + k;
-        u64 x0 = *word(e0), x1 = *word(e0 + st), x2 = *word(e0 + 2 * st), x3 = *word(e0 + 3 * st);
-        const typename AR::TW w = tw[b], wa = tw[2 * b], wb = tw[2 * b + 1];
-        ar.fwd(x0, x2, w);
-        ar.fwd(x1, x3, w);
-        ar.fwd(x0, x1, wa);
-        ar.fwd(x2, x3, wb);
-        *word(e0) = x0;
-        *word(e0 + st) = x1;
-        *word(e0 + 2 * st) = x2;
-        *word(e0 + 3 * st) = x3;
-    }
+    fwd_round4_quads(ar, word, [=](int s, int il) { return tw[(base << s) + il]; });
 }
 template <class AR, class WORD>
 __device__ __forceinline__ void inv_round4_smem(const AR& ar, const WORD& word, const typename AR::TW* __restrict__ tw, unsigned base) {
-#pragma unroll 1
-    for (int it = 0; it < 8; it++) {
-        const int k = it & 3, e0 = it < 4 ? 4 * k : k, st = it < 4 ? 1 : 4;
-        const unsigned b = it < 4 ? 4 * base + k : base;
-        u64 x0 = *word(e0), x1 = *word(e0 + st), x2 = *word(e0 + 2 * st), x3 = *word(e0 + 3 * st);
-        const typename AR::TW w = tw[b], wa = tw[2 * b], wb = tw[2 * b + 1];
-        ar.inv(x0, x1, wa);
-        ar.inv(x2, x3, wb);
-        ar.inv(x0, x2, w);
-        ar.inv(x1, x3, w);
-        *word(e0) = x0;
-        *word(e0 + st) = x1;
-        *word(e0 + 2 * st) = x2;
-        *word(e0 + 3 * st) = x3;
-    }
+    inv_round4_quads(ar, word, [=](int s, int il) { return tw[(base << (3 - s)) + il]; });
 }
-
 // the same rounds with a staged table: entry il of stage s of the round at tc[((1 << s) - 1 + il) * step + off] (forward),
 // tc[(16 - (16 >> s) + il) * step + off] (inverse)
 template <class AR, class WORD>
 __device__ __forceinline__ void fwd_round4_staged(const AR& ar, const WORD& word, const typename AR::TW* tc, int step, int off) {
-#pragma unroll 1
-    for (int it = 0; it < 8; it++) {
-        const int k = it & 3, e0 = it < 4 ? k : 4 * k, st = it < 4 ? 4 : 1;
-        const int a = it < 4 ? 0 : 3 + k, b = it < 4 ? 1 : 7 + 2 * k;
-        u64 x0 = *word(e0), x1 = *word(e0 + st), x2 = *word(e0 + 2 * st), x3 = *word(e0 + 3 * st);
-        const typename AR::TW w = tc[a * step + off], wa = tc[b * step + off], wb = tc[(b + 1) * step + off];
-        ar.fwd(x0, x2, w);
-        ar.fwd(x1, x3, w);
-        ar.fwd(x0, x1, wa);
-        ar.fwd(x2, x3, wb);
-        *word(e0) = x0;
-        *word(e0 + st) = x1;
-        *word(e0 + 2 * st) = x2;
-        *word(e0 + 3 * st) = x3;
-    }
+    fwd_round4_quads(ar, word, [=](int s, int il) { return tc[((1 << s) - 1 + il) * step + off]; });
 }
 template <class AR, class WORD>
 __device__ __forceinline__ void inv_round4_staged(const AR& ar, const WORD& word, const typename AR::TW* tc, int step, int off) {
-#pragma unroll 1
-    for (int it = 0; it < 8; it++) {
-        const int k = it & 3, e0 = it < 4 ? 4 * k : k, st = it < 4 ? 1 : 4;
-        const int a = it < 4 ? 2 * k : 12, b = it < 4 ? 8 + k : 14;
-        u64 x0 = *word(e0), x1 = *word(e0 + st), x2 = *word(e0 + 2 * st), x3 = *word(e0 + 3 * st);
-        const typename AR::TW w = tc[b * step + off], wa = tc[a * step + off], wb = tc[(a + 1) * step + off];
-        ar.inv(x0, x1, wa);
-        ar.inv(x2, x3, wb);
-        ar.inv(x0, x2, w);
-        ar.inv(x1, x3, w);
-        *word(e0) = x0;
-        *word(e0 + st) = x1;
-        *word(e0 + 2 * st) = x2;
-        *word(e0 + 3 * st) = x3;
-    }
+    inv_round4_quads(ar, word, [=](int s, int il) { return tc[(16 - (16 >> s) + il) * step + off]; });
 }
 
 template <int R2>
