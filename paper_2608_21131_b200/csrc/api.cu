@@ -1208,10 +1208,22 @@ static int rotate_hoisted(hann_ctx* c, const char* who, const u64* ct, int rot0,
     u64* lifted = ar.take<u64>((int64_t)count * 2 * LN);
     if (!c1c || !digits || !u || !lifted) return fail(c, HANN_EWORKSPACE, (std::string(who) + ": workspace too small").c_str());
     // one digit set, count keys: item i uses rotation rot0 + i
+    if (ks_hoist_available(c)) {
+        if (ntt_inv_pass_b_gathers(c, ct + LN, c1c)) {
+            RET(launch_ntt_inv_pass_b_from(c, ct + LN, 2 * LN, c1c, L, N, limbmap_q(c)));
+        } else {
+            RET(launch_copy2d(c, c1c, LN, ct + LN, LN, LN, 1));
+            RET(launch_ntt_inv_pass_b(c, c1c, L, N, limbmap_q(c)));
+        }
+        RET(launch_ks_lift(c, c1c, N, L, limbmap_q(c), digits, L, 0, true));
+        RET(launch_ks_hoist(c, digits, ct + LN, count, rot0, u));
+        RET(launch_ks_lift(c, u + LN, L1N, (int64_t)count * 2, limbmap_single(L), lifted, L, 0));
+        return launch_ks_finish(c, u, L + 1, lifted, count, true, rot0, 1, 1, ct, 0, 0, nullptr, 0, out, out + LN, ctw);
+    }
     const bool fin = ks_fused_available(c);
     RET(ks_digits_to_lifted(c, c1c, 1, digits, 0, rot0, 1, count, u, lifted, ct + LN, 2 * LN, fin));
-    if (fin) RET(launch_ks_finish(c, u, L + 1, lifted, count, true, rot0, 1, 1, ct, 0, 0, nullptr, 0, out, out + LN, ctw));
-    else RET(launch_moddown_combine(c, u, lifted, count, rot0, 1, ct, 0, nullptr, 0, out, out + LN, ctw));
+    if (fin) return launch_ks_finish(c, u, L + 1, lifted, count, true, rot0, 1, 1, ct, 0, 0, nullptr, 0, out, out + LN, ctw);
+    RET(launch_moddown_combine(c, u, lifted, count, rot0, 1, ct, 0, nullptr, 0, out, out + LN, ctw));
     return HANN_OK;
 }
 

@@ -240,8 +240,10 @@ int launch_ks_inner(hann_ctx* c, const u64* digits, int64_t digit_stride, int ro
 int launch_moddown_lift(hann_ctx* c, const u64* u, int64_t npoly, u64* lifted);
 // fused key switch of rings of 2^10 points and more (ksfused.cu)
 bool ks_fused_available(const hann_ctx* c);
+bool ks_hoist_available(const hann_ctx* c);
 int ks_fused_configure();  // once per context, its device current
 int launch_ks_apply(hann_ctx* c, const u64* digits, const u64* own, int64_t own_it, int64_t own_z, int64_t items, int nz, int rot0, int rot_zinc, u64* u);
+int launch_ks_hoist(hann_ctx* c, const u64* digits, const u64* own, int64_t items, int rot0, u64* u);
 int launch_ks_finish(hann_ctx* c, const u64* u, int u_limbs, const u64* lifted, int64_t items, bool perm_items, int rot0, int rot_inc, int nz, const u64* c0,
                      int64_t c0_it, int64_t c0_z, const u64* add, int64_t add_it, u64* out0, u64* out1, int64_t out_it, u64* next = nullptr);
 int launch_rescale_finish(hann_ctx* c, const u64* src, const u64* lifted, int64_t npoly, int keep, u64* out);

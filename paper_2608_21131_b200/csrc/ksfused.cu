@@ -321,6 +321,135 @@ __global__ void __launch_bounds__(T, 640 / T) k_ks_apply(ApplyArgs A) {
     }
 }
 
+struct HoistArgs {
+    const u64* digits;  // pass-A output of digit j for modulus i: (j * L + target of i) * N, a digit's own modulus left out
+    const u64* own;     // the polynomial being switched, transform domain, [L][N]
+    const u64* const* keytab;
+    int rot0, per;      // item `it` is rotation rot0 + it; items per CTA
+    long long items;
+    u64* u;  // [item][2][L+1][N] as k_ks_apply leaves it, the automorphism still to be applied
+    int N, logN;
+    const void *tw_fwd_f64, *tw_fwd_int, *tw_inv_f64, *tw_inv_int;
+    const LimbConst* lt;
+};
+
+// u[item][c][i] = sum_j digit(j) * key_item[j][c] modulo i = L - blockIdx.y, chunk blockIdx.x: one digit set under many keys (hoisted
+// rotations).  The CTA runs the second half of the digits' forward transforms on its chunk, then a thread keeps its position's L digit
+// words in registers and streams the keys of its items past them, the next item's words in flight.  The special prime's products, eight
+// items at a time, meet in shared memory, where the sixteen half-warps run their inverse pass B'.
+//
+// Bound: HBM, 20 MiB of key and 5 MiB of products per rotation at N = 2^16, L = 4; the special prime's integer transforms (its CTAs
+// start first) run beside the stream.  31 rotations: 181 us, in place of 12 (pass B of the digits) + 150 (products) + 50 (inverse pass B').
+// Chains of more than four primes keep those three launches: the words of eight digits and of the next item's keys do not fit the
+// registers, and read from shared memory and memory in turn they lost (membership circuit 7285 -> 7579 us).
+template <int L>
+__global__ void __launch_bounds__(256, 3) k_ks_hoist(HoistArgs A) {
+    extern __shared__ __align__(16) u64 sm[];
+    const int N = A.N, t = blockIdx.x, i = L - (int)blockIdx.y;
+    const long long L1N = (long long)(L + 1) * N;
+    double2* tc = (double2*)sm;            // [256] forward, [256] inverse
+    u64* buf = sm + 1024;                  // [L][256] digits
+    u64* acc = buf + (size_t)L * 256;      // [8 items][2][256] products modulo the special prime
+    const int it0 = blockIdx.z * A.per, it1 = it0 + A.per < A.items ? it0 + A.per : (int)A.items;
+    const int hw = threadIdx.x >> 4, j = threadIdx.x & 15, m = threadIdx.x;
+    const unsigned hmask = 0xFFFFu << (threadIdx.x & 16), m0 = (unsigned)(N >> 8);
+    const LimbConst* lc = A.lt + i;
+    const u64 q = lc->q;
+    const bool f64 = q < (1ULL << 50);
+    const ArithF64 ar(lc);
+    if (f64) stage_twiddles(tc, (const double2*)A.tw_fwd_f64 + ((size_t)i << A.logN), m0 + t);
+    else stage_twiddles((ulonglong2*)tc, (const ulonglong2*)A.tw_fwd_int + ((size_t)i << A.logN), m0 + t);
+    if (i == L && f64) stage_inverse_twiddles(tc + 256, (const double2*)A.tw_inv_f64 + ((size_t)i << A.logN), m0 + t);
+    else if (i == L) stage_inverse_twiddles((ulonglong2*)tc + 256, (const ulonglong2*)A.tw_inv_int + ((size_t)i << A.logN), m0 + t);
+    chain_wait();
+    __syncthreads();
+    for (int dj = hw; dj < L; dj += 16) {
+        const bool own = dj == i;
+        const u64* p = (own ? A.own + (long long)i * N : A.digits + ((long long)dj * L + (i < dj ? i : i - 1)) * N) + (t << 8);
+        u64* sb = buf + dj * 256;
+        double x[16];  // binary64 or integer words alike
+#pragma unroll
+        for (int e = 0; e < 16; e++) x[e] = __longlong_as_double((long long)p[j + 16 * e]);
+        if (own) {
+#pragma unroll
+            for (int e = 0; e < 16; e++) {
+                const u64 v = (u64)__double_as_longlong(x[e]);
+                sb[16 * j + (e ^ j)] = f64 ? (u64)__double_as_longlong(ar.inv_input(v)) : v;
+            }
+        } else if (f64) {
+            chunk_forward(ar, x, tc, sb, j, hmask);
+#pragma unroll
+            for (int e = 0; e < 16; e++) sb[16 * j + (e ^ j)] = (u64)__double_as_longlong(ar.reduce(x[e]));
+        } else {
+#pragma unroll
+            for (int e = 0; e < 16; e++) sb[16 * e + (j ^ e)] = (u64)__double_as_longlong(x[e]);
+            if (q < (1ULL << 57)) chunk_forward_int(ArithInt<true>(lc), (const ulonglong2*)tc, sb, j, hmask);
+            else chunk_forward_int(ArithInt<false>(lc), (const ulonglong2*)tc, sb, j, hmask);
+        }
+    }
+    __syncthreads();
+    const u64* xp = buf + swz(m);
+    const long long word = (long long)i * N + (t << 8) + m;
+    u64* out = A.u + word;
+    u64 xd[L];
+#pragma unroll
+    for (int d = 0; d < L; d++) xd[d] = xp[d << 8];
+    u64 cur[2 * L], nxt[2 * L];
+    const auto load = [&](int it, u64(&v)[2 * L]) {
+        const u64* key = A.keytab[A.rot0 + it] + word;
+#pragma unroll
+        for (int d = 0; d < 2 * L; d++) v[d] = __ldcs(key + d * L1N);
+    };
+    // the two sums of an item: balanced binary64 integers below 2^50, residues otherwise
+    const auto products = [&](u64(&r)[2]) {
+        if (f64) {
+            double ah[2] = {kAcc2Start, kAcc2Start}, al[2] = {0, 0};
+#pragma unroll
+            for (int d = 0; d < L; d++)
+#pragma unroll
+                for (int c = 0; c < 2; c++) acc2_fma(ah[c], al[c], residue_to_f64(cur[2 * d + c]), __longlong_as_double((long long)xd[d]));
+            const double2 c51 = make_double2(lc->c51_bal, lc->c51_q);
+#pragma unroll
+            for (int c = 0; c < 2; c++) r[c] = (u64)__double_as_longlong(ar.reduce(ar.acc2_value(ah[c], al[c], c51)));
+        } else {
+            u64 hi[2] = {0, 0}, lo[2] = {0, 0};
+#pragma unroll
+            for (int d = 0; d < L; d++)
+#pragma unroll
+                for (int c = 0; c < 2; c++) mac128(hi[c], lo[c], xd[d], cur[2 * d + c]);
+            r[0] = reduce128(hi[0], lo[0], *lc);
+            r[1] = reduce128(hi[1], lo[1], *lc);
+        }
+    };
+    if (it0 < it1) load(it0, cur);
+    for (int b0 = it0; b0 < it1; b0 += 8) {
+        const int nb = it1 - b0 < 8 ? it1 - b0 : 8;
+#pragma unroll 1
+        for (int b = 0; b < nb; b++) {
+            const int it = b0 + b;
+            if (it + 1 < it1) load(it + 1, nxt);
+            u64 r[2];
+            products(r);
+#pragma unroll
+            for (int c = 0; c < 2; c++) {
+                if (i < L) out[(long long)(it * 2 + c) * L1N] = r[c];
+                else acc[(b * 2 + c) * 256 + swz(m)] = r[c];
+            }
+#pragma unroll
+            for (int d = 0; d < 2 * L; d++) cur[d] = nxt[d];
+        }
+        if (i < L) continue;
+        __syncthreads();
+        if (hw < 2 * nb) {
+            u64* o = A.u + (long long)(b0 * 2 + hw) * L1N + (long long)i * N + (t << 8);
+            u64* sv = acc + hw * 256;
+            if (f64) chunk_inverse<true>(ar, tc + 256, m0 + t, sv, o, j, hmask);
+            else chunk_inverse<true>(ArithInt<false>(lc), (const ulonglong2*)tc + 256, m0 + t, sv, o, j, hmask);
+        }
+        __syncthreads();  // the products of the next items may be written
+    }
+}
+
 struct FinishArgs {
     const u64* lifted;  // [item][2][limbs][N], pass-A format
     const u64* u;       // [item][2] polynomials u_poly words apart; u_mid: binary64 words of limbs below 2^50 (see ApplyArgs)
@@ -502,6 +631,8 @@ constexpr size_t apply_smem(int IB, int L, bool share = false, bool inv = true) 
     return (inv ? 8192 : 4096) + (size_t)((share ? 2 : 1) * (2 * L + 2 * IB) + apply_threads(IB, L) / 16) * 2048;
 }
 
+constexpr size_t hoist_smem(int L) { return 8192 + (size_t)(L + 16) * 2048; }
+
 template <int IB, int T, bool SHARE = false>
 void launch_apply(hann_ctx* c, const ApplyArgs& A) {
     KProf kp(c, KC_KS_INNER);
@@ -521,10 +652,12 @@ int ks_fused_configure() {
     if (cudaFuncSetAttribute(k_ks_apply<2, 256, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apply_smem(2, 8)) != cudaSuccess) return HANN_ECUDA;
     if (cudaFuncSetAttribute(k_ks_apply<1, 256, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)apply_smem(1, HANN_MAX_PRIMES)) != cudaSuccess)
         return HANN_ECUDA;
+    static_assert(hoist_smem(4) <= 48 * 1024, "k_ks_hoist needs no opt-in");
     return HANN_OK;
 }
 
 bool ks_fused_available(const hann_ctx* c) { return c->logN >= 10 && c->ntt_tau; }
+bool ks_hoist_available(const hann_ctx* c) { return ks_fused_available(c) && c->L <= 4; }
 
 // digits: output of launch_ks_lift for the nz * items polynomials of L limbs; own (optional): the polynomials themselves, in which
 // case the digits were lifted without their own modulus (and, where the context has auxiliary primes, without the special prime).
@@ -576,6 +709,48 @@ int launch_ks_apply(hann_ctx* c, const u64* digits, const u64* own, int64_t own_
     return check_launch(c, "ks_apply");
 }
 
+// digits: output of launch_ks_lift for one polynomial of L limbs, own, whose digits were lifted without their own modulus.  Leaves
+// u[item][2][L+1][N], item `it` under the key of rotation rot0 + it, for the ModDown lift and launch_ks_finish with perm_items.  Only where
+// ks_hoist_available(c) holds.
+int launch_ks_hoist(hann_ctx* c, const u64* digits, const u64* own, int64_t items, int rot0, u64* u) {
+    if (items <= 0) return HANN_OK;
+    HoistArgs A = {};
+    A.digits = digits;
+    A.own = own;
+    A.keytab = c->keytab_dev;
+    A.rot0 = rot0;
+    A.items = items;
+    A.u = u;
+    A.N = c->N;
+    A.logN = c->logN;
+    A.tw_fwd_f64 = c->tw_fwd_f64;
+    A.tw_fwd_int = c->tw_fwd;
+    A.tw_inv_f64 = c->tw_inv_f64;
+    A.tw_inv_int = c->tw_inv;
+    A.lt = c->lt_dev;
+    // CTAs that share out the items of a chunk: smallest (waves x items of a CTA, the digits counting as two), ties to fewer
+    const long per = (long)(c->N >> 8) * (c->L + 1), slots = 148 * 3;
+    int gz = 1;
+    long best = -1;
+    for (int z = 1; z <= items && z <= 64; z++) {
+        const long cost = ((per * z + slots - 1) / slots) * (2 + (items + z - 1) / z);
+        if (best < 0 || cost < best) {
+            best = cost;
+            gz = z;
+        }
+    }
+    A.per = (int)((items + gz - 1) / gz);
+    KProf kp(c, KC_KS_INNER_KEYS);
+    auto go = [&](auto kern) { launch_chain(c, kern, dim3(c->N >> 8, c->L + 1, (unsigned)((items + A.per - 1) / A.per)), 256, hoist_smem(c->L), A); };
+    switch (c->L) {
+        case 1: go(k_ks_hoist<1>); break;
+        case 2: go(k_ks_hoist<2>); break;
+        case 3: go(k_ks_hoist<3>); break;
+        default: go(k_ks_hoist<4>); break;
+    }
+    return check_launch(c, "ks_hoist");
+}
+
 // lifted: output of launch_ks_lift (launch_ks_lift_aux) for the special-prime (auxiliary) limbs of u, whose polynomials have u_limbs limbs.  perm_items: the automorphism is still to be applied, that of
 // item `it` being rotation rot0 + it * rot_inc (otherwise rotation rot0 + z * rot_inc belongs to the c0 term z < nz).  next (optional, not
 // with perm_items): the second components after their inverse pass B', [item][L][N], for a key switch that follows.
@@ -586,7 +761,7 @@ int launch_ks_finish(hann_ctx* c, const u64* u, int u_limbs, const u64* lifted, 
     A.lifted = lifted;
     A.u = u;
     A.u_poly = (long long)u_limbs * c->N;
-    A.u_mid = perm_items ? 0 : 1;
+    A.u_mid = perm_items && !ks_hoist_available(c) ? 0 : 1;
     A.limbs = c->L;
     A.add = add;
     A.add_it = add_it;
