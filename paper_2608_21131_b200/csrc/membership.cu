@@ -135,10 +135,11 @@ struct Circuit {
             out[(size_t)i] = MCt{low.p + i * ctw_low, l - 1, (pairs[(size_t)i].first.scale * pairs[(size_t)i].second.scale) / prime(l - 1), 1};
         return out;
     }
-    MCt rotate(const MCt& a, int r) {
-        MCt o{take(a.level), a.level, a.scale};
-        if (o.p) ok(hann_rotate_hoisted(at(a.level), a.p, r, 1, o.p, sub, sub_bytes), at(a.level));
-        return o;
+    // a + rot_1(a) + rot_2(..) + ..: every slot holds the sum over its R neighbours, in place
+    void fold(const MCt& a, int R) {
+        int steps = 0;
+        while ((1 << steps) < R) steps++;
+        if (rc == HANN_OK && a.p) ok(hann_fold(at(a.level), a.p, 1, steps, sub, sub_bytes), at(a.level));
     }
 };
 
@@ -226,7 +227,7 @@ extern "C" int hann_membership_decide(hann_ctx* const* arith, int L, hann_ctx* s
 
     // 1, 2: |q_R|^2 (times lam^2) in every slot, read as a t at scale Delta; u = a t - (t_hi + t_lo) / (t_hi - t_lo)
     MCt t = C.mul(q, q);
-    for (int r = 1; r < prm->R; r <<= 1) t = C.add(t, C.rotate(t, r), 1);
+    C.fold(t, prm->R);
     t.scale = t.scale / (lam * lam) * a;
     const MCt u = C.add_const(t, -(prm->t_hi + prm->t_lo) / (prm->t_hi - prm->t_lo));
     // 3: Chebyshev basis by the product identity, then the combination at one common scale
