@@ -1273,7 +1273,8 @@ extern "C" int hann_encode_candidates(hann_ctx* c, const float* rows_dev, int64_
     // a stored plaintext is the first N/2 values of each limb's transform (the rest is their mirror image)
     const int64_t n = c->n, nblk = (n_rows + n - 1) / n, Ln = (int64_t)c->L * n, ptw = (int64_t)c->R * Ln;
     const bool fused = encode_fused_available(c);
-    for (int64_t blk = 0; blk < nblk; blk++) {
+    // one block on the context's current stream, its FFT buffer at wsp
+    auto encode_block = [&](int64_t blk, char* wsp) -> int {
         const int64_t rows_here = std::min(n, n_rows - blk * n);
         const float* rows = rows_dev + blk * n * dim;
         u64* pt = (u64*)pt_dev + blk * ptw;
@@ -1283,26 +1284,51 @@ extern "C" int hann_encode_candidates(hann_ctx* c, const float* rows_dev, int64_
             u64* polys = pt + (int64_t)p0 * Ln;
             if (fused && c->encode_sym && ntt_fwd_half_available(c, polys, n)) {
                 // half of every transform is computed, straight into place
-                RET(launch_encode_rows_fused(c, rows, rows_here, dim, p0, cnt, polys, n, ws, true));
+                RET(launch_encode_rows_fused(c, rows, rows_here, dim, p0, cnt, polys, n, wsp, true));
                 RET(launch_ntt_fwd_pass_b_half(c, polys, (int64_t)cnt * c->L, n, limbmap_q(c)));
                 continue;
             }
             // full transforms of a few plaintexts at a time in the staging area, first halves copied into place
-            u64* stage = (u64*)((char*)ws + encode_fft_bytes(c));
+            u64* stage = (u64*)(wsp + encode_fft_bytes(c));
             const int sg = encode_stage_group(c);
             for (int s0 = 0; s0 < cnt; s0 += sg) {
                 const int sn = std::min(sg, cnt - s0);
                 if (fused) {
-                    RET(launch_encode_rows_fused(c, rows, rows_here, dim, p0 + s0, sn, stage, c->N, ws, false));
+                    RET(launch_encode_rows_fused(c, rows, rows_here, dim, p0 + s0, sn, stage, c->N, wsp, false));
                     RET(launch_ntt_fwd_pass_b(c, stage, (int64_t)sn * c->L, c->N, limbmap_q(c)));
                 } else {
-                    RET(launch_encode_rows(c, rows, rows_here, dim, p0 + s0, sn, stage, ws));
+                    RET(launch_encode_rows(c, rows, rows_here, dim, p0 + s0, sn, stage, wsp));
                     RET(launch_ntt_fwd(c, stage, (int64_t)sn * c->L, c->N, limbmap_q(c)));
                 }
                 RET(launch_copy2d(c, polys + (int64_t)s0 * Ln, n, stage, c->N, n, (int64_t)sn * c->L));
             }
         }
+        return HANN_OK;
+    };
+    // Every launch of a block leaves a last wave that does not fill the machine (k_encode_h at N = 2^15, R = 128: 1.6 waves), so the
+    // blocks alternate between two streams where the half-size FFT leaves half of the FFT buffer free for a second block (us of a level,
+    // one / two streams: 64 blocks of 2^15 7566 / 6914, seven of 2^16 2043 / 1992, three 1242 / 1226).
+    const int64_t half = encode_fft_bytes(c) / 2 & ~(int64_t)255;
+    const bool two = nblk > 1 && c->encode_group >= c->R && !c->kprof && c->max_lanes > 1 && c->stream != c->lane_stream[0] && fused && c->encode_sym &&
+                     ntt_fwd_half_available(c, pt_dev, n) && encode_half_fft(c, 0, c->R) && half >= (int64_t)c->R * (n / 2) * 16;
+    if (!two) {
+        for (int64_t blk = 0; blk < nblk; blk++) RET(encode_block(blk, (char*)ws));
+        return HANN_OK;
     }
+    cudaStream_t main_stream = c->stream;
+    CK(cudaEventRecord(c->ev_fork, main_stream));
+    CK(cudaStreamWaitEvent(c->lane_stream[0], c->ev_fork, 0));
+    int rc = HANN_OK;
+    for (int64_t blk = 0; blk < nblk && rc == HANN_OK; blk++) {
+        if (blk & 1) c->stream = c->lane_stream[0];
+        rc = encode_block(blk, (char*)ws + (blk & 1) * half);
+        c->stream = main_stream;
+    }
+    // join before anything is reported
+    const cudaError_t e = cudaEventRecord(c->lane_join[0], c->lane_stream[0]), e2 = cudaStreamWaitEvent(main_stream, c->lane_join[0], 0);
+    RET(rc);
+    CK(e);
+    CK(e2);
     return HANN_OK;
 }
 

@@ -764,6 +764,9 @@ int encode_configure() {
     return HANN_OK;
 }
 
+// whether launch_encode_rows_fused takes the FFT of these plaintexts at half size (its buffer then holds n / 2 complex words each)
+bool encode_half_fft(const hann_ctx* c, int p_first, int count) { return c->logN - 8 >= 5 && c->B % 8 == 0 && count % 8 == 0 && p_first % 8 == 0; }
+
 bool encode_fused_available(const hann_ctx* c) {
     if (c->logN < 9) return false;
     for (int l = 0; l < c->L; l++)
@@ -796,7 +799,7 @@ int launch_encode_rows_fused(hann_ctx* c, const float* rows, int64_t rows_in_blo
     A.lt = c->lt_dev;
     const int n = c->n, a = c->logN - 8;
     const int chunks = n >> 8;  // >= 1 because logN >= 9
-    if (sym && a >= 5 && c->B % 8 == 0 && count % 8 == 0 && p_first % 8 == 0) {
+    if (sym && encode_half_fft(c, p_first, count)) {
         double half = 0x1p52;
         for (int l = 0; l < c->L; l++) half = std::min(half, (double)(c->mod[l] / 2));
         long long bits;

@@ -224,6 +224,7 @@ int launch_ks_lift(hann_ctx* c, u64* src, int64_t src_stride, int64_t nsrc, cons
 int launch_ks_lift_aux(hann_ctx* c, const u64* src, int64_t src_stride, int64_t nsrc, u64* dst);
 // encode a block and run pass A of the transforms in one kernel when the parameters allow it (returns false if not)
 bool encode_fused_available(const hann_ctx* c);
+bool encode_half_fft(const hann_ctx* c, int p_first, int count);
 int encode_configure();  // once per context, its device current
 int launch_encode_rows_fused(hann_ctx* c, const float* rows, int64_t rows_in_block, int dim, int p_first, int count, u64* out,
                              int64_t out_stride, void* ws, bool sym);

@@ -39,3 +39,20 @@ def test_encoded_candidates_equal_the_oracle(logN, R, B, bits, norm, dim, short)
     want = o.encode_block(full).reshape(R, ps.L, ps.N)
     pt = c.encode_candidates(torch.from_numpy(rows).to(c.device), c.workspace(1))
     assert np.array_equal(c.export(b.KIND_PT, pt, R).reshape(R, ps.L, ps.N), want)
+
+
+@pytest.mark.parametrize("logN,R,B,nb", [(13, 16, 8, 2), (13, 32, 16, 5), (14, 16, 8, 3)])
+def test_blocks_on_two_streams_encode_to_the_same_words(logN, R, B, nb):
+    """A level of several blocks alternates between two streams and the two halves of the FFT buffer; one block at a time does not."""
+    import torch
+
+    from paper_2608_21131_b200 import binding as b
+
+    ps = synth.small_params(logN, R, B, L=2)
+    c = b.Context(ps)
+    rows = torch.from_numpy(synth.toy_corpus(5, rows=nb * ps.n - 7, dim=R)).to(c.device)
+    ws = c.workspace(nb)
+    pt = c.encode_candidates(rows, ws)
+    one = torch.cat([c.encode_candidates(rows[i * ps.n:(i + 1) * ps.n].contiguous(), ws) for i in range(nb)])
+    torch.cuda.synchronize()
+    assert torch.equal(pt, one)
