@@ -48,7 +48,7 @@ def test_blocks_on_two_streams_encode_to_the_same_words(logN, R, B, nb):
 
     from paper_2608_21131_b200 import binding as b
 
-    ps = synth.small_params(logN, R, B, L=2)
+    ps = synth.ParamSet("two", logN, tuple(find_primes(50, logN + 1, 2)), find_primes(60, logN + 1, 1)[0], 40, R, B, 0)
     c = b.Context(ps)
     rows = torch.from_numpy(synth.toy_corpus(5, rows=nb * ps.n - 7, dim=R)).to(c.device)
     ws = c.workspace(nb)
