@@ -699,7 +699,9 @@ int launch_ks_apply(hann_ctx* c, const u64* digits, const u64* own, int64_t own_
     //   N = 2^15, L = 4, one rotation:    1 item 18 / 19 / 22, 2: 23 / 21 / 23, 4: 43 / 33 / 28, 8: 77 / 57 / 51, 16: 140 / 105 / 96
     //   N = 2^12, L = 2, seven rotations: 1 item 78 / 68 / 62, 16: 86 / 88 / 83
     //   N = 2^15, L = 8, one rotation:    1 item 24 / 32, 2: 45 / 42, 3: 64 / 70, 4: 82 / 77, 16: 292 / 281
-    // Four lose to two where they leave half of the last CTA empty (five and six items of four primes: 86 against 70 us).
+    // (Taken with the special prime itself; with auxiliary primes four items share the transforms of both key sets, which moved a launch of
+    // four items and three rotations from 166 to 118 us.)  Without them four lose to two where they leave half of the last CTA empty
+    // (five and six items of four primes: 86 against 70 us).
     if (items >= 4 && c->L <= 4 && aux) launch_apply<4, 256, true>(c, A);
     else if (items >= 4 && c->L <= 4) launch_apply<4, 256>(c, A);
     else if (items >= 2 && c->L <= 4) launch_apply<2, 128>(c, A);
