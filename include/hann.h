@@ -29,9 +29,10 @@
  *   - The exchange and client calls (hann_import, hann_export*, key generation, encryption, decryption) stage their data in device
  *     memory of the context: allocated at the first call that needs it, grown when a later one needs more, kept until
  *     hann_ctx_destroy, never used by the server-side calls.  Its size is that of the largest call so far: 64 polynomials of L
- *     limbs for hann_import (kind PT) and hann_export, (2 L + 1)(L + 1) polynomials of one limb for key generation, at most
- *     64 MiB (and no less than one ciphertext) for decryption.  Encryption and decryption also keep 4 MiB of page-locked host memory
- *     of the context from the first copy of 1 MiB and more on, and fill it from up to three helper threads that end with the call.
+ *     limbs for hann_import (kind PT) and hann_export, (2 L + 1)(L + 1) polynomials of one limb for key generation, 2 L (L + 1)
+ *     for hann_load_keys, at most 64 MiB (and no less than one ciphertext) for decryption.  Encryption and decryption also keep 4 MiB
+ *     of page-locked host memory of the context from the first copy of 1 MiB and more on, and fill it from up to three helper threads
+ *     that end with the call.
  *   - Canonical exchange layout (the only layout with a meaning outside the library): coefficient
  *     domain, natural coefficient order, residues in [0, q_i), uint64, index order [poly][limb][coeff];
  *     a ciphertext is 2 polynomials (c0, c1) of L limbs.  The internal device layout (transform domain,
@@ -245,8 +246,11 @@ int hann_decrypt_compact(hann_ctx *ctx, const int8_t *s, const uint64_t *ct, int
 
 /* Upload evaluation keys (canonical layout as produced by hann_keygen_from_samples; `evk` may be a host or a
  * device pointer) into the context, replacing keys with the same rotation.  Allocates device memory owned by the
- * context: 2 L (L + 1) polynomials of one limb per key, and 6 L more where the key switch has auxiliary primes (rings of 2^10 points
- * and more, three ciphertext primes below 2^50 and a special prime in [2^50, 2^61)); as much again while the call runs.  Needed later: rotations 1..B-1 for hann_query_prepare, rotation B for hann_rotate_sum. */
+ * context: 2 L (L + 1) polynomials of one limb per key, and for rotations that are multiples of B (0 among them) 6 L more
+ * where the key switch has auxiliary primes (rings of 2^10 points and more, three ciphertext primes below 2^50 of about the
+ * same size and a special prime in [2^50, 2^61)) and the device has room for them; a key without them works all the same, to
+ * the same bits.  Staged through the exchange scratch.  Where a key cannot be loaded, those before it in the list stay
+ * loaded.  Needed later: rotations 1..B-1 for hann_query_prepare, rotation B for hann_rotate_sum. */
 int hann_load_keys(hann_ctx *ctx, const uint64_t *evk, int n_rot, const int32_t *rot);
 
 /* Once per query (Sec. 3.1 Detail: the baby steps of the diagonal method; Sec. 3.4: the rotated query is computed

@@ -128,9 +128,6 @@ int64_t ks_item_words(const hann_ctx* c) {
     return L * N + L * (ks_fused_available(c) ? L : L + 1) * N + 2 * (L + 1) * N + 2 * L * N + 2 * L * N;
 }
 
-// limbs of the product u of a key-switch round (ks_round_fused) whose polynomials are not switched in place
-int ks_u_limbs(const hann_ctx* c) { return c->L + (c->aux ? kAux : 1); }
-
 // words of workspace the lazy rotate-and-sum needs per block of a round: G-1 terms (c1 coefficients, digits, and their key products
 // unless the fused kernels sum them), the summed product and one ModDown
 int64_t lazy_block_words(const hann_ctx* c) {
@@ -152,30 +149,39 @@ int64_t balanced(int64_t most, int64_t total) {
     return (total + rounds - 1) / rounds;
 }
 
+// whether a key-switch round goes through auxiliary primes: every one of its keys, of rotations rot0 + z * rot_zinc, has the words
+bool ks_aux(const hann_ctx* c, int rot0, int rot_zinc, int nz) {
+    for (int z = 0; z < nz; z++)
+        if (!c->keyaux_host[rot0 + z * rot_zinc]) return false;
+    return c->aux;
+}
+
 // the sub-buffers of a key-switch round (ks_round_fused, or ks_digits_to_lifted on smaller rings) on nz * items polynomials.  With
-// auxiliary primes u has two more limbs and a digit one target less, so a round needs no more words than ks_item_words and
+// auxiliary primes (aux) u has two more limbs and a digit one target less, so a round needs no more words than ks_item_words and
 // lazy_block_words count, except on a chain of three primes: where the arena ends there, the lifted polynomials (carved last) take
 // the place of the digits, which k_ks_apply was the last to read.
 struct RoundBuffers {
     u64 *c1c, *digits, *u, *lifted;
+    bool aux;
+    int u_limbs;  // limbs of a polynomial of u
 };
-bool carve_round(const hann_ctx* c, Arena& ar, int64_t items, int64_t nz, RoundBuffers& b) {
-    const int64_t L = c->L, N = c->N, digits = L * (ks_fused_available(c) ? (c->aux ? L - 1 : L) : L + 1) * N;
-    const int64_t u = 2 * (ks_fused_available(c) ? ks_u_limbs(c) : L + 1) * N;
+bool carve_round(const hann_ctx* c, Arena& ar, bool aux, int64_t items, int64_t nz, RoundBuffers& b) {
+    const int64_t L = c->L, N = c->N, targets = aux ? L - 1 : ks_fused_available(c) ? L : L + 1;
+    b.aux = aux;
+    b.u_limbs = (int)L + (aux ? kAux : 1);
     b.c1c = ar.take<u64>(nz * items * L * N);
-    b.digits = ar.take<u64>(nz * items * digits);
-    b.u = ar.take<u64>(items * u);
+    b.digits = ar.take<u64>(nz * items * L * targets * N);
+    b.u = ar.take<u64>(items * 2 * b.u_limbs * N);
     b.lifted = ar.take<u64>(items * 2 * L * N);
-    if (!b.lifted && c->aux && L == 3) b.lifted = b.digits;
+    if (!b.lifted && aux && L == 3) b.lifted = b.digits;
     return b.c1c && b.digits && b.u && b.lifted;
 }
 
-// the four sub-buffers of ONE key switch (hann_keyswitch, hann_keyswitch_static): input copy, digits, u, lifted
-struct KsBuffers {
-    u64 *c1c, *digits, *u, *lifted;
-};
-bool carve_keyswitch(const hann_ctx* c, Arena& ar, KsBuffers& b) {
+// the sub-buffers of ONE key switch in place (hann_keyswitch, hann_keyswitch_static): input copy, digits, u, lifted
+bool carve_keyswitch(const hann_ctx* c, Arena& ar, RoundBuffers& b) {
     const int64_t L = c->L, N = c->N;
+    b.aux = false;
+    b.u_limbs = (int)L + 1;
     b.c1c = ar.take<u64>(L * N);
     b.digits = ar.take<u64>(L * (L + 1) * N);
     b.u = ar.take<u64>(2 * (L + 1) * N);
@@ -260,10 +266,11 @@ int ks_digits_to_lifted(hann_ctx* c, u64* c1c, int64_t items, u64* digits, int64
 // as carve_round leaves them.
 // src == c1c, one polynomial (nz = items = 1) only: the inverse pass overwrites it, so its digits are lifted to their own modulus as
 // well, the product modulo the special prime takes no auxiliary primes, and the digits take L * L1N words (carve_keyswitch).
-int ks_round_fused(hann_ctx* c, const u64* src, int64_t src_it, int64_t src_z, int64_t items, int nz, int rot0, int rot_zinc, u64* c1c, u64* digits,
-                   u64* u, u64* lifted, bool inverted = false) {
+int ks_round_fused(hann_ctx* c, const u64* src, int64_t src_it, int64_t src_z, int64_t items, int nz, int rot0, int rot_zinc,
+                   const RoundBuffers& b, bool inverted = false) {
     const int L = c->L, N = c->N;
-    const int64_t LN = (int64_t)L * N, L1N = (int64_t)(L + 1) * N;
+    const int64_t LN = (int64_t)L * N;
+    u64* c1c = b.c1c;
     const bool in_place = src == c1c;
     if (in_place && (nz != 1 || items != 1)) return fail(c, HANN_EINVAL, "a key-switch round in place takes one polynomial");
     if (inverted) {
@@ -277,11 +284,11 @@ int ks_round_fused(hann_ctx* c, const u64* src, int64_t src_it, int64_t src_z, i
         RET(launch_ntt_inv_pass_b(c, c1c, nz * items * L, N, limbmap_q(c)));
     }
     // a digit's transform modulo its own prime is the polynomial that came in, where that still exists
-    const bool aux = c->aux && !in_place;
-    RET(launch_ks_lift(c, c1c, N, nz * items * L, limbmap_q(c), digits, in_place ? L + 1 : aux ? L - 1 : L, 0, !in_place));
-    RET(launch_ks_apply(c, digits, in_place ? nullptr : src, src_it, src_z, items, nz, rot0, rot_zinc, u));
-    if (aux) RET(launch_ks_lift_aux(c, u + LN, LN + kAux * (int64_t)N, items * 2, lifted));
-    else RET(launch_ks_lift(c, u + LN, L1N, items * 2, limbmap_single(L), lifted, L, 0));
+    RET(launch_ks_lift(c, c1c, N, nz * items * L, limbmap_q(c), b.digits, in_place ? L + 1 : b.aux ? L - 1 : L, 0, !in_place));
+    RET(launch_ks_apply(c, b.digits, in_place ? nullptr : src, src_it, src_z, items, nz, rot0, rot_zinc, b.aux, b.u));
+    const int64_t u_poly = (int64_t)b.u_limbs * N;
+    if (b.aux) RET(launch_ks_lift_aux(c, b.u + LN, u_poly, items * 2, b.lifted));
+    else RET(launch_ks_lift(c, b.u + LN, u_poly, items * 2, limbmap_single(L), b.lifted, L, 0));
     return HANN_OK;
 }
 
@@ -293,7 +300,7 @@ int static_scratch_resolve(hann_ctx* c, void** out);
 // bytes of 256-byte aligned workspace one hann_keyswitch needs: measured by running its own carving on an empty arena
 int64_t keyswitch_ws_bytes(const hann_ctx* c) {
     Arena ar{nullptr, 0, INT64_MAX / 2};
-    KsBuffers kb;
+    RoundBuffers kb;
     ar.base = (char*)256;  // any non-null base: the carving only does pointer arithmetic
     carve_keyswitch(c, ar, kb);
     return ar.off;
@@ -459,7 +466,7 @@ extern "C" int hann_ctx_create(const hann_params* prm, hann_ctx** out) {
               cudaHostGetDevicePointer((void**)&c->kflag, c->kflag_host, 0) == cudaSuccess &&
               cudaMalloc(&c->fft_T, nh * sizeof(double2)) == cudaSuccess && cudaMalloc(&c->fft_U, n * sizeof(double2)) == cudaSuccess &&
               cudaMalloc(&c->jinv, n * sizeof(int32_t)) == cudaSuccess && cudaMalloc(&c->galois_dev, n * sizeof(unsigned)) == cudaSuccess &&
-              cudaMalloc(&c->keytab_dev, n * sizeof(u64*)) == cudaSuccess;
+              cudaMalloc(&c->keytab_dev, n * sizeof(u64*)) == cudaSuccess && cudaMalloc(&c->keyaux_dev, n * sizeof(u64*)) == cudaSuccess;
     if (ok) {
         *c->kflag_host = 0;
         ok = cudaMemcpy(c->tw_fwd, twf.data(), twb, cudaMemcpyHostToDevice) == cudaSuccess &&
@@ -471,10 +478,11 @@ extern "C" int hann_ctx_create(const hann_params* prm, hann_ctx** out) {
              cudaMemcpy(c->fft_U, U.data(), n * sizeof(double2), cudaMemcpyHostToDevice) == cudaSuccess &&
              cudaMemcpy(c->jinv, jpos.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice) == cudaSuccess &&
              cudaMemcpy(c->galois_dev, gal.data(), n * sizeof(unsigned), cudaMemcpyHostToDevice) == cudaSuccess &&
-             cudaMemset(c->keytab_dev, 0, n * sizeof(u64*)) == cudaSuccess;
+             cudaMemset(c->keytab_dev, 0, n * sizeof(u64*)) == cudaSuccess && cudaMemset(c->keyaux_dev, 0, n * sizeof(u64*)) == cudaSuccess;
     }
     c->h_galois = gal;
     c->keytab_host.assign(n, nullptr);
+    c->keyaux_host.assign(n, nullptr);
     for (int k = 0; k < HANN_NKINDS && ok; k++)
         ok = cudaEventCreate(&c->ev[k][0]) == cudaSuccess && cudaEventCreate(&c->ev[k][1]) == cudaSuccess;
     if (ok)
@@ -515,11 +523,12 @@ extern "C" void hann_ctx_destroy(hann_ctx* c) {
     if (!c) return;
     DeviceGuard dg(c->device);
     cudaStreamSynchronize(c->stream);
-    for (u64* k : c->keytab_host)
-        if (k) cudaFree(k);
+    for (const auto* tab : {&c->keytab_host, &c->keyaux_host})
+        for (u64* k : *tab)
+            if (k) cudaFree(k);
     cudaFree(c->tw_fwd); cudaFree(c->tw_inv); cudaFree(c->tw_fwd_f64); cudaFree(c->tw_inv_f64); cudaFree(c->lt_dev);
     if (c->kflag_host) cudaFreeHost(c->kflag_host);
-    cudaFree(c->fft_T); cudaFree(c->fft_U); cudaFree(c->jinv); cudaFree(c->galois_dev); cudaFree(c->keytab_dev);
+    cudaFree(c->fft_T); cudaFree(c->fft_U); cudaFree(c->jinv); cudaFree(c->galois_dev); cudaFree(c->keytab_dev); cudaFree(c->keyaux_dev);
     if (c->scratch) cudaFree(c->scratch);
     host_copy_release(c);
     if (c->aux_stream) {
@@ -1163,6 +1172,49 @@ extern "C" int hann_decrypt_compact(hann_ctx* c, const int8_t* s, const uint64_t
 
 // ================================================================================================ server side
 
+// one key of rotation r: into the buffers that the context has for it, or into new ones, which it gets when the key is complete
+static int load_key(hann_ctx* c, const uint64_t* evk, int r) {
+    const int L = c->L, N = c->N;
+    const int64_t keyw = (int64_t)L * 2 * (L + 1) * N, auxw = (int64_t)L * 2 * kAux * N;
+    u64 *tmp = (u64*)c->scratch, *buf = c->keytab_host[r], *aux = c->keyaux_host[r];
+    if (!buf && cudaMalloc(&buf, keyw * 8) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(c, HANN_ENOMEM, "hann_load_keys: device allocation failed");
+    }
+    // The rounds that take auxiliary primes switch the giant steps (multiples of B), relinearise (0) or fold; the keys of the hoisted
+    // rotations do without their words.  Where the device has no room for them the key switch takes p itself, with the same bits.
+    if (c->aux && r % c->B == 0 && !aux && cudaMalloc(&aux, auxw * 8) != cudaSuccess) {
+        cudaGetLastError();
+        aux = nullptr;
+    }
+    auto fill = [&]() -> int {
+        CK(cudaMemcpyAsync(tmp, evk, keyw * 8, cudaMemcpyDefault, c->stream));
+        // store phi_k^{-1}(key): the inner product then runs on unpermuted digits and the automorphism is applied
+        // once, to its much smaller result
+        const unsigned kinv = c->h_galois[(c->n - r) % c->n];  // 5^{-r} = 5^{n-r} (5 has order n modulo 2N)
+        if (aux) {
+            LimbMap lm;
+            lm.period = kAux;
+            for (int k = 0; k < kAux; k++) lm.limb[k] = c->crt.limb[k];
+            RET(launch_key_aux(c, tmp, buf));  // 6 L N words of the 2 L (L + 1) N that are written below
+            RET(launch_ntt_fwd(c, buf, (int64_t)L * 2 * kAux, N, lm));
+            RET(launch_permute(c, buf, aux, auxw / N, kinv));
+        }
+        RET(launch_ntt_fwd(c, tmp, (int64_t)L * 2 * (L + 1), N, limbmap_qp(c)));
+        RET(launch_permute(c, tmp, buf, keyw / N, kinv));
+        return sync_and_check(c);
+    };
+    const int rc = fill();
+    if (rc != HANN_OK) {
+        if (buf != c->keytab_host[r]) cudaFree(buf);
+        if (aux && aux != c->keyaux_host[r]) cudaFree(aux);
+        return rc;
+    }
+    c->keytab_host[r] = buf;
+    c->keyaux_host[r] = aux;
+    return HANN_OK;
+}
+
 extern "C" int hann_load_keys(hann_ctx* c, const uint64_t* evk, int n_rot, const int32_t* rot) {
     if (!c) return HANN_EINVAL;
     if (!evk || !rot || n_rot < 0) return fail(c, HANN_EINVAL, "hann_load_keys: bad argument");
@@ -1170,38 +1222,14 @@ extern "C" int hann_load_keys(hann_ctx* c, const uint64_t* evk, int n_rot, const
     for (int i = 0; i < n_rot; i++)
         if (rot[i] < 0 || rot[i] >= c->n) return fail(c, HANN_ESHAPE, "hann_load_keys: rotation out of range");
     DeviceGuard dg(c->device);
-    const int64_t keyw = (int64_t)L * 2 * (L + 1) * N, auxw = c->aux ? (int64_t)L * 2 * kAux * N : 0;
-    RET(ensure_scratch(c, (keyw + auxw) * 8));
-    LimbMap lm_aux;
-    lm_aux.period = kAux;
-    for (int k = 0; k < kAux; k++) lm_aux.limb[k] = c->crt.limb[k];
-    for (int i = 0; i < n_rot; i++) {
-        const int r = rot[i];
-        if (!c->keytab_host[r]) {
-            u64* buf = nullptr;
-            if (cudaMalloc(&buf, (keyw + auxw) * 8) != cudaSuccess) {
-                cudaGetLastError();
-                return fail(c, HANN_ENOMEM, "hann_load_keys: device allocation failed");
-            }
-            c->keytab_host[r] = buf;
-        }
-        u64* tmp = (u64*)c->scratch;
-        CK(cudaMemcpyAsync(tmp, evk + (int64_t)i * keyw, keyw * 8, cudaMemcpyDefault, c->stream));
-        if (c->aux) {
-            RET(launch_key_aux(c, tmp, tmp + keyw));
-            RET(launch_ntt_fwd(c, tmp + keyw, (int64_t)L * 2 * kAux, N, lm_aux));
-        }
-        RET(launch_ntt_fwd(c, tmp, (int64_t)L * 2 * (L + 1), N, limbmap_qp(c)));
-        // store phi_k^{-1}(key): the inner product then runs on unpermuted digits and the automorphism is applied
-        // once, to its much smaller result
-        const unsigned k = c->h_galois[r];
-        const unsigned kinv = c->h_galois[(c->n - r) % c->n];  // 5^{-r} = 5^{n-r} (5 has order n modulo 2N)
-        (void)k;
-        RET(launch_permute(c, tmp, c->keytab_host[r], (keyw + auxw) / N, kinv));
-        RET(sync_and_check(c));
-    }
+    const int64_t keyw = (int64_t)L * 2 * (L + 1) * N;
+    RET(ensure_scratch(c, keyw * 8));
+    int rc = HANN_OK;
+    for (int i = 0; i < n_rot && rc == HANN_OK; i++) rc = load_key(c, evk + (int64_t)i * keyw, rot[i]);
+    // the keys before one that could not be loaded count: the kernels' tables say what the host's do
     CK(cudaMemcpy(c->keytab_dev, c->keytab_host.data(), c->keytab_host.size() * sizeof(u64*), cudaMemcpyHostToDevice));
-    return HANN_OK;
+    CK(cudaMemcpy(c->keyaux_dev, c->keyaux_host.data(), c->keyaux_host.size() * sizeof(u64*), cudaMemcpyHostToDevice));
+    return rc;
 }
 
 // out[i] = rot_{rot0 + i}(ct), i < count: one digit decomposition of c1, count keys, one ModDown round
@@ -1376,7 +1404,7 @@ extern "C" int hann_score_level_ctdb(hann_ctx* c, const void* baby_dev, const vo
     Arena ar{(char*)ws, 0, (int64_t)ws_bytes, c};
     u64* d = ar.take<u64>(ch * 3 * LN);
     RoundBuffers rb;
-    if (!d || !carve_round(c, ar, ch, 1, rb)) return fail(c, HANN_EWORKSPACE, "hann_score_level_ctdb: workspace too small");
+    if (!d || !carve_round(c, ar, ks_aux(c, 0, 0, 1), ch, 1, rb)) return fail(c, HANN_EWORKSPACE, "hann_score_level_ctdb: workspace too small");
     const u64* ctdb = (const u64*)ctdb_dev;
     u64* inner = (u64*)inner_dev;
     for (int64_t i0 = 0; i0 < items; i0 += ch) {
@@ -1385,8 +1413,8 @@ extern "C" int hann_score_level_ctdb(hann_ctx* c, const void* baby_dev, const vo
         // relinearise: (d0 + ks0, d1 + ks1) with (ks0, ks1) the key switch of d2 under the key of s^2 ("rotation 0": no
         // automorphism)
         if (ks_fused_available(c)) {
-            RET(ks_round_fused(c, d + 2 * LN, 3 * LN, 0, ni, 1, 0, 0, rb.c1c, rb.digits, rb.u, rb.lifted));
-            RET(launch_ks_finish(c, rb.u, ks_u_limbs(c), rb.lifted, ni, false, 0, 0, 1, nullptr, 0, 0, d, 3 * LN, inner + i0 * ctw, inner + i0 * ctw + LN, ctw));
+            RET(ks_round_fused(c, d + 2 * LN, 3 * LN, 0, ni, 1, 0, 0, rb));
+            RET(launch_ks_finish(c, rb.u, rb.u_limbs, rb.lifted, ni, false, 0, 0, 1, nullptr, 0, 0, d, 3 * LN, inner + i0 * ctw, inner + i0 * ctw + LN, ctw));
             continue;
         }
         RET(launch_copy2d(c, rb.c1c, LN, d + 2 * LN, 3 * LN, LN, ni));
@@ -1416,7 +1444,7 @@ extern "C" int hann_multiply(hann_ctx* c, const void* a_dev, const void* b_dev, 
     Arena ar{(char*)ws, 0, (int64_t)ws_bytes, c};
     u64* d = ar.take<u64>(ch * 3 * LN);
     RoundBuffers rb;
-    if (!d || !carve_round(c, ar, ch, 1, rb)) return fail(c, HANN_EWORKSPACE, "hann_multiply: workspace too small");
+    if (!d || !carve_round(c, ar, ks_aux(c, 0, 0, 1), ch, 1, rb)) return fail(c, HANN_EWORKSPACE, "hann_multiply: workspace too small");
     const u64 *a = (const u64*)a_dev, *b = (const u64*)b_dev;
     u64* out = (u64*)out_dev;
     for (int64_t i0 = 0; i0 < count; i0 += ch) {
@@ -1424,8 +1452,8 @@ extern "C" int hann_multiply(hann_ctx* c, const void* a_dev, const void* b_dev, 
         RET(launch_mul_ct(c, a + i0 * ctw, b + i0 * ctw, ni, d));
         // relinearise: (d0 + ks0, d1 + ks1), (ks0, ks1) the key switch of d2 under the key of s^2 ("rotation 0")
         if (ks_fused_available(c)) {
-            RET(ks_round_fused(c, d + 2 * LN, 3 * LN, 0, ni, 1, 0, 0, rb.c1c, rb.digits, rb.u, rb.lifted));
-            RET(launch_ks_finish(c, rb.u, ks_u_limbs(c), rb.lifted, ni, false, 0, 0, 1, nullptr, 0, 0, d, 3 * LN, out + i0 * ctw, out + i0 * ctw + LN, ctw));
+            RET(ks_round_fused(c, d + 2 * LN, 3 * LN, 0, ni, 1, 0, 0, rb));
+            RET(launch_ks_finish(c, rb.u, rb.u_limbs, rb.lifted, ni, false, 0, 0, 1, nullptr, 0, 0, d, 3 * LN, out + i0 * ctw, out + i0 * ctw + LN, ctw));
             continue;
         }
         RET(launch_copy2d(c, rb.c1c, LN, d + 2 * LN, 3 * LN, LN, ni));
@@ -1462,7 +1490,7 @@ extern "C" int hann_rotate_sum(hann_ctx* c, const void* inner_dev, int64_t n_blo
         Arena ar{wsp, 0, wsp_bytes, c};
         RoundBuffers rb;
         u64* tmp = ar.take<u64>(ch * ctw);
-        if (!tmp || !carve_round(c, ar, ch, 1, rb)) return fail(c, HANN_EWORKSPACE, "hann_rotate_sum: workspace too small");
+        if (!tmp || !carve_round(c, ar, ks_aux(c, B, 0, 1), ch, 1, rb)) return fail(c, HANN_EWORKSPACE, "hann_rotate_sum: workspace too small");
         for (int64_t b0 = b_lo; b0 < b_hi; b0 += ch) {
             const int64_t nb = std::min(ch, b_hi - b0);
             const u64* old = inner + (b0 * G + (G - 1)) * ctw;  // acc = inner[G-1]
@@ -1471,8 +1499,8 @@ extern "C" int hann_rotate_sum(hann_ctx* c, const void* inner_dev, int64_t n_blo
                 u64* out = (g % 2 == 0) ? score + b0 * ctw : tmp;
                 // c1 of every accumulator, still in the transform domain; the key-switch round takes it from there
                 if (fused) {
-                    RET(ks_round_fused(c, old + LN, old_stride, 0, nb, 1, B, 0, rb.c1c, rb.digits, rb.u, rb.lifted, g < G - 2));
-                    RET(launch_ks_finish(c, rb.u, ks_u_limbs(c), rb.lifted, nb, false, B, 0, 1, old, old_stride, 0, inner + (b0 * G + g) * ctw, (int64_t)G * ctw, out,
+                    RET(ks_round_fused(c, old + LN, old_stride, 0, nb, 1, B, 0, rb, g < G - 2));
+                    RET(launch_ks_finish(c, rb.u, rb.u_limbs, rb.lifted, nb, false, B, 0, 1, old, old_stride, 0, inner + (b0 * G + g) * ctw, (int64_t)G * ctw, out,
                                          out + LN, ctw, g > 0 ? rb.c1c : nullptr));
                     old = out;
                     old_stride = ctw;
@@ -1553,7 +1581,7 @@ extern "C" int hann_rotate_sum_lazy(hann_ctx* c, const void* inner_dev, int64_t 
         u64 *c1c = nullptr, *digits = nullptr, *u = nullptr, *up = nullptr, *lifted = nullptr;
         bool carved;
         if (fused) {
-            carved = carve_round(c, ar, ch, G - 1, rb);
+            carved = carve_round(c, ar, ks_aux(c, B, B, G - 1), ch, G - 1, rb);
         } else {
             c1c = ar.take<u64>(items_max * LN);
             digits = ar.take<u64>(items_max * L * L1N);
@@ -1568,8 +1596,8 @@ extern "C" int hann_rotate_sum_lazy(hann_ctx* c, const void* inner_dev, int64_t 
             const u64* in0 = inner + b0 * G * ctw;
             if (fused) {
                 // all giant steps summed under their own keys and automorphisms before one ModDown per block
-                RET(ks_round_fused(c, in0 + ctw + LN, (int64_t)G * ctw, ctw, nb, G - 1, B, B, rb.c1c, rb.digits, rb.u, rb.lifted));
-                RET(launch_ks_finish(c, rb.u, ks_u_limbs(c), rb.lifted, nb, false, B, B, G - 1, in0 + ctw, (int64_t)G * ctw, ctw, in0, (int64_t)G * ctw, score + b0 * ctw,
+                RET(ks_round_fused(c, in0 + ctw + LN, (int64_t)G * ctw, ctw, nb, G - 1, B, B, rb));
+                RET(launch_ks_finish(c, rb.u, rb.u_limbs, rb.lifted, nb, false, B, B, G - 1, in0 + ctw, (int64_t)G * ctw, ctw, in0, (int64_t)G * ctw, score + b0 * ctw,
                                      score + b0 * ctw + LN, ctw));
                 continue;
             }
@@ -1738,8 +1766,11 @@ extern "C" int hann_fold(hann_ctx* c, void* ct_dev, int stride, int steps, void*
     if (!ct_dev || stride < 1 || steps < 0) return fail(c, HANN_EINVAL, "hann_fold: bad argument");
     if (steps == 0) return HANN_OK;
     if (((int64_t)stride << (steps - 1)) >= c->n) return fail(c, HANN_ESHAPE, "hann_fold: rotation out of range");
-    for (int t = 0; t < steps; t++)
+    bool aux = true;  // one carving for all steps
+    for (int t = 0; t < steps; t++) {
         if (!c->keytab_host[stride << t]) return fail(c, HANN_ENOKEY, "hann_fold: the keys of rotations stride * 2^t must be loaded");
+        aux = aux && ks_aux(c, stride << t, 0, 1);
+    }
     if (!ws || ((uintptr_t)ws & 255)) return fail(c, HANN_EWORKSPACE, "hann_fold: workspace missing or not 256-byte aligned");
     const int L = c->L, N = c->N;
     const int64_t LN = (int64_t)L * N, L1N = (int64_t)(L + 1) * N, ctw = 2 * LN;
@@ -1748,15 +1779,15 @@ extern "C" int hann_fold(hann_ctx* c, void* ct_dev, int stride, int steps, void*
     Arena ar{(char*)ws, 0, (int64_t)ws_bytes, c};
     RoundBuffers rb;
     u64* tmp = ar.take<u64>(ctw);
-    if (!tmp || !carve_round(c, ar, 1, 1, rb)) return fail(c, HANN_EWORKSPACE, "hann_fold: workspace too small");
+    if (!tmp || !carve_round(c, ar, aux, 1, 1, rb)) return fail(c, HANN_EWORKSPACE, "hann_fold: workspace too small");
     u64* cur = (u64*)ct_dev;
     u64* nxt = tmp;
     for (int t = 0; t < steps; t++) {
         const int r = stride << t;
         // nxt = cur + rot_r(cur): the Horner step of the rotate-and-sum with the ciphertext itself as the addend
         if (ks_fused_available(c)) {
-            RET(ks_round_fused(c, cur + LN, ctw, 0, 1, 1, r, 0, rb.c1c, rb.digits, rb.u, rb.lifted, t > 0));
-            RET(launch_ks_finish(c, rb.u, ks_u_limbs(c), rb.lifted, 1, false, r, 0, 1, cur, ctw, 0, cur, ctw, nxt, nxt + LN, ctw,
+            RET(ks_round_fused(c, cur + LN, ctw, 0, 1, 1, r, 0, rb, t > 0));
+            RET(launch_ks_finish(c, rb.u, rb.u_limbs, rb.lifted, 1, false, r, 0, 1, cur, ctw, 0, cur, ctw, nxt, nxt + LN, ctw,
                                  t + 1 < steps ? rb.c1c : nullptr));
         } else {
             RET(ks_digits_to_lifted(c, rb.c1c, 1, rb.digits, (int64_t)L * L1N, r, 0, 1, rb.u, rb.lifted, cur + LN, ctw));
@@ -1830,15 +1861,15 @@ extern "C" int hann_keyswitch(hann_ctx* c, int rot, const void* poly_dev, void* 
     DeviceGuard dg(c->device);
     Timer tm(c, 4);
     Arena ar{(char*)ws, 0, (int64_t)ws_bytes, c};
-    KsBuffers kb;
+    RoundBuffers kb;
     if (!carve_keyswitch(c, ar, kb)) return fail(c, HANN_EWORKSPACE, "hann_keyswitch: workspace too small");
     u64 *c1c = kb.c1c, *digits = kb.digits, *u = kb.u, *lifted = kb.lifted;
     // the stored key is phi_k^{-1}(evk): switch phi_k^{-1}(d) and apply phi_k to the result
     const unsigned kinv = c->h_galois[(c->n - rot) % c->n];
     RET(launch_permute(c, (const u64*)poly_dev, c1c, L, kinv));
     if (ks_fused_available(c)) {
-        RET(ks_round_fused(c, c1c, (int64_t)L * c->N, 0, 1, 1, rot, 0, c1c, digits, u, lifted));
-        return launch_ks_finish(c, u, L + 1, lifted, 1, false, 0, 0, 1, nullptr, 0, 0, nullptr, 0, (u64*)ks0_dev, (u64*)ks1_dev, 0);
+        RET(ks_round_fused(c, c1c, (int64_t)L * c->N, 0, 1, 1, rot, 0, kb));
+        return launch_ks_finish(c, u, kb.u_limbs, lifted, 1, false, 0, 0, 1, nullptr, 0, 0, nullptr, 0, (u64*)ks0_dev, (u64*)ks1_dev, 0);
     }
     RET(ks_digits_to_lifted(c, c1c, 1, digits, 0, rot, 0, 1, u, lifted));
     RET(launch_moddown_combine(c, u, lifted, 1, rot, 0, nullptr, 0, nullptr, 0, (u64*)ks0_dev, (u64*)ks1_dev, 0));

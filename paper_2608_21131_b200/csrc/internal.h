@@ -54,7 +54,7 @@ struct hann_ctx {
     std::vector<cudaEvent_t> enc_ev;
     int max_lanes = 4;  // at most this many block ranges of hann_rotate_sum run side by side (rings of 2^10 points and more: one or two)
     u64 mod[HANN_MAXL1] = {};  // q_0..q_{L-1}, p
-    bool aux = false;          // key switches take the products modulo p through auxiliary primes
+    bool aux = false;          // key switches may take the products modulo p through auxiliary primes
     AuxCrt crt = {};
     LimbTable lt = {};
     LimbConst* lt_dev = nullptr;  // device copy of lt.c (the transform kernels read it from memory)
@@ -73,10 +73,13 @@ struct hann_ctx {
     unsigned* galois_dev = nullptr;  // [n] 5^r mod 2N
     std::vector<unsigned> h_galois;
     // evaluation keys by rotation: device buffers [L][2][L+1][N], transformed and permuted by the inverse
-    // automorphism so that the key-switch inner product reads keys and digits contiguously; with auxiliary primes followed by
-    // [L][2][3][N], the residues modulo p lifted (centred) to those primes
+    // automorphism so that the key-switch inner product reads keys and digits contiguously
     std::vector<u64*> keytab_host;
     u64** keytab_dev = nullptr;  // [n] device copy of keytab_host
+    // auxiliary words of a key, [L][2][3][N]: the residues modulo p lifted (centred) to the auxiliary primes.  Only rotations that are
+    // multiples of B have them (hann_load_keys); a key switch one of whose keys has none takes p itself
+    std::vector<u64*> keyaux_host;
+    u64** keyaux_dev = nullptr;  // [n] device copy of keyaux_host
     // growable device scratch of the exchange and client calls (never used by the server-side scoring calls)
     void* scratch = nullptr;
     int64_t scratch_bytes = 0;
@@ -257,7 +260,7 @@ int launch_moddown_lift(hann_ctx* c, const u64* u, int64_t npoly, u64* lifted);
 bool ks_fused_available(const hann_ctx* c);
 bool ks_hoist_available(const hann_ctx* c);
 int ks_fused_configure();  // once per context, its device current
-int launch_ks_apply(hann_ctx* c, const u64* digits, const u64* own, int64_t own_it, int64_t own_z, int64_t items, int nz, int rot0, int rot_zinc, u64* u);
+int launch_ks_apply(hann_ctx* c, const u64* digits, const u64* own, int64_t own_it, int64_t own_z, int64_t items, int nz, int rot0, int rot_zinc, bool aux, u64* u);
 int launch_ks_hoist(hann_ctx* c, const u64* digits, const u64* own, int64_t items, int rot0, u64* u);
 int launch_ks_finish(hann_ctx* c, const u64* u, int u_limbs, const u64* lifted, int64_t items, bool perm_items, int rot0, int rot_inc, int nz, const u64* c0,
                      int64_t c0_it, int64_t c0_z, const u64* add, int64_t add_it, u64* out0, u64* out1, int64_t out_it, u64* next = nullptr);

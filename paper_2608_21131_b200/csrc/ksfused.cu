@@ -127,7 +127,7 @@ struct ApplyArgs {
                         // auxiliary primes none for the special prime either
     int nx;             // 1, or the number of auxiliary primes that stand for the special prime
     u64 aux4;           // their limbs in 4-bit fields, behind them the other limbs
-    long long aux_key;  // and the offset of their words in a key
+    const u64* const* keyaux;  // and their words of every key
     const u64* own;     // the polynomials being switched, transform domain: own + item * own_it + z * own_z + j * N (or null)
     long long own_it, own_z;
     const u64* const* keytab;
@@ -194,9 +194,9 @@ __global__ void __launch_bounds__(T, 640 / T) k_ks_apply(ApplyArgs A) {
                            : A.digits + (((z * A.items + it0 + it) * L + dj) * A.n_tgt + (!A.own || i < dj ? i : i - 1)) * N;
         p += (sc << 8);
         if (z) __syncthreads();  // the products of the previous rotation have been taken
-        const u64* key = A.keytab[A.rot0 + z * A.rot_zinc] + (sc << 8);
-        if (SHARE || !aux) stage_keys(ks, key + (long long)i * N, (long long)(L + 1) * N, L);
-        if (aux) stage_keys(ks + ks2, key + A.aux_key + (long long)y * N, (long long)kAux * N, L);
+        const int r = A.rot0 + z * A.rot_zinc;
+        if (SHARE || !aux) stage_keys(ks, A.keytab[r] + (long long)i * N + (sc << 8), (long long)(L + 1) * N, L);
+        if (aux) stage_keys(ks + ks2, A.keyaux[r] + (long long)y * N + (sc << 8), (long long)kAux * N, L);
         if (staged != sc) {
             if (f64) stage_twiddles(tc, (const double2*)A.tw_fwd_f64 + ((size_t)i << A.logN), m0 + sc);
             else stage_twiddles((ulonglong2*)tc, (const ulonglong2*)A.tw_fwd_int + ((size_t)i << A.logN), m0 + sc);
@@ -660,18 +660,18 @@ bool ks_fused_available(const hann_ctx* c) { return c->logN >= 10 && c->ntt_tau;
 bool ks_hoist_available(const hann_ctx* c) { return ks_fused_available(c) && c->L <= 4; }
 
 // digits: output of launch_ks_lift for the nz * items polynomials of L limbs; own (optional): the polynomials themselves, in which
-// case the digits were lifted without their own modulus (and, where the context has auxiliary primes, without the special prime).
+// case the digits were lifted without their own modulus.  aux (only with own): they were lifted without the special prime as well, and
+// every key of the launch has its auxiliary words.
 // Leaves u[item][2][L + nx][N] (see ApplyArgs), the input of the ModDown lift.
-int launch_ks_apply(hann_ctx* c, const u64* digits, const u64* own, int64_t own_it, int64_t own_z, int64_t items, int nz, int rot0, int rot_zinc, u64* u) {
+int launch_ks_apply(hann_ctx* c, const u64* digits, const u64* own, int64_t own_it, int64_t own_z, int64_t items, int nz, int rot0, int rot_zinc, bool aux, u64* u) {
     if (items <= 0 || nz <= 0) return HANN_OK;
     ApplyArgs A = {};
     A.digits = digits;
-    const bool aux = c->aux && own;
     A.nx = aux ? kAux : 1;
     for (int k = 0; k < kAux; k++) A.aux4 |= (u64)c->crt.limb[k] << (4 * k);
     for (int l = 0, k = kAux; aux && l < c->L; l++)
         if (l != c->crt.limb[0] && l != c->crt.limb[1] && l != c->crt.limb[2]) A.aux4 |= (u64)l << (4 * k++);
-    A.aux_key = (long long)c->L * 2 * (c->L + 1) * c->N;
+    A.keyaux = c->keyaux_dev;
     A.n_tgt = aux ? c->L - 1 : own ? c->L : c->L + 1;
     A.own = own;
     A.own_it = own_it;

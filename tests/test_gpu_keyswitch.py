@@ -87,6 +87,57 @@ def test_rotate_sum_through_auxiliary_primes(logN, bits, pbits, nb):
     test_rotate_sum_on_edge_residues(logN, bits, pbits, nb)
 
 
+@pytest.mark.parametrize("L", [3, 4])
+def test_folds_with_and_without_auxiliary_words(L):
+    """the keys of multiples of B have words modulo the auxiliary primes, the others have not: folds of either kind, and one that
+    takes both, to the oracle's bits"""
+    from paper_2608_21131_b200 import binding as b
+
+    logN, R, B = 11, 16, 4
+    q = find_primes(50, logN + 1, L)
+    ps = synth.ParamSet("fold", logN, tuple(q), find_primes(60, logN + 1, 1)[0], 20, R, B, 0)
+    rots = [1, 2, 4, 8]
+    c, o = b.Context(ps), make_oracle(ps)
+    km = synth.key_material(ps, logN, rots=rots)
+    evk = {r: o.evk_gen(km.s, r, km.evk_a[i], km.evk_e[i]) for i, r in enumerate(rots)}
+    c.load_keys(np.stack([evk[r] for r in rots]), rots)
+    ct = edge_residues(9, q, ps.N, (1, 2))
+    for stride, steps in ((1, 2), (4, 2), (1, 4)):
+        want = ct[0]
+        for t in range(steps):
+            rot = o.rotate(want, stride << t, evk[stride << t])
+            want = np.stack([(want[:, i] + rot[:, i]) % np.uint64(q[i]) for i in range(L)], axis=1)
+        dev = c.fold(c.import_(b.KIND_CT, ct, 1), stride, steps, c.workspace(1))
+        assert np.array_equal(c.export(b.KIND_CT, dev, 1)[0], want), (stride, steps)
+
+
+def test_only_giant_step_keys_take_memory_for_auxiliary_words():
+    """loading the keys of the baby steps takes 2 L (L + 1) polynomials each and no more; those of giant steps 6 L more"""
+    import torch
+
+    from paper_2608_21131_b200 import binding as b
+
+    logN, L, R, B = 14, 4, 64, 16
+    q = find_primes(50, logN + 1, L)
+    ps = synth.ParamSet("mem", logN, tuple(q), find_primes(60, logN + 1, 1)[0], 20, R, B, 0)
+    c = b.Context(ps)
+    keys = synth.uniform_residues(3, 2, q + [ps.p], ps.N, lead=(1, L, 2))
+
+    def taken(rots):
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info(c.device)[0]
+        for r in rots:
+            c.load_keys(keys, [r])
+        torch.cuda.synchronize()
+        return before - torch.cuda.mem_get_info(c.device)[0]
+
+    taken([1])  # the exchange scratch
+    key, aux = (2 * L * w * ps.N * 8 for w in (L + 1, 3))
+    page = 2 << 20  # what the device allocates in
+    assert 14 * key <= taken(range(2, 16)) < 14 * (key + page)
+    assert 3 * (key + aux) <= taken([16, 32, 48]) < 3 * (key + aux + 2 * page)
+
+
 def test_lazy_round_of_many_giant_steps():
     """15 blocks x 511 giant steps in one round: 7,665 polynomials of nine limbs, more than one launch covers (65535 / 9).  A large
     workspace only means larger rounds: the same bits as with rounds of one block"""
