@@ -197,12 +197,12 @@ def algorithmic_work(ctx, n_blocks, n_rows):
     }
 
 
-def kernel_work(ctx, ps, n_blocks, n_rows, lazy):
+def kernel_work(ctx, aux, n_blocks, n_rows, lazy):
     """algorithmic_work as the kernels share it out: pass B of the digits runs inside the key products (classes ks_inner and
     ks_inner_keys) and that of the ModDown inside the combination, a digit modulo its own prime is not transformed, the special
     prime's inverse pass B' belongs to the key products, that of every Horner step but the first to the combination before it, with
-    auxiliary primes (three ciphertext primes below 2^50, a larger special prime) the rotate-and-sum's digits have no target modulo
-    the special prime and its ModDown three inverse transforms in place of one, and the FFT of the real slot vectors is half size."""
+    auxiliary primes (aux) the rotate-and-sum's digits have no target modulo the special prime and its ModDown three inverse transforms
+    in place of one, in a class of its own, and the FFT of the real slot vectors is half size."""
     w = algorithmic_work(ctx, n_blocks, n_rows)
     L, N, B, G, R = ctx.L, ctx.N, ctx.B, ctx.G, ctx.R
     n, logN = ctx.n, ctx.logN
@@ -211,16 +211,18 @@ def kernel_work(ctx, ps, n_blocks, n_rows, lazy):
     W = 8 * N
     items = (G - 1) * n_blocks
     moddowns = n_blocks if lazy else items
-    aux = sum(q < 1 << 50 for q in ps.q) >= 3 and 1 << 50 <= ps.p < 1 << 61
     hoist = L <= 4  # longer chains keep pass B of the query's digits and the inverse pass B' of its products as launches of their own
     pt_polys, digits = n_blocks * R * L, 0 if hoist else L * (L + 1)
     inv_polys = L + (0 if hoist else (B - 1) * 2) + (items if lazy else n_blocks) * L
     lift = [(L, L if hoist else L + 1), ((B - 1) * 2, L), (items * L, L - 1 if aux else L)]
-    moddown_ops = moddowns * 2 * ((3 if aux else 1) + L) * a * (N // 2) * 8
+    if aux:
+        w["moddown_lift"] = ("alu", moddowns * 2 * (3 + L) * a * (N // 2) * 8, moddowns * 2)
+    else:
+        lift.append((moddowns * 2, L))
     pass_a_half = (N // 2) * 7 + (a - 1) * (N // 4) * 8
     w["ntt_fwd_b"] = ("alu", (pt_polys * (N // 4) + digits * (N // 2)) * b * 8, pt_polys + digits)
     w["ntt_inv_b"] = ("alu", inv_polys * (N // 2) * b * 8, inv_polys)
-    w["lift_digits"] = ("alu", sum(src * (1 + tgt) * a * (N // 2) * 8 for src, tgt in lift) + moddown_ops, sum(src for src, _ in lift) + moddowns * 2)
+    w["lift_digits"] = ("alu", sum(src * (1 + tgt) * a * (N // 2) * 8 for src, tgt in lift), sum(src for src, _ in lift))
     extra = 2 if aux else 0  # limbs of the key and of the products beyond L + 1
     w["ks_inner"] = ("hbm", (G - 1) * L * 2 * (L + 1 + extra) * W + items * (L * L + L - (L if aux else 0)) * W + moddowns * 2 * (L + 1 + extra) * W, items)
     w["fft_a"] = ("hbm", n_blocks * R * (n * 8) + n_rows * R * 4, n_blocks * R)
@@ -399,7 +401,8 @@ def run_ours(args):
     # arithmetic ceilings measured on this device by the library's own probe kernels: register-resident binary64 modular
     # butterflies (no memory traffic) and 32 x 32 -> 64 multiply-adds
     bfly_peak, madd_peak = ctx.probe_rates()
-    work = kernel_work(ctx, ps, nb, n_rows, args.giant != "horner")
+    # (rings of 2^10 points and more launch a ModDown lift of its own only for auxiliary primes)
+    work = kernel_work(ctx, ctx.logN >= 10 and "moddown_lift" in kernels, nb, n_rows, args.giant != "horner")
     dom = max((k for k in kernels if k in work), key=lambda k: kernels[k]["ms_per_step"])
     bound, amount, units = work[dom]
     dom_s = kernels[dom]["ms_per_step"] * 1e-3

@@ -1309,7 +1309,7 @@ int launch_ks_lift_aux(hann_ctx* c, const u64* src, int64_t src_stride, int64_t 
         LiftArgs A = lift_args(c, src_stride, c->L);
         A.src = src + s0 * src_stride;
         A.dst = dst + s0 * c->L * (int64_t)c->N;
-        KProf kp(c, KC_LIFT_DIGITS);
+        KProf kp(c, KC_MODDOWN_LIFT);  // a class of its own: the profile shows which key switches take auxiliary primes
         launch_chain(c, pick_lift_aux(a), dim3(tiles, ns, lift_zsplit((long)tiles * ns, (c->L + 3) / 4, 2, 148)), 4 * kLiftThreads, lift_aux_smem(R1, R2), A, c->crt, c->L);
     }
     return check_launch(c, "ks_lift_aux");

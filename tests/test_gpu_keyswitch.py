@@ -87,6 +87,56 @@ def test_rotate_sum_through_auxiliary_primes(logN, bits, pbits, nb):
     test_rotate_sum_on_edge_residues(logN, bits, pbits, nb)
 
 
+def takes_auxiliary_primes(c, call):
+    """whether the ModDown of the call's key switches went through auxiliary primes: it is a launch class of its own"""
+    c.kernel_profile(True)
+    call()
+    c.sync()
+    launches = c.kernel_times()["moddown_lift"][1]
+    c.kernel_profile(False)
+    return launches > 0
+
+
+@pytest.mark.parametrize(
+    "logN,bits,pbits,taken",
+    [
+        (10, (50,) * 3, 60, True),
+        (11, (45,) * 5, 60, True),
+        (12, (50, 50, 50, 40), 60, True),      # the three largest are what counts
+        (10, (58, 45, 45, 45), 61, True),
+        (10, (50,) * 4, 51, True),
+        (10, (50,) * 4, 50, False),            # a special prime that the FP64 pipe transforms itself
+        (10, (50,) * 4, 62, False),            # and one above what the recombination holds
+        (10, (50, 50), 60, False),
+        (10, (50, 50, 58), 60, False),         # too few primes below 2^50
+        (10, (50, 50, 46), 60, False),         # too different in size
+        (10, (37,) * 9, 60, False),            # the products do not stay below a quarter of three primes
+    ],
+)
+def test_which_chains_take_auxiliary_primes(logN, bits, pbits, taken):
+    import torch
+
+    from paper_2608_21131_b200 import binding as b
+
+    q = []
+    for w in bits:
+        q.append(next(x for x in find_primes(w, logN + 1, len(bits)) if x not in q))
+    ps = synth.ParamSet("rule", logN, tuple(q), next(x for x in find_primes(pbits, logN + 1, len(bits) + 1) if x not in q), 20, 16, 4, 0)
+    c = b.Context(ps)
+    rots = [1, 2, 3, 4, 8, 12]
+    c.load_keys(synth.uniform_residues(3, 2, q + [ps.p], ps.N, lead=(len(rots), ps.L, 2)), rots)
+    ws = c.workspace(1)
+    inner = torch.randint(0, min(q), (c.sizeof(b.SIZE_INNER) // 8,), dtype=torch.int64, device=c.device)
+    ct = inner[: 2 * ps.L * ps.N].clone()
+    assert takes_auxiliary_primes(c, lambda: c.rotate_sum(inner, 1, ws)) == taken
+    assert takes_auxiliary_primes(c, lambda: c.rotate_sum_lazy(inner, 1, ws)) == taken
+    assert takes_auxiliary_primes(c, lambda: c.fold(ct, 4, 2, ws)) == taken
+    # keys without the words: hoisted rotations, a fold by other strides, one that takes both kinds
+    assert not takes_auxiliary_primes(c, lambda: c.query_prepare(ct, ws))
+    assert not takes_auxiliary_primes(c, lambda: c.fold(ct, 1, 2, ws))
+    assert not takes_auxiliary_primes(c, lambda: c.fold(ct, 2, 2, ws))
+
+
 @pytest.mark.parametrize("L", [3, 4])
 def test_folds_with_and_without_auxiliary_words(L):
     """the keys of multiples of B have words modulo the auxiliary primes, the others have not: folds of either kind, and one that
