@@ -30,9 +30,9 @@
  *     memory of the context: allocated at the first call that needs it, grown when a later one needs more, kept until
  *     hann_ctx_destroy, never used by the server-side calls.  Its size is that of the largest call so far: 64 polynomials of L
  *     limbs for hann_import (kind PT) and hann_export, (2 L + 1)(L + 1) polynomials of one limb for key generation, 2 L (L + 1)
- *     for hann_load_keys, at most 64 MiB (and no less than one ciphertext) for decryption.  Encryption and decryption also keep 4 MiB
- *     of page-locked host memory of the context from the first copy of 1 MiB and more on, and fill it from up to three helper threads
- *     that end with the call.
+ *     for hann_load_keys, at most 64 MiB (and no less than one ciphertext) for decryption.  Decryption also keeps 2 MiB of
+ *     page-locked host memory of the context from the first piece (up to eight ciphertexts) of 16 MiB and more on, and fills it with
+ *     the help of a thread that ends with the call.
  *   - Canonical exchange layout (the only layout with a meaning outside the library): coefficient
  *     domain, natural coefficient order, residues in [0, q_i), uint64, index order [poly][limb][coeff];
  *     a ciphertext is 2 polynomials (c0, c1) of L limbs.  The internal device layout (transform domain,

@@ -1084,18 +1084,17 @@ extern "C" int hann_encrypt_query(hann_ctx* c, const int8_t* s, const float* q, 
     std::vector<double> zh(n, 0.0);
     for (int i = 0; i < n; i += c->R)
         for (int d = 0; d < dim; d++) zh[i + d] = (double)q[d];
-    const HostCopy in[4] = {{A, (void*)a, LN * 8, nullptr}, {z, zh.data(), (int64_t)n * 8, nullptr}, {e8, (void*)e, N, nullptr}, {s8, (void*)s, N, nullptr}};
-    RET(host_copy(c, in, 4, true, c->stream));
-    RET(launch_lift_i8(c, s8, L, shat));
-    RET(launch_ntt_fwd(c, shat, L, N, limbmap_q(c)));
+    CK(cudaMemcpyAsync(z, zh.data(), n * 8, cudaMemcpyHostToDevice, c->stream));
+    CK(cudaMemcpyAsync(A, a, LN * 8, cudaMemcpyHostToDevice, c->stream));
+    CK(cudaMemcpyAsync(e8, e, N, cudaMemcpyHostToDevice, c->stream));
+    RET(upload_secret(c, s, L, s8, shat));
     RET(launch_encode_slots(c, z, M, fbuf));
     RET(launch_ntt_fwd(c, A, L, N, limbmap_q(c)));
     RET(launch_mul(c, A, shat, L, AS, L, limbmap_q(c)));
     RET(launch_ntt_inv(c, AS, L, N, limbmap_q(c)));
     RET(launch_encrypt_finish(c, AS, e8, M, AS));
-    // the uniform half is copied on the host while the device works
-    const HostCopy out[2] = {{nullptr, ct_out + LN, LN * 8, a}, {AS, ct_out, LN * 8, nullptr}};
-    RET(host_copy(c, out, 2, false, c->stream));
+    memcpy(ct_out + LN, a, LN * 8);  // on the host while the device works
+    CK(cudaMemcpyAsync(ct_out, AS, LN * 8, cudaMemcpyDeviceToHost, c->stream));
     return sync_and_check(c);
 }
 
@@ -1124,32 +1123,21 @@ static int decrypt_impl(hann_ctx* c, const int8_t* s, const uint64_t* ct, int64_
     CK(cudaMemcpyAsync(s8, s, N, cudaMemcpyHostToDevice, c->stream));
     RET(launch_lift_i8(c, s8, nl, shat));
     RET(launch_ntt_fwd(c, shat, nl, N, lm));
-    // the kernels of a piece's first half run while its second half is uploaded
-    CK(cudaEventRecord(c->ev_fork, c->stream));
-    CK(cudaStreamWaitEvent(c->up_stream, c->ev_fork, 0));
     for (int64_t i0 = 0; i0 < count; i0 += piece) {
-        const int64_t np = std::min(piece, count - i0), half = (np + 1) / 2;
-        for (int64_t h0 = 0; h0 < np; h0 += half) {
-            const int64_t nh = std::min(half, np - h0);
-            HostCopy in[8];  // a piece is at most eight ciphertexts
-            for (int64_t i = 0; i < nh; i++) {
-                const uint64_t* src = ct + (i0 + h0 + i) * 2 * LN;
-                in[2 * i] = HostCopy{C1 + (h0 + i) * LN, (void*)(src + LN), LN * 8, nullptr};
-                in[2 * i + 1] = HostCopy{C0 + (h0 + i) * LN, (void*)src, LN * 8, nullptr};
-            }
-            const int rc = host_copy(c, in, 2 * (int)nh, true, c->up_stream);
-            // (also after a failure: nothing of this call runs on the upload stream past the context's stream)
-            CK(cudaEventRecord(c->ev_join, c->up_stream));
-            CK(cudaStreamWaitEvent(c->stream, c->ev_join, 0));
-            RET(rc);
-            u64 *c0 = C0 + h0 * LN, *c1 = C1 + h0 * LN;
-            RET(launch_ntt_fwd(c, c1, nh * nl, N, lm));
-            RET(launch_mul(c, c1, shat, nl, c1, nh * nl, lm));  // c1 * s; c0 is added in the coefficient domain
-            RET(launch_ntt_inv(c, c1, nh * nl, N, lm));
-            RET(launch_decode(c, c0, c1, nh, nl, mult, exp2, buf + h0 * n, re + h0 * n, imag_or_null ? im + h0 * n : nullptr));
+        const int64_t np = std::min(piece, count - i0);
+        HostCopy in[16];  // a piece is at most eight ciphertexts
+        for (int64_t i = 0; i < np; i++) {
+            const uint64_t* src = ct + (i0 + i) * 2 * LN;
+            in[2 * i] = HostCopy{C1 + i * LN, src + LN, LN * 8};
+            in[2 * i + 1] = HostCopy{C0 + i * LN, src, LN * 8};
         }
-        const HostCopy out[2] = {{re, scores + i0 * n, np * n * 8, nullptr}, {im, imag_or_null ? imag_or_null + i0 * n : nullptr, np * n * 8, nullptr}};
-        RET(host_copy(c, out, imag_or_null ? 2 : 1, false, c->stream));
+        RET(host_upload(c, in, 2 * (int)np, c->stream));
+        RET(launch_ntt_fwd(c, C1, np * nl, N, lm));
+        RET(launch_mul(c, C1, shat, nl, C1, np * nl, lm));  // c1 * s; c0 is added in the coefficient domain
+        RET(launch_ntt_inv(c, C1, np * nl, N, lm));
+        RET(launch_decode(c, C0, C1, np, nl, mult, exp2, buf, re, imag_or_null ? im : nullptr));
+        CK(cudaMemcpyAsync(scores + i0 * n, re, (size_t)np * n * 8, cudaMemcpyDeviceToHost, c->stream));
+        if (imag_or_null) CK(cudaMemcpyAsync(imag_or_null + i0 * n, im, (size_t)np * n * 8, cudaMemcpyDeviceToHost, c->stream));
         RET(sync_and_check(c));
     }
     return HANN_OK;

@@ -83,9 +83,9 @@ struct hann_ctx {
     // growable device scratch of the exchange and client calls (never used by the server-side scoring calls)
     void* scratch = nullptr;
     int64_t scratch_bytes = 0;
-    // page-locked slots of the client calls' host copies (hostcopy.cpp): 4 MiB from the first large copy on, until the context goes
+    // page-locked slots of a decryption's uploads (hostcopy.cpp): 2 MiB from the first large one on, until the context goes
     void* pin = nullptr;
-    cudaEvent_t pin_ev[8] = {};
+    cudaEvent_t pin_ev[4] = {};
     // plaintexts encoded and transformed per launch group: small enough that the group's intermediates stay in L2
     int encode_group = 1 << 20;
     int host_limbs = 0;  // limbs of every score polynomial that hann_score_level_host downloads (L: all)
@@ -178,15 +178,14 @@ void seeded_ternary(u64 seed, u64 stream, int N, int8_t* s);                    
 void seeded_gaussian(u64 seed, u64 stream, u64 ctr0, long count, double sigma, int8_t* e);  // rounded Gaussian (Box-Muller)
 }  // namespace hm
 
-// hostcopy.cpp: `up` host -> dev, otherwise dev -> host (or, with `from`, host <- from), behind what `stream` holds.  Returns when the
-// host memory has been read or written; from or to page-locked or device memory when the copies are enqueued.
+// hostcopy.cpp: host -> dev behind what `stream` holds.  Returns when the host memory has been read; from page-locked or device memory
+// when the copies are enqueued.
 struct HostCopy {
     void* dev;
-    void* host;
+    const void* host;
     int64_t bytes;
-    const void* from;
 };
-int host_copy(hann_ctx* c, const HostCopy* list, int n, bool up, cudaStream_t stream);
+int host_upload(hann_ctx* c, const HostCopy* list, int n, cudaStream_t stream);
 void host_copy_release(hann_ctx* c);
 
 // bytes of workspace one hann_keyswitch carves (api.cu); device address of the built-in scratch (static_scratch.cu)
