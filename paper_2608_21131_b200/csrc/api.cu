@@ -310,8 +310,18 @@ int64_t keyswitch_ws_bytes(const hann_ctx* c) {
 // with a special prime in [2^50, 2^61) (a smaller one has transforms on the FP64 pipe itself), if every sum of key products a call
 // takes before its ModDown -- up to G - 1 rotations of L digits, |digit| < q_j / 2, |key| < p / 2 -- stays below a quarter of their
 // product.
+//
+// They save integer transforms and cost k_ks_apply three CTAs a chunk that transform the L digits again, except where four items of up to
+// four primes share the transforms.  On longer chains that pays while a launch leaves the machine room, up to L N = 2^17 words a
+// polynomial.  us of the launches of a Horner call with three giant steps on k blocks, through p / through auxiliary primes:
+//   L = 3, N = 2^15: k = 1 196 / 177, 8 346 / 334       L = 4, N = 2^15: k = 1 194 / 190, 8 424 / 415
+//   L = 5, N = 2^14: k = 1 188 / 178, 8 363 / 339       L = 8, N = 2^14: k = 1 211 / 204, 4 337 / 330, 8 535 / 529
+//   L = 5, N = 2^15: k = 1 214 / 209, 5 430 / 464, 8 551 / 562       L = 7, N = 2^15: k = 1 235 / 242, 8 831 / 864
+//   L = 12, N = 2^13: k = 1 218 / 206, 8 575 / 575      L = 12, N = 2^14: k = 1 266 / 269, 5 709 / 731
+//   L = 12, N = 2^15: k = 1 392 / 404, 8 1905 / 1932    L = 5, N = 2^16: k = 1 293 / 288, 8 970 / 1025
 static void choose_aux(hann_ctx* c) {
     if (!ks_fused_available(c) || c->mod[c->L] < (1ULL << 50) || c->mod[c->L] >= (1ULL << 61)) return;
+    if (c->L > 4 && (int64_t)c->L * c->N > (1 << 17)) return;
     std::vector<int> small;
     for (int i = 0; i < c->L; i++)
         if (c->mod[i] < (1ULL << 50)) small.push_back(i);

@@ -81,6 +81,8 @@ def test_rotate_sum_on_edge_residues(logN, bits, pbits, nb):
         (10, (50, 50, 48), 60, 2),         # primes of too different size, and too few of them: the special prime itself
         (10, (50, 50, 58), 60, 2),
         (14, (50,) * 4, 60, 1),            # second lift round of two stages
+        (14, (45,) * 8, 60, 1),            # the longest chain of that ring, and one that takes the special prime itself
+        (14, (45,) * 9, 60, 1),
     ],
 )
 def test_rotate_sum_through_auxiliary_primes(logN, bits, pbits, nb):
@@ -110,6 +112,10 @@ def takes_auxiliary_primes(c, call):
         (10, (50, 50), 60, False),
         (10, (50, 50, 58), 60, False),         # too few primes below 2^50
         (10, (50, 50, 46), 60, False),         # too different in size
+        (14, (45,) * 8, 60, True),             # 2^17 words a polynomial
+        (14, (45,) * 9, 60, False),            # and more, on a chain of more than four primes
+        (15, (45,) * 5, 60, False),
+        (16, (45,) * 4, 60, True),
         (10, (37,) * 9, 60, False),            # the products do not stay below a quarter of three primes
     ],
 )
