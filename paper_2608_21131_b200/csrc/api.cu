@@ -328,7 +328,10 @@ static void choose_aux(hann_ctx* c) {
     if (small.size() < kAux) return;
     std::stable_sort(small.begin(), small.end(), [&](int a, int b) { return c->mod[a] > c->mod[b]; });
     const u64 qa = c->mod[small[0]], qb = c->mod[small[1]], qc = c->mod[small[2]], p = c->mod[c->L];
-    if (qa / 2 >= qc) return;  // the digits of the recombination stay below four times the modulus they meet
+    // The digits of the recombination (k_ks_lift_aux) stay below four times the modulus they meet: the differences of two balanced residues
+    // below (q_a + q_c) / 2 <= 3.5 q_c, a product's remainder (0.75 q_c with its rounded quotient) and v1 below 0.75 q_c + q_b / 2 <= 3.75 q_c.
+    // (A bound between powers of two: primes of neighbouring sizes fall on one side of it whatever their distance from the power.)
+    if (qa / 6 >= qc) return;
     double digits = 0;
     for (int i = 0; i < c->L; i++) digits += (double)c->mod[i] / 2;
     const double terms = (double)c->N * std::max(c->G - 1, 1);

@@ -78,7 +78,9 @@ def test_rotate_sum_on_edge_residues(logN, bits, pbits, nb):
         (12, (50, 50, 50, 40), 60, 2),     # a ciphertext prime far below the auxiliary ones
         (10, (50,) * 4, 61, 2),            # the largest special prime they stand for
         (10, (50,) * 4, 51, 5),            # and the smallest
-        (10, (50, 50, 48), 60, 2),         # primes of too different size, and too few of them: the special prime itself
+        (10, (50, 50, 48), 60, 2),         # the smallest a quarter of the others
+        (10, (50, 50, 47), 60, 2),         # primes of too different size, and too few of them: the special prime itself
+        (11, (58, 45, 46, 46, 45), 60, 1),  # neighbouring sizes, whichever lies closer to its power of two
         (10, (50, 50, 58), 60, 2),
         (14, (50,) * 4, 60, 1),            # second lift round of two stages
         (14, (45,) * 8, 60, 1),            # the longest chain of that ring, and one that takes the special prime itself
@@ -111,7 +113,9 @@ def takes_auxiliary_primes(c, call):
         (10, (50,) * 4, 62, False),            # and one above what the recombination holds
         (10, (50, 50), 60, False),
         (10, (50, 50, 58), 60, False),         # too few primes below 2^50
-        (10, (50, 50, 46), 60, False),         # too different in size
+        (10, (50, 50, 48), 60, True),          # a quarter of the others
+        (10, (50, 50, 47), 60, False),         # an eighth: too different in size
+        (15, (58, 46, 45, 46), 60, True),      # the short chains of the membership circuit
         (14, (45,) * 8, 60, True),             # 2^17 words a polynomial
         (14, (45,) * 9, 60, False),            # and more, on a chain of more than four primes
         (15, (45,) * 5, 60, False),
