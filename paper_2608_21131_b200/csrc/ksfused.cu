@@ -699,11 +699,17 @@ int launch_ks_apply(hann_ctx* c, const u64* digits, const u64* own, int64_t own_
     //   N = 2^15, L = 4, one rotation:    1 item 18 / 19 / 22, 2: 23 / 21 / 23, 4: 43 / 33 / 28, 8: 77 / 57 / 51, 16: 140 / 105 / 96
     //   N = 2^12, L = 2, seven rotations: 1 item 78 / 68 / 62, 16: 86 / 88 / 83
     //   N = 2^15, L = 8, one rotation:    1 item 24 / 32, 2: 45 / 42, 3: 64 / 70, 4: 82 / 77, 16: 292 / 281
-    // (Taken with the special prime itself; with auxiliary primes four items share the transforms of both key sets, which moved a launch of
-    // four items and three rotations from 166 to 118 us.)  Without them four lose to two where they leave half of the last CTA empty
-    // (five and six items of four primes: 86 against 70 us).
-    if (items >= 4 && c->L <= 4 && aux) launch_apply<4, 256, true>(c, A);
-    else if (items >= 4 && c->L <= 4) launch_apply<4, 256>(c, A);
+    // (taken with the special prime itself).  Four items of five or six leave most of the last CTA empty.  Us of the launches of a call with
+    // three giant steps, two / four items per CTA (aux: with auxiliary primes, whose key set four items take from the same transforms):
+    //   N = 2^16, L = 4, aux:  Horner, 4 blocks 456 / 441, 5 566 / 572, 6 607 / 606, 8 758 / 713   lazy, 4 273 / 251, 5 348 / 348
+    //             without:     Horner, 4 blocks 460 / 472, 5 552 / 602, 6 604 / 643, 8 747 / 750   lazy, 5 352 / 392
+    //   N = 2^15, L = 4, aux:  Horner, 5 345 / 347, 6 358 / 357      without: 5 338 / 350, 6 350 / 362, 7 422 / 412
+    //   N = 2^16, L = 3, aux:  Horner, 4 351 / 347, 5 471 / 493, 6 491 / 508     without: 5 469 / 508, 6 489 / 523, 7 552 / 566
+    //   N = 2^15, L = 3, aux:  Horner, 5 288 / 295, 6 301 / 309      without: 5 294 / 301, 6 309 / 312, 7 352 / 340
+    //   N = 2^16, L = 2:       Horner, 5 364 / 353, 6 368 / 360      N = 2^15, L = 2: 5 232 / 226, 6 234 / 232
+    const bool ragged = (items == 5 || items == 6) && (c->L == 3 || (c->L == 4 && !aux));
+    if (items >= 4 && !ragged && c->L <= 4 && aux) launch_apply<4, 256, true>(c, A);
+    else if (items >= 4 && !ragged && c->L <= 4) launch_apply<4, 256>(c, A);
     else if (items >= 2 && c->L <= 4) launch_apply<2, 128>(c, A);
     else if (items >= 2 && c->L <= 8) launch_apply<2, 256>(c, A);
     else if (c->L <= 4) launch_apply<1, 64>(c, A);

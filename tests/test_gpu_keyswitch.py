@@ -31,6 +31,11 @@ def edge_residues(seed, q, N, lead):
         (10, (45,) * 9, 60, 2),                 # more than eight digits: two exact sums per position
         (13, (50,) * 4, 60, 1),
         (15, (50, 50), 60, 2),                  # second lift round of three stages
+        (10, (50,) * 3, 62, 5),                 # five and six items go two per CTA, four and seven four
+        (10, (50,) * 4, 62, 6),
+        (10, (50,) * 4, 62, 7),
+        (10, (50,) * 3, 60, 6),                 # (with auxiliary primes)
+        (10, (50,) * 3, 60, 4),
     ],
 )
 def test_rotate_sum_on_edge_residues(logN, bits, pbits, nb):
