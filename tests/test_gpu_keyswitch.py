@@ -96,6 +96,37 @@ def test_rotate_sum_through_auxiliary_primes(logN, bits, pbits, nb):
     test_rotate_sum_on_edge_residues(logN, bits, pbits, nb)
 
 
+@pytest.mark.parametrize("logN,bits", [(10, (50,)), (12, (50, 40)), (11, (50, 58, 45)), (12, (50,) * 4), (13, (50,) * 4), (11, (45,) * 5)])
+def test_hoisted_rotations_of_an_unaligned_ciphertext(logN, bits):
+    """a ciphertext that is only 8-byte aligned is copied before its inverse transform: the oracle's bits from either"""
+    import torch
+
+    from paper_2608_21131_b200 import binding as b
+
+    q = []
+    for w in bits:
+        q.append(next(x for x in find_primes(w, logN + 1, len(bits)) if x not in q))
+    ps = synth.ParamSet("odd", logN, tuple(q), find_primes(60, logN + 1, 1)[0], 20, 16, 4, 0)
+    rots = [1, 2, 3]
+    c, o = b.Context(ps), make_oracle(ps)
+    km = synth.key_material(ps, logN, rots=rots)
+    evk = {r: o.evk_gen(km.s, r, km.evk_a[i], km.evk_e[i]) for i, r in enumerate(rots)}
+    c.load_keys(np.stack([evk[r] for r in rots]), rots)
+    ct = edge_residues(5, q, ps.N, (1, 2))
+    dev = c.import_(b.KIND_CT, ct, 1)
+    odd = c.alloc(dev.numel() * 8 + 8)[1:]
+    odd.copy_(dev)
+    ws = c.workspace(1)
+    for src in (dev, odd):
+        baby = c.export(b.KIND_CT, c.query_prepare(src, ws), 4)
+        hoisted = c.export(b.KIND_CT, c.rotate_hoisted(src, 2, 2, ws), 2)
+        for r in rots:
+            want = o.rotate(ct[0], r, evk[r])
+            assert np.array_equal(baby[r], want), r
+            assert r == 1 or np.array_equal(hoisted[r - 2], want), r
+    torch.cuda.synchronize()
+
+
 def takes_auxiliary_primes(c, call):
     """whether the ModDown of the call's key switches went through auxiliary primes: it is a launch class of its own"""
     c.kernel_profile(True)
