@@ -23,7 +23,7 @@ struct AuxCrt {
     signed char limb[4];  // a, b, c
     double2 ab, ac, bc;   // q_a^{-1} mod q_b, q_a^{-1} mod q_c, q_b^{-1} mod q_c as (balanced, fl(. / modulus))
     u64 c1, c1s, c2, c2s;  // q_a and q_a q_b modulo p with their Shoup companions
-    u64 off;               // -2^50 (c1 + c2) modulo p, in [p, 2p)
+    u64 off;               // -2^50 (c1 + c2) modulo p, in (p, 2p]
 };
 constexpr int kAux = 3;
 

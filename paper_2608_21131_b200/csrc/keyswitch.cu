@@ -101,12 +101,13 @@ __global__ void __launch_bounds__(kThreads) k_ks_inner(const u64* digits, long l
     }
 }
 
-// Streaming form of the same inner product for L <= 4 digits.  A thread owns one position (modulus i, coefficient x)
-// and loops over the items.  When the items share one digit set and differ by key (the hoisted baby rotations:
-// KEYS_STREAM), the L digit words stay in registers and the 2L key words of each item stream past them; when the
-// items share the key (rotate-and-sum over blocks), the key words stay and the digit words stream.  The streamed
-// words of the next item are in flight while the current item is multiplied.  Rings of 2^10 points and more use the first
-// form alone: there the second one's work, and the sum over the giant steps, is k_ks_apply's (ksfused.cu).
+// Streaming form of the same inner product for L <= 4 digits, on rings of 2^7 to 2^9 points (larger ones: k_ks_hoist and k_ks_apply in
+// ksfused.cu).  A thread owns one position (modulus i, coefficient x) and loops over the items.  When the items share one digit set
+// and differ by key (the hoisted baby rotations: KEYS_STREAM), the L digit words stay in registers and the 2L key words of each item
+// stream past them; when the items share the key (rotate-and-sum over blocks), the key words stay and the digit words stream.  The
+// streamed words of the next item are in flight while the current item is multiplied.  Bound there by the launches: us of a call with
+// k_ks_inner / with it, L = 2, seven giant steps, N = 2^9: lazy order, whose steps are one launch, 1 block 77 / 61, 32 1734 / 1337;
+// Horner, 32 blocks 1435 / 1412; seven hoisted rotations 46 / 45.
 // MODE 0: moduli below 2^50, 25-bit halves, Karatsuba (3 products); MODE 1: moduli below 2^60 (the special prime),
 // 30-bit halves, 4 products (sums of 2 LL <= 8 products of 60 bits fit 64 bits); MODE 2: anything else, 128-bit
 // accumulation; MODE 3 (default): moduli below 2^50, exact two-word sums on the FP64 pipe.
@@ -696,8 +697,7 @@ void launch_ks_inner_stream(hann_ctx* c, const u64* digits, int64_t digit_stride
                             int nz = 1, int rot_zinc = 0) {
     const long long L1N = (long long)(LL + 1) * c->N;
     const int tiles = (int)(L1N / 128);
-    // CTAs that share out the items of a tile: smallest (waves x items of a CTA), ties to fewer.  72 registers: seven CTAs per SM; a
-    // CTA of 31 keys takes long enough for an almost empty third wave to cost a sixth of the launch (155 -> 148 us, at N = 2^15 91 -> 76).
+    // CTAs that share out the items of a tile: smallest (waves x items of a CTA), ties to fewer.  72 registers: seven CTAs per SM
     const long long slots = 148 * 7;
     int per = (int)nitems;
     long long best = -1;
@@ -729,7 +729,8 @@ int launch_ks_inner(hann_ctx* c, const u64* digits, int64_t digit_stride, int ro
     }
     {
         KProf kp(c, KC_KS_INNER);
-        launch_chain(c, k_ks_inner, dim3(grid_for(nitems * (c->L + 1) * c->N)), kThreads, 0, digits, digit_stride, c->keytab_dev, rot0, rot_inc, u, c->N, c->L, nitems, c->lt, c->mac_f64);
+        launch_chain(c, k_ks_inner, dim3(grid_for(nitems * (c->L + 1) * c->N)), kThreads, 0, digits, digit_stride, c->keytab_dev, rot0, rot_inc, u,
+                     c->N, c->L, nitems, c->lt, c->mac_f64);
     }
     return check_launch(c, "ks_inner");
 }

@@ -154,7 +154,7 @@ struct ApplyArgs {
 //
 // SHARE (with auxiliary primes): the CTA of an auxiliary prime takes the products with the key modulo that prime as well, instead of a
 // CTA of their own that transforms the same digits again; both key sets and sums then wait in shared memory.  At four items per CTA that
-// is 100 KiB, two CTAs per SM as without: 31 blocks of three rotations 1163 -> 840 us.  At one and two items it leaves three
+// is 104 KiB, two CTAs per SM as without: 31 blocks of three rotations 1163 -> 840 us.  At one and two items it leaves three
 // CTAs in place of five and lost (95 -> 108 us for two).
 template <int IB, int T, bool SHARE>
 __global__ void __launch_bounds__(T, 640 / T) k_ks_apply(ApplyArgs A) {
@@ -471,8 +471,8 @@ struct FinishArgs {
     const LimbConst* lt;
 };
 
-// out[item][c][i] = (u - lifted) d^{-1} + add + phi(c0), d the special prime or the chain's last, modulus i = blockIdx.y, chunk blockIdx.x, a half-warp per (item, component):
-// pass B of the lifted ModDown polynomials with the combination behind its last round.
+// out[item][c][i] = (u - lifted) d^{-1} + add + phi(c0), d the special prime or the chain's last, modulus i = blockIdx.y, chunk
+// blockIdx.x, a half-warp per (item, component): pass B of the lifted ModDown polynomials with the combination behind its last round.
 // PERM: u, lifted and c0 are still in the order before the automorphism, which differs from item to item (hoisted rotations); the
 // finished words are permuted in shared memory and stored to the item's own chunk of the result.
 // NEXT: the result's second component is what the next key switch decomposes, and the half-warp that made a chunk of it runs the
@@ -621,7 +621,8 @@ int run_finish(hann_ctx* c, FinishArgs& A, bool perm_items) {
     long long gz = (2 * 148 * 3 + per - 1) / per;
     if (gz > groups) gz = groups;
     KProf kp(c, KC_MODDOWN_COMBINE);
-    launch_chain(c, perm_items ? k_ks_finish<true, false> : A.next ? k_ks_finish<false, true> : k_ks_finish<false, false>, dim3(c->N >> 8, A.limbs, (unsigned)gz), threads, smem, A);
+    const auto kern = perm_items ? k_ks_finish<true, false> : A.next ? k_ks_finish<false, true> : k_ks_finish<false, false>;
+    launch_chain(c, kern, dim3(c->N >> 8, A.limbs, (unsigned)gz), threads, smem, A);
     return check_launch(c, "ks_finish");
 }
 
@@ -759,11 +760,12 @@ int launch_ks_hoist(hann_ctx* c, const u64* digits, const u64* own, int64_t item
     return check_launch(c, "ks_hoist");
 }
 
-// lifted: output of launch_ks_lift (launch_ks_lift_aux) for the special-prime (auxiliary) limbs of u, whose polynomials have u_limbs limbs.  perm_items: the automorphism is still to be applied, that of
-// item `it` being rotation rot0 + it * rot_inc (otherwise rotation rot0 + z * rot_inc belongs to the c0 term z < nz).  next (optional, not
-// with perm_items): the second components after their inverse pass B', [item][L][N], for a key switch that follows.
-int launch_ks_finish(hann_ctx* c, const u64* u, int u_limbs, const u64* lifted, int64_t items, bool perm_items, int rot0, int rot_inc, int nz, const u64* c0,
-                     int64_t c0_it, int64_t c0_z, const u64* add, int64_t add_it, u64* out0, u64* out1, int64_t out_it, u64* next) {
+// lifted: output of launch_ks_lift (launch_ks_lift_aux) for the special-prime (auxiliary) limbs of u, whose polynomials have u_limbs
+// limbs.  perm_items: the automorphism is still to be applied, that of item `it` being rotation rot0 + it * rot_inc (otherwise rotation
+// rot0 + z * rot_inc belongs to the c0 term z < nz).  next (optional, not with perm_items): the second components after their inverse
+// pass B', [item][L][N], for a key switch that follows.
+int launch_ks_finish(hann_ctx* c, const u64* u, int u_limbs, const u64* lifted, int64_t items, bool perm_items, int rot0, int rot_inc, int nz,
+                     const u64* c0, int64_t c0_it, int64_t c0_z, const u64* add, int64_t add_it, u64* out0, u64* out1, int64_t out_it, u64* next) {
     if (items <= 0) return HANN_OK;
     FinishArgs A = {};
     A.lifted = lifted;

@@ -918,8 +918,7 @@ __global__ void __launch_bounds__(4 * kLiftThreads, 1) k_ks_lift_aux(LiftArgs A,
 typedef void (*KernLiftAux)(LiftArgs, AuxCrt, int);
 KernLiftAux pick_lift_aux(int a) {
     switch (a) {
-        case 1: return k_ks_lift_aux<1, 0>;
-        case 2: return k_ks_lift_aux<2, 0>;
+        case 2: return k_ks_lift_aux<2, 0>;  // rings of 2^10 points and more
         case 3: return k_ks_lift_aux<3, 0>;
         case 4: return k_ks_lift_aux<4, 0>;
         case 5: return k_ks_lift_aux<4, 1>;
@@ -1310,7 +1309,8 @@ int launch_ks_lift_aux(hann_ctx* c, const u64* src, int64_t src_stride, int64_t 
         A.src = src + s0 * src_stride;
         A.dst = dst + s0 * c->L * (int64_t)c->N;
         KProf kp(c, KC_MODDOWN_LIFT);  // a class of its own: the profile shows which key switches take auxiliary primes
-        launch_chain(c, pick_lift_aux(a), dim3(tiles, ns, lift_zsplit((long)tiles * ns, (c->L + 3) / 4, 2, 148)), 4 * kLiftThreads, lift_aux_smem(R1, R2), A, c->crt, c->L);
+        const int zs = lift_zsplit((long)tiles * ns, (c->L + 3) / 4, 2, 148);
+        launch_chain(c, pick_lift_aux(a), dim3(tiles, ns, zs), 4 * kLiftThreads, lift_aux_smem(R1, R2), A, c->crt, c->L);
     }
     return check_launch(c, "ks_lift_aux");
 }
@@ -1329,8 +1329,9 @@ bool ntt_inv_pass_b_gathers(const hann_ctx* c, const void* src, const void* dst)
 }
 
 // The same with the input read from elsewhere: group g (lm.period polynomials, `stride` words apart) starts at
-// src + g * src_gstride (src_per > 0: at src + (g / src_per) * src_zstride + (g % src_per) * src_gstride); the output goes to data as above.  Only where ntt_inv_pass_b_gathers(c) holds and both pointers are
-// 16-byte aligned (the bulk-copy kernel); the caller copies and uses launch_ntt_inv_pass_b otherwise.
+// src + g * src_gstride (src_per > 0: at src + (g / src_per) * src_zstride + (g % src_per) * src_gstride); the output goes to data as
+// above.  Only where ntt_inv_pass_b_gathers(c) holds and both pointers are 16-byte aligned (the bulk-copy kernel); the caller copies
+// and uses launch_ntt_inv_pass_b otherwise.
 int launch_ntt_inv_pass_b_from(hann_ctx* c, const u64* src, int64_t src_gstride, u64* data, int64_t npoly, int64_t stride, const LimbMap& lm,
                                int64_t src_per, int64_t src_zstride) {
     return launch_ntt(c, data, npoly, stride, lm, true, true, src, src_gstride, false, src_per, src_zstride);
