@@ -152,8 +152,8 @@ int64_t balanced(int64_t most, int64_t total) {
 // whether a key-switch round goes through auxiliary primes: every one of its keys, of rotations rot0 + z * rot_zinc, has the words
 bool ks_aux(const hann_ctx* c, int rot0, int rot_zinc, int nz) {
     for (int z = 0; z < nz; z++)
-        if (!c->keyaux_host[rot0 + z * rot_zinc]) return false;
-    return c->aux;
+        if (!c->key_has_aux[rot0 + z * rot_zinc]) return false;
+    return true;
 }
 
 // the sub-buffers of a key-switch round (ks_round_fused, or ks_digits_to_lifted on smaller rings) on nz * items polynomials.  With
@@ -479,7 +479,7 @@ extern "C" int hann_ctx_create(const hann_params* prm, hann_ctx** out) {
               cudaHostGetDevicePointer((void**)&c->kflag, c->kflag_host, 0) == cudaSuccess &&
               cudaMalloc(&c->fft_T, nh * sizeof(double2)) == cudaSuccess && cudaMalloc(&c->fft_U, n * sizeof(double2)) == cudaSuccess &&
               cudaMalloc(&c->jinv, n * sizeof(int32_t)) == cudaSuccess && cudaMalloc(&c->galois_dev, n * sizeof(unsigned)) == cudaSuccess &&
-              cudaMalloc(&c->keytab_dev, n * sizeof(u64*)) == cudaSuccess && cudaMalloc(&c->keyaux_dev, n * sizeof(u64*)) == cudaSuccess;
+              cudaMalloc(&c->keytab_dev, n * sizeof(u64*)) == cudaSuccess;
     if (ok) {
         *c->kflag_host = 0;
         ok = cudaMemcpy(c->tw_fwd, twf.data(), twb, cudaMemcpyHostToDevice) == cudaSuccess &&
@@ -491,11 +491,11 @@ extern "C" int hann_ctx_create(const hann_params* prm, hann_ctx** out) {
              cudaMemcpy(c->fft_U, U.data(), n * sizeof(double2), cudaMemcpyHostToDevice) == cudaSuccess &&
              cudaMemcpy(c->jinv, jpos.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice) == cudaSuccess &&
              cudaMemcpy(c->galois_dev, gal.data(), n * sizeof(unsigned), cudaMemcpyHostToDevice) == cudaSuccess &&
-             cudaMemset(c->keytab_dev, 0, n * sizeof(u64*)) == cudaSuccess && cudaMemset(c->keyaux_dev, 0, n * sizeof(u64*)) == cudaSuccess;
+             cudaMemset(c->keytab_dev, 0, n * sizeof(u64*)) == cudaSuccess;
     }
     c->h_galois = gal;
     c->keytab_host.assign(n, nullptr);
-    c->keyaux_host.assign(n, nullptr);
+    c->key_has_aux.assign(n, 0);
     for (int k = 0; k < HANN_NKINDS && ok; k++)
         ok = cudaEventCreate(&c->ev[k][0]) == cudaSuccess && cudaEventCreate(&c->ev[k][1]) == cudaSuccess;
     if (ok)
@@ -536,12 +536,11 @@ extern "C" void hann_ctx_destroy(hann_ctx* c) {
     if (!c) return;
     DeviceGuard dg(c->device);
     cudaStreamSynchronize(c->stream);
-    for (const auto* tab : {&c->keytab_host, &c->keyaux_host})
-        for (u64* k : *tab)
-            if (k) cudaFree(k);
+    for (u64* k : c->keytab_host)
+        if (k) cudaFree(k);
     cudaFree(c->tw_fwd); cudaFree(c->tw_inv); cudaFree(c->tw_fwd_f64); cudaFree(c->tw_inv_f64); cudaFree(c->lt_dev);
     if (c->kflag_host) cudaFreeHost(c->kflag_host);
-    cudaFree(c->fft_T); cudaFree(c->fft_U); cudaFree(c->jinv); cudaFree(c->galois_dev); cudaFree(c->keytab_dev); cudaFree(c->keyaux_dev);
+    cudaFree(c->fft_T); cudaFree(c->fft_U); cudaFree(c->jinv); cudaFree(c->galois_dev); cudaFree(c->keytab_dev);
     if (c->scratch) cudaFree(c->scratch);
     host_copy_release(c);
     if (c->aux_stream) {
@@ -1173,20 +1172,22 @@ extern "C" int hann_decrypt_compact(hann_ctx* c, const int8_t* s, const uint64_t
 
 // ================================================================================================ server side
 
-// one key of rotation r: into the buffers that the context has for it, or into new ones, which it gets when the key is complete
+// one key of rotation r: into the buffer that the context has for it, or into a new one, which it gets when the key is complete
 static int load_key(hann_ctx* c, const uint64_t* evk, int r) {
     const int L = c->L, N = c->N;
     const int64_t keyw = (int64_t)L * 2 * (L + 1) * N, auxw = (int64_t)L * 2 * kAux * N;
-    u64 *tmp = (u64*)c->scratch, *buf = c->keytab_host[r], *aux = c->keyaux_host[r];
+    u64 *tmp = (u64*)c->scratch, *buf = c->keytab_host[r];
+    // The rounds that take auxiliary primes switch the giant steps (multiples of B), relinearise (0) or fold; the keys of the hoisted
+    // rotations do without their words.  Where the device has no room for them the key switch takes p itself, with the same bits.
+    bool aux = buf ? c->key_has_aux[r] != 0 : c->aux && r % c->B == 0;
+    if (!buf && aux && cudaMalloc(&buf, (keyw + auxw) * 8) != cudaSuccess) {
+        cudaGetLastError();
+        buf = nullptr;
+        aux = false;
+    }
     if (!buf && cudaMalloc(&buf, keyw * 8) != cudaSuccess) {
         cudaGetLastError();
         return fail(c, HANN_ENOMEM, "hann_load_keys: device allocation failed");
-    }
-    // The rounds that take auxiliary primes switch the giant steps (multiples of B), relinearise (0) or fold; the keys of the hoisted
-    // rotations do without their words.  Where the device has no room for them the key switch takes p itself, with the same bits.
-    if (c->aux && r % c->B == 0 && !aux && cudaMalloc(&aux, auxw * 8) != cudaSuccess) {
-        cudaGetLastError();
-        aux = nullptr;
     }
     auto fill = [&]() -> int {
         CK(cudaMemcpyAsync(tmp, evk, keyw * 8, cudaMemcpyDefault, c->stream));
@@ -1199,7 +1200,7 @@ static int load_key(hann_ctx* c, const uint64_t* evk, int r) {
             for (int k = 0; k < kAux; k++) lm.limb[k] = c->crt.limb[k];
             RET(launch_key_aux(c, tmp, buf));  // 6 L N words of the 2 L (L + 1) N that are written below
             RET(launch_ntt_fwd(c, buf, (int64_t)L * 2 * kAux, N, lm));
-            RET(launch_permute(c, buf, aux, auxw / N, kinv));
+            RET(launch_permute(c, buf, buf + keyw, auxw / N, kinv));
         }
         RET(launch_ntt_fwd(c, tmp, (int64_t)L * 2 * (L + 1), N, limbmap_qp(c)));
         RET(launch_permute(c, tmp, buf, keyw / N, kinv));
@@ -1208,11 +1209,10 @@ static int load_key(hann_ctx* c, const uint64_t* evk, int r) {
     const int rc = fill();
     if (rc != HANN_OK) {
         if (buf != c->keytab_host[r]) cudaFree(buf);
-        if (aux && aux != c->keyaux_host[r]) cudaFree(aux);
         return rc;
     }
     c->keytab_host[r] = buf;
-    c->keyaux_host[r] = aux;
+    c->key_has_aux[r] = aux;
     return HANN_OK;
 }
 
@@ -1227,9 +1227,8 @@ extern "C" int hann_load_keys(hann_ctx* c, const uint64_t* evk, int n_rot, const
     RET(ensure_scratch(c, keyw * 8));
     int rc = HANN_OK;
     for (int i = 0; i < n_rot && rc == HANN_OK; i++) rc = load_key(c, evk + (int64_t)i * keyw, rot[i]);
-    // the keys before one that could not be loaded count: the kernels' tables say what the host's do
+    // the keys before one that could not be loaded count: the kernels' table says what the host's does
     CK(cudaMemcpy(c->keytab_dev, c->keytab_host.data(), c->keytab_host.size() * sizeof(u64*), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(c->keyaux_dev, c->keyaux_host.data(), c->keyaux_host.size() * sizeof(u64*), cudaMemcpyHostToDevice));
     return rc;
 }
 

@@ -73,13 +73,12 @@ struct hann_ctx {
     unsigned* galois_dev = nullptr;  // [n] 5^r mod 2N
     std::vector<unsigned> h_galois;
     // evaluation keys by rotation: device buffers [L][2][L+1][N], transformed and permuted by the inverse
-    // automorphism so that the key-switch inner product reads keys and digits contiguously
-    std::vector<u64*> keytab_host;
-    u64** keytab_dev = nullptr;  // [n] device copy of keytab_host
-    // auxiliary words of a key, [L][2][3][N]: the residues modulo p lifted (centred) to the auxiliary primes.  Only rotations that are
+    // automorphism so that the key-switch inner product reads keys and digits contiguously; followed by the auxiliary words
+    // [L][2][3][N], the residues modulo p lifted (centred) to the auxiliary primes, where key_has_aux says so.  Only rotations that are
     // multiples of B have them (hann_load_keys); a key switch one of whose keys has none takes p itself
-    std::vector<u64*> keyaux_host;
-    u64** keyaux_dev = nullptr;  // [n] device copy of keyaux_host
+    std::vector<u64*> keytab_host;
+    std::vector<char> key_has_aux;
+    u64** keytab_dev = nullptr;  // [n] device copy of keytab_host
     // growable device scratch of the exchange and client calls (never used by the server-side scoring calls)
     void* scratch = nullptr;
     int64_t scratch_bytes = 0;

@@ -127,7 +127,7 @@ struct ApplyArgs {
                         // auxiliary primes none for the special prime either
     int nx;             // 1, or the number of auxiliary primes that stand for the special prime
     u64 aux4;           // their limbs in 4-bit fields, behind them the other limbs
-    const u64* const* keyaux;  // and their words of every key
+    long long aux_key;  // and the offset of their words in a key
     const u64* own;     // the polynomials being switched, transform domain: own + item * own_it + z * own_z + j * N (or null)
     long long own_it, own_z;
     const u64* const* keytab;
@@ -194,9 +194,9 @@ __global__ void __launch_bounds__(T, 640 / T) k_ks_apply(ApplyArgs A) {
                            : A.digits + (((z * A.items + it0 + it) * L + dj) * A.n_tgt + (!A.own || i < dj ? i : i - 1)) * N;
         p += (sc << 8);
         if (z) __syncthreads();  // the products of the previous rotation have been taken
-        const int r = A.rot0 + z * A.rot_zinc;
-        if (SHARE || !aux) stage_keys(ks, A.keytab[r] + (long long)i * N + (sc << 8), (long long)(L + 1) * N, L);
-        if (aux) stage_keys(ks + ks2, A.keyaux[r] + (long long)y * N + (sc << 8), (long long)kAux * N, L);
+        const u64* key = A.keytab[A.rot0 + z * A.rot_zinc] + (sc << 8);
+        if (SHARE || !aux) stage_keys(ks, key + (long long)i * N, (long long)(L + 1) * N, L);
+        if (aux) stage_keys(ks + ks2, key + A.aux_key + (long long)y * N, (long long)kAux * N, L);
         if (staged != sc) {
             if (f64) stage_twiddles(tc, (const double2*)A.tw_fwd_f64 + ((size_t)i << A.logN), m0 + sc);
             else stage_twiddles((ulonglong2*)tc, (const ulonglong2*)A.tw_fwd_int + ((size_t)i << A.logN), m0 + sc);
@@ -672,7 +672,7 @@ int launch_ks_apply(hann_ctx* c, const u64* digits, const u64* own, int64_t own_
     for (int k = 0; k < kAux; k++) A.aux4 |= (u64)c->crt.limb[k] << (4 * k);
     for (int l = 0, k = kAux; aux && l < c->L; l++)
         if (l != c->crt.limb[0] && l != c->crt.limb[1] && l != c->crt.limb[2]) A.aux4 |= (u64)l << (4 * k++);
-    A.keyaux = c->keyaux_dev;
+    A.aux_key = (long long)c->L * 2 * (c->L + 1) * c->N;
     A.n_tgt = aux ? c->L - 1 : own ? c->L : c->L + 1;
     A.own = own;
     A.own_it = own_it;
