@@ -248,9 +248,10 @@ int hann_decrypt_compact(hann_ctx *ctx, const int8_t *s, const uint64_t *ct, int
  * device pointer) into the context, replacing keys with the same rotation.  Allocates device memory owned by the
  * context: 2 L (L + 1) polynomials of one limb per key, and for rotations that are multiples of B (0 among them) 6 L more
  * where the key switch has auxiliary primes (rings of 2^10 points and more, L <= 4 or L N <= 2^17, three ciphertext primes
- * below 2^50 of about the same size and a special prime in [2^50, 2^61)) and the device has room for them; a key without them works all the same, to
- * the same bits.  Staged through the exchange scratch.  Where a key cannot be loaded, those before it in the list stay
- * loaded.  Needed later: rotations 1..B-1 for hann_query_prepare, rotation B for hann_rotate_sum. */
+ * below 2^50, the largest less than six times the smallest, and a special prime in [2^50, 2^61)) and the device has room
+ * for them; a key without them works all the same, to the same bits.  Staged through the exchange scratch.  Where a key
+ * cannot be loaded, those before it in the list stay loaded.  Needed later: rotations 1..B-1 for hann_query_prepare,
+ * rotation B for hann_rotate_sum. */
 int hann_load_keys(hann_ctx *ctx, const uint64_t *evk, int n_rot, const int32_t *rot);
 
 /* Once per query (Sec. 3.1 Detail: the baby steps of the diagonal method; Sec. 3.4: the rotated query is computed
