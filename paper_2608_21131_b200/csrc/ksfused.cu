@@ -8,6 +8,8 @@
 // position 16 a + b is kept at word 16 a + (b ^ a), which both rounds and the word-by-word passes reach without bank conflicts
 // (swz).  An automorphism maps every chunk of 256 positions onto one chunk, so a CTA that owns a chunk of the result reads
 // one chunk of every source and permutes inside it.
+#include <algorithm>
+
 #include "internal.h"
 #include "debugcheck.cuh"
 #include "nttcore.cuh"
@@ -737,12 +739,15 @@ int launch_ks_hoist(hann_ctx* c, const u64* digits, const u64* own, int64_t item
     A.tw_inv_f64 = c->tw_inv_f64;
     A.tw_inv_int = c->tw_inv;
     A.lt = c->lt_dev;
-    // CTAs that share out the items of a chunk: smallest (waves x items of a CTA, the digits counting as two), ties to fewer
+    // CTAs that share out the items of a chunk: smallest (waves x items of a CTA, the digits counting as two), ties to fewer; no less
+    // than the CTAs of the special prime take, an item of which is two (products and inverse passes).  Without that bound a launch below
+    // one wave took one CTA a chunk and lasted as long as those (us of a level of 1000 rows, L = 2, R = 128, B = 32, 1 / 2 / 3 / 4 / 8 CTAs:
+    // N = 2^15 293 / 260 / 265 / 264 / 274, N = 2^14 198 / 184 / 182 / 180 / 185; L = 4, N = 2^16, five waves: 692 / 695 / 706 / 711 / 755).
     const long per = (long)(c->N >> 8) * (c->L + 1), slots = 148 * 3;
     int gz = 1;
     long best = -1;
     for (int z = 1; z <= items && z <= 64; z++) {
-        const long cost = ((per * z + slots - 1) / slots) * (2 + (items + z - 1) / z);
+        const long n = (items + z - 1) / z, cost = std::max(((per * z + slots - 1) / slots) * (2 + n), 2 + 2 * n);
         if (best < 0 || cost < best) {
             best = cost;
             gz = z;
